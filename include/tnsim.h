@@ -301,7 +301,8 @@ tnsim_status tnsim_set_jacobi_config(tnsim_mps* m, int32_t cfg);
 tnsim_status tnsim_set_wait_limits(tnsim_mps* m, int64_t jacobi_idle_polls, int64_t mbarrier_polls);
 
 /* Process-wide cap on the device memory held by the states of this library (0 = no cap,
- * the default).  tnsim_mps_create computes every device allocation of the new state
+ * the default).  complex128 states made under a cap leave out the buffers of the SVD's FP32
+ * preconditioner (the same results, more slowly).  tnsim_mps_create computes every device allocation of the new state
  * before making any, and returns ENOMEM, allocating nothing, when the bytes already held
  * plus the new state's would exceed the cap.  Errors: EINVAL (negative bytes). */
 tnsim_status tnsim_set_device_memory_cap(int64_t bytes);
@@ -367,7 +368,9 @@ tnsim_status tnsim_grad(const tnsim_circuit* c, const double* theta, const tnsim
  * on m (then reset).  visit_rows and rotation_rows weight every examined / rotated
  * column pair by its column length m = 2 chi_L, so the Jacobi SVD's arithmetic is
  * 8 visit_rows + 20 rotation_rows real flops (FMA = 2): an examined pair forms
- * g = x_i^H x_j, the column norms being tracked, and a rotation updates both columns. */
+ * g = x_i^H x_j, the column norms being tracked, and a rotation updates both columns.
+ * For complex128 the sweeps, rotations and pairs are those of the FP64 iteration; the
+ * FP32 sweeps of its preconditioner are not counted. */
 typedef struct {
     int64_t gates;         /* two-qubit gates applied */
     int64_t sweeps;        /* Jacobi sweeps, summed over gates */

@@ -28,8 +28,7 @@ __device__ __forceinline__ void rr_pair(int P, int r, int v, int& a, int& b) {
 // c^2 + s^2 = 1 -- use correctly rounded square roots and reciprocals (sqrtf,
 // __frcp_rn), so their rounding errors are unbiased; the skip test and the angle t
 // (which only has to orthogonalise the pair to within rounding) use fast division.
-// c - 1 = -t^2 / (rr (1 + rr)) is formed without cancellation.  FP64 keeps IEEE
-// operations throughout.
+// c - 1 = -t^2 / (rr (1 + rr)) is formed without cancellation.
 __device__ __forceinline__ bool rot_params_fast(float a, float b, float gr, float gi, float tol2, float zthr,
                                                 float& cm1, float& sr, float& si, float& tg) {
     const float g2 = gr * gr + gi * gi;
@@ -50,19 +49,60 @@ __device__ __forceinline__ bool rot_params_fast(float a, float b, float gr, floa
     tg = t * gabs;                                        // the norms become a - t|g|, b + t|g|
     return true;
 }
-__device__ __forceinline__ bool rot_params_fast(double a, double b, double gr, double gi, double tol2, double zthr,
-                                                double& cm1, double& sr, double& si, double& tg) {
-    const double g2 = gr * gr + gi * gi;
-    if (!(a > zthr && b > zthr && g2 / b > tol2 * a)) return false;
-    const double gabs = sqrt(g2);
-    const double zeta = (b - a) / (2 * gabs);
-    const double t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-    const double rr = sqrt(1.0 + t * t);
-    cm1 = -(t * t) / (rr * (1.0 + rr));
-    const double sv = t / rr;
-    sr = sv * (gr / gabs);
-    si = sv * (gi / gabs);
-    tg = t * gabs;
+// x 2^-e in FP32 (truncated) and back, by integer operations: FP64 instructions, the
+// conversions among them, issue once in 64 cycles per scheduler.
+__device__ __forceinline__ float f32_scaled(double x, int e) {
+    const int hi = __double2hiint(x), ex = ((hi >> 20) & 0x7ff) - 1023 - e + 127;
+    if (ex <= 0) return 0.f;
+    const unsigned mant = ((unsigned)(hi & 0xfffff) << 3) | ((unsigned)__double2loint(x) >> 29);
+    return __uint_as_float(((unsigned)hi & 0x80000000u) | ((unsigned)min(ex, 254) << 23) | mant);
+}
+__device__ __forceinline__ double f64_scaled(float x, int e) {
+    const unsigned b = __float_as_uint(x);
+    const int ex = (int)((b >> 23) & 0xff) - 127 + 1023 + e;
+    if (!(b & 0x7f800000u) || ex <= 0) return 0.0;
+    return __hiloint2double((int)((b & 0x80000000u) | ((unsigned)min(ex, 2046) << 20) | ((b & 0x7fffffu) >> 3)),
+                            (int)(b << 29));
+}
+// FP64: the test and a first tau in FP32 on values scaled by the larger norm's power of two;
+// one Newton step for tau (without it a gate took 0.6 sweeps more) and the quantities that
+// make the rotation unitary in FP64: 15 FP64 instructions while t < 2^-10 (where c - 1 is
+// its series), against about 150 with FP64 square roots and divisions.
+__device__ __forceinline__ bool rot_params64(double a, double b, double gr, double gi, float tol, double zthr,
+                                             double& cm1, double& sr, double& si, double& tg) {
+    const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b), iz = __double_as_longlong(zthr);
+    if (!(ia > iz && ib > iz)) return false;              // zthr >= 0: ordered like the values
+    const int e = (int)((max(ia, ib) >> 52) & 0x7ff) - 1023;
+    const float xr = fabsf(f32_scaled(gr, e)), xi = fabsf(f32_scaled(gi, e));
+    const float mx = fmaxf(xr, xi);
+    if (!(mx > 0.f)) return false;
+    const float r = __fdividef(fminf(xr, xi), mx);
+    const float gm = mx * sqrtf(fmaf(r, r, 1.f));
+    if (!(gm > tol * sqrtf(f32_scaled(a, e) * f32_scaled(b, e)))) return false;
+    const double d = b - a;
+    const float df = f32_scaled(d, e);
+    const float tauf = __fdividef(2.f, fabsf(df) + sqrtf(fmaf(df, df, 4.f * gm * gm)));
+    double tau = f64_scaled(copysignf(tauf, df), -e);
+    const double g2 = fma(gr, gr, gi * gi);
+    // one Newton step on |g|^2 tau^2 + d tau = 1, its slope sqrt(d^2 + 4 |g|^2) in FP32
+    const float slope = copysignf(__fdividef(1.f, sqrtf(fmaf(df, df, 4.f * gm * gm))), df);
+    tau = fma(-fma(tau, fma(tau, g2, d), -1.0), f64_scaled(slope, -e), tau);
+    tg = tau * g2;
+    const double t2 = tg * tau;
+    if (__double2hiint(t2) < 0x3eb00000) {                // t^2 < 2^-20: the next term is below 2^-61
+        cm1 = t2 * fma(0.375, t2, -0.5);
+    } else {
+        const double c = rsqrt(1.0 + t2);
+        // 1 / (1 + c) by two Newton steps from FP32
+        const double h = 1.0 + c;
+        double ih = (double)__frcp_rn((float)h);
+        ih = fma(ih, fma(-h, ih, 1.0), ih);
+        ih = fma(ih, fma(-h, ih, 1.0), ih);
+        cm1 = -(t2 * c) * c * ih;
+    }
+    const double f = fma(tau, cm1, tau);
+    sr = f * gr;
+    si = f * gi;
     return true;
 }
 

@@ -1,0 +1,410 @@
+// FP64 products of the two-qubit update, and the mixed-precision preconditioner of the
+// complex128 SVD.
+//
+// GB300 issues FP64 at 1/64 of the FP32 rate, so an FP64 kernel's time is its FP64
+// instruction count over the SMs that it keeps busy, and everything else hides behind
+// it.  The products therefore use small tiles (16 x 16 complex, 64 threads): with 64 x 64
+// tiles one SM per gate did the work at m = n <= 64 (theta 88 -> 23 us, right site
+// 136 -> 28 us per layer of 4-5 gates; 20 gates at m = 180: 480 -> 370 and 790 -> 420 us).
+//
+// Preconditioner (mixed-precision Jacobi SVD: Gao, Ma and Shao 2022).  One-sided Jacobi
+// converges quadratically, so 9 of its ~12 FP64 sweeps only bring the columns from O(1)
+// to ~1e-6 of orthogonal, which FP32 can do at 64 times the rate:
+//   k_mix_build  [theta; I] in FP32 (theta scaled by a power of two to |theta|_F in [1, 2));
+//   k_jacobi     FP32 Jacobi rotations of these columns until theta V is orthogonal to
+//                kMixTol; the lower n rows become V (k_jacobi.cu, EXT);
+//   k_mix_gram   E = I - V^H V in FP64 (V is unitary to ~1e-6 only);
+//   k_mix_corr   F = E/2 + 3/8 E^2, so that V (I + F) = V (V^H V)^{-1/2} + O(E^3) is
+//                unitary to FP64 rounding (E^2 ~ 1e-12 needs four digits: FP32);
+//   k_mix_mul    X = W V, then W <- X + X F, both in FP64.
+// The FP64 Jacobi iteration then starts from W V' with V' unitary: the same SVD to the
+// same tolerance, with fewer sweeps and mostly tiny rotations.  A preconditioner that did
+// not converge or lost small columns to FP32 rounding only costs sweeps.
+// Measured with the FP64 visit of k_jacobi.cu on 20 gates at m = n = 180: SVD 139 -> 29 ms
+// (12.2 -> 4.7 FP64 sweeps per gate; of the 29 ms, FP32 rotations 4.4, these products 2.1);
+// singular values 6e-16 (relative) from LAPACK's before and after.
+#include "tnsim_internal.h"
+
+namespace tnsim {
+
+namespace {
+
+constexpr int GT = 16;             // tile edge and K step
+constexpr int GTHREADS = 64;       // 2 x 2 outputs per thread
+
+// acc += a b
+template <typename C>
+__device__ __forceinline__ void cmul_add(C& acc, const C& a, const C& b) {
+    acc.x = fma(a.x, b.x, acc.x);
+    acc.x = fma(-a.y, b.y, acc.x);
+    acc.y = fma(a.x, b.y, acc.y);
+    acc.y = fma(a.y, b.x, acc.y);
+}
+
+// 16 x 16 tile added to acc: A B over k < K, each K step summed by itself first (rounding
+// grows with sqrt(16 + K / 16) instead of sqrt(K), for 3 % more instructions): thread (rx, cy) holds rows ROW(rx, 0/1), columns cy and
+// cy + 8, with ROW(rx, i) = rx + 8 i, or 2 rx + i (PAIRED).  la(i, k) and lb(k, j) give the
+// operands' elements (zero outside them) for tile row i and tile column j; AK / BK: memory
+// runs along k (consecutive threads then load consecutive k).
+template <typename C, bool AK, bool BK, bool PAIRED, typename LA, typename LB>
+__device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[2][2]) {
+    __shared__ C As[GT][GT + 1], Bs[GT][GT + 1];
+    const int tid = threadIdx.x, rx = tid & 7, cy = tid >> 3;
+    for (int k0 = 0; k0 < K; k0 += GT) {
+#pragma unroll
+        for (int t = 0; t < GT * GT / GTHREADS; ++t) {
+            const int e = tid + GTHREADS * t, lo = e & (GT - 1), hi = e / GT;
+            C a, b;
+            a.x = a.y = b.x = b.y = 0;
+            if (k0 + (AK ? lo : hi) < K) a = la(AK ? hi : lo, k0 + (AK ? lo : hi));
+            if (k0 + (BK ? lo : hi) < K) b = lb(k0 + (BK ? lo : hi), BK ? hi : lo);
+            As[AK ? lo : hi][AK ? hi : lo] = a;
+            Bs[BK ? lo : hi][BK ? hi : lo] = b;
+        }
+        __syncthreads();
+        C part[2][2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) { part[i][j].x = 0; part[i][j].y = 0; }
+#pragma unroll 4
+        for (int kk = 0; kk < GT; ++kk) {
+            C a[2], b[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                a[i] = As[kk][PAIRED ? 2 * rx + i : rx + 8 * i];
+                b[i] = Bs[kk][cy + 8 * i];
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) cmul_add(part[i][j], a[i], b[j]);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) { acc[i][j].x += part[i][j].x; acc[i][j].y += part[i][j].y; }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// theta (see k_gemm.cu): 8 l x 8 r per CTA; tile rows (l, c), tile columns (d, r).
+__global__ void __launch_bounds__(GTHREADS) k_theta64(const GateDesc* __restrict__ gd) {
+    const GateDesc& d = gd[blockIdx.z];
+    const int q = d.q;
+    const int chiL = d.chi[q], chiM = d.chi[q + 1], chiR = d.chi[q + 2];
+    const int l0 = blockIdx.x * 8, r0 = blockIdx.y * 8;
+    if (l0 >= chiL || r0 >= chiR) return;
+    __shared__ double2 Gs[16];
+    const int tid = threadIdx.x, rx = tid & 7, cy = tid >> 3;
+    if (tid < 16) {
+        const int o = tid >> 2, i = tid & 3;
+        double re = 0.0, im = 0.0;
+        for (int j = 0; j < 4; ++j) {
+            const double gr = d.g4[2 * (o * 4 + j)], gi = d.g4[2 * (o * 4 + j) + 1];
+            // K[j][i] = uL[j>>1][i>>1] * uR[j&1][i&1]
+            double ar = ((j >> 1) == (i >> 1)) ? 1.0 : 0.0, ai = 0.0;
+            double br = ((j & 1) == (i & 1)) ? 1.0 : 0.0, bi = 0.0;
+            if (d.uL) { ar = d.uL[2 * ((j >> 1) * 2 + (i >> 1))]; ai = d.uL[2 * ((j >> 1) * 2 + (i >> 1)) + 1]; }
+            if (d.uR) { br = d.uR[2 * ((j & 1) * 2 + (i & 1))]; bi = d.uR[2 * ((j & 1) * 2 + (i & 1)) + 1]; }
+            const double kr = ar * br - ai * bi, ki = ar * bi + ai * br;
+            re += gr * kr - gi * ki;
+            im += gr * ki + gi * kr;
+        }
+        Gs[tid] = make_double2(re, im);
+    }
+    const double2* A = (const double2*)d.siteA;
+    const double2* B = (const double2*)d.siteB;
+    const int m = 2 * chiL;
+    double2 acc[2][2] = {};
+    tile_product<double2, true, false, true>(
+        chiM,
+        [&](int i, int k) {
+            const int row = 2 * l0 + i;
+            return row < m ? A[(size_t)row * chiM + k] : make_double2(0.0, 0.0);
+        },
+        [&](int k, int j) {
+            const int r = r0 + (j & 7);
+            return r < chiR ? B[((size_t)k * 2 + (j >> 3)) * chiR + r] : make_double2(0.0, 0.0);
+        },
+        acc);
+    double2* Wm = (double2*)d.W;
+    double2* T0 = (double2*)d.theta0;
+    double fro = 0.0;
+    const int l = l0 + rx, r = r0 + cy;
+    if (l < chiL && r < chiR) {
+#pragma unroll
+        for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+            for (int aa = 0; aa < 2; ++aa) {
+                double2 t = make_double2(0.0, 0.0);
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) cmul_add(t, Gs[(2 * aa + bb) * 4 + 2 * c + e], acc[c][e]);
+                const size_t idx = (size_t)(bb * chiR + r) * m + 2 * l + aa;
+                Wm[idx] = t;
+                T0[idx] = t;
+                fro = fma(t.x, t.x, fma(t.y, t.y, fro));
+            }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, o);
+    if ((tid & 31) == 0 && fro != 0.0) atomicAdd(&d.out->frob2, fro);
+}
+
+// right site (see k_right in k_gemm.cu): R[j, col] = f_j sum_row conj(W[row, perm_j]) theta0[row, col]
+__global__ void __launch_bounds__(GTHREADS) k_right64(const GateDesc* __restrict__ gd) {
+    const GateDesc& d = gd[blockIdx.z];
+    const int q = d.q;
+    const int m = 2 * d.chi[q], n = 2 * d.chi[q + 2], k = d.out->k;
+    if (qr_active(d, m, n)) return;   // QR-preconditioned: k_right_pre (k_qr.cu)
+    const int c0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+    if (c0 >= n || j0 >= k) return;
+    __shared__ int pj[GT];
+    __shared__ double fj[GT];
+    const int tid = threadIdx.x;
+    if (tid < GT) {
+        const int j = j0 + tid;
+        const double s2j = j < k ? d.s2[j] : 0.0;
+        pj[tid] = j < k ? d.perm[j] : -1;
+        if (d.canon) fj[tid] = s2j > 0.0 ? 1.0 / s2j : 0.0;
+        else fj[tid] = s2j > 0.0 ? d.out->scale / sqrt(s2j) : 0.0;
+    }
+    __syncthreads();
+    const double2* Wm = (const double2*)d.W;
+    const double2* T0 = (const double2*)d.theta0;
+    const int lk = d.canon ? *d.lam_k : 0;
+    double2 acc[2][2] = {};
+    // tile rows: columns of R (they run along its rows in memory); tile columns: rows j
+    tile_product<double2, true, true, false>(
+        m,
+        [&](int i, int row) {
+            if (c0 + i >= n) return make_double2(0.0, 0.0);
+            double2 w = T0[(size_t)(c0 + i) * m + row];
+            if ((row >> 1) < lk) {
+                const double f = d.lam[row >> 1];
+                w.x *= f;
+                w.y *= f;
+            }
+            return w;
+        },
+        [&](int row, int j) {
+            if (pj[j] < 0) return make_double2(0.0, 0.0);
+            const double2 v = Wm[(size_t)pj[j] * m + row];
+            return make_double2(v.x, -v.y);
+        },
+        acc);
+    double2* R = (double2*)d.siteB;
+    const int rx = tid & 7, cy = tid >> 3;
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int jj = cy + 8 * j, col = c0 + rx + 8 * i;
+            if (j0 + jj < k && col < n)
+                R[(size_t)(j0 + jj) * n + col] = make_double2(acc[i][j].x * fj[jj], acc[i][j].y * fj[jj]);
+        }
+}
+
+// ---------------------------------------------------------------------------
+// the preconditioner
+
+__device__ __forceinline__ bool mix_active(const GateDesc& d, int m, int n) {
+    return d.pre && n >= kMixMinCols && m + n <= kMixMaxRows;
+}
+
+// [theta; I] in FP32; a gate outside the preconditioner counts as finished in its launch
+__global__ void __launch_bounds__(256) k_mix_build(const GateDesc* __restrict__ gd, JacobiCtl* __restrict__ ctl) {
+    const GateDesc& d = gd[blockIdx.y];
+    const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
+    if (!mix_active(d, m, n)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            d.out->finished = 1;
+            atomicAdd(&ctl->n_finished, 1);
+        }
+        return;
+    }
+    const int mt = m + n;
+    const double f = mix_scale(d.out->frob2);
+    const double2* Wm = (const double2*)d.W;
+    float2* Y = (float2*)d.pre;
+    const int total = mt * n;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        const int c = t / mt, r = t - c * mt;
+        float2 y;
+        if (r < m) {
+            const double2 w = Wm[(size_t)c * m + r];
+            y = make_float2((float)(w.x * f), (float)(w.y * f));
+        } else {
+            y = make_float2(r - m == c ? 1.f : 0.f, 0.f);
+        }
+        Y[t] = y;
+    }
+}
+
+// E = I - V^H V (Hermitian: tiles on and above the diagonal, mirrored).  The first CTA of
+// a gate also readies its record for the FP64 launch: a sweep cap reached in FP32 is no
+// error, a timeout is.
+__global__ void __launch_bounds__(GTHREADS) k_mix_gram(const GateDesc* __restrict__ gd) {
+    const GateDesc& d = gd[blockIdx.z];
+    const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        GateOut* o = d.out;
+        if (!o->finished) o->status = 5;
+        else if (o->status == 4) o->status = 0;
+        o->finished = 0;
+        o->done = 0;
+        o->rot_sweep = 0;
+        o->claim = 0;
+    }
+    if (!mix_active(d, m, n)) return;
+    const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+    if (i0 >= n || j0 >= n || i0 > j0) return;
+    const int mt = m + n;
+    const float2* V = (const float2*)d.pre + m;
+    double2* E = (double2*)d.pre_x;
+    // the diagonal sums start from -1: they end near 0, and the last roundings are small
+    double2 acc[2][2] = {};
+    if (i0 == j0 && (threadIdx.x & 7) == (threadIdx.x >> 3)) acc[0][0].x = acc[1][1].x = -1.0;
+    tile_product<double2, true, true, false>(
+        n,
+        [&](int i, int k) {
+            if (i0 + i >= n) return make_double2(0.0, 0.0);
+            const float2 v = V[(size_t)(i0 + i) * mt + k];
+            return make_double2((double)v.x, -(double)v.y);
+        },
+        [&](int k, int j) {
+            if (j0 + j >= n) return make_double2(0.0, 0.0);
+            const float2 v = V[(size_t)(j0 + j) * mt + k];
+            return make_double2((double)v.x, (double)v.y);
+        },
+        acc);
+    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
+#pragma unroll
+    for (int jj = 0; jj < 2; ++jj)
+#pragma unroll
+        for (int ii = 0; ii < 2; ++ii) {
+            const int i = i0 + rx + 8 * ii, j = j0 + cy + 8 * jj;
+            if (i >= n || j >= n) continue;
+            const double re = -acc[ii][jj].x, im = -acc[ii][jj].y;
+            E[(size_t)j * n + i] = make_double2(re, im);
+            if (i0 != j0) E[(size_t)i * n + j] = make_double2(re, -im);
+        }
+}
+
+// F = E/2 + 3/8 E^2 (Hermitian)
+__global__ void __launch_bounds__(GTHREADS) k_mix_corr(const GateDesc* __restrict__ gd) {
+    const GateDesc& d = gd[blockIdx.z];
+    const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
+    if (!mix_active(d, m, n)) return;
+    const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+    if (i0 >= n || j0 >= n || i0 > j0) return;
+    const double2* E = (const double2*)d.pre_x;
+    double2* F = (double2*)d.pre_f;
+    float2 acc[2][2] = {};
+    tile_product<float2, true, true, false>(
+        n,
+        [&](int i, int k) {   // E[i, k] = conj(E[k, i])
+            if (i0 + i >= n) return make_float2(0.f, 0.f);
+            const double2 e = E[(size_t)(i0 + i) * n + k];
+            return make_float2((float)e.x, -(float)e.y);
+        },
+        [&](int k, int j) {
+            if (j0 + j >= n) return make_float2(0.f, 0.f);
+            const double2 e = E[(size_t)(j0 + j) * n + k];
+            return make_float2((float)e.x, (float)e.y);
+        },
+        acc);
+    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
+#pragma unroll
+    for (int jj = 0; jj < 2; ++jj)
+#pragma unroll
+        for (int ii = 0; ii < 2; ++ii) {
+            const int i = i0 + rx + 8 * ii, j = j0 + cy + 8 * jj;
+            if (i >= n || j >= n) continue;
+            const double2 e = E[(size_t)j * n + i];
+            const double re = fma(0.375, (double)acc[ii][jj].x, 0.5 * e.x);
+            const double im = fma(0.375, (double)acc[ii][jj].y, 0.5 * e.y);
+            F[(size_t)j * n + i] = make_double2(re, im);
+            if (i0 != j0) F[(size_t)i * n + j] = make_double2(re, -im);
+        }
+}
+
+// FIRST: X = W V; else W = X + X F
+template <bool FIRST>
+__global__ void __launch_bounds__(GTHREADS) k_mix_mul(const GateDesc* __restrict__ gd) {
+    const GateDesc& d = gd[blockIdx.z];
+    const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
+    if (!mix_active(d, m, n)) return;
+    const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+    if (i0 >= m || j0 >= n) return;
+    const int mt = m + n;
+    double2* X = (double2*)d.pre_x;
+    double2* Wm = (double2*)d.W;
+    const double2* A = FIRST ? Wm : X;
+    double2 acc[2][2] = {};
+    tile_product<double2, false, true, false>(
+        n,
+        [&](int i, int k) { return i0 + i < m ? A[(size_t)k * m + i0 + i] : make_double2(0.0, 0.0); },
+        [&](int k, int j) {
+            if (j0 + j >= n) return make_double2(0.0, 0.0);
+            if (!FIRST) return ((const double2*)d.pre_f)[(size_t)(j0 + j) * n + k];
+            const float2 v = ((const float2*)d.pre)[(size_t)(j0 + j) * mt + m + k];
+            return make_double2((double)v.x, (double)v.y);
+        },
+        acc);
+    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
+#pragma unroll
+    for (int jj = 0; jj < 2; ++jj)
+#pragma unroll
+        for (int ii = 0; ii < 2; ++ii) {
+            const int i = i0 + rx + 8 * ii, j = j0 + cy + 8 * jj;
+            if (i >= m || j >= n) continue;
+            const size_t idx = (size_t)j * m + i;
+            if (FIRST) {
+                X[idx] = acc[ii][jj];
+            } else {
+                const double2 x = X[idx];
+                Wm[idx] = make_double2(x.x + acc[ii][jj].x, x.y + acc[ii][jj].y);
+            }
+        }
+}
+
+}  // namespace
+
+cudaError_t launch_theta64(const GateDesc* d, int n_gates, int chiL_max, int chiR_max, cudaStream_t s) {
+    if (n_gates <= 0) return cudaSuccess;
+    dim3 grid((chiL_max + 7) / 8, (chiR_max + 7) / 8, n_gates);
+    k_theta64<<<grid, GTHREADS, 0, s>>>(d);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_right64(const GateDesc* d, int n_gates, int k_max, int n_max, cudaStream_t s) {
+    if (n_gates <= 0) return cudaSuccess;
+    dim3 grid((n_max + GT - 1) / GT, (k_max + GT - 1) / GT, n_gates);
+    k_right64<<<grid, GTHREADS, 0, s>>>(d);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, JacobiCtl* ctl, cudaStream_t s,
+                       int n_lead, unsigned spin_limit) {
+    if (n_gates <= 0 || n_max < kMixMinCols) return cudaSuccess;
+    const int mt = m_max + n_max < kMixMaxRows ? m_max + n_max : kMixMaxRows;   // of an active gate
+    const int mm = m_max < kMixMaxRows ? m_max : kMixMaxRows, nm = n_max < kMixMaxRows ? n_max : kMixMaxRows;
+    int bx = (int)(((long long)mt * nm + 1023) / 1024);
+    if (bx > 128) bx = 128;
+    k_mix_build<<<dim3(bx, n_gates), 256, 0, s>>>(d, ctl);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_jacobi_mix(d, n_gates, mt, nm, ctl, s, n_lead, spin_limit);
+    if (e != cudaSuccess) return e;
+    const int tn = (nm + GT - 1) / GT, tm = (mm + GT - 1) / GT;
+    k_mix_gram<<<dim3(tn, tn, n_gates), GTHREADS, 0, s>>>(d);
+    k_mix_corr<<<dim3(tn, tn, n_gates), GTHREADS, 0, s>>>(d);
+    k_mix_mul<true><<<dim3(tm, tn, n_gates), GTHREADS, 0, s>>>(d);
+    k_mix_mul<false><<<dim3(tm, tn, n_gates), GTHREADS, 0, s>>>(d);
+    return cudaGetLastError();
+}
+
+}  // namespace tnsim

@@ -13,6 +13,7 @@
 //            and U = W.S^-1, row j of S.V^H equals u_j^H theta, so the right site is
 //            the product U_kept^H . theta0 scaled per row -- no V is accumulated.
 //            In canonical form (k_canon.cu) it is V^H of diag(Lam_q) theta instead.
+//  complex128 runs both in k_fp64.cu.
 #include "tnsim_internal.h"
 
 namespace tnsim {
@@ -172,8 +173,9 @@ template <typename T>
 cudaError_t launch_theta(const GateDesc* d, int n_gates, int chiL_max, int chiR_max,
                          cudaStream_t s) {
     if (n_gates <= 0) return cudaSuccess;
+    if constexpr (sizeof(T) == 8) return launch_theta64(d, n_gates, chiL_max, chiR_max, s);
     dim3 grid((chiL_max + TH_L - 1) / TH_L, (chiR_max + TH_R - 1) / TH_R, n_gates);
-    k_theta<T><<<grid, 256, 0, s>>>(d);
+    if constexpr (sizeof(T) == 4) k_theta<T><<<grid, 256, 0, s>>>(d);
     return cudaGetLastError();
 }
 
@@ -283,8 +285,9 @@ __global__ void __launch_bounds__(256) k_right(const GateDesc* __restrict__ gd) 
 template <typename T>
 cudaError_t launch_right(const GateDesc* d, int n_gates, int k_max, int n_max, cudaStream_t s) {
     if (n_gates <= 0) return cudaSuccess;
+    if constexpr (sizeof(T) == 8) return launch_right64(d, n_gates, k_max, n_max, s);
     dim3 grid((n_max + RT_C - 1) / RT_C, (k_max + RT_J - 1) / RT_J, n_gates);
-    k_right<T><<<grid, 256, 0, s>>>(d);
+    if constexpr (sizeof(T) == 4) k_right<T><<<grid, 256, 0, s>>>(d);
     return cudaGetLastError();
 }
 

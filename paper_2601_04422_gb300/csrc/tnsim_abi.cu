@@ -49,6 +49,7 @@ constexpr int kRing = 4;           // pinned staging slots per state
 // Process-wide cap on the device memory that states hold (0 = none) and the bytes held.
 std::atomic<int64_t> g_dev_cap{0};
 std::atomic<int64_t> g_dev_held{0};
+std::atomic<int64_t> g_pre_held{0};   // of these, the preconditioner's buffers
 constexpr int kMaxChi = 512;       // largest supported chi_max
 
 struct Staging {
@@ -89,10 +90,12 @@ struct tnsim_mps {
     double* d_gates = nullptr;     // G*32 + n*8
     int* d_sticky = nullptr;
     unsigned long long* d_stats = nullptr;   // the counters of tnsim_stats
-    JacobiCtl* d_ctl = nullptr;    // control word of the persistent Jacobi launch
+    JacobiCtl* d_ctl = nullptr;    // control words of the persistent Jacobi launches (the SVD's, the preconditioner's)
+    char* d_pre = nullptr;         // complex128: G slots * 3 buffers of the preconditioner (null: none)
     int jac_cfg = 0;               // Jacobi launch configuration (tnsim_set_jacobi_config / tnsim_autotune)
     unsigned jac_spin = 0;         // idle polls of the Jacobi kernel before it gives up (0 = default)
     int tc_spin = 0;               // polls of a tensor-core mbarrier wait before it gives up (0 = default)
+    int64_t pre_bytes = 0;         // bytes of d_pre
     int64_t dev_bytes = 0;         // device bytes held, counted against the process-wide cap
     // tensor-core contraction (complex64 with gemm TF32X3 / BF16X3)
     int tc_mode = -1;              // -1 none, 0 TF32 planes, 1 BF16 planes
@@ -110,25 +113,31 @@ struct tnsim_mps {
     std::vector<Rec> recs;
 };
 
+namespace {
+
+// What the launches of one batch of gates depend on besides the descriptors.
+struct BatchShape {
+    int chiL, chiM, chiR, k;   // largest bond dimensions and kept rank (bounds)
+    int gemm, tc_mode;
+    bool canon, qr, mix;       // some gate: canonical form, QR preconditioning, FP32 preconditioning
+    double tol;
+    int sweeps, jac_cfg, lead;
+    unsigned spin;
+};
+
+}  // namespace
+
 struct tnsim_plan {
     std::vector<tnsim_mps*> states;
     cudaStream_t stream = nullptr;
     int device = 0;
     tnsim_dtype dt = TNSIM_C64;
-    int gemm = 0, tc_mode = -1;
-    int n_gates = 0, n_s1 = 0;
-    int chiL_max = 1, chiM_max = 1, chiR_max = 1, k_max = 1, caplr = 1;
-    double tol = 0.0;
-    int sweeps = 40;
+    int n_gates = 0, n_s1 = 0, caplr = 1;
     GateDesc* d_desc = nullptr;
     GateOut* d_out = nullptr;
     Site1Desc* d_s1 = nullptr;
     JacobiCtl* d_ctl = nullptr;
-    bool canon = false;            // some state of the plan is in canonical form
-    bool qr = false;               // some state of the plan selected QR preconditioning
-    int jac_cfg = 0;               // Jacobi launch configuration of the first state
-    unsigned jac_spin = 0;         // idle-poll limit of the first state
-    int lead = 0;                  // leading gates of the largest capacity (leading_jobs)
+    BatchShape shape{};            // launch shapes from the capacities, options of the states
 };
 
 struct tnsim_graph {
@@ -159,12 +168,34 @@ tnsim_status check_params(const tnsim_params* p) {
     return TNSIM_OK;
 }
 
+// The FP32 preconditioner of a complex128 state is optional: a state without its buffers
+// takes more sweeps to the same result.  They are left out where they could take memory
+// that a state needs: under a process-wide cap, and beyond an eighth of the device's
+// memory over all states.
+void alloc_preconditioner(tnsim_mps* m) {
+    if (2 * m->capmax < kMixMinCols || 4 * m->capmax > kMixMaxRows || g_dev_cap.load() > 0) return;
+    const int64_t bytes = (int64_t)((size_t)m->G * 3 * m->ws_elems * m->esz);
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); return; }
+    if (g_pre_held.fetch_add(bytes) + bytes > (int64_t)(total_b / 8) || bytes > (int64_t)(free_b / 2) ||
+        cudaMalloc((void**)&m->d_pre, (size_t)bytes) != cudaSuccess) {
+        cudaGetLastError();
+        m->d_pre = nullptr;
+        g_pre_held.fetch_sub(bytes);
+        return;
+    }
+    m->pre_bytes = bytes;
+    m->dev_bytes += bytes;
+    g_dev_held.fetch_add(bytes);
+}
+
 void free_all(tnsim_mps* m) {
     cudaFree(m->d_sites); cudaFree(m->d_chi); cudaFree(m->d_ws); cudaFree(m->d_s2);
     cudaFree(m->d_perm); cudaFree(m->d_spec); cudaFree(m->d_spec_k); cudaFree(m->d_out);
     cudaFree(m->d_desc); cudaFree(m->d_s1); cudaFree(m->d_gates); cudaFree(m->d_sticky);
     cudaFree(m->d_stats);
     cudaFree(m->d_ctl);
+    cudaFree(m->d_pre);
     cudaFree(m->d_planes);
     cudaFree(m->d_maps);
     cudaFreeHost(m->h_out); cudaFreeHost(m->h_chi);
@@ -178,7 +209,8 @@ void free_all(tnsim_mps* m) {
     m->recs.clear();
     if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);
     g_dev_held.fetch_sub(m->dev_bytes);
-    m->dev_bytes = 0;
+    g_pre_held.fetch_sub(m->pre_bytes);
+    m->dev_bytes = m->pre_bytes = 0;
 }
 
 cudaEvent_t prof_event(tnsim_mps* m) {
@@ -311,75 +343,87 @@ tnsim_status upload_desc(cudaStream_t st, const std::vector<GateJob>& jobs, Gate
         d.lam_k = m->d_spec_k + j.q;
         d.qr = qr_force >= 0 ? qr_force : (m->jac_cfg >> 1) & 1;
         d.wait_polls = m->tc_spin;
+        if (m->d_pre) {
+            const size_t pb = m->ws_elems * es;   // [theta; I] in FP32: (m + n) n * 8 <= (2 capmax)^2 * 16 bytes
+            char* pre = m->d_pre + (size_t)j.slot * 3 * pb;
+            d.pre = pre;
+            d.pre_x = pre + pb;
+            d.pre_f = pre + 2 * pb;
+        }
     }
     CUDA_TRY(cudaMemcpyAsync(d_desc, h_desc, sizeof(GateDesc) * ng, cudaMemcpyHostToDevice, st));
     return TNSIM_OK;
 }
 
+// The kernels of one batch of gates, in order; prof (may be null) times them.  ctl holds
+// two control words: the preconditioner's and the SVD's Jacobi launch.
 template <typename T>
-tnsim_status launch_gates(cudaStream_t st, const std::vector<GateJob>& jobs, const GateDesc* d_desc,
-                          double tol, int sweeps) {
+tnsim_status launch_batch(cudaStream_t st, const GateDesc* d, int ng, const BatchShape& b, JacobiCtl* ctl,
+                          tnsim_mps* prof) {
+    const int m_max = 2 * b.chiL, n_max = 2 * b.chiR;
+    auto begin = [&]() { return prof ? prof_begin(prof, st) : nullptr; };
+    auto end = [&](int cls, cudaEvent_t ev) { if (prof) prof_end(prof, st, cls, ev); };
+    cudaEvent_t ev = begin();
+    if (sizeof(T) == 8 || b.gemm == TNSIM_GEMM_FP32) {
+        CUDA_TRY(launch_theta<T>(d, ng, b.chiL, b.chiR, st));
+    } else if (b.gemm == TNSIM_GEMM_FP32_3M) {
+        CUDA_TRY(launch_theta_3m(d, ng, b.chiL, b.chiR, st));
+    } else {
+        CUDA_TRY(launch_theta_tc(b.tc_mode, d, ng, b.chiL, b.chiM, b.chiR, st));
+    }
+    end(TNSIM_K_THETA, ev);
+    if (b.canon) CUDA_TRY(launch_scale_rows<T>(d, ng, st));
+    CUDA_TRY(cudaMemsetAsync(ctl, 0, 2 * sizeof(JacobiCtl), st));
+    if (b.qr) {
+        ev = begin();
+        CUDA_TRY(launch_qr<T>(d, ng, m_max, st));
+        end(TNSIM_K_QR, ev);
+    }
+    ev = begin();
+    if (b.mix) CUDA_TRY(launch_mix(d, ng, m_max, n_max, ctl + 1, st, b.lead, b.spin));
+    CUDA_TRY(launch_jacobi<T>(d, ng, m_max, n_max, b.tol, b.sweeps, ctl, st, b.jac_cfg, b.lead, b.spin));
+    end(TNSIM_K_JACOBI, ev);
+    ev = begin();
+    CUDA_TRY(launch_truncate<T>(d, ng, n_max, st));
+    end(TNSIM_K_TRUNCATE, ev);
+    ev = begin();
+    CUDA_TRY(launch_left<T>(d, ng, m_max, b.k, st));
+    end(TNSIM_K_LEFT, ev);
+    ev = begin();
+    CUDA_TRY(launch_right<T>(d, ng, b.k, n_max, st));
+    if (b.canon) CUDA_TRY(launch_left_canon<T>(d, ng, m_max, b.k, st));
+    if (b.qr)
+        CUDA_TRY(launch_sites_pre<T>(d, ng, m_max, b.k, n_max, st,
+                                     b.gemm == TNSIM_GEMM_TF32X3 || b.gemm == TNSIM_GEMM_BF16X3));
+    end(TNSIM_K_RIGHT, ev);
+    return TNSIM_OK;
+}
+
+// One batch of gates: shapes from the bond bounds, launches, bounds for the next layer.
+tnsim_status launch_gates(tnsim_dtype dt, cudaStream_t st, const std::vector<GateJob>& jobs,
+                          const GateDesc* d_desc, double tol, int sweeps) {
     const int ng = (int)jobs.size();
     if (ng == 0) return TNSIM_OK;
-    int chiL_max = 1, chiM_max = 1, chiR_max = 1, k_max = 1;
-    for (const GateJob& j : jobs) {
-        chiL_max = std::max(chiL_max, j.m->ub[j.q]);
-        chiM_max = std::max(chiM_max, j.m->ub[j.q + 1]);
-        chiR_max = std::max(chiR_max, j.m->ub[j.q + 2]);
-        k_max = std::max(k_max, std::min({j.m->cap[j.q + 1], 2 * j.m->ub[j.q], 2 * j.m->ub[j.q + 2]}));
-    }
-    const int m_max = 2 * chiL_max, n_max = 2 * chiR_max;
     tnsim_mps* pm = jobs[0].m;   // the state whose profiler records this batch
-    cudaEvent_t ev = prof_begin(pm, st);
-    if (sizeof(T) == 8 || pm->p.gemm == TNSIM_GEMM_FP32) {
-        CUDA_TRY(launch_theta<T>(d_desc, ng, chiL_max, chiR_max, st));
-    } else if (pm->p.gemm == TNSIM_GEMM_FP32_3M) {
-        CUDA_TRY(launch_theta_3m(d_desc, ng, chiL_max, chiR_max, st));
-    } else {
-        CUDA_TRY(launch_theta_tc(pm->tc_mode, d_desc, ng, chiL_max, chiM_max, chiR_max, st));
-    }
-    prof_end(pm, st, TNSIM_K_THETA, ev);
-    bool canon = false, qr = false;
+    BatchShape b{1, 1, 1, 1, pm->p.gemm, pm->tc_mode, false, false, false, tol, sweeps, pm->jac_cfg,
+                 leading_jobs(jobs, false), pm->jac_spin};
     for (const GateJob& j : jobs) {
-        canon = canon || j.m->p.form == TNSIM_FORM_CANONICAL;
-        qr = qr || (j.m->jac_cfg & 2) != 0;
+        b.chiL = std::max(b.chiL, j.m->ub[j.q]);
+        b.chiM = std::max(b.chiM, j.m->ub[j.q + 1]);
+        b.chiR = std::max(b.chiR, j.m->ub[j.q + 2]);
+        b.k = std::max(b.k, std::min({j.m->cap[j.q + 1], 2 * j.m->ub[j.q], 2 * j.m->ub[j.q + 2]}));
+        b.canon = b.canon || j.m->p.form == TNSIM_FORM_CANONICAL;
+        b.qr = b.qr || (j.m->jac_cfg & 2) != 0;
+        b.mix = b.mix || j.m->d_pre;
     }
-    if (canon) CUDA_TRY(launch_scale_rows<T>(d_desc, ng, st));
-    CUDA_TRY(cudaMemsetAsync(pm->d_ctl, 0, sizeof(JacobiCtl), st));
-    if (qr) {
-        ev = prof_begin(pm, st);
-        CUDA_TRY(launch_qr<T>(d_desc, ng, m_max, st));
-        prof_end(pm, st, TNSIM_K_QR, ev);
-    }
-    ev = prof_begin(pm, st);
-    CUDA_TRY(launch_jacobi<T>(d_desc, ng, m_max, n_max, tol, sweeps, pm->d_ctl, st, pm->jac_cfg,
-                              leading_jobs(jobs, false), pm->jac_spin));
-    prof_end(pm, st, TNSIM_K_JACOBI, ev);
-    ev = prof_begin(pm, st);
-    CUDA_TRY(launch_truncate<T>(d_desc, ng, n_max, st));
-    prof_end(pm, st, TNSIM_K_TRUNCATE, ev);
-    ev = prof_begin(pm, st);
-    CUDA_TRY(launch_left<T>(d_desc, ng, m_max, k_max, st));
-    prof_end(pm, st, TNSIM_K_LEFT, ev);
-    ev = prof_begin(pm, st);
-    CUDA_TRY(launch_right<T>(d_desc, ng, k_max, n_max, st));
-    if (canon) CUDA_TRY(launch_left_canon<T>(d_desc, ng, m_max, k_max, st));
-    if (qr)
-        CUDA_TRY(launch_sites_pre<T>(d_desc, ng, m_max, k_max, n_max, st,
-                                     pm->p.gemm == TNSIM_GEMM_TF32X3 || pm->p.gemm == TNSIM_GEMM_BF16X3));
-    prof_end(pm, st, TNSIM_K_RIGHT, ev);
-    // bounds for the next layer
+    const tnsim_status s = dt == TNSIM_C64 ? launch_batch<float>(st, d_desc, ng, b, pm->d_ctl, pm)
+                                           : launch_batch<double>(st, d_desc, ng, b, pm->d_ctl, pm);
+    if (s != TNSIM_OK) return s;
     for (const GateJob& j : jobs) {
         tnsim_mps* m = j.m;
         m->ub[j.q + 1] = std::min({m->cap[j.q + 1], 2 * m->ub[j.q], 2 * m->ub[j.q + 2]});
     }
     return TNSIM_OK;
-}
-
-tnsim_status launch_gates_dt(tnsim_dtype dt, cudaStream_t st, const std::vector<GateJob>& jobs,
-                             const GateDesc* d_desc, double tol, int sweeps) {
-    return dt == TNSIM_C64 ? launch_gates<float>(st, jobs, d_desc, tol, sweeps)
-                           : launch_gates<double>(st, jobs, d_desc, tol, sweeps);
 }
 
 // the one-qubit updates of the qubits outside every pair
@@ -448,11 +492,11 @@ tnsim_status enqueue_layer(tnsim_mps* m, Staging* stg, int n2, const int32_t* q,
         // one pair at a time: each pair is its own launch sequence
         for (int i = 0; i < n2; ++i) {
             std::vector<GateJob> one(1, jobs[i]);
-            s = launch_gates_dt(m->dt, st, one, m->d_desc + i, tol, sweeps);
+            s = launch_gates(m->dt, st, one, m->d_desc + i, tol, sweeps);
             if (s != TNSIM_OK) return s;
         }
     } else {
-        s = launch_gates_dt(m->dt, st, jobs, m->d_desc, tol, sweeps);
+        s = launch_gates(m->dt, st, jobs, m->d_desc, tol, sweeps);
         if (s != TNSIM_OK) return s;
     }
     return TNSIM_OK;
@@ -560,7 +604,7 @@ tnsim_status tnsim_mps_create(int32_t n_qubits, tnsim_dtype dt, const tnsim_para
                                  nG * capmax2 * (sizeof(double) + sizeof(int)) +
                                  (size_t)(n_qubits + 1) * prm.chi_max * sizeof(double) + sizeof(int) * (n_qubits + 1) +
                                  nG * (sizeof(GateOut) + sizeof(GateDesc)) + (size_t)n_qubits * sizeof(Site1Desc) +
-                                 gate_doubles * sizeof(double) + sizeof(int) + sizeof(tnsim_stats) + sizeof(JacobiCtl));
+                                 gate_doubles * sizeof(double) + sizeof(int) + sizeof(tnsim_stats) + 2 * sizeof(JacobiCtl));
         if (use_tc) need += (int64_t)(nG * 8 * capmax2 * ((m->capmax + 63) / 64 * 64) * sizeof(float) +
                                       2 * sizeof(CUtensorMap));
         const int64_t cap = g_dev_cap.load();
@@ -587,7 +631,7 @@ tnsim_status tnsim_mps_create(int32_t n_qubits, tnsim_dtype dt, const tnsim_para
     ALLOC(m->d_gates, gate_doubles * sizeof(double));
     ALLOC(m->d_sticky, sizeof(int));
     ALLOC(m->d_stats, sizeof(tnsim_stats));
-    ALLOC(m->d_ctl, sizeof(JacobiCtl));
+    ALLOC(m->d_ctl, 2 * sizeof(JacobiCtl));
     HALLOC(m->h_out, nG * sizeof(GateOut));
     HALLOC(m->h_chi, sizeof(int) * (n_qubits + 1));
     for (auto& r : m->ring) {
@@ -618,6 +662,7 @@ tnsim_status tnsim_mps_create(int32_t n_qubits, tnsim_dtype dt, const tnsim_para
     }
 #undef ALLOC
 #undef HALLOC
+    if (dt == TNSIM_C128) alloc_preconditioner(m);
     if (cuda_stream) {
         m->stream = (cudaStream_t)cuda_stream;
     } else {
@@ -900,7 +945,7 @@ tnsim_status tnsim_apply_layers_batched(tnsim_mps* const* ms, int32_t n_circ, in
             if (e != cudaSuccess) { ret = fail(TNSIM_ECUDA, cudaGetErrorString(e)); break; }
             ret = upload_desc(st, jobs, h_desc, d_desc, d_out);
             if (ret != TNSIM_OK) break;
-            ret = launch_gates_dt(m0->dt, st, jobs, d_desc, tol, sweeps);
+            ret = launch_gates(m0->dt, st, jobs, d_desc, tol, sweeps);
             if (ret != TNSIM_OK) break;
             // the pinned staging is reused by the next step
             e = cudaMemcpyAsync(h_out, d_out, sizeof(GateOut) * jobs.size(), cudaMemcpyDeviceToHost, st);
@@ -949,18 +994,16 @@ tnsim_status tnsim_plan_create(tnsim_mps* const* ms, int32_t n_states, const int
     p->stream = m0->stream;
     p->device = m0->device;
     p->dt = m0->dt;
-    p->gemm = m0->p.gemm;
-    for (int i = 0; i < n_states; ++i) p->canon = p->canon || ms[i]->p.form == TNSIM_FORM_CANONICAL;
-    p->jac_cfg = m0->jac_cfg;
-    p->jac_spin = m0->jac_spin;
-    for (int i = 0; i < n_states; ++i) p->qr = p->qr || (ms[i]->jac_cfg & 2) != 0;
-    p->tc_mode = m0->tc_mode;
-    p->tol = m0->p.jacobi_tol;
+    BatchShape& b = p->shape;
+    b = {1, 1, 1, 1, m0->p.gemm, m0->tc_mode, false, false, false, m0->p.jacobi_tol, 40, m0->jac_cfg, 0, m0->jac_spin};
     std::vector<GateJob> jobs;
     std::vector<Site1Desc> s1;
     for (int i = 0; i < n_states; ++i) {
         tnsim_mps* m = ms[i];
-        p->sweeps = std::max(p->sweeps, default_sweeps(m));
+        b.sweeps = std::max(b.sweeps, default_sweeps(m));
+        b.canon = b.canon || m->p.form == TNSIM_FORM_CANONICAL;
+        b.qr = b.qr || (m->jac_cfg & 2) != 0;
+        b.mix = b.mix || m->d_pre;
         std::vector<char> used(m->n, 0);
         for (int j = 0; j < n2[i]; ++j) {
             const int q = q_ptrs[i][j];
@@ -975,10 +1018,10 @@ tnsim_status tnsim_plan_create(tnsim_mps* const* ms, int32_t n_states, const int
             jb.eps_dev = nullptr;
             jobs.push_back(jb);
             // launch shapes from the capacities: valid for any bond dimensions reached later
-            p->chiL_max = std::max(p->chiL_max, m->cap[q]);
-            p->chiM_max = std::max(p->chiM_max, m->cap[q + 1]);
-            p->chiR_max = std::max(p->chiR_max, m->cap[q + 2]);
-            p->k_max = std::max(p->k_max, m->cap[q + 1]);
+            b.chiL = std::max(b.chiL, m->cap[q]);
+            b.chiM = std::max(b.chiM, m->cap[q + 1]);
+            b.chiR = std::max(b.chiR, m->cap[q + 2]);
+            b.k = std::max(b.k, m->cap[q + 1]);
         }
         if (u1_dev[i]) {
             for (int sidx = 0; sidx < m->n; ++sidx) {
@@ -1000,12 +1043,12 @@ tnsim_status tnsim_plan_create(tnsim_mps* const* ms, int32_t n_states, const int
         return ca > cb;
     });
     p->n_gates = (int)jobs.size();
-    p->lead = leading_jobs(jobs, true);
+    b.lead = leading_jobs(jobs, true);
     p->n_s1 = (int)s1.size();
     cudaError_t e = cudaMalloc((void**)&p->d_desc, sizeof(GateDesc) * (p->n_gates + 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_out, sizeof(GateOut) * (p->n_gates + 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_s1, sizeof(Site1Desc) * (p->n_s1 + 1));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_ctl, sizeof(JacobiCtl));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_ctl, 2 * sizeof(JacobiCtl));
     if (e != cudaSuccess) {
         cudaFree(p->d_desc); cudaFree(p->d_out); cudaFree(p->d_s1); cudaFree(p->d_ctl);
         delete p;
@@ -1034,35 +1077,9 @@ tnsim_status tnsim_plan_launch(tnsim_plan* p) {
     const int ng = p->n_gates;
     if (ng == 0) return TNSIM_OK;
     CUDA_TRY(cudaMemsetAsync(p->d_out, 0, sizeof(GateOut) * ng, st));
-    CUDA_TRY(cudaMemsetAsync(p->d_ctl, 0, sizeof(JacobiCtl), st));
-    const int m_max = 2 * p->chiL_max, n_max = 2 * p->chiR_max;
-    if (p->dt == TNSIM_C128) {
-        CUDA_TRY(launch_theta<double>(p->d_desc, ng, p->chiL_max, p->chiR_max, st));
-        if (p->canon) CUDA_TRY(launch_scale_rows<double>(p->d_desc, ng, st));
-        if (p->qr) CUDA_TRY(launch_qr<double>(p->d_desc, ng, m_max, st));
-        CUDA_TRY(launch_jacobi<double>(p->d_desc, ng, m_max, n_max, p->tol, p->sweeps, p->d_ctl, st, p->jac_cfg,
-                                       p->lead, p->jac_spin));
-        CUDA_TRY(launch_truncate<double>(p->d_desc, ng, n_max, st));
-        CUDA_TRY(launch_left<double>(p->d_desc, ng, m_max, p->k_max, st));
-        CUDA_TRY(launch_right<double>(p->d_desc, ng, p->k_max, n_max, st));
-        if (p->canon) CUDA_TRY(launch_left_canon<double>(p->d_desc, ng, m_max, p->k_max, st));
-        if (p->qr) CUDA_TRY(launch_sites_pre<double>(p->d_desc, ng, m_max, p->k_max, n_max, st));
-    } else {
-        if (p->gemm == TNSIM_GEMM_FP32) CUDA_TRY(launch_theta<float>(p->d_desc, ng, p->chiL_max, p->chiR_max, st));
-        else if (p->gemm == TNSIM_GEMM_FP32_3M) CUDA_TRY(launch_theta_3m(p->d_desc, ng, p->chiL_max, p->chiR_max, st));
-        else CUDA_TRY(launch_theta_tc(p->tc_mode, p->d_desc, ng, p->chiL_max, p->chiM_max, p->chiR_max, st));
-        if (p->canon) CUDA_TRY(launch_scale_rows<float>(p->d_desc, ng, st));
-        if (p->qr) CUDA_TRY(launch_qr<float>(p->d_desc, ng, m_max, st));
-        CUDA_TRY(launch_jacobi<float>(p->d_desc, ng, m_max, n_max, p->tol, p->sweeps, p->d_ctl, st, p->jac_cfg,
-                                      p->lead, p->jac_spin));
-        CUDA_TRY(launch_truncate<float>(p->d_desc, ng, n_max, st));
-        CUDA_TRY(launch_left<float>(p->d_desc, ng, m_max, p->k_max, st));
-        CUDA_TRY(launch_right<float>(p->d_desc, ng, p->k_max, n_max, st));
-        if (p->canon) CUDA_TRY(launch_left_canon<float>(p->d_desc, ng, m_max, p->k_max, st));
-        if (p->qr)
-            CUDA_TRY(launch_sites_pre<float>(p->d_desc, ng, m_max, p->k_max, n_max, st,
-                                             p->gemm == TNSIM_GEMM_TF32X3 || p->gemm == TNSIM_GEMM_BF16X3));
-    }
+    const tnsim_status s = p->dt == TNSIM_C64 ? launch_batch<float>(st, p->d_desc, ng, p->shape, p->d_ctl, nullptr)
+                                              : launch_batch<double>(st, p->d_desc, ng, p->shape, p->d_ctl, nullptr);
+    if (s != TNSIM_OK) return s;
     // the bond upper bounds the host keeps become the capacities
     for (tnsim_mps* m : p->states)
         for (int b = 0; b <= m->n; ++b) m->ub[b] = std::max(m->ub[b], m->cap[b]);
@@ -1504,11 +1521,12 @@ tnsim_status tnsim_autotune(tnsim_mps* m, int32_t n2, const int32_t* q, const do
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(m->d_out, bak + (size_t)n2 * wbytes, sizeof(GateOut) * n2,
                                     cudaMemcpyDeviceToDevice, st);
-            if (e == cudaSuccess) e = cudaMemsetAsync(m->d_ctl, 0, sizeof(JacobiCtl), st);
+            if (e == cudaSuccess) e = cudaMemsetAsync(m->d_ctl, 0, 2 * sizeof(JacobiCtl), st);
             if (e == cudaSuccess) e = cudaEventRecord(e0, st);
             if (e == cudaSuccess && (c & 2))
                 e = m->dt == TNSIM_C64 ? launch_qr<float>(m->d_desc, n2, m_max, st)
                                        : launch_qr<double>(m->d_desc, n2, m_max, st);
+            if (e == cudaSuccess && m->d_pre) e = launch_mix(m->d_desc, n2, m_max, n_max, m->d_ctl + 1, st, lead, 0);
             if (e == cudaSuccess)
                 e = m->dt == TNSIM_C64
                         ? launch_jacobi<float>(m->d_desc, n2, m_max, n_max, default_tol(m), default_sweeps(m), m->d_ctl, st, c,

@@ -76,6 +76,11 @@ struct GateDesc {
     // QR preconditioning (k_qr.cu): for m == n the Jacobi runs on R^H of theta = Q R; the
     // left site becomes theta W' S^-2 and the right site the conjugated Jacobi columns
     int qr;
+    // complex128: the buffers of the mixed-precision preconditioner (k_fp64.cu), null = none:
+    // [theta; I] in FP32 ((m + n) x n), I - V^H V and then W V (FP64, m x n), the correction (n x n)
+    void* pre;
+    void* pre_x;
+    void* pre_f;
     // polls of a bounded mbarrier wait in the tensor-core contraction before it gives up
     // (0 = the kernel's default); the CTA then drains its copies in flight and reports
     // status 5 (ETIMEOUT)
@@ -118,6 +123,20 @@ __device__ __forceinline__ bool qr_active(const GateDesc& d, int m, int n) {
 }
 #endif
 
+// Mixed-precision preconditioner of the complex128 SVD: gates of fewer columns converge
+// in FP64 within the time of its launches; of more rows (m + n, those of its columns) two
+// column blocks no longer fit in shared memory.
+constexpr int kMixMinCols = 16;
+constexpr int kMixMaxRows = 1024;
+constexpr double kMixTol = 2e-6;
+#ifdef __CUDACC__
+// power of two that brings |theta|_F into [1, 2) in the FP32 copy of theta
+__device__ __forceinline__ double mix_scale(double frob2) {
+    if (!(frob2 > 0.0) || isinf(frob2)) return 1.0;
+    return ldexp(1.0, -(ilogb(frob2) >> 1));
+}
+#endif
+
 // One-qubit update of one site (Eq. 3).
 struct Site1Desc {
     void* site;
@@ -143,6 +162,16 @@ template <typename T>
 cudaError_t launch_jacobi(const GateDesc* d, int n_gates, int m_max, int n_max, double tol,
                           int max_sweeps, JacobiCtl* ctl, cudaStream_t s, int cfg = 0, int n_lead = 0,
                           unsigned spin_limit = 0);
+// the FP32 Jacobi of the preconditioner (columns of mt_max rows in GateDesc::pre)
+cudaError_t launch_jacobi_mix(const GateDesc* d, int n_gates, int mt_max, int n_max, JacobiCtl* ctl, cudaStream_t s,
+                              int n_lead, unsigned spin_limit);
+// the whole preconditioner: W <- W V' for every complex128 gate with buffers; ctl is its
+// own control word (zeroed before)
+cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, JacobiCtl* ctl, cudaStream_t s,
+                       int n_lead, unsigned spin_limit);
+// FP64 merge + gate contraction and right site
+cudaError_t launch_theta64(const GateDesc* d, int n_gates, int chiL_max, int chiR_max, cudaStream_t s);
+cudaError_t launch_right64(const GateDesc* d, int n_gates, int k_max, int n_max, cudaStream_t s);
 // the tensor-core Jacobi launch (complex64), called by launch_jacobi<float> for cfg bit 2
 cudaError_t launch_jacobi_tc(const GateDesc* d, int n_gates, int n_lead, int n_max, double tol, int max_sweeps,
                              JacobiCtl* ctl, cudaStream_t s, unsigned spin_limit);

@@ -1,0 +1,109 @@
+"""complex128 updates through the FP32-preconditioned SVD and the 16 x 16-tiled FP64 products.
+
+Sizes around the edges of the tiles (16), of the column blocks (8, 4), of the smallest
+preconditioned block (16 columns) and of the largest (m + n = 1024 rows), rectangular
+blocks, every contraction form, and spectra that FP32 cannot resolve.  The kept singular
+values must agree with LAPACK's within 64 eps s_max sqrt(rank) (both are backward stable:
+a few eps |theta|_2 each, and |theta|_F <= sqrt(rank) s_max), the new block with the best
+approximation at the gap of the cut, which random blocks keep above 1e-6.
+"""
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import mps as om
+
+pytestmark = pytest.mark.gpu
+EPS = np.finfo(np.float64).eps
+
+
+@pytest.fixture(scope="module")
+def T():
+    import __graft_entry__ as g
+    g.build()
+    import paper_2601_04422_gb300 as T
+    return T
+
+
+def _chain(cl, cm, cr):
+    """Bond dimensions of a chain whose middle pair has bonds cl, cm, cr."""
+    def ramp(c):
+        d = [1]
+        while d[-1] < c:
+            d.append(min(c, 2 * d[-1]))
+        return d
+    a, b = ramp(cl), ramp(cr)
+    return a + [cm] + b[::-1], len(a) - 1
+
+
+def _update(T, cl, cm, cr, chi, cfg, decay=0.0, seed=1):
+    rng = np.random.default_rng(seed)
+    dims, q = _chain(cl, cm, cr)
+    sites = [(rng.standard_normal((dims[i], 2, dims[i + 1])) + 1j * rng.standard_normal((dims[i], 2, dims[i + 1])))
+             / np.sqrt(4 * dims[i + 1]) for i in range(len(dims) - 1)]
+    sites[q + 1] = sites[q + 1] * np.exp(-decay * np.arange(cm) / max(1, cm - 1))[:, None, None]
+    n = len(sites)
+    cap = max(chi, max(dims))
+    m = T.MPS(n, dtype=T.TNSIM_C128, chi_max=cap)
+    if any(d > c for d, c in zip(dims, [min(cap, 2 ** min(b, n - b)) for b in range(n + 1)])):
+        pytest.skip("chain too short for these bonds")
+    m.import_sites(sites)
+    if cfg:
+        T.tnsim_set_jacobi_config(m.h, cfg)
+    g = W.haar_su4(rng)
+    m.apply_layer(W.Layer(np.array([q], np.int32), g[None], None))
+    ref = om.MPS(sites)
+    r = om.apply_2q(ref, q, g, cap)
+    s = m.spectrum(q + 1)
+    out = m.export_sites()
+    m.close()
+    blk = out[q].reshape(2 * cl, -1) @ out[q + 1].reshape(-1, 2 * cr)
+    blk_o = ref.sites[q].reshape(2 * cl, -1) @ ref.sites[q + 1].reshape(-1, 2 * cr)
+    return s, r, blk, blk_o, out[q]
+
+
+@pytest.mark.parametrize("cfg", [0, 1, 2])
+@pytest.mark.parametrize("c", [(3, 4, 4), (7, 8, 7), (8, 8, 8), (8, 9, 9), (9, 16, 12), (16, 17, 17), (33, 33, 20),
+                               (20, 33, 33), (64, 64, 65), (100, 60, 90)])
+def test_block_sizes(T, c, cfg):
+    s, r, blk, blk_o, u = _update(T, *c, chi=1, cfg=cfg)
+    assert len(s) == r.k
+    assert np.max(np.abs(s - r.s_kept)) <= 64 * EPS * np.sqrt(r.k) * r.s_kept[0]
+    assert np.linalg.norm(blk - blk_o) <= 1e-9 * np.linalg.norm(blk_o)
+    u = u.reshape(-1, u.shape[2])
+    assert np.abs(u.conj().T @ u - np.eye(u.shape[1])).max() <= 1e-11
+
+
+@pytest.mark.parametrize("chi", [256, 257])
+def test_largest_preconditioned_block(T, chi):
+    """m + n = 1024 rows is the last preconditioned size, 1028 the first beyond it."""
+    s, r, blk, blk_o, _ = _update(T, chi, chi, chi, chi=1, cfg=0)
+    assert len(s) == r.k and np.max(np.abs(s - r.s_kept)) <= 64 * EPS * np.sqrt(r.k) * r.s_kept[0]
+    assert np.linalg.norm(blk - blk_o) <= 1e-9 * np.linalg.norm(blk_o)
+
+
+@pytest.mark.parametrize("decay", [12.0, 30.0])
+def test_spectrum_below_fp32(T, decay):
+    """Singular values over 5 and 13 decades: the small ones are beyond FP32 and are found
+    by the FP64 iteration."""
+    s, r, blk, blk_o, _ = _update(T, 32, 32, 32, chi=64, cfg=0, decay=decay)
+    k = min(len(s), r.k)
+    assert np.max(np.abs(s[:k] - r.s_kept[:k])) <= 64 * EPS * np.sqrt(r.k) * r.s_kept[0]
+    assert np.linalg.norm(blk - blk_o) <= 1e-12 * np.linalg.norm(blk_o)
+
+
+def test_canonical_form_and_memory_cap(T):
+    """Canonical-form gates precondition diag(Lam) theta; a state made under a device-memory
+    cap has no preconditioner buffers and gives the same state."""
+    circ = W.brickwork_u2_su4(12, 8, seed=4)
+    out = []
+    for cap in (0, 1 << 40):
+        T.tnsim_set_device_memory_cap(cap)
+        try:
+            m = T.MPS(12, dtype=T.TNSIM_C128, chi_max=24, form=T.TNSIM_FORM_CANONICAL)
+        finally:
+            T.tnsim_set_device_memory_cap(0)
+        m.run(circ)
+        out.append(om.MPS(m.export_sites()))
+        m.close()
+    assert 1 - om.fidelity(*out) <= 1e-12
