@@ -24,31 +24,36 @@ __device__ __forceinline__ void rr_pair(int P, int r, int v, int& a, int& b) {
 }
 
 // Rotation parameters (c - 1, s e^{i phi}) of a column pair from a, b and g = gr + i gi.
-// The quantities that decide whether the rotation is unitary -- |e^{i phi}| = 1 and
-// c^2 + s^2 = 1 -- use correctly rounded square roots and reciprocals (sqrtf,
-// __frcp_rn), so their rounding errors are unbiased; the skip test and the angle t
-// (which only has to orthogonalise the pair to within rounding) use fast division.
-// c - 1 = -t^2 / (rr (1 + rr)) is formed without cancellation.
+// With tau = t / |g| = 2 sign(b - a) / (|b - a| + sqrt((b - a)^2 + 4 |g|^2)):
+//     t^2 = tau^2 |g|^2,   c = (1 + t^2)^{-1/2},   s e^{i phi} = c tau g,
+// so the rotation is unitary (c^2 + |s e^{i phi}|^2 = 1) for whatever tau, which only has to
+// orthogonalise the pair to within rounding and comes from the approximate reciprocal and
+// square root.  c takes one Newton step (its rounding error is then unbiased), and
+// c - 1 = -t^2 c^2 / (1 + c) is formed without cancellation with a correctly rounded
+// reciprocal: a bias of either would make the norms drift.  Three dependent special-function
+// operations instead of eight (with |g|, zeta and 1 / |g| by IEEE square roots and
+// reciprocals): the chain from g to the update is what the warps of a step wait for.
 __device__ __forceinline__ bool rot_params_fast(float a, float b, float gr, float gi, float tol2, float zthr,
                                                 float& cm1, float& sr, float& si, float& tg) {
-    const float g2 = gr * gr + gi * gi;
-    if (!(a > zthr && b > zthr && __fdividef(g2, b) > tol2 * a)) return false;
-    const float gabs = sqrtf(g2);
-    const float rg = __frcp_rn(gabs);                     // 1 / |g|
-    const float zeta = 0.5f * (b - a) * rg;
-    const float az = fabsf(zeta);
-    // t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)); for |zeta| > 2^12, 1 + zeta^2 rounds to zeta^2
-    const float den = az > 4096.f ? 2.f * az : az + sqrtf(fmaf(zeta, zeta, 1.f));
-    const float t = copysignf(__fdividef(1.f, den), zeta);
-    const float rr = sqrtf(fmaf(t, t, 1.f));
-    const float irr = __frcp_rn(rr);                      // c
-    cm1 = -(t * t) * irr * __frcp_rn(1.f + rr);
-    const float sv = t * irr;
-    sr = sv * (gr * rg);
-    si = sv * (gi * rg);
-    tg = t * gabs;                                        // the norms become a - t|g|, b + t|g|
+    const float g2 = fmaf(gr, gr, gi * gi);
+    if (!(a > zthr && b > zthr && g2 > (tol2 * a) * b)) return false;
+    const float d = b - a, ad = fabsf(d);
+    float h = fmaf(d, d, 4.f * g2);
+    // sqrt(h); beyond the range of h: |d| dominates
+    const float rt = h < 1e38f ? h * rsqrtf(h) : ad;
+    const float tau = copysignf(__fdividef(2.f, ad + rt), d);
+    tg = tau * g2;                                        // the norms become a - t|g|, b + t|g|
+    const float t2 = tg * tau;
+    const float u = 1.f + t2;
+    const float c0 = rsqrtf(u);
+    const float c = fmaf(0.5f * c0, fmaf(-u * c0, c0, 1.f), c0);
+    const float f = c * tau;
+    sr = f * gr;
+    si = f * gi;
+    cm1 = -(t2 * c) * c * __frcp_rn(1.f + c);
     return true;
 }
+
 // x 2^-e in FP32 (truncated) and back, by integer operations: FP64 instructions, the
 // conversions among them, issue once in 64 cycles per scheduler.
 __device__ __forceinline__ float f32_scaled(double x, int e) {

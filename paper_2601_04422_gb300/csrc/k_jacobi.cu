@@ -58,22 +58,13 @@ __device__ __forceinline__ int rotate_pair(C* __restrict__ xi, C* __restrict__ x
         gr += __shfl_xor_sync(0xffffffffu, gr, o);
         gi += __shfl_xor_sync(0xffffffffu, gi, o);
     }
-    const T g2 = gr * gr + gi * gi;
-    if (!(a > zthr && b > zthr && g2 / b > tol2 * a)) return 0;
-    const T gabs = sqrt(g2);
-    const T zeta = (b - a) / (2 * gabs);
-    const T t = copysign(T(1), zeta) / (fabs(zeta) + sqrt(T(1) + zeta * zeta));
-    // c = 1/rr, s = t/rr with rr = sqrt(1 + t^2), and c - 1 = -t^2 / (rr (1 + rr)) formed
-    // directly.  Each new element is x + d, where the small correction d = (c-1) x + ...
-    // is summed first and then added to x with a single rounding.  Near convergence
-    // |(c-1) x| is below half an ulp of x: added to an already rounded x + ... it would
-    // always round away, leaving c = 1 and growing the pair's norm by a factor 1 + t^2
-    // per rotation (a systematic drift of the singular values in FP32).
-    const T rr = sqrt(T(1) + t * t);
-    const T cm1 = -(t * t) / (rr * (T(1) + rr));
-    const T s = t / rr;
-    const T er = gr / gabs, ei = gi / gabs;
-    const T sr = s * er, si = s * ei;     // s e^{i phi}
+    T cm1, sr, si, tg;
+    if (!rot_params_fast(a, b, gr, gi, tol2, zthr, cm1, sr, si, tg)) return 0;
+    // Each new element is x + d, where the small correction d = (c-1) x + ... is summed
+    // first and then added to x with a single rounding.  Near convergence |(c-1) x| is
+    // below half an ulp of x: added to an already rounded x + ... it would always round
+    // away, leaving c = 1 and growing the pair's norm by a factor 1 + t^2 per rotation (a
+    // systematic drift of the singular values in FP32).
     for (int r = lane; r < m; r += 32) {
         const C u = xi[r], v = xj[r];
         C nu, nv;
