@@ -72,7 +72,7 @@ __device__ __forceinline__ double f64_scaled(float x, int e) {
 // FP64: the test and a first tau in FP32 on values scaled by the larger norm's power of two;
 // one Newton step for tau (without it a gate took 0.6 sweeps more) and the quantities that
 // make the rotation unitary in FP64: 15 FP64 instructions while t < 2^-10 (where c - 1 is
-// its series), against about 150 with FP64 square roots and divisions.
+// its series), 20 beyond, against about 150 with FP64 square roots and divisions.
 __device__ __forceinline__ bool rot_params64(double a, double b, double gr, double gi, float tol, double zthr,
                                              double& cm1, double& sr, double& si, double& tg) {
     const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b), iz = __double_as_longlong(zthr);
@@ -97,13 +97,12 @@ __device__ __forceinline__ bool rot_params64(double a, double b, double gr, doub
     if (__double2hiint(t2) < 0x3eb00000) {                // t^2 < 2^-20: the next term is below 2^-61
         cm1 = t2 * fma(0.375, t2, -0.5);
     } else {
-        const double c = rsqrt(1.0 + t2);
-        // 1 / (1 + c) by two Newton steps from FP32
-        const double h = 1.0 + c;
-        double ih = (double)__frcp_rn((float)h);
-        ih = fma(ih, fma(-h, ih, 1.0), ih);
-        ih = fma(ih, fma(-h, ih, 1.0), ih);
-        cm1 = -(t2 * c) * c * ih;
+        // c = u^{-1/2} from an FP32 estimate c0: with e = 1 - u c0^2 (~1e-7),
+        // c = c0 (1 + e/2 + 3/8 e^2 + O(e^3)); c - 1 is exact here
+        const double u = 1.0 + t2;
+        const double c0 = f64_scaled(rsqrtf(f32_scaled(u, 0)), 0);
+        const double ee = fma(-u * c0, c0, 1.0);
+        cm1 = fma(c0 * ee, fma(0.375, ee, 0.5), c0) - 1.0;
     }
     const double f = fma(tau, cm1, tau);
     sr = f * gr;

@@ -17,14 +17,15 @@
 // Schedule.  The columns are cut into blocks of BC.  A sweep visits every pair of
 // blocks once in round-robin ("circle") order: P - 1 rounds of P/2 disjoint block
 // pairs.  A visit stages both blocks in shared memory, rotates the BC x BC cross
-// pairs in BC rounds of BC disjoint pairs (one warp per pair, lanes over rows,
-// warp-shuffle reductions; each warp keeps its block-I column in registers, and the
-// column norms are tracked rather than recomputed per pair) and, in
-// the first round of a sweep, the pairs inside each block as well, then writes the
+// pairs in BC rounds of BC disjoint pairs and, in the first round of a sweep, the pairs
+// inside each block as well (Visit32, visit64 below), then writes the
 // blocks back.  Each sweep therefore rotates every column pair exactly once.  A sweep
 // that rotates nothing ends the gate's iteration; reaching max_sweeps sets ENOCONV.
 //
-// The launch is persistent: one CTA per SM (as occupancy allows) claims visits of
+// Two kernels run this schedule with the same arithmetic: k_jacobi_cl, one cluster per gate,
+// where all gates are resident at once; else k_jacobi, a queue.
+//
+// k_jacobi is persistent: as many CTAs as the SMs hold claim visits of
 // any gate from a device-side queue, so gates of different sizes and all rounds of
 // a layer share the machine without waves.  The visits of a round are independent;
 // a gate's next round opens when the last visit of the current one is reported.  An
@@ -35,140 +36,217 @@
 // in flight.
 #include <float.h>
 
+#include <algorithm>
+#include <atomic>
+
+#include <cooperative_groups.h>
+
 #include "jacobi_sched.cuh"
 #include "tnsim_internal.h"
 
+namespace cg = cooperative_groups;
+
 namespace tnsim {
 
-template <typename T, typename C>
-__device__ __forceinline__ int rotate_pair(C* __restrict__ xi, C* __restrict__ xj, int m, int md, int lane,
-                                           T tol2, T zthr) {
-    T a = 0, b = 0, gr = 0, gi = 0;
-    for (int r = lane; r < md; r += 32) {
-        const C u = xi[r], v = xj[r];
-        a = fma(u.x, u.x, fma(u.y, u.y, a));
-        b = fma(v.x, v.x, fma(v.y, v.y, b));
-        gr = fma(u.x, v.x, fma(u.y, v.y, gr));
-        gi = fma(u.x, v.y, fma(-u.y, v.x, gi));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-        gr += __shfl_xor_sync(0xffffffffu, gr, o);
-        gi += __shfl_xor_sync(0xffffffffu, gi, o);
-    }
-    T cm1, sr, si, tg;
-    if (!rot_params_fast(a, b, gr, gi, tol2, zthr, cm1, sr, si, tg)) return 0;
-    // Each new element is x + d, where the small correction d = (c-1) x + ... is summed
-    // first and then added to x with a single rounding.  Near convergence |(c-1) x| is
-    // below half an ulp of x: added to an already rounded x + ... it would always round
-    // away, leaving c = 1 and growing the pair's norm by a factor 1 + t^2 per rotation (a
-    // systematic drift of the singular values in FP32).
-    for (int r = lane; r < m; r += 32) {
-        const C u = xi[r], v = xj[r];
-        C nu, nv;
-        // nu = c u - conj(s e) v = u + [(c-1) u - conj(s e) v]
-        nu.x = u.x + fma(-si, v.y, fma(-sr, v.x, cm1 * u.x));
-        nu.y = u.y + fma(si, v.x, fma(-sr, v.y, cm1 * u.y));
-        // nv = (s e) u + c v = v + [(c-1) v + (s e) u]
-        nv.x = v.x + fma(-si, u.y, fma(sr, u.x, cm1 * v.x));
-        nv.y = v.y + fma(si, u.x, fma(sr, u.y, cm1 * v.y));
-        xi[r] = nu;
-        xj[r] = nv;
-    }
-    return 1;
-}
+// One visit in FP32.  A pair belongs to a group of LP lanes, each holding RPL rows of a
+// column.  16 rows a lane up to m = 512 (LP = m / 16): the shuffles of the inner product
+// and the rotation parameters are then shared by 32 / LP pairs of a warp, and a CTA of
+// 16 LP threads leaves room for others on its SM that run while this one waits (with a
+// whole warp per pair these took ~110 of ~180 issue slots per pair and step at m = 128).
+// Shared memory holds a block as 16-byte units (two rows) [RPL / 2][BC columns][LP lanes],
+// rows padded with zeros to RPL LP: the accesses have constant offsets, no bounds and no
+// bank conflicts.
+// Block I's columns stay in registers over the BC rounds of the cross pairs; in the first
+// round of a sweep the pairs inside each block come first.  Column norms are tracked:
+// exact at the start of the visit, then a - t|g| and b + t|g| (the eigenvalues of the
+// pair's 2 x 2 Gram matrix).
+// Inner products and norms run over the first md rows (EXT: fewer than the stored m).
+template <int BC, int LP, int RPL, bool EXT>
+struct Visit32 {
+    static constexpr int U = RPL / 2, PITCH = BC * LP;      // units per lane and column; units per row of units
+    static constexpr int BLOCK = U * PITCH;                  // units of a block
+    float4 *XI, *XJ;                                         // the two blocks
+    int w, l, kd;   // this thread's group and lane, its units inside the first md rows
 
-// Rows owned by a lane in the register-resident layout: element k of a lane is row
-// 64 (k / 2) + 2 lane + (k % 2), so each lane moves two consecutive rows with one
-// 16-byte shared-memory access.
-__device__ __forceinline__ int reg_row(int lane, int k) { return 64 * (k >> 1) + 2 * lane + (k & 1); }
-
-// Rotation of a column pair whose first column lives in registers (layout above) and
-// whose second column lives in shared memory: the second column is read once, kept in
-// registers for the update and written back once (FULL: m == 32 * RPL, so no row needs
-// a bounds test).  The two column norms are tracked instead of recomputed: a (the
-// register column's, in a register) and *bj (the shared column's, in shared memory).
-// Only g = x_i^H x_j is formed; after a rotation the norms are a - t|g| and b + t|g|
-// (the eigenvalues of the pair's 2 x 2 Gram matrix).  The caller recomputes both
-// exactly when a visit starts, so the tracked values drift over at most BC rotations.
-template <typename T, typename C, int RPL, bool FULL, bool EXT>
-__device__ __forceinline__ int rotate_reg_tracked(C (&xi)[RPL], C* __restrict__ xjs, int m, int md, int lane, T tol2,
-                                                  T zthr, T& a, T* bj) {
-    C xj[RPL];
-    T gr = 0, gi = 0;
-#pragma unroll
-    for (int k = 0; k < RPL; k += 2) {
-        const int r = reg_row(lane, k);
-        if (FULL || r < m) {
-            if constexpr (sizeof(C) == 8) {
-                const float4 v = *reinterpret_cast<const float4*>(xjs + r);
-                xj[k].x = v.x; xj[k].y = v.y; xj[k + 1].x = v.z; xj[k + 1].y = v.w;
-            } else {
-                xj[k] = xjs[r];
-                xj[k + 1] = xjs[r + 1];
-            }
-        } else {
-            xj[k].x = 0; xj[k].y = 0; xj[k + 1].x = 0; xj[k + 1].y = 0;
-        }
-        if (EXT && r >= md) continue;
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const C u = xi[k + e], v = xj[k + e];
-            gr = fma(u.x, v.x, fma(u.y, v.y, gr));
-            gi = fma(u.x, v.y, fma(-u.y, v.x, gi));
-        }
+    __device__ __forceinline__ Visit32(float4* xi, float4* xj, int md)
+        : XI(xi), XJ(xj), w(threadIdx.x / LP), l(threadIdx.x % LP), kd((md / 2 - l + LP - 1) / LP) {}
+    // column c of the two blocks (c < 2 BC): this lane's first unit
+    __device__ __forceinline__ float4* unit(int c) const {
+        return (c >= BC ? XJ : XI) + (c & (BC - 1)) * LP + l;
     }
+    static __device__ __forceinline__ float sum(float v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        gr += __shfl_xor_sync(0xffffffffu, gr, o);
-        gi += __shfl_xor_sync(0xffffffffu, gi, o);
+        for (int o = LP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
     }
-    const T b = *bj;
-    T cm1, sr, si, tg;
-    if (!rot_params_fast(a, b, gr, gi, tol2, zthr, cm1, sr, si, tg)) return 0;
-    a -= tg;
-    __syncwarp();
-    if (lane == 0) *bj = b + tg;
+    __device__ __forceinline__ float norm2(int c) const {
+        const float4* p = unit(c);
+        float a = 0.f;
 #pragma unroll
-    for (int k = 0; k < RPL; k += 2) {
-        const int r = reg_row(lane, k);
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const C u = xi[k + e], v = xj[k + e];
-            C nu, nv;
-            nu.x = u.x + fma(-si, v.y, fma(-sr, v.x, cm1 * u.x));
-            nu.y = u.y + fma(si, v.x, fma(-sr, v.y, cm1 * u.y));
-            nv.x = v.x + fma(-si, u.y, fma(sr, u.x, cm1 * v.x));
-            nv.y = v.y + fma(si, u.x, fma(sr, u.y, cm1 * v.y));
-            xi[k + e] = nu;
-            xj[k + e] = nv;
+        for (int k = 0; k < U; ++k) {
+            const float4 x = p[k * PITCH];
+            if (!EXT || k < kd) a = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, a))));
         }
-        if (FULL || r < m) {
-            if constexpr (sizeof(C) == 8) {
-                *reinterpret_cast<float4*>(xjs + r) = make_float4(xj[k].x, xj[k].y, xj[k + 1].x, xj[k + 1].y);
-            } else {
-                xjs[r] = xj[k];
-                xjs[r + 1] = xj[k + 1];
+        return sum(a);
+    }
+    // x + d with the small correction d = (c-1) x + ... summed first and then added to x
+    // with a single rounding.  Near convergence |(c-1) x| is below half an ulp of x: added
+    // to an already rounded x + ... it would always round away, leaving c = 1 and growing
+    // the pair's norm by a factor 1 + t^2 per rotation (a systematic drift of the singular
+    // values in FP32).
+    static __device__ __forceinline__ void rot2(float& ax, float& ay, float& bx, float& by, float cm1, float sr,
+                                                float si) {
+        const float ux = ax, uy = ay, vx = bx, vy = by;
+        ax = ux + fmaf(-si, vy, fmaf(-sr, vx, cm1 * ux));
+        ay = uy + fmaf(si, vx, fmaf(-sr, vy, cm1 * uy));
+        bx = vx + fmaf(-si, uy, fmaf(sr, ux, cm1 * vx));
+        by = vy + fmaf(si, ux, fmaf(sr, uy, cm1 * vy));
+    }
+    // The pair of the register column u (norm a) and the shared column cv (norm b), which
+    // is read once and written back once; tg: a -> a - tg, b -> b + tg.
+    __device__ __forceinline__ bool rotate(float4 (&u)[U], int cv, bool act, float tol2, float zthr, float a, float b,
+                                           float& tg) const {
+        float4* p = unit(cv);
+        float4 v[U];
+        float gr = 0.f, gi = 0.f, hr = 0.f, hi = 0.f;   // two chains each: a chain of 2 RPL FMAs waits 4 cycles on each
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            v[k] = p[k * PITCH];
+            if (!EXT || k < kd) {
+                gr = fmaf(u[k].x, v[k].x, fmaf(u[k].y, v[k].y, gr));
+                gi = fmaf(u[k].x, v[k].y, fmaf(-u[k].y, v[k].x, gi));
+                hr = fmaf(u[k].z, v[k].z, fmaf(u[k].w, v[k].w, hr));
+                hi = fmaf(u[k].z, v[k].w, fmaf(-u[k].w, v[k].z, hi));
             }
         }
+        gr = sum(gr + hr);
+        gi = sum(gi + hi);
+        float cm1, sr, si;
+        if (!act || !rot_params_fast(a, b, gr, gi, tol2, zthr, cm1, sr, si, tg)) return false;
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            rot2(u[k].x, u[k].y, v[k].x, v[k].y, cm1, sr, si);
+            rot2(u[k].z, u[k].w, v[k].z, v[k].w, cm1, sr, si);
+            p[k * PITCH] = v[k];
+        }
+        return true;
     }
-    return 1;
-}
+    __device__ __forceinline__ void load(float4 (&u)[U], int c) const {
+        const float4* p = unit(c);
+#pragma unroll
+        for (int k = 0; k < U; ++k) u[k] = p[k * PITCH];
+    }
+    __device__ __forceinline__ void store(int c, const float4 (&u)[U]) const {
+        float4* p = unit(c);
+#pragma unroll
+        for (int k = 0; k < U; ++k) p[k * PITCH] = u[k];
+    }
 
-// squared norm of a register column (reg_row layout), summed over the warp; EXT: of its
-// first md rows only
-template <typename T, typename C, int RPL, bool EXT>
-__device__ __forceinline__ T reg_norm2(const C (&x)[RPL], int md, int lane) {
-    T a = 0;
-#pragma unroll
-    for (int k = 0; k < RPL; ++k)
-        if (!EXT || reg_row(lane, k) < md) a = fma(x[k].x, x[k].x, fma(x[k].y, x[k].y, a));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    return a;
-}
+    // exact norms of all columns, and the pairs inside both blocks (intra)
+    __device__ __forceinline__ void begin(int nI, int nJ, bool intra, float tol2, float zthr, float* __restrict__ nrm,
+                                          int& my_rot, int& my_vis) const {
+        const float na0 = norm2(w), nb0 = norm2(BC + w);
+        if (l == 0) {
+            nrm[w] = na0;
+            nrm[BC + w] = nb0;
+        }
+        __syncthreads();
+        if (!intra) return;
+        // pairs inside block I (the first half of the groups) and inside block J (the rest)
+        constexpr int half = BC / 2;
+        const int base = w < half ? 0 : BC, nblk = w < half ? nI : nJ;
+        float4 u[U];
+#pragma unroll 1
+        for (int t = 0; t < BC - 1; ++t) {
+            int a, b;
+            rr_pair(BC, t, w < half ? w : w - half, a, b);
+            const bool act = a < nblk && b < nblk;
+            a += base;
+            b += base;
+            load(u, a);
+            const float na = nrm[a], nb = nrm[b];
+            float tg;
+            const bool rot = rotate(u, b, act, tol2, zthr, na, nb, tg);
+            my_vis += act && l == 0;
+            __syncwarp();
+            if (rot) {
+                store(a, u);
+                if (l == 0) {
+                    ++my_rot;
+                    nrm[a] = na - tg;
+                    nrm[b] = nb + tg;
+                }
+            }
+            __syncthreads();
+        }
+    }
+
+    // The cross pairs: block I's columns in registers (u, loaded by the caller, and the
+    // caller's to store).  The CTA's groups form two halves, each with its own barrier: in
+    // the first BC / 2 rounds half h rotates I_h with J_h, in the others with the other half
+    // of J.  A half's loads, shuffles and parameters then run beside the other's updates
+    // (one barrier for all in every round: 50.2 against 43.6 ms for the chi 256 layer).
+    __device__ __forceinline__ void cross(float4 (&u)[U], int nI, int nJ, float tol2, float zthr,
+                                          float* __restrict__ nrm, int& my_rot, int& my_vis) const {
+        constexpr int H = BC / 2;
+        constexpr bool halves = H * LP % 32 == 0;   // named barriers count whole warps
+        const int h = w / H;
+        float a_i = nrm[w];
+#pragma unroll 1
+        for (int t = 0; t < BC; ++t) {
+            const int b = ((w + t) & (H - 1)) + H * (h ^ (t / H));
+            const bool act = w < nI && b < nJ;
+            const float nb = nrm[BC + b];
+            float tg;
+            const bool rot = rotate(u, BC + b, act, tol2, zthr, a_i, nb, tg);
+            my_vis += act && l == 0;
+            __syncwarp();
+            if (rot) {
+                a_i -= tg;
+                if (l == 0) {
+                    ++my_rot;
+                    nrm[BC + b] = nb + tg;
+                }
+            }
+            if (!halves || (t & (H - 1)) == H - 1) __syncthreads();
+            else asm volatile("bar.sync %0, %1;" ::"r"(1 + h), "n"(H * LP) : "memory");
+        }
+    }
+
+    // blocks in: 16-byte asynchronous copies (through L2, no registers held), every copy of
+    // both blocks in flight at once; zeros past the stored rows and columns.  The caller's
+    // barrier follows the wait.
+    __device__ __forceinline__ void copy_in(const float2* WI, int nI, const float2* WJ, int nJ, int m) const {
+        const int units = m / 2;
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        for (int c = warp; c < 2 * BC; c += nw) {
+            const int cc = c & (BC - 1);
+            const float2* src = (c < BC ? WI : WJ) + (size_t)cc * m;
+            const int have = cc < (c < BC ? nI : nJ) ? units : 0;
+            float4* dst = (c >= BC ? XJ : XI) + cc * LP;
+#pragma unroll 4
+            for (int i = lane; i < U * LP; i += 32) {
+                float4* p = dst + (i / LP) * PITCH + i % LP;
+                if (i < have) cp_async16(p, src + 2 * i);
+                else *p = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+    }
+    // blocks out (L2 stores), by the warps from warp0 on
+    __device__ __forceinline__ void copy_out(float2* WI, int nI, float2* WJ, int nJ, int m, int warp0) const {
+        const int units = m / 2;
+        const int warp = (int)(threadIdx.x >> 5) - warp0, lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5) - warp0;
+        for (int c = warp; c < nI + nJ; c += nw) {
+            const bool isI = c < nI;
+            const int cc = isI ? c : c - nI;
+            float4* dst = reinterpret_cast<float4*>((isI ? WI : WJ) + (size_t)cc * m);
+            const float4* src = (isI ? XI : XJ) + cc * LP;
+#pragma unroll 4
+            for (int i = lane; i < units; i += 32) __stcg(dst + i, src[(i / LP) * PITCH + i % LP]);
+        }
+    }
+};
 
 // shared-memory block back to W (L2 stores) by the threads from first_thread on
 template <typename C>
@@ -213,12 +291,13 @@ __device__ __forceinline__ void pair64(int t, int w, bool intra, int nI, int nJ,
     }
 }
 template <int BC>
-__device__ __forceinline__ void visit64(double2* __restrict__ X, int m, int nI, int nJ, bool intra, float tol,
+__device__ __forceinline__ void visit64(double2* __restrict__ XI, double2* __restrict__ XJ, int m, int nI, int nJ, bool intra, float tol,
                                         double zthr, double2* __restrict__ red, double* __restrict__ nrm,
                                         Par64* __restrict__ par, int& my_rot, int& my_vis) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto col = [&](int c) { return c < BC ? XI + (size_t)c * m : XJ + (size_t)(c - BC) * m; };
     for (int c = warp; c < 2 * BC; c += BC) {
-        const double2* x = X + (size_t)c * m;
+        const double2* x = col(c);
         double a = 0.0;
         if (c < BC ? c < nI : c - BC < nJ)
             for (int r = lane; r < m; r += 32) a = fma(x[r].x, x[r].x, fma(x[r].y, x[r].y, a));
@@ -227,13 +306,13 @@ __device__ __forceinline__ void visit64(double2* __restrict__ X, int m, int nI, 
         if (lane == 0) nrm[c] = a;
     }
     __syncthreads();
-    const int steps = (intra ? BC - 1 : 0) + (nJ > 0 ? BC : 0);
+    const int steps = (intra ? BC - 1 : 0) + (nI > 0 && nJ > 0 ? BC : 0);
     for (int t = 0; t < steps; ++t) {
         int ca, cb;
         bool act;
         pair64<BC>(t, warp, intra, nI, nJ, ca, cb, act);
-        double2* xa = X + (size_t)ca * m;
-        double2* xb = X + (size_t)cb * m;
+        double2* xa = col(ca);
+        double2* xb = col(cb);
         double2 g = make_double2(0.0, 0.0);
         if (act) {
 #pragma unroll 4
@@ -306,13 +385,15 @@ __device__ __forceinline__ void visit64(double2* __restrict__ X, int m, int nI, 
 // a CTA with nothing to claim only waits for work that running CTAs are doing.
 // EXT (FP32): the columns of the complex128 gates' preconditioner, [theta; I] in GateDesc::pre
 // (k_mixed.cu); rotated over all m + n rows, the inner products and norms over the first m.
-template <typename T, int BC, int RPL, int MINB, bool EXT>
-__global__ void __launch_bounds__(BC * 32, MINB)
+// LP, RPL: lanes per pair and rows per lane of the launch's largest m (FP32; 32 and 0 for FP64).
+template <typename T, int BC, int LP, int RPL, int MINB, bool EXT>
+__global__ void __launch_bounds__(BC * LP, MINB)
 k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in, int max_sweeps,
          JacobiCtl* __restrict__ ctl, unsigned spin_limit) {
     using C = typename CT<T>::type;
+    static_assert(BC * LP >= 64, "warp 0 claims while the others write back");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* X = reinterpret_cast<C*>(smem_raw);       // [2*BC][m], column-major
+    C* X = reinterpret_cast<C*>(smem_raw);       // FP64: [2*BC][m], column-major
     __shared__ int s_g, s_rnd, s_v, s_exit, s_rot, s_vis;
     __shared__ T s_bn[2 * BC];                   // tracked squared norms (FP32: of block J's columns; FP64: of both)
     __shared__ double2 s_red[sizeof(T) == 8 ? BC * kRed64 : 1];
@@ -414,94 +495,48 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
             rr_pair(P, round, v, I, J);
             if (I >= nb) { I = J; J = -1; }
             else if (J >= nb) J = -1;
-            if (J >= 0 && J < I) { const int t = I; I = J; J = t; }
         }
         const bool intra = (round == 0);
         int my_rot = 0, my_vis = 0;
         if (J >= 0 || intra) {
             const int colI = I * BC, nI = min(BC, n - colI);
             const int colJ = J >= 0 ? J * BC : 0, nJ = J >= 0 ? min(BC, n - colJ) : 0;
-            copy_blocks_in(X, Wm + (size_t)colI * m, nI * m, X + (size_t)BC * m, Wm + (size_t)colJ * m,
-                           J >= 0 ? nJ * m : 0);
+            using V32 = Visit32<BC, LP, RPL, EXT>;
+            float4* const xs = reinterpret_cast<float4*>(smem_raw);
+            const V32 vis(xs, xs + V32::BLOCK, md);
+            if constexpr (sizeof(T) == 8)
+                copy_blocks_in(X, Wm + (size_t)colI * m, nI * m, X + (size_t)BC * m, Wm + (size_t)colJ * m,
+                               J >= 0 ? nJ * m : 0);
+            else
+                vis.copy_in(Wm + (size_t)colI * m, nI, Wm + (size_t)colJ * m, nJ, m);
             __syncthreads();
-            if constexpr (sizeof(T) == 8) {
-                // a gate of one block runs all its sweeps in this visit
-                for (;;) {
-                    int rot = 0;
-                    visit64<BC>(X, m, nI, nJ, intra, (float)tol, zthr, s_red, s_bn, s_par, rot, my_vis);
-                    my_rot += rot;
-                    if (nb > 1) break;
-                    last_rot = __syncthreads_or(rot);
-                    if (!last_rot || ++sweep >= max_sweeps) break;
-                }
-            } else {
-            if (intra) {
-                // pairs inside block I (warps 0..BC/2-1) and inside block J (the rest)
-                for (int t = 0; t < BC - 1; ++t) {
-                    const int half = BC / 2;
-                    const int w = warp < half ? warp : warp - half;
-                    const int base = warp < half ? 0 : BC;
-                    const int nblk = warp < half ? nI : nJ;
-                    int a, b;
-                    rr_pair(BC, t, w, a, b);
-                    if (a < nblk && b < nblk) {
-                        my_vis += (lane == 0);
-                        my_rot += rotate_pair<T>(X + (size_t)(base + a) * m, X + (size_t)(base + b) * m,
-                                                 m, md, lane, tol2, zthr);
-                    }
-                    __syncthreads();
-                }
-            }
-            if (J >= 0) {
-                // cross pairs: warp w keeps column I_w in registers and meets every
-                // column of J once, J_{(w + sft) mod BC} in round sft
-                C xi[RPL];
-                const C* ci = X + (size_t)warp * m;
-#pragma unroll
-                for (int k = 0; k < RPL; ++k) {
-                    const int r = reg_row(lane, k);
-                    if (warp < nI && r < m) {
-                        xi[k] = ci[r];
-                    } else {
-                        xi[k].x = 0;
-                        xi[k].y = 0;
+            // a gate of one block runs all its sweeps in this visit
+            for (;;) {
+                int rot = 0;
+                if constexpr (sizeof(T) == 8) {
+                    visit64<BC>(X, X + (size_t)BC * m, m, nI, nJ, intra, (float)tol, zthr, s_red, s_bn, s_par, rot, my_vis);
+                } else {
+                    vis.begin(nI, nJ, intra, tol2, zthr, s_bn, rot, my_vis);
+                    if (nJ > 0) {
+                        float4 u[V32::U];
+                        vis.load(u, vis.w);
+                        vis.cross(u, nI, nJ, tol2, zthr, s_bn, rot, my_vis);
+                        vis.store(vis.w, u);
+                        __syncthreads();
                     }
                 }
-                const bool full = (m == 32 * RPL);
-                // exact norms at the start of the cross pairs: a of the register column,
-                // s_bn[w] of block J's column w
-                T a_i = reg_norm2<T, C, RPL, EXT>(xi, md, lane);
-                if (warp < nJ) {
-                    const C* cj = X + (size_t)(BC + warp) * m;
-                    T bn = 0;
-                    for (int r = lane; r < md; r += 32) bn = fma(cj[r].x, cj[r].x, fma(cj[r].y, cj[r].y, bn));
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) bn += __shfl_xor_sync(0xffffffffu, bn, o);
-                    if (lane == 0) s_bn[warp] = bn;
-                }
-                __syncthreads();
-                for (int sft = 0; sft < BC; ++sft) {
-                    const int b = (warp + sft) % BC;
-                    if (warp < nI && b < nJ) {
-                        my_vis += (lane == 0);
-                        C* xjs = X + (size_t)(BC + b) * m;
-                        my_rot += full ? rotate_reg_tracked<T, C, RPL, true, EXT>(xi, xjs, m, md, lane, tol2, zthr, a_i, &s_bn[b])
-                                       : rotate_reg_tracked<T, C, RPL, false, EXT>(xi, xjs, m, md, lane, tol2, zthr, a_i, &s_bn[b]);
-                    }
-                    __syncthreads();
-                }
-                C* co = X + (size_t)warp * m;
-#pragma unroll
-                for (int k = 0; k < RPL; ++k) {
-                    const int r = reg_row(lane, k);
-                    if (warp < nI && r < m) co[r] = xi[k];
-                }
-                __syncthreads();
-            }
+                my_rot += rot;
+                if (nb > 1) break;
+                last_rot = __syncthreads_or(rot);
+                if (!last_rot || ++sweep >= max_sweeps) break;
             }
             if (warp > 0) {
-                copy_block_out_from(Wm + (size_t)colI * m, X, nI * m, 32);
-                if (J >= 0) copy_block_out_from(Wm + (size_t)colJ * m, X + (size_t)BC * m, nJ * m, 32);
+                if constexpr (sizeof(T) == 8) {
+                    copy_block_out_from(Wm + (size_t)colI * m, X, nI * m, 32);
+                    if (J >= 0) copy_block_out_from(Wm + (size_t)colJ * m, X + (size_t)BC * m, nJ * m, 32);
+                } else {
+                    vis.copy_out(Wm + (size_t)colI * m, nI, Wm + (size_t)colJ * m, nJ, m, 1);
+                }
             }
         }
         // warp 0 claims the next visit while the other warps write the blocks back (a CTA
@@ -515,6 +550,8 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
             nxt_rnd = frnd;
             nxt_v = fv;
         }
+        my_rot = __reduce_add_sync(0xffffffffu, my_rot);
+        my_vis = __reduce_add_sync(0xffffffffu, my_vis);
         if (lane == 0 && my_rot) atomicAdd(&s_rot, my_rot);
         if (lane == 0 && my_vis) atomicAdd(&s_vis, my_vis);
         __threadfence();   // every thread's block stores before the report
@@ -555,18 +592,231 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
     }
 }
 
-template <typename T, int BC, int RPL, int MINB, bool EXT = false>
+// One thread-block cluster per gate: the whole iteration with the columns in (distributed)
+// shared memory.  In the persistent kernel a visit of a 128-row gate spends 12 k of its 40 k
+// cycles on the claim, the copies through L2, the fence, the report and waiting for the
+// round's other visits; a layer whose gates all fit on the GPU at once gains nothing from
+// its queue.  Here CTA v of the cluster is seat v of the tournament: in round r it holds the
+// blocks a = r + v and b = r - v modulo P - 1 (a = P - 1 and b = r for v = 0), rotates
+// their pairs as above, and passes a to seat v - 1 and b to seat v + 1 (a turns into seat
+// 0's b, the last seat's b into its own a) through distributed shared memory.  After the
+// P - 1 rounds of a sweep every block is back, and the seats' rotation counts decide
+// whether the iteration ends.  Seats beyond the gate's P / 2 only keep the barriers.
+//   FP32: three block slots; b stays in its slot, a's columns are in registers, so two slots
+// are free for the next round's blocks once every seat has loaded a (the first cluster
+// barrier of a round, arrived at early).  FP64: four slots, two free.
+template <typename T, int BC, int LP, int RPL, int MINB, bool EXT>
+__global__ void __launch_bounds__(BC * LP, MINB)
+k_jacobi_cl(const GateDesc* __restrict__ gd, double tol_in, int max_sweeps) {
+    using C = typename CT<T>::type;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ T s_n[2 * BC];
+    __shared__ double2 s_red[sizeof(T) == 8 ? BC * kRed64 : 1];
+    __shared__ Par64 s_par[sizeof(T) == 8 ? BC : 1];
+    __shared__ int s_cnt[2][8];      // the seats' rotations in this sweep, by parity of the sweep
+    __shared__ int s_rot, s_vis;
+    cg::cluster_group cl = cg::this_cluster();
+    const int seats = (int)cl.num_blocks(), v = (int)cl.block_rank();
+    const GateDesc& d = gd[blockIdx.x / seats];
+    GateOut* out = d.out;
+    if (EXT && out->finished) return;   // outside the preconditioner: the whole cluster leaves
+    const Tour tg = tour_of<BC>(d);
+    const int md = tg.m, n = tg.n, nb = tg.nb, P = tg.P, R = tg.R;
+    const int m = EXT ? md + n : md, last = P / 2 - 1;
+    C* Wm = EXT ? (C*)d.pre : (C*)d.W;
+    const double tol = tol_in > 0.0 ? tol_in
+                                    : (sizeof(T) == 4 ? 2.0 * Eps<T>::v : fmax(sqrt((double)md), 4.0) * Eps<T>::v);
+    const T tol2 = (T)(tol * tol);
+    double frob2 = out->frob2;
+    if (EXT) {
+        const double f = mix_scale(frob2);
+        frob2 *= f * f;
+    }
+    const T zthr = (T)(Eps<T>::v * Eps<T>::v * (double)max(md, n) * frob2);
+    const bool seat = v <= last;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) s_rot = s_vis = 0;
+
+    using V32 = Visit32<BC, LP, sizeof(T) == 4 ? RPL : 2, EXT>;
+    // a block slot in 16-byte units (a multiple of two elements: m is even)
+    const int slot_units = sizeof(T) == 4 ? V32::BLOCK : BC * m;
+    float4* const xs = reinterpret_cast<float4*>(smem_raw);
+    auto slot = [&](int k) { return xs + (size_t)k * slot_units; };
+    auto cols = [&](int b) { return b < nb ? min(BC, n - b * BC) : 0; };
+    // seats and slots of this CTA's outgoing blocks
+    const int to_a = v == 0 ? 0 : v - 1, to_b = v == last ? v : v + 1;
+    const bool a_stays_a = v != 1, b_turns_a = v == last && v > 0;
+    int sa = 1, sb = 0;                 // slots of a and b; FP64: pairs (0, 1) and (2, 3) in turn
+    int blk_a = P - 1, blk_b = 0;
+    if (v > 0) { blk_a = v; blk_b = P - 1 - v; }
+    if (seat) {
+        if constexpr (sizeof(T) == 4) {
+            V32(slot(sa), slot(sb), md)
+                .copy_in(Wm + (size_t)blk_a * BC * m, cols(blk_a), Wm + (size_t)blk_b * BC * m, cols(blk_b), m);
+        } else {
+            copy_blocks_in((C*)slot(sa), Wm + (size_t)blk_a * BC * m, cols(blk_a) * m, (C*)slot(sb),
+                           Wm + (size_t)blk_b * BC * m, cols(blk_b) * m);
+        }
+    }
+    cl.sync();   // every seat runs before anything is written into it
+    int sweep = 0, my_rot = 0, my_vis = 0, rs = 0;
+    for (;; ++sweep) {
+        int rot = 0;
+        for (int r = 0; r < R; ++r) {
+            int a = P - 1, b = r;
+            if (v > 0) {
+                a = (r + v) % (P - 1);
+                b = (r - v + P - 1) % (P - 1);
+            }
+            const int nA = seat ? cols(a) : 0, nB = seat ? cols(b) : 0;
+            if constexpr (sizeof(T) == 4) {
+                const V32 vis(slot(sa), slot(sb), md);
+                float4 u[V32::U];
+                const int na = (sb + 1) % 3, nbs = (sb + 2) % 3;   // slots of the next a and b
+                if (seat) {
+                    vis.begin(nA, nB, r == 0, tol2, zthr, s_n, rot, my_vis);
+                    vis.load(u, vis.w);
+                }
+                asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+                if (seat && nA > 0 && nB > 0) vis.cross(u, nA, nB, tol2, zthr, s_n, rot, my_vis);
+                __syncthreads();
+                if (r == R - 1) {
+                    // this seat's count, to every CTA
+                    const int wr = __reduce_add_sync(0xffffffffu, rot);
+                    if (lane == 0 && wr) atomicAdd(&s_rot, wr);
+                    __syncthreads();
+                    if (tid < seats) cl.map_shared_rank(&s_cnt[sweep & 1][v], tid)[0] = s_rot;
+                }
+                asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+                if (seat) {
+                    float4* da = cl.map_shared_rank(slot(a_stays_a ? na : nbs), to_a) + vis.w * LP + vis.l;
+#pragma unroll
+                    for (int k = 0; k < V32::U; ++k) da[k * V32::PITCH] = u[k];
+                    float4* db = cl.map_shared_rank(slot(b_turns_a ? na : nbs), to_b);
+                    const float4* src = slot(sb);
+#pragma unroll 4
+                    for (int i = tid; i < V32::BLOCK; i += BC * LP) db[i] = src[i];
+                }
+                sa = na;
+                sb = nbs;
+            } else {
+                const int na = (sa + 2) & 3, nbs = (sb + 2) & 3;
+                if (seat) {
+                    visit64<BC>((double2*)slot(sa), (double2*)slot(sb), m, nA, nB, r == 0, (float)tol, (double)zthr, s_red,
+                                (double*)s_n, s_par, rot, my_vis);
+                    float4* da = cl.map_shared_rank(slot(a_stays_a ? na : nbs), to_a);
+                    float4* db = cl.map_shared_rank(slot(b_turns_a ? na : nbs), to_b);
+                    const float4 *pa = slot(sa), *pb = slot(sb);
+#pragma unroll 2
+                    for (int i = tid; i < slot_units; i += BC * LP) {
+                        da[i] = pa[i];
+                        db[i] = pb[i];
+                    }
+                }
+                if (r == R - 1) {
+                    const int wr = __reduce_add_sync(0xffffffffu, rot);
+                    if (lane == 0 && wr) atomicAdd(&s_rot, wr);
+                    __syncthreads();
+                    if (tid < seats) cl.map_shared_rank(&s_cnt[sweep & 1][v], tid)[0] = s_rot;
+                }
+                sa = na;
+                sb = nbs;
+            }
+            __syncwarp();
+            cl.sync();   // the next round's blocks have arrived
+        }
+        my_rot += rot;
+        rs = 0;
+        for (int k = 0; k < seats; ++k) rs += s_cnt[sweep & 1][k];
+        __syncthreads();
+        if (tid == 0) s_rot = 0;
+        __syncthreads();
+        if (rs == 0 || sweep + 1 >= max_sweeps) break;
+    }
+    // every block is back at its first seat
+    if (seat) {
+        if constexpr (sizeof(T) == 4) {
+            V32(slot(sa), slot(sb), md)
+                .copy_out(Wm + (size_t)blk_a * BC * m, cols(blk_a), Wm + (size_t)blk_b * BC * m, cols(blk_b), m, 0);
+        } else {
+            copy_block_out_from(Wm + (size_t)blk_a * BC * m, (const C*)slot(sa), cols(blk_a) * m, 0);
+            copy_block_out_from(Wm + (size_t)blk_b * BC * m, (const C*)slot(sb), cols(blk_b) * m, 0);
+        }
+        if (!EXT) {
+            my_rot = __reduce_add_sync(0xffffffffu, my_rot);
+            my_vis = __reduce_add_sync(0xffffffffu, my_vis);
+            if (lane == 0 && my_rot) atomicAdd(&s_rot, my_rot);
+            if (lane == 0 && my_vis) atomicAdd(&s_vis, my_vis);
+            __syncthreads();
+            if (tid == 0) {
+                atomicAdd(&out->rotations, (unsigned long long)s_rot);
+                atomicAdd(&out->visits, (unsigned long long)s_vis);
+            }
+        }
+    }
+    if (v == 0 && tid == 0) {
+        out->sweeps = sweep + 1;
+        if (rs != 0 && out->status < 4) out->status = 4;
+        out->finished = 1;
+    }
+}
+
+constexpr size_t kOneCta = 116 << 10;   // dynamic shared memory that leaves no room for a second CTA
+
+// Launch k_jacobi_cl when all the gates' clusters are resident at once; *used tells.
+template <typename T, int BC, int LP, int RPL, int MINB, bool EXT = false>
+static cudaError_t launch_cl(const GateDesc* d, int n_gates, int m_max, int n_max, double tol, int max_sweeps,
+                             cudaStream_t s, bool* used) {
+    using C = typename CT<T>::type;
+    *used = false;
+    const int nb = (n_max + BC - 1) / BC;
+    int seats = 1;
+    while (2 * seats < nb) seats *= 2;
+    if (seats > 8) return cudaSuccess;
+    const auto kernel = k_jacobi_cl<T, BC, LP, RPL, MINB, EXT>;
+    const size_t smem = sizeof(T) == 4 ? (size_t)3 * BC * LP * RPL * sizeof(C) : (size_t)4 * BC * m_max * sizeof(C);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = seats;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(n_gates * seats));
+    cfg.blockDim = dim3(BC * LP);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int fit = 0, dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if (n_gates * seats <= sms && smem < kOneCta) {
+        // one CTA per SM, where every SM's pipes and schedulers are its own: the cluster
+        // scheduler otherwise packs two on an SM beside idle ones
+        cfg.dynamicSmemBytes = kOneCta;
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOneCta)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg)) != cudaSuccess) return e;
+        if (n_gates > fit) cfg.dynamicSmemBytes = smem;
+    }
+    if (n_gates > fit && (e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg)) != cudaSuccess) return e;
+    if (n_gates > fit) return cudaSuccess;
+    *used = true;
+    return cudaLaunchKernelEx(&cfg, kernel, d, tol, max_sweeps < 1 ? 1 : max_sweeps);
+}
+
+template <typename T, int BC, int LP, int RPL, int MINB, bool EXT = false>
 static cudaError_t launch_bc(const GateDesc* d, int n_gates, int n_lead, int m_max, int n_max, double tol,
                              int max_sweeps, JacobiCtl* ctl, cudaStream_t s, unsigned spin_limit) {
     using C = typename CT<T>::type;
-    const auto kernel = k_jacobi<T, BC, RPL, MINB, EXT>;
-    const size_t smem = (size_t)2 * BC * m_max * sizeof(C);
+    const auto kernel = k_jacobi<T, BC, LP, RPL, MINB, EXT>;
+    const size_t smem = sizeof(T) == 8 ? (size_t)2 * BC * m_max * sizeof(C) : (size_t)2 * BC * LP * RPL * sizeof(C);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, BC * 32, smem)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, BC * LP, smem)) != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorLaunchOutOfResources;
     // no more CTAs than visits that can run at once
     const int nb = (n_max + BC - 1) / BC;
@@ -575,16 +825,17 @@ static cudaError_t launch_bc(const GateDesc* d, int n_gates, int n_lead, int m_m
     if (grid > visits) grid = visits;
     if (grid < 1) grid = 1;
     const int lead = (n_lead < 1 || n_lead > n_gates) ? n_gates : n_lead;
-    kernel<<<(unsigned)grid, BC * 32, smem, s>>>(d, n_gates, lead, tol, max_sweeps < 1 ? 1 : max_sweeps, ctl,
+    kernel<<<(unsigned)grid, BC * LP, smem, s>>>(d, n_gates, lead, tol, max_sweeps < 1 ? 1 : max_sweeps, ctl,
                                                  spin_limit ? spin_limit : kSpinLimit);
     return cudaGetLastError();
 }
 
-// Block width BC and rows per lane RPL (= ceil(m_max / 32)) per precision: the two
-// staged blocks take 2 BC m_max elements of shared memory (at most 128 KB).  Two
+// Block width BC and lanes per pair LP per precision: the two staged blocks take
+// 2 BC m elements of shared memory (at most 128 KB), and the register columns leave
+// 16 warps per SM, in one CTA at m = 512 and in up to eight at m = 64.  Two
 // configurations per shape: cfg 0 -- wide blocks (fewer rounds per sweep); cfg 1 --
 // half-width blocks, more CTAs per SM (independent barriers, twice the rounds).  FP64
-// visits keep no column in registers (RPL has no meaning): 8-column blocks of up to 256
+// visits keep no column in registers: 8-column blocks of up to 256
 // rows let two or three CTAs share an SM's FP64 pipe and fill each other's waits.  Bit 1 of a
 // state's configuration (QR preconditioning, k_qr.cu) does not change this launch.
 // tnsim_autotune times every configuration on a real layer.
@@ -594,18 +845,32 @@ cudaError_t launch_jacobi(const GateDesc* d, int n_gates, int m_max, int n_max, 
                           unsigned spin_limit) {
     if (n_gates <= 0) return cudaSuccess;
     const bool narrow = (cfg & 1) != 0;
-#define TNSIM_JAC(BC, RPL, MINB) launch_bc<T, BC, RPL, MINB>(d, n_gates, n_lead, m_max, n_max, tol, max_sweeps, ctl, s, spin_limit)
+#define TNSIM_CL(BC, LP, RPL, MINB) launch_cl<T, BC, LP, RPL, MINB>(d, n_gates, m_max, n_max, tol, max_sweeps, s, &used)
+#define TNSIM_JAC(BC, LP, RPL, MINB) launch_bc<T, BC, LP, RPL, MINB>(d, n_gates, n_lead, m_max, n_max, tol, max_sweeps, ctl, s, spin_limit)
     if constexpr (sizeof(T) == 4) {
         if ((cfg & 4) && m_max <= jacobi_tc_max_rows())
             return launch_jacobi_tc(d, n_gates, n_lead, n_max, tol, max_sweeps, ctl, s, spin_limit);
-        if (m_max <= 64) return narrow ? TNSIM_JAC(8, 2, 2) : TNSIM_JAC(16, 2, 1);
-        if (m_max <= 128) return narrow ? TNSIM_JAC(8, 4, 2) : TNSIM_JAC(16, 4, 1);
-        if (m_max <= 256) return narrow ? TNSIM_JAC(8, 8, 2) : TNSIM_JAC(16, 8, 1);
-        if (m_max <= 512) return narrow ? TNSIM_JAC(8, 16, 2) : TNSIM_JAC(16, 16, 1);
-        return TNSIM_JAC(8, 32, 1);
+        if (!narrow) {
+            bool used = false;
+            cudaError_t e = cudaSuccess;
+            if (m_max <= 64) e = TNSIM_CL(16, 4, 16, 1);
+            else if (m_max <= 128) e = TNSIM_CL(16, 8, 16, 1);
+            else if (m_max <= 256) e = TNSIM_CL(16, 16, 16, 2);
+            if (e != cudaSuccess || used) return e;
+        }
+        if (m_max <= 64) return narrow ? TNSIM_JAC(8, 8, 16, 8) : TNSIM_JAC(16, 4, 16, 8);
+        if (m_max <= 128) return narrow ? TNSIM_JAC(8, 8, 16, 8) : TNSIM_JAC(16, 8, 16, 4);
+        if (m_max <= 256) return narrow ? TNSIM_JAC(8, 16, 16, 4) : TNSIM_JAC(16, 16, 16, 2);
+        if (m_max <= 512) return narrow ? TNSIM_JAC(8, 32, 16, 2) : TNSIM_JAC(16, 32, 16, 1);
+        return TNSIM_JAC(8, 32, 32, 1);
     } else {
-        if (m_max <= 512) return narrow ? TNSIM_JAC(4, 0, 2) : TNSIM_JAC(8, 0, 2);
-        return TNSIM_JAC(4, 0, 1);
+        if (!narrow && m_max <= 256) {
+            bool used = false;
+            const cudaError_t e = TNSIM_CL(8, 32, 0, 1);
+            if (e != cudaSuccess || used) return e;
+        }
+        if (m_max <= 512) return narrow ? TNSIM_JAC(4, 32, 0, 2) : TNSIM_JAC(8, 32, 0, 2);
+        return TNSIM_JAC(4, 32, 0, 1);
     }
 #undef TNSIM_JAC
 }
@@ -615,11 +880,20 @@ cudaError_t launch_jacobi_mix(const GateDesc* d, int n_gates, int mt_max, int n_
     if (n_gates <= 0) return cudaSuccess;
     // sweep cap: more than these do not make the preconditioner better
     constexpr int sweeps = 20;
-#define TNSIM_MIX(BC, RPL) launch_bc<float, BC, RPL, 1, true>(d, n_gates, n_lead, mt_max, n_max, kMixTol, sweeps, ctl, s, spin_limit)
-    if (mt_max <= 128) return TNSIM_MIX(16, 4);
-    if (mt_max <= 256) return TNSIM_MIX(16, 8);
-    if (mt_max <= 512) return TNSIM_MIX(16, 16);
-    return TNSIM_MIX(8, 32);
+#define TNSIM_MIXCL(BC, LP, RPL, MINB) launch_cl<float, BC, LP, RPL, MINB, true>(d, n_gates, mt_max, n_max, kMixTol, sweeps, s, &used)
+    bool used = false;
+    cudaError_t e = cudaSuccess;
+    if (mt_max <= 64) e = TNSIM_MIXCL(16, 4, 16, 1);
+    else if (mt_max <= 128) e = TNSIM_MIXCL(16, 8, 16, 1);
+    else if (mt_max <= 256) e = TNSIM_MIXCL(16, 16, 16, 1);
+    else if (mt_max <= 512) e = TNSIM_MIXCL(16, 32, 16, 1);
+    if (e != cudaSuccess || used) return e;
+#define TNSIM_MIX(BC, LP, RPL, MINB) launch_bc<float, BC, LP, RPL, MINB, true>(d, n_gates, n_lead, mt_max, n_max, kMixTol, sweeps, ctl, s, spin_limit)
+    if (mt_max <= 64) return TNSIM_MIX(16, 4, 16, 8);
+    if (mt_max <= 128) return TNSIM_MIX(16, 8, 16, 4);
+    if (mt_max <= 256) return TNSIM_MIX(16, 16, 16, 2);
+    if (mt_max <= 512) return TNSIM_MIX(16, 32, 16, 1);
+    return TNSIM_MIX(8, 32, 32, 1);
 #undef TNSIM_MIX
 }
 

@@ -36,7 +36,7 @@ def _chain(cl, cm, cr):
     return a + [cm] + b[::-1], len(a) - 1
 
 
-def _update(T, cl, cm, cr, chi, cfg, decay=0.0, seed=1):
+def _update(T, cl, cm, cr, chi, cfg, decay=0.0, seed=1, dtype=None):
     rng = np.random.default_rng(seed)
     dims, q = _chain(cl, cm, cr)
     sites = [(rng.standard_normal((dims[i], 2, dims[i + 1])) + 1j * rng.standard_normal((dims[i], 2, dims[i + 1])))
@@ -44,7 +44,7 @@ def _update(T, cl, cm, cr, chi, cfg, decay=0.0, seed=1):
     sites[q + 1] = sites[q + 1] * np.exp(-decay * np.arange(cm) / max(1, cm - 1))[:, None, None]
     n = len(sites)
     cap = max(chi, max(dims))
-    m = T.MPS(n, dtype=T.TNSIM_C128, chi_max=cap)
+    m = T.MPS(n, dtype=T.TNSIM_C128 if dtype is None else dtype, chi_max=cap)
     if any(d > c for d, c in zip(dims, [min(cap, 2 ** min(b, n - b)) for b in range(n + 1)])):
         pytest.skip("chain too short for these bonds")
     m.import_sites(sites)
