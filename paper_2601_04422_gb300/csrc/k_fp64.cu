@@ -23,74 +23,16 @@
 // Measured with the FP64 visit of k_jacobi.cu on 20 gates at m = n = 180: SVD 139 -> 29 ms
 // (12.2 -> 4.7 FP64 sweeps per gate; of the 29 ms, FP32 rotations 4.4, these products 2.1);
 // singular values 6e-16 (relative) from LAPACK's before and after.
+#include "tile16.cuh"
 #include "tnsim_internal.h"
 
 namespace tnsim {
 
 namespace {
 
-constexpr int GT = 16;             // tile edge and K step
-constexpr int GTHREADS = 64;       // 2 x 2 outputs per thread
-
-// acc += a b
-template <typename C>
-__device__ __forceinline__ void cmul_add(C& acc, const C& a, const C& b) {
-    acc.x = fma(a.x, b.x, acc.x);
-    acc.x = fma(-a.y, b.y, acc.x);
-    acc.y = fma(a.x, b.y, acc.y);
-    acc.y = fma(a.y, b.x, acc.y);
-}
-
-// 16 x 16 tile added to acc: A B over k < K, each K step summed by itself first (rounding
-// grows with sqrt(16 + K / 16) instead of sqrt(K), for 3 % more instructions): thread (rx, cy) holds rows ROW(rx, 0/1), columns cy and
-// cy + 8, with ROW(rx, i) = rx + 8 i, or 2 rx + i (PAIRED).  la(i, k) and lb(k, j) give the
-// operands' elements (zero outside them) for tile row i and tile column j; AK / BK: memory
-// runs along k (consecutive threads then load consecutive k).
-template <typename C, bool AK, bool BK, bool PAIRED, typename LA, typename LB>
-__device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[2][2]) {
-    __shared__ C As[GT][GT + 1], Bs[GT][GT + 1];
-    const int tid = threadIdx.x, rx = tid & 7, cy = tid >> 3;
-    for (int k0 = 0; k0 < K; k0 += GT) {
-#pragma unroll
-        for (int t = 0; t < GT * GT / GTHREADS; ++t) {
-            const int e = tid + GTHREADS * t, lo = e & (GT - 1), hi = e / GT;
-            C a, b;
-            a.x = a.y = b.x = b.y = 0;
-            if (k0 + (AK ? lo : hi) < K) a = la(AK ? hi : lo, k0 + (AK ? lo : hi));
-            if (k0 + (BK ? lo : hi) < K) b = lb(k0 + (BK ? lo : hi), BK ? hi : lo);
-            As[AK ? lo : hi][AK ? hi : lo] = a;
-            Bs[BK ? lo : hi][BK ? hi : lo] = b;
-        }
-        __syncthreads();
-        C part[2][2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) { part[i][j].x = 0; part[i][j].y = 0; }
-#pragma unroll 4
-        for (int kk = 0; kk < GT; ++kk) {
-            C a[2], b[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                a[i] = As[kk][PAIRED ? 2 * rx + i : rx + 8 * i];
-                b[i] = Bs[kk][cy + 8 * i];
-            }
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 2; ++j) cmul_add(part[i][j], a[i], b[j]);
-        }
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) { acc[i][j].x += part[i][j].x; acc[i][j].y += part[i][j].y; }
-        __syncthreads();
-    }
-}
-
 // ---------------------------------------------------------------------------
 // theta (see k_gemm.cu): 8 l x 8 r per CTA; tile rows (l, c), tile columns (d, r).
-__global__ void __launch_bounds__(GTHREADS) k_theta64(const GateDesc* __restrict__ gd) {
+__global__ void __launch_bounds__(TILE_THREADS) k_theta64(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.z];
     const int q = d.q;
     const int chiL = d.chi[q], chiM = d.chi[q + 1], chiR = d.chi[q + 2];
@@ -118,7 +60,7 @@ __global__ void __launch_bounds__(GTHREADS) k_theta64(const GateDesc* __restrict
     const double2* B = (const double2*)d.siteB;
     const int m = 2 * chiL;
     double2 acc[2][2] = {};
-    tile_product<double2, true, false, true>(
+    tile_product<double2, true, false, true, true, MulAdd>(
         chiM,
         [&](int i, int k) {
             const int row = 2 * l0 + i;
@@ -142,7 +84,7 @@ __global__ void __launch_bounds__(GTHREADS) k_theta64(const GateDesc* __restrict
 #pragma unroll
                 for (int c = 0; c < 2; ++c)
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) cmul_add(t, Gs[(2 * aa + bb) * 4 + 2 * c + e], acc[c][e]);
+                    for (int e = 0; e < 2; ++e) MulAdd::op(t, Gs[(2 * aa + bb) * 4 + 2 * c + e], acc[c][e]);
                 const size_t idx = (size_t)(bb * chiR + r) * m + 2 * l + aa;
                 Wm[idx] = t;
                 T0[idx] = t;
@@ -155,17 +97,17 @@ __global__ void __launch_bounds__(GTHREADS) k_theta64(const GateDesc* __restrict
 }
 
 // right site (see k_right in k_gemm.cu): R[j, col] = f_j sum_row conj(W[row, perm_j]) theta0[row, col]
-__global__ void __launch_bounds__(GTHREADS) k_right64(const GateDesc* __restrict__ gd) {
+__global__ void __launch_bounds__(TILE_THREADS) k_right64(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.z];
     const int q = d.q;
     const int m = 2 * d.chi[q], n = 2 * d.chi[q + 2], k = d.out->k;
     if (qr_active(d, m, n)) return;   // QR-preconditioned: k_right_pre (k_qr.cu)
-    const int c0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+    const int c0 = blockIdx.x * TILE, j0 = blockIdx.y * TILE;
     if (c0 >= n || j0 >= k) return;
-    __shared__ int pj[GT];
-    __shared__ double fj[GT];
+    __shared__ int pj[TILE];
+    __shared__ double fj[TILE];
     const int tid = threadIdx.x;
-    if (tid < GT) {
+    if (tid < TILE) {
         const int j = j0 + tid;
         const double s2j = j < k ? d.s2[j] : 0.0;
         pj[tid] = j < k ? d.perm[j] : -1;
@@ -178,7 +120,7 @@ __global__ void __launch_bounds__(GTHREADS) k_right64(const GateDesc* __restrict
     const int lk = d.canon ? *d.lam_k : 0;
     double2 acc[2][2] = {};
     // tile rows: columns of R (they run along its rows in memory); tile columns: rows j
-    tile_product<double2, true, true, false>(
+    tile_product<double2, true, true, false, true, MulAdd>(
         m,
         [&](int i, int row) {
             if (c0 + i >= n) return make_double2(0.0, 0.0);
@@ -247,7 +189,7 @@ __global__ void __launch_bounds__(256) k_mix_build(const GateDesc* __restrict__ 
 // E = I - V^H V (Hermitian: tiles on and above the diagonal, mirrored).  The first CTA of
 // a gate also readies its record for the FP64 launch: a sweep cap reached in FP32 is no
 // error, a timeout is.
-__global__ void __launch_bounds__(GTHREADS) k_mix_gram(const GateDesc* __restrict__ gd) {
+__global__ void __launch_bounds__(TILE_THREADS) k_mix_gram(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.z];
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
@@ -260,7 +202,7 @@ __global__ void __launch_bounds__(GTHREADS) k_mix_gram(const GateDesc* __restric
         o->claim = 0;
     }
     if (!mix_active(d, m, n)) return;
-    const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+    const int i0 = blockIdx.x * TILE, j0 = blockIdx.y * TILE;
     if (i0 >= n || j0 >= n || i0 > j0) return;
     const int mt = m + n;
     const float2* V = (const float2*)d.pre + m;
@@ -268,7 +210,7 @@ __global__ void __launch_bounds__(GTHREADS) k_mix_gram(const GateDesc* __restric
     // the diagonal sums start from -1: they end near 0, and the last roundings are small
     double2 acc[2][2] = {};
     if (i0 == j0 && (threadIdx.x & 7) == (threadIdx.x >> 3)) acc[0][0].x = acc[1][1].x = -1.0;
-    tile_product<double2, true, true, false>(
+    tile_product<double2, true, true, false, true, MulAdd>(
         n,
         [&](int i, int k) {
             if (i0 + i >= n) return make_double2(0.0, 0.0);
@@ -295,16 +237,16 @@ __global__ void __launch_bounds__(GTHREADS) k_mix_gram(const GateDesc* __restric
 }
 
 // F = E/2 + 3/8 E^2 (Hermitian)
-__global__ void __launch_bounds__(GTHREADS) k_mix_corr(const GateDesc* __restrict__ gd) {
+__global__ void __launch_bounds__(TILE_THREADS) k_mix_corr(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.z];
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
     if (!mix_active(d, m, n)) return;
-    const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+    const int i0 = blockIdx.x * TILE, j0 = blockIdx.y * TILE;
     if (i0 >= n || j0 >= n || i0 > j0) return;
     const double2* E = (const double2*)d.pre_x;
     double2* F = (double2*)d.pre_f;
     float2 acc[2][2] = {};
-    tile_product<float2, true, true, false>(
+    tile_product<float2, true, true, false, true, MulAdd>(
         n,
         [&](int i, int k) {   // E[i, k] = conj(E[k, i])
             if (i0 + i >= n) return make_float2(0.f, 0.f);
@@ -334,18 +276,18 @@ __global__ void __launch_bounds__(GTHREADS) k_mix_corr(const GateDesc* __restric
 
 // FIRST: X = W V; else W = X + X F
 template <bool FIRST>
-__global__ void __launch_bounds__(GTHREADS) k_mix_mul(const GateDesc* __restrict__ gd) {
+__global__ void __launch_bounds__(TILE_THREADS) k_mix_mul(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.z];
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
     if (!mix_active(d, m, n)) return;
-    const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+    const int i0 = blockIdx.x * TILE, j0 = blockIdx.y * TILE;
     if (i0 >= m || j0 >= n) return;
     const int mt = m + n;
     double2* X = (double2*)d.pre_x;
     double2* Wm = (double2*)d.W;
     const double2* A = FIRST ? Wm : X;
     double2 acc[2][2] = {};
-    tile_product<double2, false, true, false>(
+    tile_product<double2, false, true, false, true, MulAdd>(
         n,
         [&](int i, int k) { return i0 + i < m ? A[(size_t)k * m + i0 + i] : make_double2(0.0, 0.0); },
         [&](int k, int j) {
@@ -377,14 +319,14 @@ __global__ void __launch_bounds__(GTHREADS) k_mix_mul(const GateDesc* __restrict
 cudaError_t launch_theta64(const GateDesc* d, int n_gates, int chiL_max, int chiR_max, cudaStream_t s) {
     if (n_gates <= 0) return cudaSuccess;
     dim3 grid((chiL_max + 7) / 8, (chiR_max + 7) / 8, n_gates);
-    k_theta64<<<grid, GTHREADS, 0, s>>>(d);
+    k_theta64<<<grid, TILE_THREADS, 0, s>>>(d);
     return cudaGetLastError();
 }
 
 cudaError_t launch_right64(const GateDesc* d, int n_gates, int k_max, int n_max, cudaStream_t s) {
     if (n_gates <= 0) return cudaSuccess;
-    dim3 grid((n_max + GT - 1) / GT, (k_max + GT - 1) / GT, n_gates);
-    k_right64<<<grid, GTHREADS, 0, s>>>(d);
+    dim3 grid((n_max + TILE - 1) / TILE, (k_max + TILE - 1) / TILE, n_gates);
+    k_right64<<<grid, TILE_THREADS, 0, s>>>(d);
     return cudaGetLastError();
 }
 
@@ -399,11 +341,11 @@ cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, Jac
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_jacobi_mix(d, n_gates, mt, nm, ctl, s, n_lead, spin_limit);
     if (e != cudaSuccess) return e;
-    const int tn = (nm + GT - 1) / GT, tm = (mm + GT - 1) / GT;
-    k_mix_gram<<<dim3(tn, tn, n_gates), GTHREADS, 0, s>>>(d);
-    k_mix_corr<<<dim3(tn, tn, n_gates), GTHREADS, 0, s>>>(d);
-    k_mix_mul<true><<<dim3(tm, tn, n_gates), GTHREADS, 0, s>>>(d);
-    k_mix_mul<false><<<dim3(tm, tn, n_gates), GTHREADS, 0, s>>>(d);
+    const int tn = (nm + TILE - 1) / TILE, tm = (mm + TILE - 1) / TILE;
+    k_mix_gram<<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
+    k_mix_corr<<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
+    k_mix_mul<true><<<dim3(tm, tn, n_gates), TILE_THREADS, 0, s>>>(d);
+    k_mix_mul<false><<<dim3(tm, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     return cudaGetLastError();
 }
 

@@ -1285,62 +1285,122 @@ tnsim_status tnsim_expect_pauli(tnsim_mps* m, int32_t n_terms, const char* pauli
     if (s != TNSIM_OK) return s;
     int chi_cap = 1;
     for (int b = 0; b <= n; ++b) chi_cap = std::max(chi_cap, m->ub[b]);
-    const size_t env = (size_t)chi_cap * chi_cap * m->esz;
+    const size_t es = m->esz, env = (size_t)chi_cap * chi_cap * es;
     // operators: I, X, Y, Z as 2x2 complex128
     const double ops[4][8] = {{1, 0, 0, 0, 0, 0, 1, 0},
                               {0, 0, 1, 0, 1, 0, 0, 0},
                               {0, 0, 0, -1, 0, 1, 0, 0},
                               {1, 0, 0, 0, 0, 0, -1, 0}};
-    char* d_L = nullptr; char* d_R = nullptr; char* d_tmp = nullptr; char* d_E = nullptr;
-    double* d_ops = nullptr; double* d_res = nullptr;
-    cudaError_t e = cudaMalloc((void**)&d_L, env * (n + 1));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_R, env * (n + 1));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_tmp, env * 2);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_E, env * 2);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_ops, sizeof(ops));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_res, sizeof(double) * 2 * n_terms);
-    if (e == cudaSuccess) e = cudaMemcpy(d_ops, ops, sizeof(ops), cudaMemcpyHostToDevice);
-    // identity boundary environments: L_0 = [[1]], R_n = [[1]]
-    std::vector<char> one(m->esz, 0);
-    if (m->dt == TNSIM_C64) { float f = 1.0f; std::memcpy(one.data(), &f, 4); }
-    else { double f = 1.0; std::memcpy(one.data(), &f, 8); }
-    if (e == cudaSuccess) e = cudaMemcpy(d_L, one.data(), m->esz, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(d_R + env * n, one.data(), m->esz, cudaMemcpyHostToDevice);
-    auto transfer = [&](int q, int op, const char* ein, char* eout, int left) -> cudaError_t {
-        return (m->dt == TNSIM_C64)
-                   ? launch_transfer<float>(site_ptr(m, q), m->d_chi, q, d_ops + 8 * op, ein, d_tmp, eout,
-                                            chi_cap, left, m->stream)
-                   : launch_transfer<double>(site_ptr(m, q), m->d_chi, q, d_ops + 8 * op, ein, d_tmp, eout,
-                                             chi_cap, left, m->stream);
-    };
-    for (int q = 0; q < n && e == cudaSuccess; ++q) e = transfer(q, 0, d_L + env * q, d_L + env * (q + 1), 1);
-    for (int q = n - 1; q >= 0 && e == cudaSuccess; --q) e = transfer(q, 0, d_R + env * (q + 1), d_R + env * q, 0);
-    for (int t = 0; t < n_terms && e == cudaSuccess; ++t) {
+    auto opi = [](char c) { return c == 'I' ? 0 : c == 'X' ? 1 : c == 'Y' ? 2 : 3; };
+    // the support [a, b] of every term (the identity: a = n, closed at the right end)
+    struct Sup { int a, b; };
+    std::vector<Sup> sup(n_terms);
+    int l_need = 0, r_need = n;
+    for (int t = 0; t < n_terms; ++t) {
         const char* ps = paulis + (size_t)t * n;
-        int a = -1, b = -1;
+        int a = n, b = n - 1;
         for (int q = 0; q < n; ++q)
-            if (ps[q] != 'I') { if (a < 0) a = q; b = q; }
-        auto opi = [](char c) { return c == 'I' ? 0 : c == 'X' ? 1 : c == 'Y' ? 2 : 3; };
-        if (a < 0) {
-            e = (m->dt == TNSIM_C64) ? launch_close<float>(d_L + env * n, d_R + env * n, m->d_chi, n, d_res + 2 * t, m->stream)
-                                     : launch_close<double>(d_L + env * n, d_R + env * n, m->d_chi, n, d_res + 2 * t, m->stream);
-            continue;
-        }
-        const char* cur = d_L + env * a;
-        int pp = 0;
-        for (int q = a; q <= b && e == cudaSuccess; ++q) {
-            char* dst = d_E + env * pp;
-            e = transfer(q, opi(ps[q]), cur, dst, 1);
-            cur = dst;
-            pp ^= 1;
-        }
-        if (e == cudaSuccess)
-            e = (m->dt == TNSIM_C64) ? launch_close<float>(cur, d_R + env * (b + 1), m->d_chi, b + 1, d_res + 2 * t, m->stream)
-                                     : launch_close<double>(cur, d_R + env * (b + 1), m->d_chi, b + 1, d_res + 2 * t, m->stream);
+            if (ps[q] != 'I') { if (a == n) a = q; b = q; }
+        sup[t] = {a, b};
+        l_need = std::max(l_need, a);
+        r_need = std::min(r_need, b + 1);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
-    if (e == cudaSuccess) e = cudaMemcpy(out, d_res, sizeof(double) * 2 * n_terms, cudaMemcpyDeviceToHost);
-    cudaFree(d_L); cudaFree(d_R); cudaFree(d_tmp); cudaFree(d_E); cudaFree(d_ops); cudaFree(d_res);
+    // One allocation: the environments L_0..L_n and R_0..R_n, two scratch buffers of the
+    // chains, per term of a batch two running environments and a scratch buffer, and the
+    // lists of the steps.  Terms of a batch advance together, one site per launch.
+    const int batch = (int)std::min<size_t>(n_terms, std::max<size_t>(1, ((size_t)256 << 20) / (4 * env)));
+    size_t off = 0;
+    auto take = [&](size_t bytes) { const size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
+    const size_t o_L = take(env * (n + 1)), o_R = take(env * (n + 1)), o_tmp = take(env * 4), o_ops = take(sizeof(ops));
+    const size_t o_term = take(env * 4 * batch), o_parts = take(sizeof(double) * 2 * CLOSE_PARTS * n_terms);
+    const size_t o_res = take(sizeof(double) * 2 * n_terms);
+    size_t n_steps = 2 * (size_t)n;
+    for (int t0 = 0; t0 < n_terms; t0 += batch) {
+        int len = 0;
+        for (int t = t0; t < std::min(n_terms, t0 + batch); ++t) len = std::max(len, sup[t].b - sup[t].a + 1);
+        n_steps += (size_t)len * batch;
+    }
+    const size_t o_list = take(sizeof(TransferDesc) * n_steps), o_close = take(sizeof(CloseDesc) * n_terms);
+    char* base = nullptr;
+    CUDA_TRY(cudaMalloc((void**)&base, off));
+    char *d_L = base + o_L, *d_R = base + o_R;
+    const double* d_ops = (const double*)(base + o_ops);
+    std::vector<TransferDesc> list(n_steps);
+    std::vector<CloseDesc> closes(n_terms);
+    // both chains at once: step i takes L_i to L_{i+1} and R_{n-i} to R_{n-i-1}
+    for (int i = 0; i < n; ++i) {
+        const int q = n - 1 - i;
+        list[2 * i] = {i < l_need ? site_ptr(m, i) : nullptr, m->d_chi, d_ops, d_L + env * i, base + o_tmp,
+                       d_L + env * (i + 1), i, 1};
+        list[2 * i + 1] = {q >= r_need ? site_ptr(m, q) : nullptr, m->d_chi, d_ops, d_R + env * (q + 1),
+                           base + o_tmp + 2 * env, d_R + env * q, q, 0};
+    }
+    std::vector<std::pair<size_t, int>> launches;   // (first step of the list, how many)
+    size_t pos = 2 * (size_t)n;
+    for (int t0 = 0; t0 < n_terms; t0 += batch) {
+        const int nb = std::min(batch, n_terms - t0);
+        int len = 0;
+        for (int t = t0; t < t0 + nb; ++t) len = std::max(len, sup[t].b - sup[t].a + 1);
+        for (int step = 0; step < len; ++step) {
+            for (int t = t0; t < t0 + nb; ++t) {
+                char* buf = base + o_term + env * 4 * (t - t0);
+                const int q = sup[t].a + step;
+                TransferDesc& d = list[pos + (t - t0)];
+                d = {nullptr, m->d_chi, nullptr, nullptr, buf + 2 * env, buf + env * (step & 1), q, 1};
+                if (q > sup[t].b) continue;
+                d.site = site_ptr(m, q);
+                d.op = d_ops + 8 * opi(paulis[(size_t)t * n + q]);
+                d.e_in = step == 0 ? d_L + env * q : buf + env * ((step - 1) & 1);
+            }
+            launches.push_back({pos, nb});
+            pos += nb;
+        }
+        for (int t = t0; t < t0 + nb; ++t) {
+            const int steps = sup[t].b - sup[t].a + 1;
+            const char* buf = base + o_term + env * 4 * (t - t0);
+            closes[t] = {steps > 0 ? (const void*)(buf + env * ((steps - 1) & 1)) : (const void*)(d_L + env * n),
+                         d_R + env * (sup[t].b + 1), m->d_chi, sup[t].b + 1, 0};
+        }
+        launches.push_back({(size_t)t0, -nb});   // close this batch's terms
+    }
+    cudaStream_t st = m->stream;
+    const bool c64 = m->dt == TNSIM_C64;
+    // identity boundary environments: L_0 = [[1]], R_n = [[1]]
+    std::vector<char> one(es, 0);
+    if (c64) { float f = 1.0f; std::memcpy(one.data(), &f, 4); }
+    else { double f = 1.0; std::memcpy(one.data(), &f, 8); }
+    cudaError_t e = cudaMemcpyAsync(base + o_ops, ops, sizeof(ops), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_L, one.data(), es, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_R + env * n, one.data(), es, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(base + o_list, list.data(), sizeof(TransferDesc) * n_steps, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(base + o_close, closes.data(), sizeof(CloseDesc) * n_terms, cudaMemcpyHostToDevice, st);
+    const TransferDesc* dl = (const TransferDesc*)(base + o_list);
+    const CloseDesc* dc = (const CloseDesc*)(base + o_close);
+    double* parts = (double*)(base + o_parts);
+    double* res = (double*)(base + o_res);
+    auto steps = [&](size_t first, int count) {
+        return c64 ? launch_transfers<float>(dl + first, TransferDesc{}, count, chi_cap, st)
+                   : launch_transfers<double>(dl + first, TransferDesc{}, count, chi_cap, st);
+    };
+    for (int i = 0; i < n && e == cudaSuccess; ++i)
+        if (i < l_need || n - 1 - i >= r_need) e = steps(2 * (size_t)i, 2);
+    for (const auto& l : launches) {
+        if (e != cudaSuccess) break;
+        if (l.second > 0) {
+            e = steps(l.first, l.second);
+        } else {
+            const size_t t0 = l.first;
+            double* p = parts + 2 * CLOSE_PARTS * t0;
+            e = c64 ? launch_close<float>(dc + t0, -l.second, p, res + 2 * t0, st)
+                    : launch_close<double>(dc + t0, -l.second, p, res + 2 * t0, st);
+        }
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out, res, sizeof(double) * 2 * n_terms, cudaMemcpyDeviceToHost, st);
+    const cudaError_t es2 = cudaStreamSynchronize(st);   // the host lists are read by the copies
+    if (e == cudaSuccess) e = es2;
+    cudaFree(base);
     if (e != cudaSuccess) return fail(TNSIM_ECUDA, std::string("expect_pauli: ") + cudaGetErrorString(e));
     return TNSIM_OK;
 }

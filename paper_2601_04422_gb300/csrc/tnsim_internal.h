@@ -211,9 +211,28 @@ template <typename T>
 cudaError_t launch_transfer(const void* site, const int* chi, int q, const double* op,
                             const void* e_in, void* tmp, void* e_out, int chi_cap,
                             int from_left, cudaStream_t s);
+// One transfer step (site null: none) and one closure, as lists in device memory
+struct TransferDesc {
+    const void* site;
+    const int* chi;
+    const double* op;     // 2 x 2 complex128
+    const void* e_in;
+    void* tmp;            // 2 chi_cap^2 elements
+    void* e_out;
+    int q, left;
+};
+struct CloseDesc {
+    const void* e;
+    const void* rt;
+    const int* chi;
+    int bond, pad_;
+};
+// count steps of list (or `one` when list is null), independent of one another
 template <typename T>
-cudaError_t launch_close(const void* E, const void* Rt, const int* chi, int bond, double* out,
-                         cudaStream_t s);
+cudaError_t launch_transfers(const TransferDesc* list, const TransferDesc& one, int count, int chi_cap, cudaStream_t s);
+constexpr int CLOSE_PARTS = 16;   // parts: count * CLOSE_PARTS * 2 doubles of scratch
+template <typename T>
+cudaError_t launch_close(const CloseDesc* list, int count, double* parts, double* out, cudaStream_t s);
 
 // Merge + gate contraction with FP32 3M arithmetic (SIMT).
 cudaError_t launch_theta_3m(const GateDesc* d, int n_gates, int chiL_max, int chiR_max, cudaStream_t s);
