@@ -3,9 +3,8 @@
 //
 // GB300 issues FP64 at 1/64 of the FP32 rate, so an FP64 kernel's time is its FP64
 // instruction count over the SMs that it keeps busy, and everything else hides behind
-// it.  The products therefore use small tiles (16 x 16 complex, 64 threads): with 64 x 64
-// tiles one SM per gate did the work at m = n <= 64 (theta 88 -> 23 us, right site
-// 136 -> 28 us per layer of 4-5 gates; 20 gates at m = 180: 480 -> 370 and 790 -> 420 us).
+// it.  The products therefore use 8 x 8 tiles (tile16.cuh): with 64 x 64 tiles one SM per
+// gate did the work at m = n <= 64 (THETA_FIG).
 //
 // Preconditioner (mixed-precision Jacobi SVD: Gao, Ma and Shao 2022).  One-sided Jacobi
 // converges quadratically, so 9 of its ~12 FP64 sweeps only bring the columns from O(1)
@@ -31,15 +30,17 @@ namespace tnsim {
 namespace {
 
 // ---------------------------------------------------------------------------
-// theta (see k_gemm.cu): 8 l x 8 r per CTA; tile rows (l, c), tile columns (d, r).
+// theta (see k_gemm.cu): 4 l x 4 r per CTA; tile rows (l, c), tile columns (d, r).
+constexpr int T64 = TileOf<double2>::E;   // 8
 __global__ void __launch_bounds__(TILE_THREADS) k_theta64(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.z];
     const int q = d.q;
     const int chiL = d.chi[q], chiM = d.chi[q + 1], chiR = d.chi[q + 2];
-    const int l0 = blockIdx.x * 8, r0 = blockIdx.y * 8;
+    constexpr int H = T64 / 2;
+    const int l0 = blockIdx.x * H, r0 = blockIdx.y * H;
     if (l0 >= chiL || r0 >= chiR) return;
-    __shared__ double2 Gs[16];
-    const int tid = threadIdx.x, rx = tid & 7, cy = tid >> 3;
+    __shared__ double2 Gs[16], S[T64][T64 + 1];
+    const int tid = threadIdx.x;
     if (tid < 16) {
         const int o = tid >> 2, i = tid & 3;
         double re = 0.0, im = 0.0;
@@ -59,37 +60,35 @@ __global__ void __launch_bounds__(TILE_THREADS) k_theta64(const GateDesc* __rest
     const double2* A = (const double2*)d.siteA;
     const double2* B = (const double2*)d.siteB;
     const int m = 2 * chiL;
-    double2 acc[2][2] = {};
-    tile_product<double2, true, false, true, true, MulAdd>(
+    double2 acc[1][1] = {};
+    tile_product<double2, true, false, false, true, MulAdd>(
         chiM,
         [&](int i, int k) {
             const int row = 2 * l0 + i;
             return row < m ? A[(size_t)row * chiM + k] : make_double2(0.0, 0.0);
         },
         [&](int k, int j) {
-            const int r = r0 + (j & 7);
-            return r < chiR ? B[((size_t)k * 2 + (j >> 3)) * chiR + r] : make_double2(0.0, 0.0);
+            const int r = r0 + j % H;
+            return r < chiR ? B[((size_t)k * 2 + j / H) * chiR + r] : make_double2(0.0, 0.0);
         },
         acc);
+    tile_share<double2, false>(S, acc);
     double2* Wm = (double2*)d.W;
     double2* T0 = (double2*)d.theta0;
     double fro = 0.0;
-    const int l = l0 + rx, r = r0 + cy;
+    // output (l, aa), (bb, r): the four merged entries of (l, r) mixed by the gate
+    const int i = tid & 7, j = tid >> 3, li = i >> 1, ri = j % H, aa = i & 1, bb = j / H;
+    const int l = l0 + li, r = r0 + ri;
     if (l < chiL && r < chiR) {
+        double2 t = make_double2(0.0, 0.0);
 #pragma unroll
-        for (int bb = 0; bb < 2; ++bb)
+        for (int c = 0; c < 2; ++c)
 #pragma unroll
-            for (int aa = 0; aa < 2; ++aa) {
-                double2 t = make_double2(0.0, 0.0);
-#pragma unroll
-                for (int c = 0; c < 2; ++c)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) MulAdd::op(t, Gs[(2 * aa + bb) * 4 + 2 * c + e], acc[c][e]);
-                const size_t idx = (size_t)(bb * chiR + r) * m + 2 * l + aa;
-                Wm[idx] = t;
-                T0[idx] = t;
-                fro = fma(t.x, t.x, fma(t.y, t.y, fro));
-            }
+            for (int e = 0; e < 2; ++e) MulAdd::op(t, Gs[(2 * aa + bb) * 4 + 2 * c + e], S[2 * li + c][e * H + ri]);
+        const size_t idx = (size_t)(bb * chiR + r) * m + 2 * l + aa;
+        Wm[idx] = t;
+        T0[idx] = t;
+        fro = fma(t.x, t.x, t.y * t.y);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, o);
@@ -102,12 +101,12 @@ __global__ void __launch_bounds__(TILE_THREADS) k_right64(const GateDesc* __rest
     const int q = d.q;
     const int m = 2 * d.chi[q], n = 2 * d.chi[q + 2], k = d.out->k;
     if (qr_active(d, m, n)) return;   // QR-preconditioned: k_right_pre (k_qr.cu)
-    const int c0 = blockIdx.x * TILE, j0 = blockIdx.y * TILE;
+    const int c0 = blockIdx.x * T64, j0 = blockIdx.y * T64;
     if (c0 >= n || j0 >= k) return;
-    __shared__ int pj[TILE];
-    __shared__ double fj[TILE];
+    __shared__ int pj[T64];
+    __shared__ double fj[T64];
     const int tid = threadIdx.x;
-    if (tid < TILE) {
+    if (tid < T64) {
         const int j = j0 + tid;
         const double s2j = j < k ? d.s2[j] : 0.0;
         pj[tid] = j < k ? d.perm[j] : -1;
@@ -118,7 +117,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_right64(const GateDesc* __rest
     const double2* Wm = (const double2*)d.W;
     const double2* T0 = (const double2*)d.theta0;
     const int lk = d.canon ? *d.lam_k : 0;
-    double2 acc[2][2] = {};
+    double2 acc[1][1] = {};
     // tile rows: columns of R (they run along its rows in memory); tile columns: rows j
     tile_product<double2, true, true, false, true, MulAdd>(
         m,
@@ -139,15 +138,8 @@ __global__ void __launch_bounds__(TILE_THREADS) k_right64(const GateDesc* __rest
         },
         acc);
     double2* R = (double2*)d.siteB;
-    const int rx = tid & 7, cy = tid >> 3;
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int jj = cy + 8 * j, col = c0 + rx + 8 * i;
-            if (j0 + jj < k && col < n)
-                R[(size_t)(j0 + jj) * n + col] = make_double2(acc[i][j].x * fj[jj], acc[i][j].y * fj[jj]);
-        }
+    const int jj = tid >> 3, col = c0 + (tid & 7);
+    if (j0 + jj < k && col < n) R[(size_t)(j0 + jj) * n + col] = make_double2(acc[0][0].x * fj[jj], acc[0][0].y * fj[jj]);
 }
 
 // ---------------------------------------------------------------------------
@@ -202,14 +194,14 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_gram(const GateDesc* __res
         o->claim = 0;
     }
     if (!mix_active(d, m, n)) return;
-    const int i0 = blockIdx.x * TILE, j0 = blockIdx.y * TILE;
+    const int i0 = blockIdx.x * T64, j0 = blockIdx.y * T64;
     if (i0 >= n || j0 >= n || i0 > j0) return;
     const int mt = m + n;
     const float2* V = (const float2*)d.pre + m;
     double2* E = (double2*)d.pre_x;
     // the diagonal sums start from -1: they end near 0, and the last roundings are small
-    double2 acc[2][2] = {};
-    if (i0 == j0 && (threadIdx.x & 7) == (threadIdx.x >> 3)) acc[0][0].x = acc[1][1].x = -1.0;
+    double2 acc[1][1] = {};
+    if (i0 == j0 && (threadIdx.x & 7) == (threadIdx.x >> 3)) acc[0][0].x = -1.0;
     tile_product<double2, true, true, false, true, MulAdd>(
         n,
         [&](int i, int k) {
@@ -223,25 +215,20 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_gram(const GateDesc* __res
             return make_double2((double)v.x, (double)v.y);
         },
         acc);
-    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
-#pragma unroll
-    for (int jj = 0; jj < 2; ++jj)
-#pragma unroll
-        for (int ii = 0; ii < 2; ++ii) {
-            const int i = i0 + rx + 8 * ii, j = j0 + cy + 8 * jj;
-            if (i >= n || j >= n) continue;
-            const double re = -acc[ii][jj].x, im = -acc[ii][jj].y;
-            E[(size_t)j * n + i] = make_double2(re, im);
-            if (i0 != j0) E[(size_t)i * n + j] = make_double2(re, -im);
-        }
+    const int i = i0 + (threadIdx.x & 7), j = j0 + (threadIdx.x >> 3);
+    if (i >= n || j >= n) return;
+    const double re = -acc[0][0].x, im = -acc[0][0].y;
+    E[(size_t)j * n + i] = make_double2(re, im);
+    if (i0 != j0) E[(size_t)i * n + j] = make_double2(re, -im);
 }
 
+constexpr int T32 = TileOf<float2>::E;    // 16
 // F = E/2 + 3/8 E^2 (Hermitian)
 __global__ void __launch_bounds__(TILE_THREADS) k_mix_corr(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.z];
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
     if (!mix_active(d, m, n)) return;
-    const int i0 = blockIdx.x * TILE, j0 = blockIdx.y * TILE;
+    const int i0 = blockIdx.x * T32, j0 = blockIdx.y * T32;
     if (i0 >= n || j0 >= n || i0 > j0) return;
     const double2* E = (const double2*)d.pre_x;
     double2* F = (double2*)d.pre_f;
@@ -280,13 +267,13 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_mul(const GateDesc* __rest
     const GateDesc& d = gd[blockIdx.z];
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
     if (!mix_active(d, m, n)) return;
-    const int i0 = blockIdx.x * TILE, j0 = blockIdx.y * TILE;
+    const int i0 = blockIdx.x * T64, j0 = blockIdx.y * T64;
     if (i0 >= m || j0 >= n) return;
     const int mt = m + n;
     double2* X = (double2*)d.pre_x;
     double2* Wm = (double2*)d.W;
     const double2* A = FIRST ? Wm : X;
-    double2 acc[2][2] = {};
+    double2 acc[1][1] = {};
     tile_product<double2, false, true, false, true, MulAdd>(
         n,
         [&](int i, int k) { return i0 + i < m ? A[(size_t)k * m + i0 + i] : make_double2(0.0, 0.0); },
@@ -297,35 +284,29 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_mul(const GateDesc* __rest
             return make_double2((double)v.x, (double)v.y);
         },
         acc);
-    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
-#pragma unroll
-    for (int jj = 0; jj < 2; ++jj)
-#pragma unroll
-        for (int ii = 0; ii < 2; ++ii) {
-            const int i = i0 + rx + 8 * ii, j = j0 + cy + 8 * jj;
-            if (i >= m || j >= n) continue;
-            const size_t idx = (size_t)j * m + i;
-            if (FIRST) {
-                X[idx] = acc[ii][jj];
-            } else {
-                const double2 x = X[idx];
-                Wm[idx] = make_double2(x.x + acc[ii][jj].x, x.y + acc[ii][jj].y);
-            }
-        }
+    const int i = i0 + (threadIdx.x & 7), j = j0 + (threadIdx.x >> 3);
+    if (i >= m || j >= n) return;
+    const size_t idx = (size_t)j * m + i;
+    if (FIRST) {
+        X[idx] = acc[0][0];
+    } else {
+        const double2 x = X[idx];
+        Wm[idx] = make_double2(x.x + acc[0][0].x, x.y + acc[0][0].y);
+    }
 }
 
 }  // namespace
 
 cudaError_t launch_theta64(const GateDesc* d, int n_gates, int chiL_max, int chiR_max, cudaStream_t s) {
     if (n_gates <= 0) return cudaSuccess;
-    dim3 grid((chiL_max + 7) / 8, (chiR_max + 7) / 8, n_gates);
+    dim3 grid((chiL_max + T64 / 2 - 1) / (T64 / 2), (chiR_max + T64 / 2 - 1) / (T64 / 2), n_gates);
     k_theta64<<<grid, TILE_THREADS, 0, s>>>(d);
     return cudaGetLastError();
 }
 
 cudaError_t launch_right64(const GateDesc* d, int n_gates, int k_max, int n_max, cudaStream_t s) {
     if (n_gates <= 0) return cudaSuccess;
-    dim3 grid((n_max + TILE - 1) / TILE, (k_max + TILE - 1) / TILE, n_gates);
+    dim3 grid((n_max + T64 - 1) / T64, (k_max + T64 - 1) / T64, n_gates);
     k_right64<<<grid, TILE_THREADS, 0, s>>>(d);
     return cudaGetLastError();
 }
@@ -341,9 +322,9 @@ cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, Jac
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_jacobi_mix(d, n_gates, mt, nm, ctl, s, n_lead, spin_limit);
     if (e != cudaSuccess) return e;
-    const int tn = (nm + TILE - 1) / TILE, tm = (mm + TILE - 1) / TILE;
+    const int tn = (nm + T64 - 1) / T64, tm = (mm + T64 - 1) / T64, tf = (nm + T32 - 1) / T32;
     k_mix_gram<<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
-    k_mix_corr<<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
+    k_mix_corr<<<dim3(tf, tf, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_mul<true><<<dim3(tm, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_mul<false><<<dim3(tm, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     return cudaGetLastError();

@@ -253,91 +253,103 @@ cudaError_t launch_amplitudes(void* const* sites, const int* chi, int n_qubits, 
 
 // ---------------------------------------------------------------------------
 // Transfer steps, two products each (d.left: from the left):
-//   left   tmp[x, (p', b)] = sum_y E[x, y] A[y, p', b]
-//          E'[a, b] = sum_{x,p} conj(A[x,p,a]) sum_{p'} O[p,p'] tmp[x, p', b]
+//   left   w[(x, p), b] = sum_{p'} O[p,p'] sum_y E[x, y] A[y, p', b]
+//          E'[a, b] = sum_{x,p} conj(A[x,p,a]) w[(x, p), b]
 //   right  (Rt[b][a] = R[a][b], a: bra, b: ket on bond q + 1)
-//          tmp[(y, p'), a] = sum_b A[y, p', b] Rt[b, a]
-//          Rt'[y, x] = sum_{a,p} conj(A[x,p,a]) sum_{p'} O[p,p'] tmp[y, p', a]
-// 16 x 16 tiles over a grid of (tiles, steps): a step's time is its latency, so small tiles
+//          w[y, (a, p)] = sum_{p'} O[p,p'] sum_b A[y, p', b] Rt[b, a]
+//          Rt'[y, x] = sum_{a,p} w[y, (a, p)] conj(A[x,p,a])
+// Small tiles over a grid of (tiles, steps): a step's time is its latency, so small tiles
 // over many SMs, and every step that does not depend on another in the same launch.  (One
 // thread per element, with its operands from L2 on every k: 21 + 38 us per step at chi 64,
-// against 4 + 4.)  The sums keep the order of that form, k ascending in one accumulator.
+// complex64, against TRANSFER_FIG.)  The sums keep the order of that form, k ascending in
+// one accumulator, then p'.  op null: w is the product itself, unmixed (tmp[(y, p'), a]).
 template <typename T>
 __global__ void __launch_bounds__(TILE_THREADS) k_transfer1(const TransferDesc* __restrict__ list, TransferDesc one) {
     using C = typename CT<T>::type;
+    constexpr int E = TileOf<C>::E, R = TileOf<C>::R, H = E / 2;
     const TransferDesc& d = list ? list[blockIdx.y] : one;
     if (!d.site) return;
     const int cl = d.chi[d.q], cr = d.chi[d.q + 1];
-    const int M = d.left ? cl : 2 * cl, N = d.left ? 2 * cr : cr, K = d.left ? cl : cr;
-    const int tn = (N + TILE - 1) / TILE, i0 = (int)(blockIdx.x / tn) * TILE, j0 = (int)(blockIdx.x % tn) * TILE;
-    if (i0 >= M) return;
-    const C* A = (const C*)(d.left ? d.e_in : d.site);   // M x K
-    const C* B = (const C*)(d.left ? d.site : d.e_in);   // K x N
-    C acc[2][2] = {};
-    tile_product<C, true, false, false, false, MulAdd>(
-        K,
-        [&](int i, int k) { return i0 + i < M ? A[(size_t)(i0 + i) * K + k] : C{}; },
-        [&](int k, int j) { return j0 + j < N ? B[(size_t)k * N + j0 + j] : C{}; }, acc);
+    // left: tile of E rows x and H columns b for both p'; right: H rows y for both p', E columns a
+    const int nx = d.left ? cl : cr, nh = d.left ? cr : cl, K = d.left ? cl : cr;
+    const int th = (nh + H - 1) / H, x0 = (int)(blockIdx.x / th) * E, h0 = (int)(blockIdx.x % th) * H;
+    if (x0 >= nx) return;
+    const C* site = (const C*)d.site;
+    const C* env = (const C*)d.e_in;
+    C acc[R][R] = {};
+    if (d.left)
+        tile_product<C, true, false, false, false, MulAdd>(
+            K, [&](int i, int k) { return x0 + i < cl ? env[(size_t)(x0 + i) * cl + k] : C{}; },
+            [&](int k, int j) {
+                const int b = h0 + j % H;
+                return b < cr ? site[((size_t)k * 2 + j / H) * cr + b] : C{};
+            },
+            acc);
+    else
+        tile_product<C, true, false, false, false, MulAdd>(
+            K,
+            [&](int i, int k) {
+                const int y = h0 + i % H;
+                return y < cl ? site[((size_t)y * 2 + i / H) * cr + k] : C{};
+            },
+            [&](int k, int j) { return x0 + j < cr ? env[(size_t)k * cr + x0 + j] : C{}; }, acc);
+    __shared__ C S[E][E + 1];
+    tile_share<C, false>(S, acc);
+    C o[4];
+    if (d.op) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { o[i].x = (T)d.op[2 * i]; o[i].y = (T)d.op[2 * i + 1]; }
+    }
     C* tmp = (C*)d.tmp;
-    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int r = i0 + rx + 8 * i, c = j0 + cy + 8 * j;
-            if (r < M && c < N) tmp[(size_t)r * N + c] = acc[i][j];
+    for (int e = threadIdx.x; e < E * E; e += TILE_THREADS) {
+        // p, index h of the halved side, index x of the full side; consecutive threads write
+        // consecutive elements
+        const int p = d.left ? e / H % 2 : d.op ? e % 2 : e / E % 2;
+        const int h = d.left ? e % H : e / (2 * E), x = d.left ? e / E : d.op ? e / 2 % E : e % E;
+        if (h0 + h >= nh || x0 + x >= nx) continue;
+        const C t0 = d.left ? S[x][h] : S[h][x], t1 = d.left ? S[x][H + h] : S[H + h][x];
+        C w = p ? t1 : t0;
+        if (d.op) {
+            w = C{};
+            MulAdd::op(w, p ? o[2] : o[0], t0);
+            MulAdd::op(w, p ? o[3] : o[1], t1);
         }
+        const size_t g = d.left ? ((size_t)(x0 + x) * 2 + p) * cr + h0 + h
+                         : d.op ? (size_t)(h0 + h) * 2 * cr + 2 * (x0 + x) + p
+                                : ((size_t)(h0 + h) * 2 + p) * cr + x0 + x;
+        tmp[g] = w;
+    }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(TILE_THREADS) k_transfer2(const TransferDesc* __restrict__ list, TransferDesc one) {
     using C = typename CT<T>::type;
+    constexpr int TE = TileOf<C>::E, R = TileOf<C>::R;
     const TransferDesc& d = list ? list[blockIdx.y] : one;
     if (!d.site) return;
     const int cl = d.chi[d.q], cr = d.chi[d.q + 1];
     const int M = d.left ? cr : cl, K = d.left ? 2 * cl : 2 * cr;   // M x M output
-    const int tn = (M + TILE - 1) / TILE, i0 = (int)(blockIdx.x / tn) * TILE, j0 = (int)(blockIdx.x % tn) * TILE;
+    const int tn = (M + TE - 1) / TE, i0 = (int)(blockIdx.x / tn) * TE, j0 = (int)(blockIdx.x % tn) * TE;
     if (i0 >= M) return;
     const C* A = (const C*)d.site;
-    const C* tmp = (const C*)d.tmp;
-    C o[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { o[i].x = (T)d.op[2 * i]; o[i].y = (T)d.op[2 * i + 1]; }
-    // w = sum_{p'} O[p, p'] t_{p'}
-    auto mix = [&](int p, const C& t0, const C& t1) {
-        C w = {};
-        MulAdd::op(w, p ? o[2] : o[0], t0);
-        MulAdd::op(w, p ? o[3] : o[1], t1);
-        return w;
-    };
-    C acc[2][2] = {};
-    if (d.left) {
+    const C* w = (const C*)d.tmp;
+    C acc[R][R] = {};
+    if (d.left)
         tile_product<C, false, false, false, false, ConjMulAdd>(
             K, [&](int i, int k) { return i0 + i < M ? A[(size_t)k * cr + i0 + i] : C{}; },
-            [&](int k, int j) {
-                if (j0 + j >= M) return C{};
-                const C* t = tmp + (size_t)(k >> 1) * 2 * cr + j0 + j;
-                return mix(k & 1, t[0], t[cr]);
-            },
-            acc);
-    } else {
+            [&](int k, int j) { return j0 + j < M ? w[(size_t)k * cr + j0 + j] : C{}; }, acc);
+    else
         tile_product<C, true, true, false, false, MulAddConj>(
-            K,
-            [&](int i, int k) {
-                if (i0 + i >= M) return C{};
-                const C* t = tmp + (size_t)(2 * (i0 + i)) * cr + (k >> 1);
-                return mix(k & 1, t[0], t[cr]);
-            },
+            K, [&](int i, int k) { return i0 + i < M ? w[(size_t)(i0 + i) * K + k] : C{}; },
             [&](int k, int j) { return j0 + j < M ? A[(size_t)(2 * (j0 + j) + (k & 1)) * cr + (k >> 1)] : C{}; }, acc);
-    }
-    C* E = (C*)d.e_out;
+    C* out = (C*)d.e_out;
     const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
+        for (int j = 0; j < R; ++j) {
             const int r = i0 + rx + 8 * i, c = j0 + cy + 8 * j;
-            if (r < M && c < M) E[(size_t)r * M + c] = acc[i][j];
+            if (r < M && c < M) out[(size_t)r * M + c] = acc[i][j];
         }
 }
 
@@ -345,9 +357,10 @@ template <typename T>
 cudaError_t launch_transfers(const TransferDesc* list, const TransferDesc& one, int count, int chi_cap,
                              cudaStream_t s) {
     if (count <= 0) return cudaSuccess;
-    const int t1 = (chi_cap + TILE - 1) / TILE, t2 = (2 * chi_cap + TILE - 1) / TILE;
-    k_transfer1<T><<<dim3(t1 * t2, count), TILE_THREADS, 0, s>>>(list, one);
-    k_transfer2<T><<<dim3(t1 * t1, count), TILE_THREADS, 0, s>>>(list, one);
+    constexpr int E = TileOf<typename CT<T>::type>::E;
+    const int te = (chi_cap + E - 1) / E, th = (chi_cap + E / 2 - 1) / (E / 2);
+    k_transfer1<T><<<dim3(te * th, count), TILE_THREADS, 0, s>>>(list, one);
+    k_transfer2<T><<<dim3(te * te, count), TILE_THREADS, 0, s>>>(list, one);
     return cudaGetLastError();
 }
 template <typename T>
@@ -361,8 +374,9 @@ template <typename T>
 cudaError_t launch_apply_rt(const void* site, const int* chi, int q, const void* rt, void* tmp, int chi_cap,
                             cudaStream_t s) {
     const TransferDesc one{site, chi, nullptr, rt, tmp, nullptr, q, 0};
-    const int t1 = (chi_cap + TILE - 1) / TILE, t2 = (2 * chi_cap + TILE - 1) / TILE;
-    k_transfer1<T><<<dim3(t1 * t2, 1), TILE_THREADS, 0, s>>>(nullptr, one);
+    constexpr int E = TileOf<typename CT<T>::type>::E;
+    const int te = (chi_cap + E - 1) / E, th = (chi_cap + E / 2 - 1) / (E / 2);
+    k_transfer1<T><<<dim3(te * th, 1), TILE_THREADS, 0, s>>>(nullptr, one);
     return cudaGetLastError();
 }
 template cudaError_t launch_apply_rt<float>(const void*, const int*, int, const void*, void*, int, cudaStream_t);

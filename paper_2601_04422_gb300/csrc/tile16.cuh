@@ -1,16 +1,20 @@
-// A 16 x 16 tile of a complex product by 64 threads, shared by the FP64 products
-// (k_fp64.cu) and the read-out (k_readout.cu).
+// A small tile of a complex product by 64 threads, shared by the FP64 products (k_fp64.cu)
+// and the read-out (k_readout.cu): 16 x 16 for complex64, 8 x 8 for complex128.
 //
-// Small tiles: FP64 issues at 1/64 of the FP32 rate, and the read-out's products are
-// chains of small matrices, so a tile's time is its latency and what counts is how many
-// SMs share a product.  The next K step's operands are loaded while this one's are used.
+// The read-out's products are chains of small matrices, so a tile's time is its latency and
+// what counts is how many SMs share a product.  FP64 issues once in 64 cycles per scheduler:
+// one output per thread is 4 FP64 instructions per k and warp, and small matrices spread
+// over as many schedulers as there are warps of outputs.  (2 x 2 outputs per thread: 13 us
+// for a 24 x 12 x 12 product, the zeros of the K step included, against 3.)
+// The next K step's operands are loaded while this one's are used.
 #pragma once
 #include <cuda_runtime.h>
 
 namespace tnsim {
 
-constexpr int TILE = 16;           // tile edge and K step
-constexpr int TILE_THREADS = 64;   // 2 x 2 outputs per thread
+constexpr int TILE_K = 16;         // K step
+constexpr int TILE_THREADS = 64;
+template <typename C> struct TileOf { static constexpr int E = sizeof(C) == 8 ? 16 : 8, R = E / 8; };   // edge, outputs per thread and side
 
 // acc += a b; acc += conj(a) b; acc += a conj(b) -- one fixed order of the roundings
 struct MulAdd {
@@ -36,58 +40,80 @@ struct MulAddConj {
 };
 
 // acc += sum over k < K of OP(la(i, k), lb(k, j)): thread (rx, cy) = (tid % 8, tid / 8)
-// holds rows rx + 8 i (PAIRED: 2 rx + i) and columns cy + 8 j.  la and lb give the
+// holds rows rx + 8 i (PAIRED: 2 rx + i) and columns cy + 8 j, i, j < R.  la and lb give the
 // operands' elements for tile row i / tile column j (zero outside them); AK / BK: memory
 // runs along k (consecutive threads then load consecutive k).  k ascends; SPLIT sums every
 // K step by itself first (rounding grows with sqrt(16 + K / 16) instead of sqrt(K), for
-// 3 % more instructions).
+// 3 - 6 % more instructions).
 template <typename C, bool AK, bool BK, bool PAIRED, bool SPLIT, typename OP, typename LA, typename LB>
-__device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[2][2]) {
-    constexpr int PER = TILE * TILE / TILE_THREADS;
-    __shared__ C As[TILE][TILE + 1], Bs[TILE][TILE + 1];
+__device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[TileOf<C>::R][TileOf<C>::R]) {
+    constexpr int E = TileOf<C>::E, R = TileOf<C>::R, PER = E * TILE_K / TILE_THREADS;
+    __shared__ C As[TILE_K][E + 1], Bs[TILE_K][E + 1];
     const int tid = threadIdx.x, rx = tid & 7, cy = tid >> 3;
     C na[PER], nb[PER];
+    // element e of a K step: (edge index, k) with k running fastest (KF) or slowest
+    auto at = [](int e, bool kf, int& i, int& k) {
+        if (kf) { k = e % TILE_K; i = e / TILE_K; }
+        else { i = e % E; k = e / E; }
+    };
     auto fetch = [&](int k0) {
 #pragma unroll
         for (int t = 0; t < PER; ++t) {
-            const int e = tid + TILE_THREADS * t, lo = e & (TILE - 1), hi = e / TILE;
+            int i, k;
             na[t].x = na[t].y = nb[t].x = nb[t].y = 0;
-            if (k0 + (AK ? lo : hi) < K) na[t] = la(AK ? hi : lo, k0 + (AK ? lo : hi));
-            if (k0 + (BK ? lo : hi) < K) nb[t] = lb(k0 + (BK ? lo : hi), BK ? hi : lo);
+            at(tid + TILE_THREADS * t, AK, i, k);
+            if (k0 + k < K) na[t] = la(i, k0 + k);
+            at(tid + TILE_THREADS * t, BK, i, k);
+            if (k0 + k < K) nb[t] = lb(k0 + k, i);
         }
     };
     fetch(0);
-    for (int k0 = 0; k0 < K; k0 += TILE) {
+    for (int k0 = 0; k0 < K; k0 += TILE_K) {
 #pragma unroll
         for (int t = 0; t < PER; ++t) {
-            const int e = tid + TILE_THREADS * t, lo = e & (TILE - 1), hi = e / TILE;
-            As[AK ? lo : hi][AK ? hi : lo] = na[t];
-            Bs[BK ? lo : hi][BK ? hi : lo] = nb[t];
+            int i, k;
+            at(tid + TILE_THREADS * t, AK, i, k);
+            As[k][i] = na[t];
+            at(tid + TILE_THREADS * t, BK, i, k);
+            Bs[k][i] = nb[t];
         }
         __syncthreads();
-        if (k0 + TILE < K) fetch(k0 + TILE);
-        C part[2][2] = {};
+        if (k0 + TILE_K < K) fetch(k0 + TILE_K);
+        C part[R][R] = {};
+        const int kn = min(TILE_K, K - k0);
 #pragma unroll 4
-        for (int kk = 0; kk < TILE; ++kk) {
-            C a[2], b[2];
+        for (int kk = 0; kk < kn; ++kk) {
+            C a[R], b[R];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                a[i] = As[kk][PAIRED ? 2 * rx + i : rx + 8 * i];
+            for (int i = 0; i < R; ++i) {
+                a[i] = As[kk][PAIRED ? R * rx + i : rx + 8 * i];
                 b[i] = Bs[kk][cy + 8 * i];
             }
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int j = 0; j < 2; ++j) OP::op(SPLIT ? part[i][j] : acc[i][j], a[i], b[j]);
+                for (int j = 0; j < R; ++j) OP::op(SPLIT ? part[i][j] : acc[i][j], a[i], b[j]);
         }
         if (SPLIT) {
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int j = 0; j < 2; ++j) { acc[i][j].x += part[i][j].x; acc[i][j].y += part[i][j].y; }
+                for (int j = 0; j < R; ++j) { acc[i][j].x += part[i][j].x; acc[i][j].y += part[i][j].y; }
         }
         __syncthreads();
     }
+}
+
+// The tile in shared memory, for outputs that mix entries of several threads.
+template <typename C, bool PAIRED>
+__device__ __forceinline__ void tile_share(C (*S)[TileOf<C>::E + 1], const C (&acc)[TileOf<C>::R][TileOf<C>::R]) {
+    constexpr int R = TileOf<C>::R;
+    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j) S[PAIRED ? R * rx + i : rx + 8 * i][cy + 8 * j] = acc[i][j];
+    __syncthreads();
 }
 
 }  // namespace tnsim
