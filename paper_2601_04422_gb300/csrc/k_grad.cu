@@ -2,7 +2,7 @@
 //
 // Conventions: for a complex intermediate X the kernels carry Xb = dE/d(conj X), so
 // that dE = 2 Re <Xb, dX>.  The forward is the library's own layer path; the
-// backward of one two-qubit update (k_gate_bwd, one CTA per gate) follows the
+// backward of one two-qubit update (k_gate_bwd, one cluster per gate) follows the
 // chain rule of its steps:
 //   right site c Y (Y = U^H T, c = |T|_F / |Y|_F):  Yb = c Bb - (dc c / 2K2) Y,
 //     dc = 2 Re <Bb, Y>, plus (dc c / 2F2) T into Tb;
@@ -16,15 +16,18 @@
 //     s_j <= sqrt(eps) s_max get no inverse factors (a pseudo-inverse cutoff);
 //   gate contraction theta = G (uL x uR) M and merge M = A B: the adjoints of the
 //     linear maps, and the 4 x 4 adjoint of G (uL x uR) for the one-qubit gates.
-// The final-state adjoint uses transfer-matrix environments (k_env_axpy,
-// k_site_adj2, k_adj_combine); k_rot_grad turns the 2 x 2 adjoints of every layer's
+// The final-state adjoint uses transfer-matrix environments (k_env_sum,
+// k_site_adj in k_readout.cu, k_adj_combine); k_rot_grad turns the 2 x 2 adjoints of every layer's
 // one-qubit gates into angle derivatives.
 #include <float.h>
 
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
 #include "tnsim_internal.h"
 
+namespace cg = cooperative_groups;
 namespace tnsim {
 
 namespace {
@@ -43,77 +46,71 @@ __device__ __forceinline__ void cmac(C& acc, const C& a, const C& b) {
     acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
 }
 
-// Operand of cta_gemm: element (i, j) = p[i * rs + j * cs], conjugated if conj.
+// Operand of cl_gemm: element (i, j) = p[i * rs + j * cs], conjugated if conj.  Read from
+// L2: other CTAs of the cluster write most operands between the cluster's barriers.
 template <typename C>
 struct Op {
     const C* p;
     int64_t rs, cs;
     bool conj;
     __device__ __forceinline__ C at(int i, int j) const {
-        C v = p[(int64_t)i * rs + (int64_t)j * cs];
+        C v = __ldcg(p + (int64_t)i * rs + (int64_t)j * cs);
         if (conj) v.y = -v.y;
         return v;
     }
 };
 
-constexpr int GT = 64, GK = 16;
+// Tile edge and K step.  One CTA of 256 threads per gate in 64 x 64 tiles of 4 x 4 outputs
+// issued the whole tile's FP64 instructions, mostly zeros, for a 24 x 24 block: 65 us per K
+// step (0.97 ms per gate).  A gate is a cluster of kBwdRanks CTAs now, in 16 x 16 tiles of
+// one output per thread.
+constexpr int GT = 16, GK = 16, kBwdRanks = 8;
+
+__device__ __forceinline__ void cluster_sync() {
+    __threadfence();
+    cg::this_cluster().sync();
+}
 
 // out(i, j) = alpha * sum_k a(i, k) b(k, j) (+ out(i, j) when acc), for i < M, j < N;
-// out element (i, j) at o[i * ors + j * ocs].  Whole CTA (256 threads), 64 x 64 tiles.
+// out element (i, j) at o[i * ors + j * ocs].  Whole cluster, tiles in turn; ends with the
+// cluster's barrier.
 template <typename T, typename C>
-__device__ void cta_gemm(int M, int N, int K, Op<C> a, Op<C> b, C* o, int64_t ors, int64_t ocs, T alpha, bool acc,
-                         C (*As)[GT + 1], C (*Bs)[GT]) {
+__device__ void cl_gemm(int M, int N, int K, Op<C> a, Op<C> b, C* o, int64_t ors, int64_t ocs, T alpha, bool acc,
+                        C (*As)[GT + 1], C (*Bs)[GT + 1], int rank) {
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int tm = (M + GT - 1) / GT, tn = (N + GT - 1) / GT;
-    for (int tile = 0; tile < tm * tn; ++tile) {
+    for (int tile = rank; tile < tm * tn; tile += kBwdRanks) {
         const int m0 = (tile / tn) * GT, n0 = (tile % tn) * GT;
-        C r[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) r[i][j] = cz<C>();
+        C r = cz<C>(), na, nb;
+        auto fetch = [&](int k0) {
+            na = (m0 + ty < M && k0 + tx < K) ? a.at(m0 + ty, k0 + tx) : cz<C>();   // row ty, k tx
+            nb = (k0 + ty < K && n0 + tx < N) ? b.at(k0 + ty, n0 + tx) : cz<C>();   // k ty, column tx
+        };
+        fetch(0);
         for (int k0 = 0; k0 < K; k0 += GK) {
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const int e = tid + 256 * t;
-                const int ii = e / GK, kk = e % GK;          // a: 64 rows x 16
-                As[kk][ii] = (m0 + ii < M && k0 + kk < K) ? a.at(m0 + ii, k0 + kk) : cz<C>();
-                const int kb = e / GT, jj = e % GT;          // b: 16 x 64 columns
-                Bs[kb][jj] = (k0 + kb < K && n0 + jj < N) ? b.at(k0 + kb, n0 + jj) : cz<C>();
-            }
+            As[tx][ty] = na;
+            Bs[ty][tx] = nb;
             __syncthreads();
+            if (k0 + GK < K) fetch(k0 + GK);
+            const int kn = min(GK, K - k0);
 #pragma unroll 4
-            for (int kk = 0; kk < GK; ++kk) {
-                C av[4], bv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) av[i] = As[kk][ty + 16 * i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) cmac(r[i][j], av[i], bv[j]);
-            }
+            for (int kk = 0; kk < kn; ++kk) cmac(r, As[kk][ty], Bs[kk][tx]);
             __syncthreads();
         }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int ii = m0 + ty + 16 * i;
-            if (ii >= M) continue;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int jj = n0 + tx + 16 * j;
-                if (jj >= N) continue;
-                C* dst = o + (int64_t)ii * ors + (int64_t)jj * ocs;
-                C v;
-                v.x = alpha * r[i][j].x;
-                v.y = alpha * r[i][j].y;
-                if (acc) { v.x += dst->x; v.y += dst->y; }
-                *dst = v;
+        if (m0 + ty < M && n0 + tx < N) {
+            C* dst = o + (int64_t)(m0 + ty) * ors + (int64_t)(n0 + tx) * ocs;
+            C v;
+            v.x = alpha * r.x;
+            v.y = alpha * r.y;
+            if (acc) {
+                const C w = __ldcg(dst);
+                v.x += w.x;
+                v.y += w.y;
             }
+            *dst = v;
         }
     }
-    __syncthreads();
+    cluster_sync();
 }
 
 // block-wide sum of n doubles per thread (n <= 32); result in out[] of every thread
@@ -136,19 +133,25 @@ __device__ void block_sum(double (&v)[NV], double* red /* NV * 32 */) {
     __syncthreads();
 }
 
-// The backward of one two-qubit update (one CTA of 256 threads per gate).
+// The backward of one two-qubit update (a cluster of kBwdRanks CTAs of 256 threads per gate).
 template <typename T>
 __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict__ gd) {
     using C = typename CT<T>::type;
-    const GradGateDesc& d = gd[blockIdx.x];
+    const GradGateDesc& d = gd[blockIdx.x / kBwdRanks];
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank();
     __shared__ C As[GK][GT + 1];
-    __shared__ C Bs[GK][GT];
-    __shared__ double red[32 * 32];
+    __shared__ C Bs[GK][GT + 1];
+    __shared__ double s_part[kBwdRanks][32];
+    __shared__ double red[8 * 32];
     __shared__ C Gt[16];
     __shared__ double s_sc[4];
     const int chiL = d.chiL, chiM = d.chiM, chiR = d.chiR, k = d.k;
     const int m = 2 * chiL, n = 2 * chiR;
     const int tid = threadIdx.x, nt = blockDim.x;
+    // of the cluster, for the elementwise passes; the mixing pass spreads its few elements
+    // over the ranks' schedulers (mid)
+    const int gid = rank * nt + tid, gn = kBwdRanks * nt, mid = tid * kBwdRanks + rank;
     const C* Tm = (const C*)d.theta0;        // column-major m x n
     const C* W = (const C*)d.W;              // column-major m x n
     const C* U = (const C*)d.u_post;         // m x k row-major
@@ -171,21 +174,31 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
     C* Mm = S + 7 * R;                       // m x n (merge)
     C* Mb = S + 8 * R;                       // m x n, or k x n
 
-    // scalars: k, norms, nonzero count, renormalisation
-    if (tid == 0) {
+    // scalars: k, norms, nonzero count, renormalisation (one warp: a thread's sum of n
+    // FP64 terms takes 64 n cycles)
+    if (tid < 32) {
         double f2 = 0.0, k2 = 0.0;
-        for (int j = 0; j < n; ++j) f2 += d.s2[j];
-        for (int j = 0; j < k; ++j) k2 += d.s2[j];
         const double thr = EpsG<T>::v * (double)max(m, n);
+        const double smax2 = d.s2[0], cut = thr * thr * smax2;
         int nz = 0;
-        const double smax2 = d.s2[0];
-        for (int j = 0; j < min(m, n); ++j)
-            if (d.s2[j] > thr * thr * smax2) nz = j + 1;
-        if (nz < k) nz = k;
-        s_sc[0] = f2;
-        s_sc[1] = k2;
-        s_sc[2] = (double)nz;
-        s_sc[3] = (d.renorm && k2 > 0.0) ? sqrt(f2 / k2) : 1.0;
+        for (int j = tid; j < n; j += 32) {
+            const double v = d.s2[j];
+            f2 += v;
+            if (j < k) k2 += v;
+            if (j < min(m, n) && v > cut) nz = j + 1;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            f2 += __shfl_xor_sync(0xffffffffu, f2, o);
+            k2 += __shfl_xor_sync(0xffffffffu, k2, o);
+            nz = max(nz, __shfl_xor_sync(0xffffffffu, nz, o));
+        }
+        if (tid == 0) {
+            s_sc[0] = f2;
+            s_sc[1] = k2;
+            s_sc[2] = (double)max(nz, k);
+            s_sc[3] = (d.renorm && k2 > 0.0) ? sqrt(f2 / k2) : 1.0;
+        }
     }
     __syncthreads();
     const double F2 = s_sc[0], K2 = s_sc[1], c = s_sc[3];
@@ -202,7 +215,7 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
     // Yb = c Bb - (dc c / 2K2) Y
     {
         const T a1 = (T)c, a2 = ren ? (T)(-dldc * c / (2.0 * K2) / c) : (T)0;
-        for (int i = tid; i < k * n; i += nt) {
+        for (int i = gid; i < k * n; i += gn) {
             const C b = Bb[i], y = cY[i];
             C v;
             v.x = a1 * b.x + a2 * y.x;
@@ -210,27 +223,29 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
             Yb[i] = v;
         }
     }
-    __syncthreads();
+    cluster_sync();
     // Tb = U Yb + (dc c / 2F2) T
-    cta_gemm<T, C>(m, n, k, Op<C>{U, k, 1, false}, Op<C>{Yb, n, 1, false}, Tb, n, 1, (T)1, false, As, Bs);
+    cl_gemm<T, C>(m, n, k, Op<C>{U, k, 1, false}, Op<C>{Yb, n, 1, false}, Tb, n, 1, (T)1, false, As, Bs, rank);
     if (ren) {
         const T a3 = (T)(dldc * c / (2.0 * F2));
-        for (int i = tid; i < m * n; i += nt) {
+        for (int i = gid; i < m * n; i += gn) {
             const int row = i / n, col = i % n;
             const C t = Tm[(size_t)col * m + row];
-            Tb[i].x += a3 * t.x;
-            Tb[i].y += a3 * t.y;
+            C v = __ldcg(Tb + i);
+            v.x += a3 * t.x;
+            v.y += a3 * t.y;
+            Tb[i] = v;
         }
-        __syncthreads();
+        cluster_sync();
     }
     // Ut = Ub + T Yb^H
-    for (int i = tid; i < m * k; i += nt) Ut[i] = Ub[i];
-    __syncthreads();
-    cta_gemm<T, C>(m, k, n, Op<C>{Tm, 1, m, false}, Op<C>{Yb, 1, n, true}, Ut, k, 1, (T)1, true, As, Bs);
+    for (int i = gid; i < m * k; i += gn) Ut[i] = Ub[i];
+    cluster_sync();
+    cl_gemm<T, C>(m, k, n, Op<C>{Tm, 1, m, false}, Op<C>{Yb, 1, n, true}, Ut, k, 1, (T)1, true, As, Bs, rank);
     const bool need_null = nz < m, need_disc = nz > k;
     if (need_null || need_disc) {
         // Ua[:, j] = W[:, perm[j]] / s_j for j < nz (column-major m x nz)
-        for (int i = tid; i < m * nz; i += nt) {
+        for (int i = gid; i < m * nz; i += gn) {
             const int j = i / m, row = i % m;
             const double s2j = d.s2[j];
             const T f = s2j > 0.0 ? (T)(1.0 / sqrt(s2j)) : (T)0;
@@ -239,21 +254,21 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
             w.y *= f;
             Ua[i] = w;
         }
-        __syncthreads();
+        cluster_sync();
         // Q1 = Ua^H Ut (nz x k)
-        cta_gemm<T, C>(nz, k, m, Op<C>{Ua, m, 1, true}, Op<C>{Ut, k, 1, false}, Q1, k, 1, (T)1, false, As, Bs);
+        cl_gemm<T, C>(nz, k, m, Op<C>{Ua, m, 1, true}, Op<C>{Ut, k, 1, false}, Q1, k, 1, (T)1, false, As, Bs, rank);
     }
     // directions below tau s_max get no inverse factors (pseudo-inverse cutoff, tau = sqrt(eps))
     const double tau2s = EpsG<T>::v * d.s2[0];
     if (need_null) {
         // (I - P) Ut = (I - P) Ub exactly ((I - P) T = 0); X1 = Ub - Ua (Ua^H Ub), then
         // Tb += X1 S_k^-2 Y.  Mb holds Ua^H Ub (nz x k) meanwhile.
-        cta_gemm<T, C>(nz, k, m, Op<C>{Ua, m, 1, true}, Op<C>{Ub, k, 1, false}, Mb, k, 1, (T)1, false, As, Bs);
-        for (int i = tid; i < m * k; i += nt) X1[i] = Ub[i];
-        __syncthreads();
-        cta_gemm<T, C>(m, k, nz, Op<C>{Ua, 1, m, false}, Op<C>{Mb, k, 1, false}, X1, k, 1, (T)-1, true, As, Bs);
+        cl_gemm<T, C>(nz, k, m, Op<C>{Ua, m, 1, true}, Op<C>{Ub, k, 1, false}, Mb, k, 1, (T)1, false, As, Bs, rank);
+        for (int i = gid; i < m * k; i += gn) X1[i] = Ub[i];
+        cluster_sync();
+        cl_gemm<T, C>(m, k, nz, Op<C>{Ua, 1, m, false}, Op<C>{Mb, k, 1, false}, X1, k, 1, (T)-1, true, As, Bs, rank);
         // X2 = S_k^-2 Y (k x n), Y = cY / c
-        for (int i = tid; i < k * n; i += nt) {
+        for (int i = gid; i < k * n; i += gn) {
             const int j = i / n;
             const T f = d.s2[j] > tau2s ? (T)(1.0 / (c * d.s2[j])) : (T)0;
             C y = cY[i];
@@ -261,8 +276,8 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
             y.y *= f;
             X2[i] = y;
         }
-        __syncthreads();
-        cta_gemm<T, C>(m, n, k, Op<C>{X1, k, 1, false}, Op<C>{X2, n, 1, false}, Tb, n, 1, (T)1, true, As, Bs);
+        cluster_sync();
+        cl_gemm<T, C>(m, n, k, Op<C>{X1, k, 1, false}, Op<C>{X2, n, 1, false}, Tb, n, 1, (T)1, true, As, Bs, rank);
     }
     if (need_disc) {
         const int dd = nz - k;
@@ -273,27 +288,27 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
         // separated singular values alone
         const double e2s = EpsG<T>::v * EpsG<T>::v * d.s2[0];
         // X1 = G o B_D (dd x k), B_D = rows k.. of Q1
-        for (int i = tid; i < dd * k; i += nt) {
+        for (int i = gid; i < dd * k; i += gn) {
             const int l = i / k, j = i % k;
             const double dj = d.s2[j] - d.s2[k + l];
             const double sum = sqrt(d.s2[j]) + sqrt(fmax(d.s2[k + l], 0.0));
             const double eps_b = e2s * sum * sum;
             const T g = d.s2[j] > tau2s ? (T)(dj / (dj * dj + eps_b)) : (T)0;
-            C b = Q1[(size_t)(k + l) * k + j];
+            C b = __ldcg(Q1 + (size_t)(k + l) * k + j);
             b.x *= g;
             b.y *= g;
             X1[i] = b;
         }
-        __syncthreads();
+        cluster_sync();
         // Z T = U_D (Gb Y): X2 = Gb Y (dd x n), Tb += Ua_D X2
-        cta_gemm<T, C>(dd, n, k, Op<C>{X1, k, 1, false}, Op<C>{cY, n, 1, false}, X2, n, 1, (T)(1.0 / c), false, As, Bs);
-        cta_gemm<T, C>(m, n, dd, Op<C>{Ua + (size_t)k * m, 1, m, false}, Op<C>{X2, n, 1, false}, Tb, n, 1, (T)1, true,
-                       As, Bs);
+        cl_gemm<T, C>(dd, n, k, Op<C>{X1, k, 1, false}, Op<C>{cY, n, 1, false}, X2, n, 1, (T)(1.0 / c), false, As, Bs, rank);
+        cl_gemm<T, C>(m, n, dd, Op<C>{Ua + (size_t)k * m, 1, m, false}, Op<C>{X2, n, 1, false}, Tb, n, 1, (T)1, true,
+                       As, Bs, rank);
         // Z^H T = U Gb^H (U_D^H T): X2 = U_D^H T (dd x n), Mb (scratch) = Gb^H X2 (k x n), Tb += U Mb
-        cta_gemm<T, C>(dd, n, m, Op<C>{Ua + (size_t)k * m, m, 1, true}, Op<C>{Tm, 1, m, false}, X2, n, 1, (T)1, false,
-                       As, Bs);
-        cta_gemm<T, C>(k, n, dd, Op<C>{X1, 1, k, true}, Op<C>{X2, n, 1, false}, Mb, n, 1, (T)1, false, As, Bs);
-        cta_gemm<T, C>(m, n, k, Op<C>{U, k, 1, false}, Op<C>{Mb, n, 1, false}, Tb, n, 1, (T)1, true, As, Bs);
+        cl_gemm<T, C>(dd, n, m, Op<C>{Ua + (size_t)k * m, m, 1, true}, Op<C>{Tm, 1, m, false}, X2, n, 1, (T)1, false,
+                       As, Bs, rank);
+        cl_gemm<T, C>(k, n, dd, Op<C>{X1, 1, k, true}, Op<C>{X2, n, 1, false}, Mb, n, 1, (T)1, false, As, Bs, rank);
+        cl_gemm<T, C>(m, n, k, Op<C>{U, k, 1, false}, Op<C>{Mb, n, 1, false}, Tb, n, 1, (T)1, true, As, Bs, rank);
     }
     // effective gate G (uL x uR) in shared memory
     if (tid < 16) {
@@ -313,18 +328,18 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
         Gt[tid].y = (T)im;
     }
     // merge M = A B (m x n row-major)
-    cta_gemm<T, C>(m, n, chiM, Op<C>{Apre, chiM, 1, false}, Op<C>{Bpre, n, 1, false}, Mm, n, 1, (T)1, false, As, Bs);
+    cl_gemm<T, C>(m, n, chiM, Op<C>{Apre, chiM, 1, false}, Op<C>{Bpre, n, 1, false}, Mm, n, 1, (T)1, false, As, Bs, rank);
     // Mb[(l,c),(d,r)] = sum_ab conj(Gt[2a+b][2c+d]) Tb[(l,a),(b,r)]; Gtb = sum_{l,r} Tb conj(M)
     double gacc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) gacc[i] = 0.0;
-    for (int i = tid; i < chiL * chiR; i += nt) {
+    for (int i = mid; i < chiL * chiR; i += gn) {
         const int l = i / chiR, r = i % chiR;
         C tb[4], mm[4];
 #pragma unroll
         for (int ab = 0; ab < 4; ++ab) {
-            tb[ab] = Tb[(size_t)(2 * l + (ab >> 1)) * n + (ab & 1) * chiR + r];
-            mm[ab] = Mm[(size_t)(2 * l + (ab >> 1)) * n + (ab & 1) * chiR + r];
+            tb[ab] = __ldcg(Tb + (size_t)(2 * l + (ab >> 1)) * n + (ab & 1) * chiR + r);
+            mm[ab] = __ldcg(Mm + (size_t)(2 * l + (ab >> 1)) * n + (ab & 1) * chiR + r);
         }
 #pragma unroll
         for (int cd = 0; cd < 4; ++cd) {
@@ -342,97 +357,91 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
                 gacc[2 * (ab * 4 + cd) + 1] += (double)a.y * b.x - (double)a.x * b.y;
             }
     }
-    block_sum<32>(gacc, red);
+    // sums of the 32 values over the warp: lane i ends up with value i (31 additions instead
+    // of the 160 of 32 separate reductions), then over the warps and the ranks
+    const int lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < o; ++i) {
+            const bool up = (lane & o) != 0;
+            const double send = up ? gacc[i] : gacc[i + o], keep = up ? gacc[i + o] : gacc[i];
+            gacc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    red[warp * 32 + lane] = gacc[0];
     __syncthreads();
+    if (tid < 32) {
+        double v = red[lane];
+        for (int w = 1; w < nt / 32; ++w) v += red[w * 32 + lane];
+        cl.map_shared_rank(&s_part[rank][0], 0)[lane] = v;
+    }
+    cluster_sync();   // the partial sums and Mb
     // site adjoints: Ab = Mb B^H (m x chiM), Bb = A^H Mb (chiM x n)
-    cta_gemm<T, C>(m, chiM, n, Op<C>{Mb, n, 1, false}, Op<C>{Bpre, 1, n, true}, (C*)d.ab_pre, chiM, 1, (T)1, false,
-                   As, Bs);
-    cta_gemm<T, C>(chiM, n, m, Op<C>{Apre, 1, chiM, true}, Op<C>{Mb, n, 1, false}, (C*)d.bb_pre, n, 1, (T)1, false,
-                   As, Bs);
+    cl_gemm<T, C>(m, chiM, n, Op<C>{Mb, n, 1, false}, Op<C>{Bpre, 1, n, true}, (C*)d.ab_pre, chiM, 1, (T)1, false,
+                   As, Bs, rank);
+    cl_gemm<T, C>(chiM, n, m, Op<C>{Apre, 1, chiM, true}, Op<C>{Mb, n, 1, false}, (C*)d.bb_pre, n, 1, (T)1, false,
+                   As, Bs, rank);
     // Kb = G^H Gtb; uLb[a,c] = sum_bd Kb[(ab),(cd)] conj(uR[b,d]); uRb[b,d] = sum_ac Kb[...] conj(uL[a,c])
-    if (tid == 0) {
-        double kb[32];
-        for (int rI = 0; rI < 4; ++rI)
-            for (int cI = 0; cI < 4; ++cI) {
-                double re = 0.0, im = 0.0;
-                for (int j = 0; j < 4; ++j) {
-                    const double gr = d.g4[2 * (j * 4 + rI)], gi = -d.g4[2 * (j * 4 + rI) + 1];   // conj(G[j][rI])
-                    const double xr = gacc[2 * (j * 4 + cI)], xi = gacc[2 * (j * 4 + cI) + 1];
-                    re += gr * xr - gi * xi;
-                    im += gr * xi + gi * xr;
+    if (rank == 0 && tid < 32) {
+        __shared__ double s_g[32], s_kb[32];
+        double v = s_part[0][lane];
+        for (int w = 1; w < kBwdRanks; ++w) v += s_part[w][lane];
+        s_g[lane] = v;
+        __syncwarp();
+        if (lane < 16) {
+            const int rI = lane >> 2, cI = lane & 3;
+            double re = 0.0, im = 0.0;
+            for (int j = 0; j < 4; ++j) {
+                const double gr = d.g4[2 * (j * 4 + rI)], gi = -d.g4[2 * (j * 4 + rI) + 1];   // conj(G[j][rI])
+                const double xr = s_g[2 * (j * 4 + cI)], xi = s_g[2 * (j * 4 + cI) + 1];
+                re += gr * xr - gi * xi;
+                im += gr * xi + gi * xr;
+            }
+            s_kb[2 * lane] = re;
+            s_kb[2 * lane + 1] = im;
+        }
+        __syncwarp();
+        if (lane < 8) {
+            // lanes 0-3: uLb[a][cc] += Kb[(a b),(cc dd)] conj(uR[b][dd]);
+            // lanes 4-7: uRb[a][cc] (as [b][d] = [a][cc]) += Kb[(b' a),(d' cc)] conj(uL[b'][d'])
+            const bool left = lane < 4;
+            const int a = (lane >> 1) & 1, cc = lane & 1;
+            const double* u = left ? d.uR : d.uL;
+            double re = 0.0, im = 0.0;
+            for (int b = 0; b < 2; ++b)
+                for (int dd = 0; dd < 2; ++dd) {
+                    const double ur = u ? u[2 * (b * 2 + dd)] : (b == dd ? 1.0 : 0.0), ui = u ? u[2 * (b * 2 + dd) + 1] : 0.0;
+                    const int e = left ? (2 * a + b) * 4 + 2 * cc + dd : (2 * b + a) * 4 + 2 * dd + cc;
+                    const double kr = s_kb[2 * e], ki = s_kb[2 * e + 1];
+                    re += kr * ur + ki * ui;
+                    im += ki * ur - kr * ui;
                 }
-                kb[2 * (rI * 4 + cI)] = re;
-                kb[2 * (rI * 4 + cI) + 1] = im;
-            }
-        auto u_at = [](const double* u, int r, int cc, double& ur, double& ui) {
-            if (u) { ur = u[2 * (r * 2 + cc)]; ui = u[2 * (r * 2 + cc) + 1]; }
-            else { ur = (r == cc) ? 1.0 : 0.0; ui = 0.0; }
-        };
-        for (int a = 0; a < 2; ++a)
-            for (int cc = 0; cc < 2; ++cc) {
-                double lr = 0.0, li = 0.0, rr = 0.0, ri = 0.0;
-                for (int b = 0; b < 2; ++b)
-                    for (int dd = 0; dd < 2; ++dd) {
-                        double vr, vi;
-                        // uLb[a][cc] += Kb[(a b),(cc dd)] conj(uR[b][dd])
-                        u_at(d.uR, b, dd, vr, vi);
-                        const double kr = kb[2 * ((2 * a + b) * 4 + 2 * cc + dd)], ki = kb[2 * ((2 * a + b) * 4 + 2 * cc + dd) + 1];
-                        lr += kr * vr + ki * vi;
-                        li += ki * vr - kr * vi;
-                        // uRb[a][cc] (as [b][d] = [a][cc]) += Kb[(b' a),(d' cc)] conj(uL[b'][d'])
-                        u_at(d.uL, b, dd, vr, vi);
-                        const double kr2 = kb[2 * ((2 * b + a) * 4 + 2 * dd + cc)], ki2 = kb[2 * ((2 * b + a) * 4 + 2 * dd + cc) + 1];
-                        rr += kr2 * vr + ki2 * vi;
-                        ri += ki2 * vr - kr2 * vi;
-                    }
-                d.ubar_l[2 * (a * 2 + cc)] += lr;
-                d.ubar_l[2 * (a * 2 + cc) + 1] += li;
-                d.ubar_r[2 * (a * 2 + cc)] += rr;
-                d.ubar_r[2 * (a * 2 + cc) + 1] += ri;
-            }
+            double* out = (left ? d.ubar_l : d.ubar_r) + 2 * (a * 2 + cc);
+            out[0] += re;
+            out[1] += im;
+        }
     }
 }
 
 // ---------------------------------------------------------------------------
 // final-state adjoint helpers (environments are compact chi x chi, chi read on the device)
 
+// dst += sum of a list's environments, in its order (one CTA row per dst)
 template <typename T>
-__global__ void k_env_axpy(typename CT<T>::type* __restrict__ dst, const typename CT<T>::type* __restrict__ src,
-                           const int* __restrict__ chi, int bond, double coef, int zero_first) {
-    const int c = chi[bond];
+__global__ void k_env_sum(const EnvSumDesc* __restrict__ list, const EnvTerm* __restrict__ terms) {
+    using C = typename CT<T>::type;
+    const EnvSumDesc d = list[blockIdx.y];
+    const int c = d.chi[d.bond];
+    C* dst = (C*)d.dst;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < c * c; i += gridDim.x * blockDim.x) {
-        auto v = zero_first ? cz<typename CT<T>::type>() : dst[i];
-        if (src) {
-            v.x += (T)coef * src[i].x;
-            v.y += (T)coef * src[i].y;
+        C v = dst[i];
+        for (int t = d.first; t < d.first + d.n; ++t) {
+            const C s = ((const C*)terms[t].src)[i];
+            v.x += (T)terms[t].coef * s.x;
+            v.y += (T)terms[t].coef * s.y;
         }
         dst[i] = v;
     }
-}
-
-// out[l, p, r] += coef sum_{l'} E[l, l'] sum_{p'} O[p, p'] tmp[l', p', r]
-// (tmp = A Rt from the right-transfer pass; E: left environment, bra x ket)
-template <typename T>
-__global__ void k_site_adj2(const typename CT<T>::type* __restrict__ E, const double* __restrict__ op,
-                            const typename CT<T>::type* __restrict__ tmp, const int* __restrict__ chi, int q,
-                            double coef, typename CT<T>::type* __restrict__ out) {
-    using C = typename CT<T>::type;
-    const int cl = chi[q], cr = chi[q + 1];
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)cl * 2 * cr) return;
-    const int l = (int)(t / (2 * cr)), rem = (int)(t % (2 * cr)), p = rem / cr, r = rem % cr;
-    C o0, o1;
-    o0.x = (T)op[2 * (p * 2)]; o0.y = (T)op[2 * (p * 2) + 1];
-    o1.x = (T)op[2 * (p * 2 + 1)]; o1.y = (T)op[2 * (p * 2 + 1) + 1];
-    C acc = cz<C>();
-    for (int lp = 0; lp < cl; ++lp) {
-        C w = cz<C>();
-        cmac(w, o0, tmp[((size_t)lp * 2 + 0) * cr + r]);
-        cmac(w, o1, tmp[((size_t)lp * 2 + 1) * cr + r]);
-        cmac(acc, E[(size_t)l * cl + lp], w);
-    }
-    out[t].x += (T)coef * acc.x;
-    out[t].y += (T)coef * acc.y;
 }
 
 // Ab = (AH - (Hsum / N) AN) / N with Hsum, N the 1 x 1 closing environments (device)
@@ -574,8 +583,17 @@ __global__ void __launch_bounds__(256) k_site1_bwd(const Site1Bwd* __restrict__ 
 template <typename T>
 cudaError_t launch_gate_bwd(const GradGateDesc* d, int n_gates, cudaStream_t s) {
     if (n_gates <= 0) return cudaSuccess;
-    k_gate_bwd<T><<<n_gates, 256, 0, s>>>(d);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kBwdRanks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(n_gates * kBwdRanks));
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_gate_bwd<T>, d);
 }
 template <typename T>
 cudaError_t launch_site1_bwd(const Site1Bwd* d, int n_sites, cudaStream_t s) {
@@ -584,19 +602,9 @@ cudaError_t launch_site1_bwd(const Site1Bwd* d, int n_sites, cudaStream_t s) {
     return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_env_axpy(void* dst, const void* src, const int* chi, int bond, double coef, int zero_first,
-                            int chi_cap, cudaStream_t s) {
-    using C = typename CT<T>::type;
-    const int blocks = (chi_cap * chi_cap + 255) / 256;
-    k_env_axpy<T><<<blocks > 0 ? blocks : 1, 256, 0, s>>>((C*)dst, (const C*)src, chi, bond, coef, zero_first);
-    return cudaGetLastError();
-}
-template <typename T>
-cudaError_t launch_site_adj2(const void* E, const double* op, const void* tmp, const int* chi, int q, double coef,
-                             void* out, int chi_cap, cudaStream_t s) {
-    using C = typename CT<T>::type;
-    const int64_t tot = (int64_t)chi_cap * 2 * chi_cap;
-    k_site_adj2<T><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>((const C*)E, op, (const C*)tmp, chi, q, coef, (C*)out);
+cudaError_t launch_env_sums(const EnvSumDesc* d, const EnvTerm* terms, int count, int chi_cap, cudaStream_t s) {
+    if (count <= 0) return cudaSuccess;
+    k_env_sum<T><<<dim3((chi_cap * chi_cap + 127) / 128, count), 128, 0, s>>>(d, terms);
     return cudaGetLastError();
 }
 template <typename T>
@@ -621,9 +629,7 @@ cudaError_t launch_rot_grad(const RotLayer* rl, int n_layers, int n, const doubl
 #define TNSIM_GRAD_INST(T)                                                                                      \
     template cudaError_t launch_gate_bwd<T>(const GradGateDesc*, int, cudaStream_t);                              \
     template cudaError_t launch_site1_bwd<T>(const Site1Bwd*, int, cudaStream_t);                                 \
-    template cudaError_t launch_env_axpy<T>(void*, const void*, const int*, int, double, int, int, cudaStream_t); \
-    template cudaError_t launch_site_adj2<T>(const void*, const double*, const void*, const int*, int, double,   \
-                                             void*, int, cudaStream_t);                                           \
+    template cudaError_t launch_env_sums<T>(const EnvSumDesc*, const EnvTerm*, int, int, cudaStream_t);           \
     template cudaError_t launch_adj_combine<T>(void*, const void*, const void*, const void*, int64_t, cudaStream_t);
 TNSIM_GRAD_INST(float)
 TNSIM_GRAD_INST(double)

@@ -262,7 +262,7 @@ cudaError_t launch_amplitudes(void* const* sites, const int* chi, int n_qubits, 
 // over many SMs, and every step that does not depend on another in the same launch.  (One
 // thread per element, with its operands from L2 on every k: 21 + 38 us per step at chi 64,
 // complex64, against TRANSFER_FIG.)  The sums keep the order of that form, k ascending in
-// one accumulator, then p'.  op null: w is the product itself, unmixed (tmp[(y, p'), a]).
+// one accumulator, then p'.
 template <typename T>
 __global__ void __launch_bounds__(TILE_THREADS) k_transfer1(const TransferDesc* __restrict__ list, TransferDesc one) {
     using C = typename CT<T>::type;
@@ -296,27 +296,20 @@ __global__ void __launch_bounds__(TILE_THREADS) k_transfer1(const TransferDesc* 
     __shared__ C S[E][E + 1];
     tile_share<C, false>(S, acc);
     C o[4];
-    if (d.op) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { o[i].x = (T)d.op[2 * i]; o[i].y = (T)d.op[2 * i + 1]; }
-    }
+    for (int i = 0; i < 4; ++i) { o[i].x = (T)d.op[2 * i]; o[i].y = (T)d.op[2 * i + 1]; }
     C* tmp = (C*)d.tmp;
     for (int e = threadIdx.x; e < E * E; e += TILE_THREADS) {
         // p, index h of the halved side, index x of the full side; consecutive threads write
         // consecutive elements
-        const int p = d.left ? e / H % 2 : d.op ? e % 2 : e / E % 2;
-        const int h = d.left ? e % H : e / (2 * E), x = d.left ? e / E : d.op ? e / 2 % E : e % E;
+        const int p = d.left ? e / H % 2 : e % 2;
+        const int h = d.left ? e % H : e / (2 * E), x = d.left ? e / E : e / 2 % E;
         if (h0 + h >= nh || x0 + x >= nx) continue;
         const C t0 = d.left ? S[x][h] : S[h][x], t1 = d.left ? S[x][H + h] : S[H + h][x];
-        C w = p ? t1 : t0;
-        if (d.op) {
-            w = C{};
-            MulAdd::op(w, p ? o[2] : o[0], t0);
-            MulAdd::op(w, p ? o[3] : o[1], t1);
-        }
-        const size_t g = d.left ? ((size_t)(x0 + x) * 2 + p) * cr + h0 + h
-                         : d.op ? (size_t)(h0 + h) * 2 * cr + 2 * (x0 + x) + p
-                                : ((size_t)(h0 + h) * 2 + p) * cr + x0 + x;
+        C w = {};
+        MulAdd::op(w, p ? o[2] : o[0], t0);
+        MulAdd::op(w, p ? o[3] : o[1], t1);
+        const size_t g = d.left ? ((size_t)(x0 + x) * 2 + p) * cr + h0 + h : (size_t)(h0 + h) * 2 * cr + 2 * (x0 + x) + p;
         tmp[g] = w;
     }
 }
@@ -353,6 +346,36 @@ __global__ void __launch_bounds__(TILE_THREADS) k_transfer2(const TransferDesc* 
         }
 }
 
+// out[l, p, r] += coef sum_{l'} E[l, l'] w[l', (r, p)]  (E: left environment, bra x ket)
+template <typename T>
+__global__ void __launch_bounds__(TILE_THREADS) k_site_adj(const SiteAdjDesc* __restrict__ list) {
+    using C = typename CT<T>::type;
+    constexpr int TE = TileOf<C>::E, R = TileOf<C>::R;
+    const SiteAdjDesc& d = list[blockIdx.y];
+    const int cl = d.chi[d.q], cr = d.chi[d.q + 1], N = 2 * cr;
+    const int tn = (N + TE - 1) / TE, i0 = (int)(blockIdx.x / tn) * TE, j0 = (int)(blockIdx.x % tn) * TE;
+    if (i0 >= cl) return;
+    const C* E = (const C*)d.E;
+    const C* w = (const C*)d.w;
+    C acc[R][R] = {};
+    tile_product<C, true, false, false, false, MulAdd>(
+        cl, [&](int i, int k) { return i0 + i < cl ? E[(size_t)(i0 + i) * cl + k] : C{}; },
+        [&](int k, int j) { return j0 + j < N ? w[(size_t)k * N + j0 + j] : C{}; }, acc);
+    C* out = (C*)d.out;
+    const T f = (T)d.coef;
+    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const int l = i0 + rx + 8 * i, c = j0 + cy + 8 * j;
+            if (l >= cl || c >= N) continue;
+            C* o = out + ((size_t)l * 2 + (c & 1)) * cr + (c >> 1);
+            o->x += f * acc[i][j].x;
+            o->y += f * acc[i][j].y;
+        }
+}
+
 template <typename T>
 cudaError_t launch_transfers(const TransferDesc* list, const TransferDesc& one, int count, int chi_cap,
                              cudaStream_t s) {
@@ -371,16 +394,16 @@ cudaError_t launch_transfer(const void* site, const int* chi, int q, const doubl
 }
 
 template <typename T>
-cudaError_t launch_apply_rt(const void* site, const int* chi, int q, const void* rt, void* tmp, int chi_cap,
-                            cudaStream_t s) {
-    const TransferDesc one{site, chi, nullptr, rt, tmp, nullptr, q, 0};
+cudaError_t launch_site_adjs(const TransferDesc* t, const SiteAdjDesc* a, int count, int chi_cap, cudaStream_t s) {
+    if (count <= 0) return cudaSuccess;
     constexpr int E = TileOf<typename CT<T>::type>::E;
-    const int te = (chi_cap + E - 1) / E, th = (chi_cap + E / 2 - 1) / (E / 2);
-    k_transfer1<T><<<dim3(te * th, 1), TILE_THREADS, 0, s>>>(nullptr, one);
+    const int te = (chi_cap + E - 1) / E, th = (chi_cap + E / 2 - 1) / (E / 2), t2 = (2 * chi_cap + E - 1) / E;
+    k_transfer1<T><<<dim3(te * th, count), TILE_THREADS, 0, s>>>(t, TransferDesc{});
+    k_site_adj<T><<<dim3(te * t2, count), TILE_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
-template cudaError_t launch_apply_rt<float>(const void*, const int*, int, const void*, void*, int, cudaStream_t);
-template cudaError_t launch_apply_rt<double>(const void*, const int*, int, const void*, void*, int, cudaStream_t);
+template cudaError_t launch_site_adjs<float>(const TransferDesc*, const SiteAdjDesc*, int, int, cudaStream_t);
+template cudaError_t launch_site_adjs<double>(const TransferDesc*, const SiteAdjDesc*, int, int, cudaStream_t);
 template cudaError_t launch_transfers<float>(const TransferDesc*, const TransferDesc&, int, int, cudaStream_t);
 template cudaError_t launch_transfers<double>(const TransferDesc*, const TransferDesc&, int, int, cudaStream_t);
 

@@ -1693,11 +1693,26 @@ tnsim_status tnsim_grad(const tnsim_circuit* c, const double* theta, const tnsim
     double* d_g4 = (double*)dalloc(sizeof(double) * 32 * std::max<int64_t>(n_gates_all, 1));
     RotLayer* d_rl = (RotLayer*)dalloc(sizeof(RotLayer) * std::max(nl, 1));
     char* d_ckpt = dalloc((AB + sizeof(int) * (n + 1) + 255) / 256 * 256 * (size_t)(nl + 1));
+    // environments L0, R0, LH, RH, the full ones of every term, the chains' two scratch buffers
     char* d_env = dalloc(env * (size_t)(4 * (n + 1) + 4) + env * 2 * terms.size());
     char* d_adj = dalloc(AB * 4);
     char* d_scr = dalloc(9 * cm * cm * es * (size_t)m->G);
-    GradGateDesc* d_gdesc = (GradGateDesc*)dalloc(sizeof(GradGateDesc) * m->G);
-    Site1Bwd* d_s1 = (Site1Bwd*)dalloc(sizeof(Site1Bwd) * n);
+    GradGateDesc* d_gdesc = (GradGateDesc*)dalloc(sizeof(GradGateDesc) * std::max<int64_t>(n_gates_all, 1));
+    Site1Bwd* d_s1 = (Site1Bwd*)dalloc(sizeof(Site1Bwd) * std::max((int64_t)n * nl, (int64_t)1));
+    // The gated blocks and decompositions of every layer are kept for the backward where they
+    // fit into a quarter of the free memory and no cap is set; else the backward recomputes each layer.
+    const size_t ws_b = (size_t)m->G * 2 * m->ws_elems * es, s2_b = (size_t)m->G * 2 * m->capmax * sizeof(double),
+                 pm_b = (size_t)m->G * 2 * m->capmax * sizeof(int);
+    const size_t keep_b = (ws_b + s2_b + pm_b + 255) / 256 * 256;
+    char* d_keep = nullptr;
+    {
+        size_t free_b = 0, total_b = 0;
+        if (g_dev_cap.load() <= 0 && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+            keep_b * (size_t)std::max(nl, 1) <= free_b / 4) {
+            d_keep = dalloc(keep_b * (size_t)std::max(nl, 1));
+            if (!d_keep) cudaGetLastError();
+        }
+    }
     double* d_ops = (double*)dalloc(sizeof(double) * 32);
     if (!d_theta || !d_axes || !d_u1 || !d_ubar || !d_grad || !d_g4 || !d_rl || !d_ckpt || !d_env || !d_adj || !d_scr ||
         !d_gdesc || !d_s1 || !d_ops)
@@ -1737,8 +1752,25 @@ tnsim_status tnsim_grad(const tnsim_circuit* c, const double* theta, const tnsim
         cudaEventRecord(stg->done, st);
         return r;
     };
+    // the workspace of layer L's decompositions
+    struct Work { char* ws; double* s2; int* perm; };
+    const Work own{m->d_ws, m->d_s2, m->d_perm};
+    auto layer_work = [&](int L) -> Work {
+        if (!d_keep) return own;
+        char* w = d_keep + keep_b * (size_t)L;
+        return {w, (double*)(w + ws_b), (int*)(w + ws_b + s2_b)};
+    };
+    struct Restore { tnsim_mps* m; Work w; ~Restore() { m->d_ws = w.ws; m->d_s2 = w.s2; m->d_perm = w.perm; } } restore{m, own};
+    // finite contents, as in a state's own workspace: a contraction that timed out leaves W unwritten
+    if (d_keep) CUDA_TRY(cudaMemsetAsync(d_keep, 0, keep_b * (size_t)std::max(nl, 1), st));
     // ---- forward with a checkpoint before every layer (and of the final state)
     for (int L = 0; L <= nl; ++L) {
+        if (L < nl) {
+            const Work w = layer_work(L);
+            m->d_ws = w.ws;
+            m->d_s2 = w.s2;
+            m->d_perm = w.perm;
+        }
         CUDA_TRY(cudaMemcpyAsync(ck_sites(L), m->d_sites, AB, cudaMemcpyDeviceToDevice, st));
         CUDA_TRY(cudaMemcpyAsync(ck_chi(L), m->d_chi, sizeof(int) * (n + 1), cudaMemcpyDeviceToDevice, st));
         if (L < nl) {
@@ -1761,9 +1793,8 @@ tnsim_status tnsim_grad(const tnsim_circuit* c, const double* theta, const tnsim
     char* R0 = L0 + env * (n + 1);
     char* LH = R0 + env * (n + 1);
     char* RH = LH + env * (n + 1);
-    char* tmp = RH + env * (n + 1);            // 2 env
-    char* part = tmp + env * 2;                // 2 env (running partial)
-    char* full = part + env * 2;               // 2 env per term (left full, right full)
+    char* tmp = RH + env * (n + 1);            // 4 env: scratch of two chains
+    char* full = tmp + env * 4;                // 2 env per term (left full, right full)
     char* AH = d_adj;                          // adjoint of <H> (arena layout)
     char* AN = d_adj + AB;                     // adjoint of the norm
     char* ABc = d_adj + 2 * AB;                // adjoint of the current (post-layer) state
@@ -1776,75 +1807,172 @@ tnsim_status tnsim_grad(const tnsim_circuit* c, const double* theta, const tnsim
     CUDA_TRY(cudaMemcpyAsync(L0, one.data(), es, cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMemcpyAsync(R0 + env * n, one.data(), es, cudaMemcpyHostToDevice, st));
     const bool c64 = dt == TNSIM_C64;
-    auto transfer = [&](int q, const double* op, const char* ein, char* eout, int left) -> cudaError_t {
-        return c64 ? launch_transfer<float>(site_ptr(m, q), dchi, q, op, ein, tmp, eout, cap_max, left, st)
-                   : launch_transfer<double>(site_ptr(m, q), dchi, q, op, ein, tmp, eout, cap_max, left, st);
-    };
-    auto site_adj = [&](int q, const char* E, const double* op, const char* Rt, double coef, char* out) -> cudaError_t {
-        cudaError_t e = c64 ? launch_apply_rt<float>(site_ptr(m, q), dchi, q, Rt, tmp, cap_max, st)
-                            : launch_apply_rt<double>(site_ptr(m, q), dchi, q, Rt, tmp, cap_max, st);
-        if (e != cudaSuccess) return e;
-        return c64 ? launch_site_adj2<float>(E, op, tmp, dchi, q, coef, out + m->site_off[q], cap_max, st)
-                   : launch_site_adj2<double>(E, op, tmp, dchi, q, coef, out + m->site_off[q], cap_max, st);
-    };
-    auto axpy = [&](char* dst, const char* src, int bond, double coef, int zero_first) -> cudaError_t {
-        return c64 ? launch_env_axpy<float>(dst, src, dchi, bond, coef, zero_first, cap_max, st)
-                   : launch_env_axpy<double>(dst, src, dchi, bond, coef, zero_first, cap_max, st);
+    // Lists of independent steps, one launch each, all uploaded at once.  (One launch per
+    // transfer and term, with device copies between them, was ~1000 launches of 5 us for
+    // 59 terms of 30 qubits.)
+    std::vector<TransferDesc> tl;
+    std::vector<SiteAdjDesc> al;
+    std::vector<EnvSumDesc> sl;
+    std::vector<EnvTerm> el;
+    struct Launch { int kind; size_t first; int count; };   // 0: transfers, 1: site adjoints, 2: environment sums
+    std::vector<Launch> plan;
+    auto step = [&](int q, const double* op, const char* in, char* w, char* outp, int left) {
+        tl.push_back({site_ptr(m, q), dchi, op, in, w, outp, q, left});
     };
     const double* opI = d_ops;
-    for (int q = 0; q < n; ++q) CUDA_TRY(transfer(q, opI, L0 + env * q, L0 + env * (q + 1), 1));
-    for (int q = n - 1; q >= 0; --q) CUDA_TRY(transfer(q, opI, R0 + env * (q + 1), R0 + env * q, 0));
-    // every non-identity term: the sites it covers, and its full left / right environments
-    for (size_t t = 0; t < terms.size(); ++t) {
-        const Term& tm = terms[t];
-        const char* ps = h->paulis + (size_t)tm.idx * n;
-        char* Lfull = full + env * 2 * t;
-        char* Rfull = Lfull + env;
-        // every site of the support: left partial over a..q-1, right partial over q+1..b
-        // (recomputed per site; Pauli supports are short)
-        for (int q = tm.a; q <= tm.b; ++q) {
-            // left partial over a..q-1 into part[0]
-            CUDA_TRY(cudaMemcpyAsync(part, L0 + env * tm.a, env, cudaMemcpyDeviceToDevice, st));
-            for (int x = tm.a; x < q; ++x) {
-                CUDA_TRY(transfer(x, d_ops + 8 * opi(ps[x]), part, part + env, 1));
-                CUDA_TRY(cudaMemcpyAsync(part, part + env, env, cudaMemcpyDeviceToDevice, st));
+    // both environment chains
+    for (int i = 0; i < n; ++i) {
+        const int q = n - 1 - i;
+        plan.push_back({0, tl.size(), 2});
+        step(i, opI, L0 + env * i, tmp, L0 + env * (i + 1), 1);
+        step(q, opI, R0 + env * (q + 1), tmp + 2 * env, R0 + env * q, 0);
+    }
+    // Every non-identity term: left partials over a..x-1 and right ones over x+1..b of its
+    // sites, its full environments, and its site adjoints, in batches that fit the scratch:
+    // per term 2 (len - 1) partials and 4 env, and one w = O A Rt (2 env) per site adjoint of
+    // a launch (each launch takes at most one adjoint per site: their order is fixed).
+    struct Adj { int q; const char* E; const double* op; const char* rt; double coef; char* out; };
+    const size_t max_scr = (size_t)512 << 20;
+    size_t scr_need = 0;
+    std::vector<std::pair<size_t, size_t>> batches;
+    for (size_t t0 = 0; t0 < terms.size();) {
+        size_t t1 = t0, need = 0;
+        while (t1 < terms.size()) {
+            const size_t add = env * (2 * (size_t)(terms[t1].b - terms[t1].a) + 4);
+            if (t1 > t0 && need + add > max_scr) break;
+            need += add;
+            ++t1;
+        }
+        scr_need = std::max(scr_need, need);
+        batches.push_back({t0, t1});
+        t0 = t1;
+    }
+    char* d_tscr = dalloc(scr_need + env * 2 * 2 * (size_t)n + 256);
+    if (!d_tscr) return fail(TNSIM_ENOMEM, "tnsim_grad: device allocation failed");
+    char* d_w = d_tscr + scr_need;             // 2 env for each of 2n site adjoints
+    auto add_adjoints = [&](const std::vector<Adj>& v) {
+        // round r: the r-th adjoint of every (site, output)
+        std::vector<int> seen(2 * (size_t)n, 0);
+        std::vector<std::vector<size_t>> rounds;
+        for (size_t i = 0; i < v.size(); ++i) {
+            const size_t r = (size_t)seen[2 * v[i].q + (v[i].out == AN)]++;
+            if (r >= rounds.size()) rounds.resize(r + 1);
+            rounds[r].push_back(i);
+        }
+        for (const auto& r : rounds) {
+            // transfer and adjoint lists advance together: the same index in both
+            while (al.size() < tl.size()) al.push_back(SiteAdjDesc{});
+            plan.push_back({1, tl.size(), (int)r.size()});
+            for (size_t k = 0; k < r.size(); ++k) {
+                const Adj& a = v[r[k]];
+                char* w = d_w + env * 2 * k;
+                step(a.q, a.op, a.rt, w, nullptr, 0);
+                al.push_back({a.E, w, dchi, a.out + m->site_off[a.q], a.coef, a.q, 0});
             }
-            // right partial over q+1..b into Rfull (scratch)
-            CUDA_TRY(cudaMemcpyAsync(Rfull, R0 + env * (tm.b + 1), env, cudaMemcpyDeviceToDevice, st));
-            for (int x = tm.b; x > q; --x) {
-                CUDA_TRY(transfer(x, d_ops + 8 * opi(ps[x]), Rfull, part + env, 0));
-                CUDA_TRY(cudaMemcpyAsync(Rfull, part + env, env, cudaMemcpyDeviceToDevice, st));
+        }
+    };
+    for (const auto& bt : batches) {
+        std::vector<char*> lp(bt.second - bt.first), tw(bt.second - bt.first);
+        size_t off = 0;
+        int len_max = 0;
+        for (size_t t = bt.first; t < bt.second; ++t) {
+            const int len = terms[t].b - terms[t].a + 1;
+            lp[t - bt.first] = d_tscr + off;                       // len - 1 left, len - 1 right partials
+            off += env * 2 * (size_t)(len - 1);
+            tw[t - bt.first] = d_tscr + off;                       // two scratch buffers of 2 env
+            off += env * 4;
+            len_max = std::max(len_max, len);
+        }
+        // environments after i sites from the left / right end of term t's support
+        auto left_env = [&](size_t t, int i) -> char* {
+            const int len = terms[t].b - terms[t].a + 1;
+            return i == 0 ? L0 + env * terms[t].a : i == len ? full + env * 2 * t : lp[t - bt.first] + env * (i - 1);
+        };
+        auto right_env = [&](size_t t, int i) -> char* {
+            const int len = terms[t].b - terms[t].a + 1;
+            return i == 0 ? R0 + env * (terms[t].b + 1)
+                          : i == len ? full + env * 2 * t + env : lp[t - bt.first] + env * (len - 1 + i - 1);
+        };
+        for (int i = 0; i < len_max; ++i) {
+            const size_t first = tl.size();
+            for (size_t t = bt.first; t < bt.second; ++t) {
+                const Term& tm = terms[t];
+                if (i > tm.b - tm.a) continue;
+                const char* ps = h->paulis + (size_t)tm.idx * n;
+                step(tm.a + i, d_ops + 8 * opi(ps[tm.a + i]), left_env(t, i), tw[t - bt.first], left_env(t, i + 1), 1);
+                step(tm.b - i, d_ops + 8 * opi(ps[tm.b - i]), right_env(t, i), tw[t - bt.first] + 2 * env,
+                     right_env(t, i + 1), 0);
             }
-            CUDA_TRY(site_adj(q, part, d_ops + 8 * opi(ps[q]), Rfull, tm.coef, AH));
+            plan.push_back({0, first, (int)(tl.size() - first)});
         }
-        // full environments of the term
-        CUDA_TRY(cudaMemcpyAsync(Lfull, L0 + env * tm.a, env, cudaMemcpyDeviceToDevice, st));
-        for (int x = tm.a; x <= tm.b; ++x) {
-            CUDA_TRY(transfer(x, d_ops + 8 * opi(ps[x]), Lfull, part, 1));
-            CUDA_TRY(cudaMemcpyAsync(Lfull, part, env, cudaMemcpyDeviceToDevice, st));
+        std::vector<Adj> adj;
+        for (size_t t = bt.first; t < bt.second; ++t) {
+            const Term& tm = terms[t];
+            const char* ps = h->paulis + (size_t)tm.idx * n;
+            for (int q = tm.a; q <= tm.b; ++q)
+                adj.push_back({q, left_env(t, q - tm.a), d_ops + 8 * opi(ps[q]), right_env(t, tm.b - q), tm.coef, AH});
         }
-        CUDA_TRY(cudaMemcpyAsync(Rfull, R0 + env * (tm.b + 1), env, cudaMemcpyDeviceToDevice, st));
-        for (int x = tm.b; x >= tm.a; --x) {
-            CUDA_TRY(transfer(x, d_ops + 8 * opi(ps[x]), Rfull, part, 0));
-            CUDA_TRY(cudaMemcpyAsync(Rfull, part, env, cudaMemcpyDeviceToDevice, st));
-        }
+        add_adjoints(adj);
     }
     // LH[q]: terms entirely left of bond q; RH[q]: terms entirely right of it
-    CUDA_TRY(axpy(LH, L0, 0, id_coef, 1));
-    for (int q = 0; q < n; ++q) {
-        CUDA_TRY(transfer(q, opI, LH + env * q, LH + env * (q + 1), 1));
+    auto env_sum = [&](char* dst, int bond, size_t first_term) {
+        sl.push_back({dst, dchi, bond, (int)first_term, (int)(el.size() - first_term), 0});
+    };
+    el.push_back({L0, id_coef});
+    env_sum(LH, 0, 0);
+    plan.push_back({2, 0, 1});
+    for (int i = 0; i < n; ++i) {
+        const int q = n - 1 - i;
+        plan.push_back({0, tl.size(), 2});
+        step(i, opI, LH + env * i, tmp, LH + env * (i + 1), 1);
+        step(q, opI, RH + env * (q + 1), tmp + 2 * env, RH + env * q, 0);
+        const size_t first = sl.size();
+        size_t e0 = el.size();
         for (size_t t = 0; t < terms.size(); ++t)
-            if (terms[t].b == q) CUDA_TRY(axpy(LH + env * (q + 1), full + env * 2 * t, q + 1, terms[t].coef, 0));
-    }
-    for (int q = n - 1; q >= 0; --q) {
-        CUDA_TRY(transfer(q, opI, RH + env * (q + 1), RH + env * q, 0));
+            if (terms[t].b == i) el.push_back({full + env * 2 * t, terms[t].coef});
+        if (el.size() > e0) env_sum(LH + env * (i + 1), i + 1, e0);
+        e0 = el.size();
         for (size_t t = 0; t < terms.size(); ++t)
-            if (terms[t].a == q) CUDA_TRY(axpy(RH + env * q, full + env * 2 * t + env, q, terms[t].coef, 0));
+            if (terms[t].a == q) el.push_back({full + env * 2 * t + env, terms[t].coef});
+        if (el.size() > e0) env_sum(RH + env * q, q, e0);
+        if (sl.size() > first) plan.push_back({2, first, (int)(sl.size() - first)});
     }
-    for (int q = 0; q < n; ++q) {
-        CUDA_TRY(site_adj(q, LH + env * q, opI, R0 + env * (q + 1), 1.0, AH));
-        CUDA_TRY(site_adj(q, L0 + env * q, opI, RH + env * (q + 1), 1.0, AH));
-        CUDA_TRY(site_adj(q, L0 + env * q, opI, R0 + env * (q + 1), 1.0, AN));
+    {
+        std::vector<Adj> adj;
+        for (int q = 0; q < n; ++q) {
+            adj.push_back({q, LH + env * q, opI, R0 + env * (q + 1), 1.0, AH});
+            adj.push_back({q, L0 + env * q, opI, RH + env * (q + 1), 1.0, AH});
+            adj.push_back({q, L0 + env * q, opI, R0 + env * (q + 1), 1.0, AN});
+        }
+        add_adjoints(adj);
+    }
+    auto rnd = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t b_tl = rnd(sizeof(TransferDesc) * tl.size()), b_al = rnd(sizeof(SiteAdjDesc) * (al.size() + 1)),
+                 b_sl = rnd(sizeof(EnvSumDesc) * sl.size()), b_el = rnd(sizeof(EnvTerm) * el.size());
+    char* d_lists = dalloc(b_tl + b_al + b_sl + b_el);
+    if (!d_lists) return fail(TNSIM_ENOMEM, "tnsim_grad: device allocation failed");
+    const TransferDesc* d_tl = (const TransferDesc*)d_lists;
+    const SiteAdjDesc* d_al = (const SiteAdjDesc*)(d_lists + b_tl);
+    const EnvSumDesc* d_sl = (const EnvSumDesc*)(d_lists + b_tl + b_al);
+    const EnvTerm* d_el = (const EnvTerm*)(d_lists + b_tl + b_al + b_sl);
+    CUDA_TRY(cudaMemcpyAsync((void*)d_tl, tl.data(), sizeof(TransferDesc) * tl.size(), cudaMemcpyHostToDevice, st));
+    if (!al.empty()) CUDA_TRY(cudaMemcpyAsync((void*)d_al, al.data(), sizeof(SiteAdjDesc) * al.size(), cudaMemcpyHostToDevice, st));
+    CUDA_TRY(cudaMemcpyAsync((void*)d_sl, sl.data(), sizeof(EnvSumDesc) * sl.size(), cudaMemcpyHostToDevice, st));
+    CUDA_TRY(cudaMemcpyAsync((void*)d_el, el.data(), sizeof(EnvTerm) * el.size(), cudaMemcpyHostToDevice, st));
+    int chi_top = 1;   // the final bond dimensions bound every environment
+    for (int b = 0; b <= n; ++b) chi_top = std::max(chi_top, chi_at(nl, b));
+    for (const Launch& l : plan) {
+        cudaError_t e;
+        if (l.kind == 0)
+            e = c64 ? launch_transfers<float>(d_tl + l.first, TransferDesc{}, l.count, chi_top, st)
+                    : launch_transfers<double>(d_tl + l.first, TransferDesc{}, l.count, chi_top, st);
+        else if (l.kind == 1)
+            e = c64 ? launch_site_adjs<float>(d_tl + l.first, d_al + l.first, l.count, chi_top, st)
+                    : launch_site_adjs<double>(d_tl + l.first, d_al + l.first, l.count, chi_top, st);
+        else
+            e = c64 ? launch_env_sums<float>(d_sl + l.first, d_el, l.count, chi_top, st)
+                    : launch_env_sums<double>(d_sl + l.first, d_el, l.count, chi_top, st);
+        CUDA_TRY(e);
     }
     // energy = LH[n] / L0[n]
     double hs[2] = {0, 0}, nr[2] = {0, 0};
@@ -1864,79 +1992,90 @@ tnsim_status tnsim_grad(const tnsim_circuit* c, const double* theta, const tnsim
     CUDA_TRY(c64 ? launch_adj_combine<float>(AH, AN, LH + env * n, L0 + env * n, arena_elems, st)
                  : launch_adj_combine<double>(AH, AN, LH + env * n, L0 + env * n, arena_elems, st));
     CUDA_TRY(cudaMemcpyAsync(ABc, AH, AB, cudaMemcpyDeviceToDevice, st));
-    // ---- backward, layer by layer: restore, recompute, differentiate every gate
-    std::vector<GradGateDesc> hg(m->G);
-    std::vector<Site1Bwd> hs1(n);
+    // ---- backward, layer by layer: (restore, recompute,) differentiate every gate
+    std::vector<GradGateDesc> hg((size_t)n_gates_all);
+    std::vector<Site1Bwd> hs1;
+    std::vector<size_t> s1_off(nl + 1, 0);
+    {
+        char *cur = ABc, *nxt = ABn;
+        for (int L = nl - 1; L >= 0; --L, std::swap(cur, nxt)) {
+            const int32_t* ql = c->q + gate_off[L];
+            const double* u1 = layer_u1(L);
+            const Work work = layer_work(L);
+            std::vector<char> paired(n, 0);
+            for (int i = 0; i < c->n2[L]; ++i) {
+                const int q = ql[i];
+                paired[q] = paired[q + 1] = 1;
+                GradGateDesc& d = hg[gate_off[L] + i];
+                std::memset(&d, 0, sizeof(d));
+                char* ws = work.ws + (size_t)i * 2 * m->ws_elems * es;
+                d.a_pre = ck_sites(L) + m->site_off[q];
+                d.b_pre = ck_sites(L) + m->site_off[q + 1];
+                d.u_post = ck_sites(L + 1) + m->site_off[q];
+                d.y_post = ck_sites(L + 1) + m->site_off[q + 1];
+                d.theta0 = ws;
+                d.W = ws + m->ws_elems * es;
+                d.s2 = work.s2 + (size_t)i * 2 * m->capmax;
+                d.perm = work.perm + (size_t)i * 2 * m->capmax;
+                d.g4 = d_g4 + (gate_off[L] + i) * 32;
+                d.uL = u1 ? u1 + (size_t)q * 8 : nullptr;
+                d.uR = u1 ? u1 + (size_t)(q + 1) * 8 : nullptr;
+                d.ub_post = cur + m->site_off[q];
+                d.bb_post = cur + m->site_off[q + 1];
+                d.ab_pre = nxt + m->site_off[q];
+                d.bb_pre = nxt + m->site_off[q + 1];
+                double* ub0 = u1 ? d_ubar + u1_off[L] : d_ubar + (size_t)8 * std::max<int64_t>(n_theta, 1);
+                d.ubar_l = u1 ? ub0 + (size_t)q * 8 : ub0 + (size_t)i * 16;
+                d.ubar_r = u1 ? ub0 + (size_t)(q + 1) * 8 : ub0 + (size_t)i * 16 + 8;
+                d.scratch = d_scr + (size_t)i * 9 * cm * cm * es;
+                d.chiL = chi_at(L, q);
+                d.chiM = chi_at(L, q + 1);
+                d.chiR = chi_at(L, q + 2);
+                d.k = chi_at(L + 1, q + 1);
+                d.renorm = prm.renormalize ? 1 : 0;
+                d.cm = (int)cm;
+            }
+            s1_off[L] = hs1.size();
+            for (int q = 0; q < n; ++q) {
+                if (paired[q] || !u1) continue;
+                hs1.push_back({cur + m->site_off[q], ck_sites(L) + m->site_off[q], nxt + m->site_off[q], u1 + (size_t)q * 8,
+                               d_ubar + u1_off[L] + (size_t)q * 8, chi_at(L, q), chi_at(L, q + 1)});
+            }
+        }
+    }
+    if (n_gates_all > 0)
+        CUDA_TRY(cudaMemcpyAsync(d_gdesc, hg.data(), sizeof(GradGateDesc) * n_gates_all, cudaMemcpyHostToDevice, st));
+    if (!hs1.empty()) CUDA_TRY(cudaMemcpyAsync(d_s1, hs1.data(), sizeof(Site1Bwd) * hs1.size(), cudaMemcpyHostToDevice, st));
     for (int L = nl - 1; L >= 0; --L) {
-        CUDA_TRY(cudaMemcpyAsync(m->d_sites, ck_sites(L), AB, cudaMemcpyDeviceToDevice, st));
-        CUDA_TRY(cudaMemcpyAsync(m->d_chi, ck_chi(L), sizeof(int) * (n + 1), cudaMemcpyDeviceToDevice, st));
-        for (int b = 0; b <= n; ++b) m->ub[b] = chi_at(L, b);
-        s = run_layer(L);
-        if (s != TNSIM_OK) return s;
+        if (!d_keep) {
+            CUDA_TRY(cudaMemcpyAsync(m->d_sites, ck_sites(L), AB, cudaMemcpyDeviceToDevice, st));
+            CUDA_TRY(cudaMemcpyAsync(m->d_chi, ck_chi(L), sizeof(int) * (n + 1), cudaMemcpyDeviceToDevice, st));
+            for (int b = 0; b <= n; ++b) m->ub[b] = chi_at(L, b);
+            s = run_layer(L);
+            if (s != TNSIM_OK) return s;
+        }
         CUDA_TRY(cudaMemsetAsync(ABn, 0, AB, st));
         const int n2 = c->n2[L];
-        const int32_t* ql = c->q + gate_off[L];
-        const double* u1 = layer_u1(L);
-        std::vector<char> paired(n, 0);
-        for (int i = 0; i < n2; ++i) {
-            const int q = ql[i];
-            paired[q] = paired[q + 1] = 1;
-            GradGateDesc& d = hg[i];
-            std::memset(&d, 0, sizeof(d));
-            char* ws = m->d_ws + (size_t)i * 2 * m->ws_elems * es;
-            d.a_pre = ck_sites(L) + m->site_off[q];
-            d.b_pre = ck_sites(L) + m->site_off[q + 1];
-            d.u_post = ck_sites(L + 1) + m->site_off[q];
-            d.y_post = ck_sites(L + 1) + m->site_off[q + 1];
-            d.theta0 = ws;
-            d.W = ws + m->ws_elems * es;
-            d.s2 = m->d_s2 + (size_t)i * 2 * m->capmax;
-            d.perm = m->d_perm + (size_t)i * 2 * m->capmax;
-            d.g4 = d_g4 + (gate_off[L] + i) * 32;
-            d.uL = u1 ? u1 + (size_t)q * 8 : nullptr;
-            d.uR = u1 ? u1 + (size_t)(q + 1) * 8 : nullptr;
-            d.ub_post = ABc + m->site_off[q];
-            d.bb_post = ABc + m->site_off[q + 1];
-            d.ab_pre = ABn + m->site_off[q];
-            d.bb_pre = ABn + m->site_off[q + 1];
-            double* ub0 = u1 ? d_ubar + u1_off[L] : d_ubar + (size_t)8 * std::max<int64_t>(n_theta, 1);
-            d.ubar_l = u1 ? ub0 + (size_t)q * 8 : ub0 + (size_t)i * 16;
-            d.ubar_r = u1 ? ub0 + (size_t)(q + 1) * 8 : ub0 + (size_t)i * 16 + 8;
-            d.scratch = d_scr + (size_t)i * 9 * cm * cm * es;
-            d.chiL = chi_at(L, q);
-            d.chiM = chi_at(L, q + 1);
-            d.chiR = chi_at(L, q + 2);
-            d.k = chi_at(L + 1, q + 1);
-            d.renorm = prm.renormalize ? 1 : 0;
-            d.cm = (int)cm;
-        }
         if (n2 > 0) {
-            CUDA_TRY(cudaMemcpyAsync(d_gdesc, hg.data(), sizeof(GradGateDesc) * n2, cudaMemcpyHostToDevice, st));
-            CUDA_TRY(c64 ? launch_gate_bwd<float>(d_gdesc, n2, st) : launch_gate_bwd<double>(d_gdesc, n2, st));
+            const GradGateDesc* gd2 = d_gdesc + gate_off[L];
+            CUDA_TRY(c64 ? launch_gate_bwd<float>(gd2, n2, st) : launch_gate_bwd<double>(gd2, n2, st));
         }
-        int ns = 0;
-        for (int q = 0; q < n; ++q) {
-            if (paired[q]) continue;
-            const size_t bytes = (size_t)chi_at(L, q) * 2 * chi_at(L, q + 1) * es;
-            if (!u1) {
+        if (!layer_u1(L)) {
+            std::vector<char> paired(n, 0);
+            for (int i = 0; i < n2; ++i) paired[c->q[gate_off[L] + i]] = paired[c->q[gate_off[L] + i] + 1] = 1;
+            for (int q = 0; q < n; ++q) {
+                if (paired[q]) continue;
+                const size_t bytes = (size_t)chi_at(L, q) * 2 * chi_at(L, q + 1) * es;
                 CUDA_TRY(cudaMemcpyAsync(ABn + m->site_off[q], ABc + m->site_off[q], bytes, cudaMemcpyDeviceToDevice, st));
-                continue;
             }
-            Site1Bwd& d = hs1[ns++];
-            d.ab_post = ABc + m->site_off[q];
-            d.a_pre = ck_sites(L) + m->site_off[q];
-            d.ab_pre = ABn + m->site_off[q];
-            d.u = u1 + (size_t)q * 8;
-            d.ubar = d_ubar + u1_off[L] + (size_t)q * 8;
-            d.cl = chi_at(L, q);
-            d.cr = chi_at(L, q + 1);
         }
-        if (ns > 0) {
-            CUDA_TRY(cudaMemcpyAsync(d_s1, hs1.data(), sizeof(Site1Bwd) * ns, cudaMemcpyHostToDevice, st));
-            CUDA_TRY(c64 ? launch_site1_bwd<float>(d_s1, ns, st) : launch_site1_bwd<double>(d_s1, ns, st));
+        // the one-qubit descriptors were filled from the last layer down
+        const size_t s1_beg = s1_off[L];
+        const size_t s1_end = L == 0 ? hs1.size() : s1_off[L - 1];
+        if (s1_end > s1_beg) {
+            const int ns = (int)(s1_end - s1_beg);
+            CUDA_TRY(c64 ? launch_site1_bwd<float>(d_s1 + s1_beg, ns, st) : launch_site1_bwd<double>(d_s1 + s1_beg, ns, st));
         }
-        // the host arrays above are read by the copies before the next layer reuses them
-        CUDA_TRY(cudaStreamSynchronize(st));
         std::swap(ABc, ABn);
     }
     if (n_theta > 0) {

@@ -313,22 +313,35 @@ template <typename T>
 cudaError_t launch_gate_bwd(const GradGateDesc* d, int n_gates, cudaStream_t s);
 template <typename T>
 cudaError_t launch_site1_bwd(const Site1Bwd* d, int n_sites, cudaStream_t s);
+// Site adjoint: out[l, p, r] += coef sum_{l'} E[l, l'] w[l', (r, p)], w the right product of
+// the TransferDesc of the same index (w = O A Rt).
+struct SiteAdjDesc {
+    const void* E;
+    const void* w;
+    const int* chi;
+    void* out;
+    double coef;
+    int q, pad_;
+};
 template <typename T>
-cudaError_t launch_env_axpy(void* dst, const void* src, const int* chi, int bond, double coef, int zero_first,
-                            int chi_cap, cudaStream_t s);
+cudaError_t launch_site_adjs(const TransferDesc* t, const SiteAdjDesc* a, int count, int chi_cap, cudaStream_t s);
+// dst += the sum of terms [first, first + n) of a list (environments of one bond)
+struct EnvTerm {
+    const void* src;
+    double coef;
+};
+struct EnvSumDesc {
+    void* dst;
+    const int* chi;
+    int bond, first, n, pad_;
+};
 template <typename T>
-cudaError_t launch_site_adj2(const void* E, const double* op, const void* tmp, const int* chi, int q, double coef,
-                             void* out, int chi_cap, cudaStream_t s);
+cudaError_t launch_env_sums(const EnvSumDesc* d, const EnvTerm* terms, int count, int chi_cap, cudaStream_t s);
 template <typename T>
 cudaError_t launch_adj_combine(void* ah, const void* an, const void* hsum, const void* nrm, int64_t count,
                                cudaStream_t s);
 cudaError_t launch_rot_build(const RotLayer* rl, int n_layers, int n, double* u1, cudaStream_t s);
 cudaError_t launch_rot_grad(const RotLayer* rl, int n_layers, int n, const double* ub, double* grad, cudaStream_t s);
-// tmp[y, p, a] = sum_b A_q[y, p, b] Rt[b, a]: a site times a (transposed) right environment
-template <typename T>
-cudaError_t launch_apply_rt(const void* site, const int* chi, int q, const void* rt, void* tmp, int chi_cap,
-                            cudaStream_t s);
-
 // Set the thread-local message returned by tnsim_last_error().
 void set_last_error(const char* msg);
 

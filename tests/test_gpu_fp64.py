@@ -11,6 +11,7 @@ import numpy as np
 import pytest
 
 import workloads as W
+from oracle import grad as OG
 from oracle import mps as om
 
 pytestmark = pytest.mark.gpu
@@ -107,3 +108,33 @@ def test_canonical_form_and_memory_cap(T):
         out.append(om.MPS(m.export_sites()))
         m.close()
     assert 1 - om.fidelity(*out) <= 1e-12
+
+
+@pytest.mark.parametrize("dt,tol", [("C128", 1e-9), ("C64", 1e-3)])
+def test_gradient_recomputes_layers_under_a_cap(T, dt, tol):
+    """Without a cap the gradient keeps every layer's decomposition, with one it recomputes
+    them; rows of Pauli strings of every length share the environments' launches.  At cutoff
+    1e-4 the kept values stay above 1e-2 s_max, so both precisions resolve the gradient
+    (complex64 within the bar of the other gradient tests)."""
+    n, nl = 9, 5
+    circ, ang = W.hea_circuit(n, nl, seed=3)
+    layers = [(l.pairs, l.g4) for l in circ.layers]
+    axes = ["YZ" if i % 2 == 0 else "" for i in range(len(layers))]
+    theta = [ang[i // 2] if i % 2 == 0 else np.zeros((n, 0)) for i in range(len(layers))]
+    rng = np.random.default_rng(1)
+    paulis = ["I" * n, "Z" * n, "X" + "I" * (n - 1)] + ["".join(rng.choice(list("IIXYZ"), n)) for _ in range(20)]
+    coeffs = rng.standard_normal(len(paulis))
+    p = T.tnsim_params_default(getattr(T, "TNSIM_" + dt))
+    p.chi_max, p.cutoff = 6, 1e-4
+    out = []
+    for cap in (0, 1 << 40):
+        T.tnsim_set_device_memory_cap(cap)
+        try:
+            e, g = T.tnsim_grad(n, layers, axes, theta, paulis, coeffs, getattr(T, "TNSIM_" + dt), p)
+        finally:
+            T.tnsim_set_device_memory_cap(0)
+        out.append(np.concatenate([[e]] + [x.reshape(-1) for x in g]))
+    ref = OG.grad(n, layers, axes, theta, paulis, list(coeffs), 6, 1e-4)
+    want = np.concatenate([[ref[0]]] + [x.reshape(-1) for x in ref[1]])
+    for o in out:
+        assert np.max(np.abs(o - want)) <= tol * np.max(np.abs(want))
