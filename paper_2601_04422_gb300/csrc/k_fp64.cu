@@ -4,24 +4,35 @@
 // GB300 issues FP64 at 1/64 of the FP32 rate, so an FP64 kernel's time is its FP64
 // instruction count over the SMs that it keeps busy, and everything else hides behind
 // it.  The products therefore use 8 x 8 tiles (tile16.cuh): with 64 x 64 tiles one SM per
-// gate did the work at m = n <= 64 (THETA_FIG).
+// gate did the work (theta and right site of 5 gates at m = n = 64: 88 + 136 -> 9 + 13 us;
+// of 20 gates at m = 180: 480 + 790 -> 330 + 350 us).
 //
 // Preconditioner (mixed-precision Jacobi SVD: Gao, Ma and Shao 2022).  One-sided Jacobi
 // converges quadratically, so 9 of its ~12 FP64 sweeps only bring the columns from O(1)
 // to ~1e-6 of orthogonal, which FP32 can do at 64 times the rate:
-//   k_mix_build  [theta; I] in FP32 (theta scaled by a power of two to |theta|_F in [1, 2));
-//   k_jacobi     FP32 Jacobi rotations of these columns until theta V is orthogonal to
+//   k_mix_build  [W; I] in FP32 (W, at first theta, scaled by a power of two to |W|_F in
+//                [2^28, 2^29): the squares and their products stay in FP32's range for
+//                columns down to 2^-52 |W|_F);
+//   k_jacobi     FP32 Jacobi rotations of these columns until W V is orthogonal to
 //                kMixTol; the lower n rows become V (k_jacobi.cu, EXT);
 //   k_mix_gram   E = I - V^H V in FP64 (V is unitary to ~1e-6 only);
 //   k_mix_corr   F = E/2 + 3/8 E^2, so that V (I + F) = V (V^H V)^{-1/2} + O(E^3) is
 //                unitary to FP64 rounding (E^2 ~ 1e-12 needs four digits: FP32);
 //   k_mix_mul    X = W V, then W <- X + X F, both in FP64.
+// This is done twice.  In the first pass the columns of theta, all of about the same
+// norm, hide singular values s in FP32 roundings: the small columns of W come out
+// orthogonal to ~1e-7 s_max / s only (and below 1e-7 s_max not at all).  W's columns now
+// have the singular values as norms, each rounded to FP32 relative to its own norm, so
+// the second pass resolves all of them down to FP64's zero, in two or three FP32 sweeps.
 // The FP64 Jacobi iteration then starts from W V' with V' unitary: the same SVD to the
 // same tolerance, with fewer sweeps and mostly tiny rotations.  A preconditioner that did
-// not converge or lost small columns to FP32 rounding only costs sweeps.
-// Measured with the FP64 visit of k_jacobi.cu on 20 gates at m = n = 180: SVD 139 -> 29 ms
-// (12.2 -> 4.7 FP64 sweeps per gate; of the 29 ms, FP32 rotations 4.4, these products 2.1);
-// singular values 6e-16 (relative) from LAPACK's before and after.
+// not converge only costs sweeps.
+// Measured with the FP64 visit of k_jacobi.cu on 20 gates at m = n = 180: SVD 139 ms
+// without, 29 with one pass (12.2 -> 4.7 FP64 sweeps per gate), 23 with two (3.6); 4 gates
+// at m = n = 64: 3.2 ms with one pass (6.7 sweeps), 2.1 with two (4.2).  Singular values
+// 6e-16 (relative) from LAPACK's in all three.
+#include <float.h>
+
 #include "tile16.cuh"
 #include "tnsim_internal.h"
 
@@ -149,7 +160,7 @@ __device__ __forceinline__ bool mix_active(const GateDesc& d, int m, int n) {
     return d.pre && n >= kMixMinCols && m + n <= kMixMaxRows;
 }
 
-// [theta; I] in FP32; a gate outside the preconditioner counts as finished in its launch
+// [W; I] in FP32; a gate outside the preconditioner counts as finished in its launch
 __global__ void __launch_bounds__(256) k_mix_build(const GateDesc* __restrict__ gd, JacobiCtl* __restrict__ ctl) {
     const GateDesc& d = gd[blockIdx.y];
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
@@ -318,15 +329,19 @@ cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, Jac
     const int mm = m_max < kMixMaxRows ? m_max : kMixMaxRows, nm = n_max < kMixMaxRows ? n_max : kMixMaxRows;
     int bx = (int)(((long long)mt * nm + 1023) / 1024);
     if (bx > 128) bx = 128;
-    k_mix_build<<<dim3(bx, n_gates), 256, 0, s>>>(d, ctl);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_jacobi_mix(d, n_gates, mt, nm, ctl, s, n_lead, spin_limit);
-    if (e != cudaSuccess) return e;
     const int tn = (nm + T64 - 1) / T64, tm = (mm + T64 - 1) / T64, tf = (nm + T32 - 1) / T32;
-    k_mix_gram<<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
-    k_mix_corr<<<dim3(tf, tf, n_gates), TILE_THREADS, 0, s>>>(d);
-    k_mix_mul<true><<<dim3(tm, tn, n_gates), TILE_THREADS, 0, s>>>(d);
-    k_mix_mul<false><<<dim3(tm, tn, n_gates), TILE_THREADS, 0, s>>>(d);
+    for (int pass = 0; pass < 2; ++pass) {
+        cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(JacobiCtl), s);
+        if (e != cudaSuccess) return e;
+        k_mix_build<<<dim3(bx, n_gates), 256, 0, s>>>(d, ctl);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_jacobi_mix(d, n_gates, mt, nm, pass ? DBL_EPSILON : FLT_EPSILON, ctl, s, n_lead, spin_limit);
+        if (e != cudaSuccess) return e;
+        k_mix_gram<<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
+        k_mix_corr<<<dim3(tf, tf, n_gates), TILE_THREADS, 0, s>>>(d);
+        k_mix_mul<true><<<dim3(tm, tn, n_gates), TILE_THREADS, 0, s>>>(d);
+        k_mix_mul<false><<<dim3(tm, tn, n_gates), TILE_THREADS, 0, s>>>(d);
+    }
     return cudaGetLastError();
 }
 

@@ -130,10 +130,10 @@ constexpr int kMixMinCols = 16;
 constexpr int kMixMaxRows = 1024;
 constexpr double kMixTol = 2e-6;
 #ifdef __CUDACC__
-// power of two that brings |theta|_F into [1, 2) in the FP32 copy of theta
+// power of two that brings |W|_F into [2^28, 2^29) in the FP32 copy of W
 __device__ __forceinline__ double mix_scale(double frob2) {
     if (!(frob2 > 0.0) || isinf(frob2)) return 1.0;
-    return ldexp(1.0, -(ilogb(frob2) >> 1));
+    return ldexp(1.0, 28 - (ilogb(frob2) >> 1));
 }
 #endif
 
@@ -162,11 +162,12 @@ template <typename T>
 cudaError_t launch_jacobi(const GateDesc* d, int n_gates, int m_max, int n_max, double tol,
                           int max_sweeps, JacobiCtl* ctl, cudaStream_t s, int cfg = 0, int n_lead = 0,
                           unsigned spin_limit = 0);
-// the FP32 Jacobi of the preconditioner (columns of mt_max rows in GateDesc::pre)
-cudaError_t launch_jacobi_mix(const GateDesc* d, int n_gates, int mt_max, int n_max, JacobiCtl* ctl, cudaStream_t s,
-                              int n_lead, unsigned spin_limit);
+// the FP32 Jacobi of the preconditioner (columns of mt_max rows in GateDesc::pre; those
+// below zeps sqrt(max(m, n)) |W|_F count as zero)
+cudaError_t launch_jacobi_mix(const GateDesc* d, int n_gates, int mt_max, int n_max, double zeps, JacobiCtl* ctl,
+                              cudaStream_t s, int n_lead, unsigned spin_limit);
 // the whole preconditioner: W <- W V' for every complex128 gate with buffers; ctl is its
-// own control word (zeroed before)
+// own control word
 cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, JacobiCtl* ctl, cudaStream_t s,
                        int n_lead, unsigned spin_limit);
 // FP64 merge + gate contraction and right site
