@@ -773,8 +773,7 @@ static cudaError_t launch_cl(const GateDesc* d, int n_gates, int m_max, int n_ma
     using C = typename CT<T>::type;
     *used = false;
     const int nb = (n_max + BC - 1) / BC;
-    int seats = 1;
-    while (2 * seats < nb) seats *= 2;
+    const int seats = (nb + 1) / 2;
     if (seats > 8) return cudaSuccess;
     const auto kernel = k_jacobi_cl<T, BC, LP, RPL, MINB, EXT>;
     const size_t smem = sizeof(T) == 4 ? (size_t)3 * BC * LP * RPL * sizeof(C) : (size_t)4 * BC * m_max * sizeof(C);
@@ -889,12 +888,14 @@ cudaError_t launch_jacobi_mix(const GateDesc* d, int n_gates, int mt_max, int n_
     if (mt_max <= 64) e = TNSIM_MIXCL(16, 4, 16, 1);
     else if (mt_max <= 128) e = TNSIM_MIXCL(16, 8, 16, 1);
     else if (mt_max <= 256) e = TNSIM_MIXCL(16, 16, 16, 1);
+    else if (mt_max <= 384) e = TNSIM_MIXCL(16, 32, 12, 1);
     else if (mt_max <= 512) e = TNSIM_MIXCL(16, 32, 16, 1);
     if (e != cudaSuccess || used) return e;
 #define TNSIM_MIX(BC, LP, RPL, MINB) launch_bc<float, BC, LP, RPL, MINB, true>(d, n_gates, n_lead, mt_max, n_max, kMixTol, sweeps, ctl, s, spin_limit, zeps)
     if (mt_max <= 64) return TNSIM_MIX(16, 4, 16, 8);
     if (mt_max <= 128) return TNSIM_MIX(16, 8, 16, 4);
     if (mt_max <= 256) return TNSIM_MIX(16, 16, 16, 2);
+    if (mt_max <= 384) return TNSIM_MIX(16, 32, 12, 1);
     if (mt_max <= 512) return TNSIM_MIX(16, 32, 16, 1);
     return TNSIM_MIX(8, 32, 32, 1);
 #undef TNSIM_MIX
