@@ -383,14 +383,13 @@ __device__ __forceinline__ void visit64(double2* __restrict__ XI, double2* __res
 // of a sweep, decides convergence).  Gates are scanned in descriptor order, which
 // the host sorts by decreasing size.  A CTA never waits while holding a claim, so
 // a CTA with nothing to claim only waits for work that running CTAs are doing.
-// EXT (FP32): the columns of the complex128 gates' preconditioner, [W; I] in GateDesc::pre
-// (k_fp64.cu); rotated over all m + n rows, the inner products and norms over the first m;
-// columns below zeps sqrt(max(m, n)) |W|_F count as zero.
+// EXT (FP32): the columns of the complex128 gates' preconditioner, [theta; I] in GateDesc::pre
+// (k_fp64.cu); rotated over all m + n rows, the inner products and norms over the first m.
 // LP, RPL: lanes per pair and rows per lane of the launch's largest m (FP32; 32 and 0 for FP64).
 template <typename T, int BC, int LP, int RPL, int MINB, bool EXT>
 __global__ void __launch_bounds__(BC * LP, MINB)
 k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in, int max_sweeps,
-         JacobiCtl* __restrict__ ctl, unsigned spin_limit, double zeps) {
+         JacobiCtl* __restrict__ ctl, unsigned spin_limit) {
     using C = typename CT<T>::type;
     static_assert(BC * LP >= 64, "warp 0 claims while the others write back");
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -486,8 +485,7 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
             const double f = mix_scale(frob2);
             frob2 *= f * f;
         }
-        const double ze = EXT ? zeps : Eps<T>::v;
-        const T zthr = (T)(ze * ze * (double)max(md, n) * frob2);
+        const T zthr = (T)(Eps<T>::v * Eps<T>::v * (double)max(md, n) * frob2);
 
         int I, J;
         if (nb == 1) {
@@ -609,7 +607,7 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
 // barrier of a round, arrived at early).  FP64: four slots, two free.
 template <typename T, int BC, int LP, int RPL, int MINB, bool EXT>
 __global__ void __launch_bounds__(BC * LP, MINB)
-k_jacobi_cl(const GateDesc* __restrict__ gd, double tol_in, int max_sweeps, double zeps) {
+k_jacobi_cl(const GateDesc* __restrict__ gd, double tol_in, int max_sweeps) {
     using C = typename CT<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ T s_n[2 * BC];
@@ -634,8 +632,7 @@ k_jacobi_cl(const GateDesc* __restrict__ gd, double tol_in, int max_sweeps, doub
         const double f = mix_scale(frob2);
         frob2 *= f * f;
     }
-    const double ze = EXT ? zeps : Eps<T>::v;
-    const T zthr = (T)(ze * ze * (double)max(md, n) * frob2);
+    const T zthr = (T)(Eps<T>::v * Eps<T>::v * (double)max(md, n) * frob2);
     const bool seat = v <= last;
     const int tid = threadIdx.x, lane = tid & 31;
     if (tid == 0) s_rot = s_vis = 0;
@@ -769,7 +766,7 @@ constexpr size_t kOneCta = 116 << 10;   // dynamic shared memory that leaves no 
 // Launch k_jacobi_cl when all the gates' clusters are resident at once; *used tells.
 template <typename T, int BC, int LP, int RPL, int MINB, bool EXT = false>
 static cudaError_t launch_cl(const GateDesc* d, int n_gates, int m_max, int n_max, double tol, int max_sweeps,
-                             cudaStream_t s, bool* used, double zeps = 0.0) {
+                             cudaStream_t s, bool* used) {
     using C = typename CT<T>::type;
     *used = false;
     const int nb = (n_max + BC - 1) / BC;
@@ -804,12 +801,12 @@ static cudaError_t launch_cl(const GateDesc* d, int n_gates, int m_max, int n_ma
     if (n_gates > fit && (e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg)) != cudaSuccess) return e;
     if (n_gates > fit) return cudaSuccess;
     *used = true;
-    return cudaLaunchKernelEx(&cfg, kernel, d, tol, max_sweeps < 1 ? 1 : max_sweeps, zeps);
+    return cudaLaunchKernelEx(&cfg, kernel, d, tol, max_sweeps < 1 ? 1 : max_sweeps);
 }
 
 template <typename T, int BC, int LP, int RPL, int MINB, bool EXT = false>
 static cudaError_t launch_bc(const GateDesc* d, int n_gates, int n_lead, int m_max, int n_max, double tol,
-                             int max_sweeps, JacobiCtl* ctl, cudaStream_t s, unsigned spin_limit, double zeps = 0.0) {
+                             int max_sweeps, JacobiCtl* ctl, cudaStream_t s, unsigned spin_limit) {
     using C = typename CT<T>::type;
     const auto kernel = k_jacobi<T, BC, LP, RPL, MINB, EXT>;
     const size_t smem = sizeof(T) == 8 ? (size_t)2 * BC * m_max * sizeof(C) : (size_t)2 * BC * LP * RPL * sizeof(C);
@@ -828,7 +825,7 @@ static cudaError_t launch_bc(const GateDesc* d, int n_gates, int n_lead, int m_m
     if (grid < 1) grid = 1;
     const int lead = (n_lead < 1 || n_lead > n_gates) ? n_gates : n_lead;
     kernel<<<(unsigned)grid, BC * LP, smem, s>>>(d, n_gates, lead, tol, max_sweeps < 1 ? 1 : max_sweeps, ctl,
-                                                 spin_limit ? spin_limit : kSpinLimit, zeps);
+                                                 spin_limit ? spin_limit : kSpinLimit);
     return cudaGetLastError();
 }
 
@@ -877,12 +874,12 @@ cudaError_t launch_jacobi(const GateDesc* d, int n_gates, int m_max, int n_max, 
 #undef TNSIM_JAC
 }
 
-cudaError_t launch_jacobi_mix(const GateDesc* d, int n_gates, int mt_max, int n_max, double zeps, JacobiCtl* ctl,
-                              cudaStream_t s, int n_lead, unsigned spin_limit) {
+cudaError_t launch_jacobi_mix(const GateDesc* d, int n_gates, int mt_max, int n_max, JacobiCtl* ctl, cudaStream_t s,
+                              int n_lead, unsigned spin_limit) {
     if (n_gates <= 0) return cudaSuccess;
     // sweep cap: more than these do not make the preconditioner better
     constexpr int sweeps = 20;
-#define TNSIM_MIXCL(BC, LP, RPL, MINB) launch_cl<float, BC, LP, RPL, MINB, true>(d, n_gates, mt_max, n_max, kMixTol, sweeps, s, &used, zeps)
+#define TNSIM_MIXCL(BC, LP, RPL, MINB) launch_cl<float, BC, LP, RPL, MINB, true>(d, n_gates, mt_max, n_max, kMixTol, sweeps, s, &used)
     bool used = false;
     cudaError_t e = cudaSuccess;
     if (mt_max <= 64) e = TNSIM_MIXCL(16, 4, 16, 1);
@@ -891,7 +888,7 @@ cudaError_t launch_jacobi_mix(const GateDesc* d, int n_gates, int mt_max, int n_
     else if (mt_max <= 384) e = TNSIM_MIXCL(16, 32, 12, 1);
     else if (mt_max <= 512) e = TNSIM_MIXCL(16, 32, 16, 1);
     if (e != cudaSuccess || used) return e;
-#define TNSIM_MIX(BC, LP, RPL, MINB) launch_bc<float, BC, LP, RPL, MINB, true>(d, n_gates, n_lead, mt_max, n_max, kMixTol, sweeps, ctl, s, spin_limit, zeps)
+#define TNSIM_MIX(BC, LP, RPL, MINB) launch_bc<float, BC, LP, RPL, MINB, true>(d, n_gates, n_lead, mt_max, n_max, kMixTol, sweeps, ctl, s, spin_limit)
     if (mt_max <= 64) return TNSIM_MIX(16, 4, 16, 8);
     if (mt_max <= 128) return TNSIM_MIX(16, 8, 16, 4);
     if (mt_max <= 256) return TNSIM_MIX(16, 16, 16, 2);

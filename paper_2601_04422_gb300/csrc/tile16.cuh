@@ -60,7 +60,8 @@ __device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[TileO
 #pragma unroll
         for (int t = 0; t < PER; ++t) {
             int i, k;
-            na[t].x = na[t].y = nb[t].x = nb[t].y = 0;
+            na[t] = C{};
+            nb[t] = C{};
             at(tid + TILE_THREADS * t, AK, i, k);
             if (k0 + k < K) na[t] = la(i, k0 + k);
             at(tid + TILE_THREADS * t, BK, i, k);

@@ -91,7 +91,7 @@ struct tnsim_mps {
     int* d_sticky = nullptr;
     unsigned long long* d_stats = nullptr;   // the counters of tnsim_stats
     JacobiCtl* d_ctl = nullptr;    // control words of the persistent Jacobi launches (the SVD's, the preconditioner's)
-    char* d_pre = nullptr;         // complex128: G slots * 3 buffers of the preconditioner (null: none)
+    char* d_pre = nullptr;         // complex128: G slots * 4 buffers of the preconditioner (null: none)
     int jac_cfg = 0;               // Jacobi launch configuration (tnsim_set_jacobi_config / tnsim_autotune)
     unsigned jac_spin = 0;         // idle polls of the Jacobi kernel before it gives up (0 = default)
     int tc_spin = 0;               // polls of a tensor-core mbarrier wait before it gives up (0 = default)
@@ -174,7 +174,7 @@ tnsim_status check_params(const tnsim_params* p) {
 // memory over all states.
 void alloc_preconditioner(tnsim_mps* m) {
     if (2 * m->capmax < kMixMinCols || 4 * m->capmax > kMixMaxRows || g_dev_cap.load() > 0) return;
-    const int64_t bytes = (int64_t)((size_t)m->G * 3 * m->ws_elems * m->esz);
+    const int64_t bytes = (int64_t)((size_t)m->G * 4 * m->ws_elems * m->esz);
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); return; }
     if (g_pre_held.fetch_add(bytes) + bytes > (int64_t)(total_b / 8) || bytes > (int64_t)(free_b / 2) ||
@@ -345,10 +345,11 @@ tnsim_status upload_desc(cudaStream_t st, const std::vector<GateJob>& jobs, Gate
         d.wait_polls = m->tc_spin;
         if (m->d_pre) {
             const size_t pb = m->ws_elems * es;   // [theta; I] in FP32: (m + n) n * 8 <= (2 capmax)^2 * 16 bytes
-            char* pre = m->d_pre + (size_t)j.slot * 3 * pb;
+            char* pre = m->d_pre + (size_t)j.slot * 4 * pb;
             d.pre = pre;
             d.pre_x = pre + pb;
-            d.pre_f = pre + 2 * pb;
+            d.pre_b = pre + 2 * pb;
+            d.pre_d = pre + 3 * pb;
         }
     }
     CUDA_TRY(cudaMemcpyAsync(d_desc, h_desc, sizeof(GateDesc) * ng, cudaMemcpyHostToDevice, st));

@@ -77,10 +77,11 @@ struct GateDesc {
     // left site becomes theta W' S^-2 and the right site the conjugated Jacobi columns
     int qr;
     // complex128: the buffers of the mixed-precision preconditioner (k_fp64.cu), null = none:
-    // [theta; I] in FP32 ((m + n) x n), I - V^H V and then W V (FP64, m x n), the correction (n x n)
+    // [theta; I] in FP32 ((m + n) x n), then a step's angles; three FP64 matrices (m x n or n x n)
     void* pre;
     void* pre_x;
-    void* pre_f;
+    void* pre_b;
+    void* pre_d;
     // polls of a bounded mbarrier wait in the tensor-core contraction before it gives up
     // (0 = the kernel's default); the CTA then drains its copies in flight and reports
     // status 5 (ETIMEOUT)
@@ -129,11 +130,15 @@ __device__ __forceinline__ bool qr_active(const GateDesc& d, int m, int n) {
 constexpr int kMixMinCols = 16;
 constexpr int kMixMaxRows = 1024;
 constexpr double kMixTol = 2e-6;
+// Refinement steps (k_fp64.cu): the largest angle of a pair (the second step's, and its
+// fallback), and the largest row sums of |K^2| (first step) and of |K| (second) at which
+// the neglected terms, K^6 / 16 and K^4 / 8, stay below 3e-17.
+constexpr float kRefCap0 = 0x1p-9f, kRefCap1 = 0x1p-14f, kRefCap2 = 0x1p-18f, kRefRow0 = 0x1p-17f, kRefRow1 = 0x1p-13f;
 #ifdef __CUDACC__
-// power of two that brings |W|_F into [2^28, 2^29) in the FP32 copy of W
+// power of two that brings |theta|_F into [1, 2) in the FP32 copy of theta
 __device__ __forceinline__ double mix_scale(double frob2) {
     if (!(frob2 > 0.0) || isinf(frob2)) return 1.0;
-    return ldexp(1.0, 28 - (ilogb(frob2) >> 1));
+    return ldexp(1.0, -(ilogb(frob2) >> 1));
 }
 #endif
 
@@ -162,12 +167,11 @@ template <typename T>
 cudaError_t launch_jacobi(const GateDesc* d, int n_gates, int m_max, int n_max, double tol,
                           int max_sweeps, JacobiCtl* ctl, cudaStream_t s, int cfg = 0, int n_lead = 0,
                           unsigned spin_limit = 0);
-// the FP32 Jacobi of the preconditioner (columns of mt_max rows in GateDesc::pre; those
-// below zeps sqrt(max(m, n)) |W|_F count as zero)
-cudaError_t launch_jacobi_mix(const GateDesc* d, int n_gates, int mt_max, int n_max, double zeps, JacobiCtl* ctl,
-                              cudaStream_t s, int n_lead, unsigned spin_limit);
+// the FP32 Jacobi of the preconditioner (columns of mt_max rows in GateDesc::pre)
+cudaError_t launch_jacobi_mix(const GateDesc* d, int n_gates, int mt_max, int n_max, JacobiCtl* ctl, cudaStream_t s,
+                              int n_lead, unsigned spin_limit);
 // the whole preconditioner: W <- W V' for every complex128 gate with buffers; ctl is its
-// own control word
+// own control word (zeroed before)
 cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, JacobiCtl* ctl, cudaStream_t s,
                        int n_lead, unsigned spin_limit);
 // FP64 merge + gate contraction and right site

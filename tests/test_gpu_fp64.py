@@ -93,6 +93,42 @@ def test_spectrum_below_fp32(T, decay):
     assert np.linalg.norm(blk - blk_o) <= 1e-12 * np.linalg.norm(blk_o)
 
 
+@pytest.mark.parametrize("kind", ["equal", "pairs", "rank", "tail"])
+def test_close_and_vanishing_singular_values(T, kind):
+    """Pairs of singular values too close for a refinement step's angles, at and below its
+    limits, null columns, and a tail of 17 decades.  Untruncated: the block itself comes back
+    to a few eps |theta|_F of each of the two SVDs, and the left site is an isometry on the
+    columns above the tail (normalised columns of singular value s are orthogonal to
+    eps s_max / s)."""
+    rng = np.random.default_rng(7)
+    c, k = 24, 48
+    s = np.linspace(1.0, 0.5, k)
+    if kind == "equal":
+        s[:] = 1.0
+    elif kind == "pairs":
+        s[1::2] = s[::2] * (1 + 10.0 ** -np.linspace(1, 15, k // 2))
+    elif kind == "rank":
+        s[k // 3:] = 0.0
+    else:
+        s = 10.0 ** -np.linspace(0, 17, k)
+    u = np.linalg.qr(rng.standard_normal((k, k)) + 1j * rng.standard_normal((k, k)))[0]
+    v = np.linalg.qr(rng.standard_normal((k, k)) + 1j * rng.standard_normal((k, k)))[0]
+    dims, q = _chain(c, k, c)
+    sites = [rng.standard_normal((dims[i], 2, dims[i + 1])) + 0j for i in range(len(dims) - 1)]
+    sites[q], sites[q + 1] = u.reshape(c, 2, k), (s[:, None] * v).reshape(k, 2, c)
+    m = T.MPS(len(sites), dtype=T.TNSIM_C128, chi_max=64, renormalize=False)
+    m.import_sites(sites)
+    m.apply_layer(W.Layer(np.array([q], np.int32), np.eye(4, dtype=complex)[None], None))
+    got, out = m.spectrum(q + 1), m.export_sites()
+    m.close()
+    blk = out[q].reshape(k, -1) @ out[q + 1].reshape(-1, k)
+    assert np.linalg.norm(blk - (u * s) @ v) <= 64 * EPS * np.linalg.norm(s)
+    want = np.sort(s)[::-1][:len(got)]
+    assert np.max(np.abs(got - want)) <= 64 * EPS * np.linalg.norm(s)
+    iso = out[q].reshape(k, -1)[:, got >= 1e-3]
+    assert np.abs(iso.conj().T @ iso - np.eye(iso.shape[1])).max() <= 1e-11
+
+
 def test_canonical_form_and_memory_cap(T):
     """Canonical-form gates precondition diag(Lam) theta; a state made under a device-memory
     cap has no preconditioner buffers and gives the same state."""
