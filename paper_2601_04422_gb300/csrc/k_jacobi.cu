@@ -42,6 +42,7 @@
 #include <cooperative_groups.h>
 
 #include "jacobi_sched.cuh"
+#include "tc_common.cuh"
 #include "tnsim_internal.h"
 
 namespace cg = cooperative_groups;
@@ -53,9 +54,9 @@ namespace tnsim {
 // and the rotation parameters are then shared by 32 / LP pairs of a warp, and a CTA of
 // 16 LP threads leaves room for others on its SM that run while this one waits (with a
 // whole warp per pair these took ~110 of ~180 issue slots per pair and step at m = 128).
-// Shared memory holds a block as 16-byte units (two rows) [RPL / 2][BC columns][LP lanes],
-// rows padded with zeros to RPL LP: the accesses have constant offsets, no bounds and no
-// bank conflicts.
+// Shared memory holds a block as 16-byte units (two rows) [RPL / 2][BC columns][LP lanes]
+// (a whole warp per pair: columns contiguous, [BC][RPL / 2][LP]), rows padded with zeros to
+// RPL LP: the accesses have constant offsets, no bounds and no bank conflicts.
 // Block I's columns stay in registers over the BC rounds of the cross pairs; in the first
 // round of a sweep the pairs inside each block come first.  Column norms are tracked:
 // exact at the start of the visit, then a - t|g| and b + t|g| (the eigenvalues of the
@@ -63,8 +64,9 @@ namespace tnsim {
 // Inner products and norms run over the first md rows (EXT: fewer than the stored m).
 template <int BC, int LP, int RPL, bool EXT>
 struct Visit32 {
-    static constexpr int U = RPL / 2, PITCH = BC * LP;      // units per lane and column; units per row of units
-    static constexpr int BLOCK = U * PITCH;                  // units of a block
+    static constexpr int U = RPL / 2, BLOCK = U * BC * LP;   // units per lane and column; units of a block
+    static constexpr int COL = LP == 32 ? U * LP : LP;       // from a column to the next
+    static constexpr int PITCH = LP == 32 ? LP : BC * LP;    // from a lane's unit to its next
     float4 *XI, *XJ;                                         // the two blocks
     int w, l, kd;   // this thread's group and lane, its units inside the first md rows
 
@@ -72,22 +74,27 @@ struct Visit32 {
         : XI(xi), XJ(xj), w(threadIdx.x / LP), l(threadIdx.x % LP), kd((md / 2 - l + LP - 1) / LP) {}
     // column c of the two blocks (c < 2 BC): this lane's first unit
     __device__ __forceinline__ float4* unit(int c) const {
-        return (c >= BC ? XJ : XI) + (c & (BC - 1)) * LP + l;
+        return (c >= BC ? XJ : XI) + (c & (BC - 1)) * COL + l;
     }
+    // all visiting threads (a prefetching warp may share the CTA)
+    static __device__ __forceinline__ void sync() { asm volatile("bar.sync 0, %0;" ::"n"(BC * LP) : "memory"); }
     static __device__ __forceinline__ float sum(float v) {
 #pragma unroll
         for (int o = LP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         return v;
     }
-    __device__ __forceinline__ float norm2(int c) const {
-        const float4* p = unit(c);
+    __device__ __forceinline__ float norm2(const float4 (&x)[U]) const {
         float a = 0.f;
 #pragma unroll
-        for (int k = 0; k < U; ++k) {
-            const float4 x = p[k * PITCH];
-            if (!EXT || k < kd) a = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, a))));
-        }
+        for (int k = 0; k < U; ++k)
+            if (!EXT || k < kd)
+                a = fmaf(x[k].x, x[k].x, fmaf(x[k].y, x[k].y, fmaf(x[k].z, x[k].z, fmaf(x[k].w, x[k].w, a))));
         return sum(a);
+    }
+    __device__ __forceinline__ float norm2(int c) const {
+        float4 x[U];
+        load(x, c);
+        return norm2(x);
     }
     // x + d with the small correction d = (c-1) x + ... summed first and then added to x
     // with a single rounding.  Near convergence |(c-1) x| is below half an ulp of x: added
@@ -142,16 +149,15 @@ struct Visit32 {
         for (int k = 0; k < U; ++k) p[k * PITCH] = u[k];
     }
 
-    // exact norms of all columns, and the pairs inside both blocks (intra)
-    __device__ __forceinline__ void begin(int nI, int nJ, bool intra, float tol2, float zthr, float* __restrict__ nrm,
+    // The pairs inside both blocks, from exact norms.
+    __device__ __forceinline__ void inner(int nI, int nJ, float tol2, float zthr, float* __restrict__ nrm,
                                           int& my_rot, int& my_vis) const {
         const float na0 = norm2(w), nb0 = norm2(BC + w);
         if (l == 0) {
             nrm[w] = na0;
             nrm[BC + w] = nb0;
         }
-        __syncthreads();
-        if (!intra) return;
+        sync();
         // pairs inside block I (the first half of the groups) and inside block J (the rest)
         constexpr int half = BC / 2;
         const int base = w < half ? 0 : BC, nblk = w < half ? nI : nJ;
@@ -177,7 +183,7 @@ struct Visit32 {
                     nrm[b] = nb + tg;
                 }
             }
-            __syncthreads();
+            sync();
         }
     }
 
@@ -186,12 +192,22 @@ struct Visit32 {
     // the first BC / 2 rounds half h rotates I_h with J_h, in the others with the other half
     // of J.  A half's loads, shuffles and parameters then run beside the other's updates
     // (one barrier for all in every round: 50.2 against 43.6 ms for the chi 256 layer).
-    __device__ __forceinline__ void cross(float4 (&u)[U], int nI, int nJ, float tol2, float zthr,
+    // Exact norms first unless inner() left tracked ones; the first pair of a group are its
+    // own columns, so they need no barrier.
+    __device__ __forceinline__ void cross(float4 (&u)[U], int nI, int nJ, bool tracked, float tol2, float zthr,
                                           float* __restrict__ nrm, int& my_rot, int& my_vis) const {
         constexpr int H = BC / 2;
         constexpr bool halves = H * LP % 32 == 0;   // named barriers count whole warps
         const int h = w / H;
-        float a_i = nrm[w];
+        float a_i;
+        if (tracked) {
+            a_i = nrm[w];
+        } else {
+            a_i = norm2(u);
+            const float b0 = norm2(BC + w);
+            if (l == 0) nrm[BC + w] = b0;
+            __syncwarp();
+        }
 #pragma unroll 1
         for (int t = 0; t < BC; ++t) {
             const int b = ((w + t) & (H - 1)) + H * (h ^ (t / H));
@@ -208,7 +224,7 @@ struct Visit32 {
                     nrm[BC + b] = nb + tg;
                 }
             }
-            if (!halves || (t & (H - 1)) == H - 1) __syncthreads();
+            if (!halves || (t & (H - 1)) == H - 1) sync();
             else asm volatile("bar.sync %0, %1;" ::"r"(1 + h), "n"(H * LP) : "memory");
         }
     }
@@ -218,12 +234,12 @@ struct Visit32 {
     // barrier follows the wait.
     __device__ __forceinline__ void copy_in(const float2* WI, int nI, const float2* WJ, int nJ, int m) const {
         const int units = m / 2;
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = BC * LP / 32;
         for (int c = warp; c < 2 * BC; c += nw) {
             const int cc = c & (BC - 1);
             const float2* src = (c < BC ? WI : WJ) + (size_t)cc * m;
             const int have = cc < (c < BC ? nI : nJ) ? units : 0;
-            float4* dst = (c >= BC ? XJ : XI) + cc * LP;
+            float4* dst = (c >= BC ? XJ : XI) + cc * COL;
 #pragma unroll 4
             for (int i = lane; i < U * LP; i += 32) {
                 float4* p = dst + (i / LP) * PITCH + i % LP;
@@ -233,15 +249,40 @@ struct Visit32 {
         }
         asm volatile("cp.async.wait_all;\n" ::: "memory");
     }
+    // One block by one warp, a bulk copy per column counted on the mbarrier bar, zeros
+    // likewise.  (512-byte copies, from [RPL / 2][BC][LP], took 25 k cycles for two blocks.)
+    static __device__ __forceinline__ void bulk_in(float4* slot, const float2* W, int nc, int m, uint32_t bar) {
+        static_assert(LP == 32, "columns contiguous");
+        for (int c = 0; c < BC; ++c) {
+            const int have = c < nc ? m / 2 : 0;
+            float4* dst = slot + c * COL;
+            for (int i = have + (threadIdx.x & 31); i < COL; i += 32) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        const int c = threadIdx.x & 31;
+        if (c < nc)
+            asm volatile(
+                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                    smem_u32(slot + c * COL)),
+                "l"(W + (size_t)c * m), "r"(m * 8), "r"(bar)
+                : "memory");
+    }
+    // block I's columns straight from the registers
+    __device__ __forceinline__ void regs_out(const float4 (&u)[U], float2* WI, int nI, int m) const {
+        if (w >= nI) return;
+        float4* dst = reinterpret_cast<float4*>(WI + (size_t)w * m);
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (k * LP + l < m / 2) __stcg(dst + k * LP + l, u[k]);
+    }
     // blocks out (L2 stores), by the warps from warp0 on
     __device__ __forceinline__ void copy_out(float2* WI, int nI, float2* WJ, int nJ, int m, int warp0) const {
         const int units = m / 2;
-        const int warp = (int)(threadIdx.x >> 5) - warp0, lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5) - warp0;
+        const int warp = (int)(threadIdx.x >> 5) - warp0, lane = threadIdx.x & 31, nw = BC * LP / 32 - warp0;
         for (int c = warp; c < nI + nJ; c += nw) {
             const bool isI = c < nI;
             const int cc = isI ? c : c - nI;
             float4* dst = reinterpret_cast<float4*>((isI ? WI : WJ) + (size_t)cc * m);
-            const float4* src = (isI ? XI : XJ) + cc * LP;
+            const float4* src = (isI ? XI : XJ) + cc * COL;
 #pragma unroll 4
             for (int i = lane; i < units; i += 32) __stcg(dst + i, src[(i / LP) * PITCH + i % LP]);
         }
@@ -516,11 +557,11 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
                 if constexpr (sizeof(T) == 8) {
                     visit64<BC>(X, X + (size_t)BC * m, m, nI, nJ, intra, (float)tol, zthr, s_red, s_bn, s_par, rot, my_vis);
                 } else {
-                    vis.begin(nI, nJ, intra, tol2, zthr, s_bn, rot, my_vis);
+                    if (intra) vis.inner(nI, nJ, tol2, zthr, s_bn, rot, my_vis);
                     if (nJ > 0) {
                         float4 u[V32::U];
                         vis.load(u, vis.w);
-                        vis.cross(u, nI, nJ, tol2, zthr, s_bn, rot, my_vis);
+                        vis.cross(u, nI, nJ, intra, tol2, zthr, s_bn, rot, my_vis);
                         vis.store(vis.w, u);
                         __syncthreads();
                     }
@@ -589,6 +630,290 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
             }
         }
         __syncthreads();
+    }
+}
+
+// The persistent kernel for FP32 columns so long that one CTA fills an SM (m > 256), with a
+// warp beside the visiting threads: a visit's claim, copies, fences and report took 20 of its
+// 49 k cycles at m = 512, and no other CTA covers them there.  In the cross pairs block I's
+// columns are in registers, so its slot and a third one take the next visit's blocks: the
+// extra warp claims the visit, has both blocks copied in, stores the finished visit's block
+// J from its slot and reports it, while the others are at work on the next.
+//   MID    the visiting threads arrive when block I's slot is free, the warp waits
+//   READY  all: the visit is through, the next one's blocks are in place
+// The warp claims ahead only while there are more visits than CTAs: a claim held while
+// another CTA idles would delay its gate's round.  A CTA still never waits while it holds a
+// claim, except for its own visit's end and copies.  Registers: 512 threads of 104 and a
+// group of four warps (three leave) of 40 are within the launch's 640 x 96; with one extra
+// warp and no redistribution 96 a thread spilled (37.5 against 41.4 ms).
+// 100 qubits at chi 256, 50 gates of m = n = 512: 44.1 -> 37.5 ms.  At m <= 256 the CTAs of
+// an SM cover for each other: this kernel took 4.5 against 4.3 ms for 32 gates at m = 256.
+struct VisitInfo {
+    float2 *WI, *WJ;             // the two blocks' columns
+    GateOut* out;
+    int nI, nJ, m, md;           // their columns (nI = 0: no work, nJ = 0: block I alone), stored rows, rows of the products
+    int intra, single;           // first round of a sweep; a gate of one block
+    float tol2, zthr;
+    int V, rnd, R, leave;        // visits of a round, round and rounds of a sweep (report); no more visits
+};
+template <int BC, int LP, int RPL, bool EXT>
+__global__ void __launch_bounds__(BC * LP + 128, 1)
+k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in, int max_sweeps,
+            JacobiCtl* __restrict__ ctl, unsigned spin_limit) {
+    using V32 = Visit32<BC, LP, RPL, EXT>;
+    constexpr int NT = BC * LP, NW = NT / 32;
+    constexpr unsigned kPolls = 1u << 24;   // of a wait for this CTA's own copies or threads
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float4* const xs = reinterpret_cast<float4*>(smem_raw);   // slots: block I in 0, block J in 1 and 2 in turn
+    __shared__ VisitInfo s_info[2];
+    __shared__ int s_rot[2], s_vis[2], s_last[2];   // of a visit: rotations, pairs; one-block gates: 2 sweep + (it rotated)
+    __shared__ int s_claimed;                       // the last visit claimed
+    __shared__ int s_done;                          // warps whose part is stored and fenced, over all visits
+    __shared__ float s_bn[2 * BC];
+    __shared__ short s_V[kScanTable];
+    __shared__ __align__(8) uint64_t s_full;
+    const uint32_t bar = smem_u32(&s_full);
+    const int lane = threadIdx.x & 31;
+    auto mid_arrive = [] { asm volatile("fence.proxy.async.shared::cta;\nbar.arrive 3, %0;" ::"n"(NT + 32) : "memory"); };
+    auto mid_wait = [] { asm volatile("bar.sync 3, %0;" ::"n"(NT + 32) : "memory"); };
+    auto ready = [] { asm volatile("fence.proxy.async.shared::cta;\nbar.sync 4, %0;" ::"n"(NT + 32) : "memory"); };
+    for (int g = threadIdx.x; g < n_gates && g < kScanTable; g += blockDim.x)
+        s_V[g] = (short)tour_of<BC>(gd[g]).V;
+    if (threadIdx.x < 2) s_rot[threadIdx.x] = s_vis[threadIdx.x] = s_last[threadIdx.x] = 0;
+    if (threadIdx.x == 2) s_done = s_claimed = 0;
+    if (threadIdx.x == 3) {
+        mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\nfence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncthreads();
+
+    if (threadIdx.x >= NT) {
+        // ---- the prefetching warp (of a group of four: registers move by groups)
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        if (threadIdx.x >= NT + 32) return;
+        int scan0 = (int)(((long long)blockIdx.x * n_lead) / gridDim.x);
+        unsigned spins = 0, last_progress = 0;
+        uint32_t phase = 0;
+        // a finished visit: block J out, then count it, and advance its gate after the
+        // round's last one
+        auto store_J = [&](int p) {
+            const VisitInfo& q = s_info[p];
+            if (lane < q.nJ)
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(q.WJ + (size_t)lane * q.m),
+                             "r"(smem_u32(xs + (size_t)(1 + p) * V32::BLOCK + lane * V32::COL)), "r"(q.m * 8)
+                             : "memory");
+            asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group 0;\nfence.proxy.async;" ::: "memory");
+            __threadfence();
+            __syncwarp();
+        };
+        auto report = [&](int p) {
+            if (lane == 0) {
+                const VisitInfo& q = s_info[p];
+                GateOut* out = q.out;
+                if (s_rot[p]) {
+                    atomicAdd(&out->rot_sweep, s_rot[p]);
+                    if (!EXT) atomicAdd(&out->rotations, (unsigned long long)s_rot[p]);
+                }
+                if (s_vis[p] && !EXT) atomicAdd(&out->visits, (unsigned long long)s_vis[p]);
+                __threadfence();
+                if (atomicAdd(&out->done, 1) + 1 == q.V) {
+                    out->done = 0;
+                    bool fin = false;
+                    int sweep = q.rnd / q.R;
+                    if (q.rnd - sweep * q.R == q.R - 1) {
+                        int rs = atomicExch(&out->rot_sweep, 0);
+                        if (q.single) {
+                            sweep = s_last[p] >> 1;
+                            rs = s_last[p] & 1;
+                        }
+                        if (rs == 0 || sweep + 1 >= max_sweeps) {
+                            fin = true;
+                            out->sweeps = min(sweep + 1, max_sweeps);
+                            // keep a timeout the contraction reported (5) before this launch
+                            if (rs != 0 && out->status < 4) out->status = 4;
+                        }
+                    }
+                    __threadfence();
+                    if (fin) {
+                        atomicExch(&out->finished, 1);
+                        atomicAdd(&ctl->n_finished, 1);
+                    } else {
+                        atomicExch(&out->claim, (unsigned long long)(q.rnd + 1) << 32);
+                    }
+                    atomicAdd(&ctl->progress, 1u);
+                }
+                s_rot[p] = s_vis[p] = s_last[p] = 0;
+            }
+            __syncwarp();
+        };
+        for (int i = 0;; ++i) {
+            const int p = i & 1;
+            bool reported = i == 0;
+            if (i > 0) mid_wait();
+            int found = 0, fg = -1, frnd = 0, fv = 0, leave = 0;
+            for (;;) {
+                if (!reported && __all_sync(0xffffffffu, *((volatile int*)&s_done) == i * NW)) {
+                    store_J(p ^ 1);
+                    report(p ^ 1);
+                    reported = true;
+                }
+                const int fin = *((volatile int*)&ctl->n_finished), err = *((volatile int*)&ctl->error);
+                if (__any_sync(0xffffffffu, err || (reported && fin >= n_gates))) {
+                    leave = 1;
+                    break;
+                }
+                // ahead of the running visit's end only with work for every CTA
+                if (__all_sync(0xffffffffu, reported || (long long)(n_gates - fin) * s_V[0] * 2 > (long long)gridDim.x * 3))
+                    claim_scan<BC>(gd, n_gates, s_V, scan0, lane, found, fg, frnd, fv);
+                if (found) break;
+                if (reported) {
+                    if (lane == 0) {
+                        const unsigned pr = *((volatile unsigned*)&ctl->progress);
+                        if (pr != last_progress) {
+                            last_progress = pr;
+                            spins = 0;
+                        } else if (++spins > spin_limit) {
+                            atomicExch(&ctl->error, 1);
+                        }
+                    }
+                    __syncwarp();
+                }
+                __nanosleep(256);
+            }
+            if (found) {
+                if (lane == 0) *((volatile int*)&s_claimed) = i;
+                __threadfence();   // order the claim before reading the blocks of the previous round
+                scan0 = fg;
+                const GateDesc& d = gd[fg];
+                const int md = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2], m = EXT ? md + n : md;
+                const int nb = (n + BC - 1) / BC, P = nb + (nb & 1), R = nb == 1 ? 1 : P - 1, round = frnd % R;
+                int I = 0, J = -1;
+                if (nb > 1) {
+                    rr_pair(P, round, fv, I, J);
+                    if (I >= nb) { I = J; J = -1; }
+                    else if (J >= nb) J = -1;
+                }
+                const int nI = J >= 0 || round == 0 ? min(BC, n - I * BC) : 0, nJ = J >= 0 ? min(BC, n - J * BC) : 0;
+                float2* W = EXT ? (float2*)d.pre : (float2*)d.W;
+                float2 *WI = W + (size_t)I * BC * m, *WJ = W + (size_t)(J >= 0 ? J : 0) * BC * m;
+                if (nI > 0) {
+                    asm volatile("fence.proxy.async;" ::: "memory");
+                    if (lane == 0) mbar_expect_tx(bar, (uint32_t)((nI + nJ) * m) * 8u);
+                    __syncwarp();
+                    V32::bulk_in(xs, WI, nI, m, bar);
+                    V32::bulk_in(xs + (size_t)(1 + p) * V32::BLOCK, WJ, nJ, m, bar);
+                }
+                if (lane == 0) {
+                    VisitInfo& q = s_info[p];
+                    q.WI = WI;
+                    q.WJ = WJ;
+                    q.out = d.out;
+                    q.nI = nI;
+                    q.nJ = nJ;
+                    q.m = m;
+                    q.md = md;
+                    q.intra = round == 0;
+                    q.single = nb == 1;
+                    q.V = nb == 1 ? 1 : P / 2;
+                    q.rnd = frnd;
+                    q.R = R;
+                    q.leave = 0;
+                    // tolerances: see k_jacobi
+                    const double tol = tol_in > 0.0 ? tol_in : 2.0 * Eps<float>::v;
+                    q.tol2 = (float)(tol * tol);
+                    double frob2 = d.out->frob2;
+                    if (EXT) {
+                        const double f = mix_scale(frob2);
+                        frob2 *= f * f;
+                    }
+                    q.zthr = (float)(Eps<float>::v * Eps<float>::v * (double)max(md, n) * frob2);
+                }
+                if (nI > 0) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(bar, phase, kPolls))) {
+                        if (lane == 0) atomicExch(&ctl->error, 1);
+                        leave = 1;
+                        mbar_wait(bar, phase, kPolls);   // not before the copies have landed
+                    }
+                    phase ^= 1;
+                }
+            }
+            if (leave && lane == 0) s_info[p].leave = 1;
+            __syncwarp();
+            ready();
+            if (!reported) {
+                store_J(p ^ 1);
+                // the visiting threads fence their part early in the next visit or on their way out
+                bool done = false;
+                for (unsigned k = 0; k < kPolls && !done; ++k) done = *((volatile int*)&s_done) >= i * NW;
+                if (__all_sync(0xffffffffu, done)) {
+                    __threadfence();
+                    report(p ^ 1);
+                } else if (lane == 0) {
+                    atomicExch(&ctl->error, 1);
+                }
+            }
+            if (leave) return;
+        }
+    }
+
+    // ---- the visiting threads
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+    bool pending = false;   // the last visit's stores are not fenced yet
+    auto signal = [&] {
+        __threadfence();   // every thread's block stores before the report
+        __syncwarp();
+        if (lane == 0) atomicAdd(&s_done, 1);
+        pending = false;
+    };
+    ready();
+    for (int i = 0;; ++i) {
+        const int p = i & 1;
+        const VisitInfo& q = s_info[p];
+        if (q.leave) {
+            if (pending) signal();
+            return;
+        }
+        const V32 vis(xs, xs + (size_t)(1 + p) * V32::BLOCK, q.md);
+        int my_rot = 0, my_vis = 0;
+        if (q.nJ > 0) {
+            const int nI = q.nI, nJ = q.nJ;
+            const bool intra = q.intra;
+            const float tol2 = q.tol2, zthr = q.zthr;
+            if (intra) vis.inner(nI, nJ, tol2, zthr, s_bn, my_rot, my_vis);
+            float4 u[V32::U];
+            vis.load(u, vis.w);
+            mid_arrive();
+            if (pending) signal();
+            vis.cross(u, nI, nJ, intra, tol2, zthr, s_bn, my_rot, my_vis);
+            vis.regs_out(u, q.WI, nI, q.m);
+        } else {
+            if (pending) signal();
+            if (q.nI > 0) {
+                // a gate of one block runs all its sweeps in this visit
+                for (int sweep = 0;; ++sweep) {
+                    int rot = 0;
+                    vis.inner(q.nI, 0, q.tol2, q.zthr, s_bn, rot, my_vis);
+                    my_rot += rot;
+                    if (!q.single) break;
+                    unsigned any;
+                    asm volatile("{\n.reg .pred a, b;\nsetp.ne.u32 a, %1, 0;\nbarrier.cta.red.or.pred b, 0, %2, a;\nselp.u32 %0, 1, 0, b;\n}"
+                                 : "=r"(any) : "r"((unsigned)rot), "n"(NT) : "memory");
+                    if (threadIdx.x == 0) s_last[p] = 2 * sweep + (int)any;
+                    if (!any || sweep + 1 >= max_sweeps) break;
+                }
+                vis.copy_out(q.WI, q.nI, q.WJ, 0, q.m, 0);
+            }
+            mid_arrive();
+        }
+        my_rot = __reduce_add_sync(0xffffffffu, my_rot);
+        my_vis = __reduce_add_sync(0xffffffffu, my_vis);
+        if (lane == 0 && my_rot) atomicAdd(&s_rot[p], my_rot);
+        if (lane == 0 && my_vis) atomicAdd(&s_vis[p], my_vis);
+        // a fence waits until the stores have landed: with the next visit in hand, later
+        pending = true;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (*((volatile int*)&s_claimed) != i + 1) signal();
+        ready();
     }
 }
 
@@ -674,11 +999,11 @@ k_jacobi_cl(const GateDesc* __restrict__ gd, double tol_in, int max_sweeps) {
                 float4 u[V32::U];
                 const int na = (sb + 1) % 3, nbs = (sb + 2) % 3;   // slots of the next a and b
                 if (seat) {
-                    vis.begin(nA, nB, r == 0, tol2, zthr, s_n, rot, my_vis);
+                    if (r == 0) vis.inner(nA, nB, tol2, zthr, s_n, rot, my_vis);
                     vis.load(u, vis.w);
                 }
                 asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-                if (seat && nA > 0 && nB > 0) vis.cross(u, nA, nB, tol2, zthr, s_n, rot, my_vis);
+                if (seat && nA > 0 && nB > 0) vis.cross(u, nA, nB, r == 0, tol2, zthr, s_n, rot, my_vis);
                 __syncthreads();
                 if (r == R - 1) {
                     // this seat's count, to every CTA
@@ -689,7 +1014,7 @@ k_jacobi_cl(const GateDesc* __restrict__ gd, double tol_in, int max_sweeps) {
                 }
                 asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
                 if (seat) {
-                    float4* da = cl.map_shared_rank(slot(a_stays_a ? na : nbs), to_a) + vis.w * LP + vis.l;
+                    float4* da = cl.map_shared_rank(slot(a_stays_a ? na : nbs), to_a) + vis.w * V32::COL + vis.l;
 #pragma unroll
                     for (int k = 0; k < V32::U; ++k) da[k * V32::PITCH] = u[k];
                     float4* db = cl.map_shared_rank(slot(b_turns_a ? na : nbs), to_b);
@@ -804,6 +1129,24 @@ static cudaError_t launch_cl(const GateDesc* d, int n_gates, int m_max, int n_ma
     return cudaLaunchKernelEx(&cfg, kernel, d, tol, max_sweeps < 1 ? 1 : max_sweeps);
 }
 
+template <int BC, int LP, int RPL, bool EXT = false>
+static cudaError_t launch_pf(const GateDesc* d, int n_gates, int n_lead, int n_max, double tol, int max_sweeps,
+                             JacobiCtl* ctl, cudaStream_t s, unsigned spin_limit) {
+    const auto kernel = k_jacobi_pf<BC, LP, RPL, EXT>;
+    const size_t smem = (size_t)3 * BC * LP * RPL * sizeof(float2);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    const int nb = (n_max + BC - 1) / BC;
+    const long long visits = (long long)n_gates * ((nb == 1) ? 1 : (nb + (nb & 1)) / 2);
+    const int lead = (n_lead < 1 || n_lead > n_gates) ? n_gates : n_lead;
+    kernel<<<(unsigned)(visits < sms ? visits : sms), BC * LP + 128, smem, s>>>(
+        d, n_gates, lead, tol, max_sweeps < 1 ? 1 : max_sweeps, ctl, spin_limit ? spin_limit : kSpinLimit);
+    return cudaGetLastError();
+}
+
 template <typename T, int BC, int LP, int RPL, int MINB, bool EXT = false>
 static cudaError_t launch_bc(const GateDesc* d, int n_gates, int n_lead, int m_max, int n_max, double tol,
                              int max_sweeps, JacobiCtl* ctl, cudaStream_t s, unsigned spin_limit) {
@@ -860,7 +1203,7 @@ cudaError_t launch_jacobi(const GateDesc* d, int n_gates, int m_max, int n_max, 
         if (m_max <= 64) return narrow ? TNSIM_JAC(8, 8, 16, 8) : TNSIM_JAC(16, 4, 16, 8);
         if (m_max <= 128) return narrow ? TNSIM_JAC(8, 8, 16, 8) : TNSIM_JAC(16, 8, 16, 4);
         if (m_max <= 256) return narrow ? TNSIM_JAC(8, 16, 16, 4) : TNSIM_JAC(16, 16, 16, 2);
-        if (m_max <= 512) return narrow ? TNSIM_JAC(8, 32, 16, 2) : TNSIM_JAC(16, 32, 16, 1);
+        if (m_max <= 512) return narrow ? TNSIM_JAC(8, 32, 16, 2) : launch_pf<16, 32, 16>(d, n_gates, n_lead, n_max, tol, max_sweeps, ctl, s, spin_limit);
         return TNSIM_JAC(8, 32, 32, 1);
     } else {
         if (!narrow && m_max <= 256) {
