@@ -489,7 +489,8 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_corr(const GateDesc* __res
     const double2 *E = (const double2*)d.pre_b, *Q = (const double2*)d.pre_d;
     const float2* K = (const float2*)d.pre;
     const bool skip = mix_rows_above(mix_rows(d, n, 0), n, kRowUnit0, kRefRow0);
-    float2 acc[2][2] = {};
+    constexpr int R = TileOf<float2>::R;
+    float2 acc[R][R] = {};
     auto herm = [&](const double2* M, float f) {   // f M[i, k] = f conj(M[k, i])
         return [=](int c, int k) {
             if (i0 + c >= n) return make_float2(0.f, 0.f);
@@ -520,9 +521,9 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_corr(const GateDesc* __res
     Df* F = mix_bufs(d, 0).F;
     const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
 #pragma unroll
-    for (int jj = 0; jj < 2; ++jj)
+    for (int jj = 0; jj < R; ++jj)
 #pragma unroll
-        for (int ii = 0; ii < 2; ++ii) {
+        for (int ii = 0; ii < R; ++ii) {
             const int i = i0 + rx + 8 * ii, j = j0 + cy + 8 * jj;
             if (i >= n || j >= n) continue;
             const size_t t = (size_t)j * n + i;

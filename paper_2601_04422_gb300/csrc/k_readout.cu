@@ -261,7 +261,7 @@ cudaError_t launch_amplitudes(void* const* sites, const int* chi, int n_qubits, 
 // Small tiles over a grid of (tiles, steps): a step's time is its latency, so small tiles
 // over many SMs, and every step that does not depend on another in the same launch.  (One
 // thread per element, with its operands from L2 on every k: 21 + 38 us per step at chi 64,
-// complex64, against 9 + 10.)  The sums keep the order of that form, k ascending in
+// complex64, against 7 + 9.)  The sums keep the order of that form, k ascending in
 // one accumulator, then p'.
 template <typename T>
 __global__ void __launch_bounds__(TILE_THREADS) k_transfer1(const TransferDesc* __restrict__ list, TransferDesc one) {

@@ -1,20 +1,21 @@
 // A small tile of a complex product by 64 threads, shared by the FP64 products (k_fp64.cu)
-// and the read-out (k_readout.cu): 16 x 16 for complex64, 8 x 8 for complex128.
+// and the read-out (k_readout.cu): 8 x 8, one output per thread.
 //
 // The read-out's products are chains of small matrices, so a tile's time is its latency and
-// what counts is how many SMs share a product.  FP64 issues once in 64 cycles per scheduler:
-// one output per thread is 4 FP64 instructions per k and warp, and small matrices spread
-// over as many schedulers as there are warps of outputs.  (2 x 2 outputs per thread: 13 us
-// for a 24 x 12 x 12 product, the zeros of the K step included, against 3.)
+// what counts is how many SMs and schedulers share a product.  FP64 issues once in 64 cycles
+// per scheduler: one output per thread is 4 FP64 instructions per k and warp.  (2 x 2 outputs
+// per thread: 13 us for a complex128 24 x 12 x 12 product, the zeros of the K step included,
+// against 3; a transfer of the read-out at chi 128, complex64, 24.5 us with 16 x 16 tiles in
+// K steps of 16, 17 with 8 x 8 in steps of 64: fewer waits for a step's operands.)
 // The next K step's operands are loaded while this one's are used.
 #pragma once
 #include <cuda_runtime.h>
 
 namespace tnsim {
 
-constexpr int TILE_K = 16;         // K step
 constexpr int TILE_THREADS = 64;
-template <typename C> struct TileOf { static constexpr int E = sizeof(C) == 8 ? 16 : 8, R = E / 8; };   // edge, outputs per thread and side
+// edge, outputs per thread and side, K step
+template <typename C> struct TileOf { static constexpr int E = 8, R = 1, K = sizeof(C) == 8 ? 64 : 16; };
 
 // acc += a b; acc += conj(a) b; acc += a conj(b) -- one fixed order of the roundings
 struct MulAdd {
@@ -47,7 +48,7 @@ struct MulAddConj {
 // 3 - 6 % more instructions).
 template <typename C, bool AK, bool BK, bool PAIRED, bool SPLIT, typename OP, typename LA, typename LB>
 __device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[TileOf<C>::R][TileOf<C>::R]) {
-    constexpr int E = TileOf<C>::E, R = TileOf<C>::R, PER = E * TILE_K / TILE_THREADS;
+    constexpr int E = TileOf<C>::E, R = TileOf<C>::R, TILE_K = TileOf<C>::K, PER = E * TILE_K / TILE_THREADS;
     __shared__ C As[TILE_K][E + 1], Bs[TILE_K][E + 1];
     const int tid = threadIdx.x, rx = tid & 7, cy = tid >> 3;
     C na[PER], nb[PER];
