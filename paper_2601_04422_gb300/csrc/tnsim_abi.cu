@@ -1422,7 +1422,7 @@ tnsim_status tnsim_sample(tnsim_mps* m, int64_t n_shots, const double* uniforms,
     if (s != TNSIM_OK) return s;
     int chi_cap = 1;
     for (int b = 0; b <= n; ++b) chi_cap = std::max(chi_cap, m->ub[b]);
-    const size_t es = m->esz, env = (size_t)chi_cap * chi_cap * es;
+    const size_t es = m->esz, env = ((size_t)chi_cap * chi_cap * es + 15) / 16 * 16;
     const size_t S = (size_t)n_shots;
     cudaStream_t st = m->stream;
     // one stream-ordered allocation for everything
@@ -1430,19 +1430,18 @@ tnsim_status tnsim_sample(tnsim_mps* m, int64_t n_shots, const double* uniforms,
     auto take = [&](size_t bytes) { const size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
     const size_t o_R = take(env * (n + 1)), o_tmp = take(env * 2), o_op = take(8 * sizeof(double));
     const size_t o_u = take(sizeof(double) * nu), o_bits = take((size_t)nu);
-    const size_t o_v0 = take(S * chi_cap * es), o_v1 = take(S * chi_cap * es);
-    const size_t o_w = take(S * 2 * chi_cap * es), o_y = take(S * 2 * chi_cap * es);
-    const size_t o_p = take(sizeof(double) * 2 * S), o_flag = take(sizeof(int) * 2 * S);
+    const size_t o_w = take(S * 2 * chi_cap * es), o_w1 = take(S * 2 * chi_cap * es);
+    const size_t o_p = take(sizeof(double) * 2 * S), o_p1 = take(sizeof(double) * 2 * S);
+    const size_t o_flag = take(sizeof(int) * 2 * S);
     const size_t o_id = take(sizeof(int) * 2 * S), o_par = take(sizeof(int) * S), o_node = take(sizeof(int) * S);
     const size_t o_cnt = take(sizeof(int) + sizeof(unsigned long long) + 8);
     char* base = nullptr;
     CUDA_TRY(cudaMallocAsync((void**)&base, off, st));
     SampleWork w;
-    w.v_cur = base + o_v0;
-    w.v_next = base + o_v1;
     w.w = base + o_w;
-    w.y = base + o_y;
-    w.p = (double*)(base + o_p);
+    w.w_next = base + o_w1;
+    w.p_cur = (double*)(base + o_p);
+    w.p_next = (double*)(base + o_p1);
     w.flag = (int*)(base + o_flag);
     w.id = (int*)(base + o_id);
     w.parent = (int*)(base + o_par);
@@ -1457,7 +1456,10 @@ tnsim_status tnsim_sample(tnsim_mps* m, int64_t n_shots, const double* uniforms,
     cudaError_t e = cudaMemcpyAsync(base + o_op, ident, sizeof(ident), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_u, uniforms, sizeof(double) * nu, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_R + env * n, one.data(), es, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_v0, one.data(), es, cudaMemcpyHostToDevice, st);
+    // the root: one node of weight 1 whose row is [1]
+    if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_w, one.data(), es, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_p, ident, sizeof(double), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.parent, 0, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_cnt, &c0, sizeof(c0), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.node_of, 0, sizeof(int) * S, st);
     // right environments R_n = [[1]], R_q from R_{q+1} (identity operator)
@@ -1474,7 +1476,6 @@ tnsim_status tnsim_sample(tnsim_mps* m, int64_t n_shots, const double* uniforms,
                                             n_shots, (int)bound, (const double*)(base + o_u), (uint8_t*)(base + o_bits), w, st)
                 : launch_sample_site<double>(site_ptr(m, q), m->ub[q], m->ub[q + 1], base + o_R + env * (q + 1), q, n,
                                              n_shots, (int)bound, (const double*)(base + o_u), (uint8_t*)(base + o_bits), w, st);
-        std::swap(w.v_cur, w.v_next);
     }
     Cnt c1 = {0, 0, 0ull};
     if (e == cudaSuccess) e = cudaMemcpyAsync(bits_out, base + o_bits, (size_t)nu, cudaMemcpyDeviceToHost, st);

@@ -250,11 +250,10 @@ cudaError_t encode_plane_maps(int mode, void* planes, int slots, int rows, int k
 
 // Work buffers of perfect sampling (k_sample.cu); node arrays hold at most `shots` entries
 struct SampleWork {
-    void* v_cur;                   // [nodes][chi_max] prefix row vectors of this site
-    void* v_next;                  // [nodes][chi_max] those of the next site
-    void* w;                       // [nodes][2 chi_max]  v A_q
-    void* y;                       // [2 nodes][chi_max]  (v A_q^b) Rt_{q+1}
-    double* p;                     // [2 nodes] outcome weights
+    void* w;                       // [nodes][2 chi_max] v A of the last site: rows (parent node, bit)
+    void* w_next;                  // this site's
+    double* p_cur;                 // [2 nodes] outcome weights of the last site
+    double* p_next;                // this site's
     int* flag;                     // [2 nodes] child (node, bit) drawn by some shot
     int* id;                       // [2 nodes] next-site index of each child, -1 if none
     int* parent;                   // [shots] child (2 node + bit) of each next-site node
