@@ -27,9 +27,10 @@ constexpr int TR_THREADS = 512;
 constexpr int TR_MAXN = 1024;
 constexpr int CN_COLS = 32;        // columns per CTA of k_colnorm2 (8 warps, 4 columns each)
 
-// a comes after b in the sorted order (descending value, ascending index)
+// a comes after b in the sorted order (descending value, ascending index); by the bits, see above()
 __device__ __forceinline__ bool after(double ka, int ia, double kb, int ib) {
-    return ka < kb || (ka == kb && ia > ib);
+    const long long a = __double_as_longlong(ka), b = __double_as_longlong(kb);
+    return a < b || (a == b && ia > ib);
 }
 
 // Squared column norms of the converged W, spread over many CTAs: grid (column chunks
@@ -71,23 +72,17 @@ __global__ void __launch_bounds__(256) k_colnorm2(const GateDesc* __restrict__ g
     }
 }
 
-// block-wide sum of one double per thread (TR_THREADS threads); every thread gets it
-__device__ __forceinline__ double tr_block_sum(double v, double* red) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-#pragma unroll 1
-    for (int w = 0; w < TR_THREADS / 32; ++w) t += red[w];
-    return t;
-}
+// order of two non-negative doubles (or the sort's -1 padding) by their bits: an FP64
+// compare issues like every FP64 instruction once in 64 cycles per scheduler
+__device__ __forceinline__ bool above(double a, double b) { return __double_as_longlong(a) > __double_as_longlong(b); }
 
 // Sort the squared norms, pick the kept rank, discarded weight and renormalisation.
 // One CTA per gate: bitonic sort (descending value, then ascending column), then
 // parallel reductions and a suffix scan of the sorted values for the cutoff rule.
+// What it costs is FP64 instructions, so only the warps that hold values sum, comparisons
+// are made on bits, counts by ballots, the rank test on squares, and one warp forms the
+// discarded weight and the scale while the others take the square roots (all 16 warps
+// doing everything: 26 - 41 us per layer at n = 8 - 256; 9 - 17 now).
 template <typename T>
 __global__ void __launch_bounds__(TR_THREADS) k_truncate(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.x];
@@ -95,13 +90,12 @@ __global__ void __launch_bounds__(TR_THREADS) k_truncate(const GateDesc* __restr
     const int chiL = d.chi[q], chiM = d.chi[q + 1], chiR = d.chi[q + 2];
     const int m = 2 * chiL, n = 2 * chiR;
     GateOut* out = d.out;
+    constexpr int NW = TR_THREADS / 32;
 
     __shared__ double key[TR_MAXN];
     __shared__ int idx[TR_MAXN];
-    __shared__ double red[TR_THREADS / 32];
-    __shared__ double wsum[TR_THREADS / 32];
-    __shared__ int s_k;
-    __shared__ double s_scale;
+    __shared__ double red[NW], wsum[NW];
+    __shared__ double s_total, s_disc, s_scale;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int P2 = 1;
@@ -135,54 +129,84 @@ __global__ void __launch_bounds__(TR_THREADS) k_truncate(const GateDesc* __restr
     }
 
     // each thread owns up to two consecutive sorted entries: 2 tid, 2 tid + 1
-    const int j0 = 2 * tid, j1 = 2 * tid + 1;
+    const int j0 = 2 * tid, j1 = 2 * tid + 1, nw = (n + 63) >> 6;   // warps with entries
     const double v0 = j0 < n ? key[j0] : 0.0, v1 = j1 < n ? key[j1] : 0.0;
-    const double total = tr_block_sum(v0 + v1, red);
+    double pair = 0.0;
+    if (warp < nw) {
+        pair = v0 + v1;
+        double v = pair;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) red[warp] = v;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        double t = red[0];
+        for (int w = 1; w < nw; ++w) t += red[w];
+        if (lane == 0) s_total = t;
+    }
+    __syncthreads();
+    const double total = s_total;
+    const long long tb = __double_as_longlong(total);
+    const bool some = tb > 0 && tb <= 0x7ff0000000000000ll;   // not NaN either
     int k = 1;
-    double eps = 0.0, scale = 1.0;
-    if (total > 0.0) {
-        const double smax = sqrt(key[0]);
-        const double thr = EpsT<T>::v * (double)max(m, n) * smax;
-        // the values are sorted, so the nonzero ones are a prefix
-        const double nzc = tr_block_sum((double)((j0 < n && sqrt(v0) > thr) + (j1 < n && sqrt(v1) > thr)), red);
-        const int nonzero = (int)nzc;
+    if (some) {
+        // sqrt(v) > eps max(m, n) s_max; the values are sorted, so these are a prefix
+        const double f = EpsT<T>::v * (double)max(m, n);
+        bool z0 = false, z1 = false;
+        if (warp < nw) {
+            const double thr2 = f * f * key[0];
+            z0 = j0 < n && above(v0, thr2);
+            z1 = j1 < n && above(v1, thr2);
+        }
+        int nonzero = __syncthreads_count(z0);
+        nonzero += __syncthreads_count(z1);
         // the rank of an m x n matrix is at most min(m, n); this also bounds the new
         // site shapes by the slot capacities
         k = max(1, min(min(d.chi_max, nonzero), min(m, n)));
         // suffix sums S_j = sum_{i >= j} key[i] (a reverse inclusive scan over the thread
         // pairs): S is non-increasing in j, so the entries with S_j > lim form a prefix
-        const double pair = v0 + v1;
         double incl = pair;     // inclusive scan from the last thread down
+        if (warp < nw) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double y = __shfl_down_sync(0xffffffffu, incl, o);
-            if (lane + o < 32) incl += y;
+            for (int o = 1; o < 32; o <<= 1) {
+                const double y = __shfl_down_sync(0xffffffffu, incl, o);
+                if (lane + o < 32) incl += y;
+            }
+            if (lane == 0) wsum[warp] = incl;      // the warp's total (its lane 0 holds all 32)
         }
         __syncthreads();
-        if (lane == 0) wsum[warp] = incl;      // the warp's total (its lane 0 holds all 32)
-        __syncthreads();
-        double later = 0.0;                    // the sum of every later warp
-        for (int w = warp + 1; w < TR_THREADS / 32; ++w) later += wsum[w];
-        const double S0 = incl + later;        // S_{j0}
-        const double S1 = S0 - v0;             // S_{j1}
+        double S0 = 0.0, S1 = 0.0;                 // S_{j0}, S_{j1}
+        if (warp < nw) {
+            double later = 0.0;                    // the sum of every later warp
+            for (int w = warp + 1; w < nw; ++w) later += wsum[w];
+            S0 = incl + later;
+            S1 = S0 - v0;
+        }
         if (d.cutoff > 0.0) {
-            const double lim = d.cutoff * total;
-            const double kkc = tr_block_sum((double)((j0 < n && S0 > lim) + (j1 < n && S1 > lim)), red);
-            k = max(1, min(k, (int)kkc));
+            bool c0 = false, c1 = false;
+            if (warp < nw) {
+                const double lim = d.cutoff * total;
+                c0 = j0 < n && above(S0, lim);
+                c1 = j1 < n && above(S1, lim);
+            }
+            int kc = __syncthreads_count(c0);
+            kc += __syncthreads_count(c1);
+            k = max(1, min(k, kc));
         }
-        __syncthreads();
         // discarded and kept weights: S_k and total - S_k
-        if (j0 == k && k < n) s_scale = S0;
-        if (j1 == k && k < n) s_scale = S1;
-        if (tid == 0 && k >= n) s_scale = 0.0;
-        __syncthreads();
-        const double disc = s_scale, kept = total - disc;
-        eps = disc / total;
-        if (d.renorm && kept > 0.0) scale = sqrt(total / kept);
-        __syncthreads();
+        if (j0 == k && k < n) s_disc = S0;
+        if (j1 == k && k < n) s_disc = S1;
+        if (tid == 0 && k >= n) s_disc = 0.0;
     }
-    if (tid == 0) {
-        s_k = k;
+    __syncthreads();
+    if (tid == TR_THREADS - 32) {
+        double eps = 0.0, scale = 1.0;
+        if (some) {
+            const double disc = s_disc, kept = total - disc;
+            eps = disc / total;
+            if (d.renorm && kept > 0.0) scale = sqrt(total / kept);
+        }
         s_scale = scale;
         out->k = k;
         out->eps = eps;
@@ -204,13 +228,22 @@ __global__ void __launch_bounds__(TR_THREADS) k_truncate(const GateDesc* __restr
         atomicAdd(&d.stats[7], (u64)k * (u64)m * (u64)n);
         if (qr_active(d, m, n)) atomicAdd(&d.stats[8], (u64)2 * (u64)n * (u64)n * (u64)n / 3);
     }
+    double root[TR_MAXN / TR_THREADS];
+#pragma unroll
+    for (int t = 0; t < TR_MAXN / TR_THREADS; ++t) {
+        const int j = tid + t * TR_THREADS;
+        root[t] = 0.0;
+        if (j < n) {
+            d.s2[j] = key[j];
+            d.perm[j] = idx[j];
+            if (j < k) root[t] = sqrt(key[j]);
+        }
+    }
     __syncthreads();
-    k = s_k;
-    scale = s_scale;
-    for (int j = tid; j < n; j += TR_THREADS) {
-        d.s2[j] = key[j];
-        d.perm[j] = idx[j];
-        if (j < k) d.spectrum[j] = sqrt(key[j]) * scale;
+#pragma unroll
+    for (int t = 0; t < TR_MAXN / TR_THREADS; ++t) {
+        const int j = tid + t * TR_THREADS;
+        if (j < k && j < n) d.spectrum[j] = root[t] * s_scale;
     }
 }
 
