@@ -312,6 +312,24 @@ cudaError_t launch_left(const GateDesc* d, int n_gates, int m_max, int k_max, cu
 }
 
 // ---------------------------------------------------------------------------
+// grid (x, sites): one transfer and this launch for up to 128 sites instead of a
+// synchronous copy each (100 product-state sites: 740 -> 59 us)
+__global__ void __launch_bounds__(128) k_unpack_sites(const __grid_constant__ SiteCopies c) {
+    const auto& t = c.site[blockIdx.y];
+    const uint4* src = (const uint4*)c.src + t.at;
+    uint4* dst = (uint4*)t.dst;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < t.units; i += gridDim.x * blockDim.x) dst[i] = src[i];
+}
+
+cudaError_t launch_unpack_sites(const SiteCopies& c, cudaStream_t s) {
+    if (c.count <= 0) return cudaSuccess;
+    unsigned most = 1;
+    for (int i = 0; i < c.count; ++i) most = c.site[i].units > most ? c.site[i].units : most;
+    const unsigned bx = (most + 1023) / 1024;
+    k_unpack_sites<<<dim3(bx > 64 ? 64 : bx, c.count), 128, 0, s>>>(c);
+    return cudaGetLastError();
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_site1q(const Site1Desc* __restrict__ sd) {
     using C = typename CT<T>::type;

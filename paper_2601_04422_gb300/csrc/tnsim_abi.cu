@@ -103,6 +103,8 @@ struct tnsim_mps {
     CUtensorMap* d_maps = nullptr; // two tensor maps (A boxes, B boxes)
     int tc_rows = 0, tc_k = 0;
     GateOut* h_out = nullptr;      // pinned readback
+    double* h_spec = nullptr;      // pinned readback of one bond's spectrum and its count, under spec_mu
+    std::mutex spec_mu;
     int* h_chi = nullptr;          // pinned readback
     Staging ring[kRing];
     int ring_pos = 0;
@@ -198,7 +200,7 @@ void free_all(tnsim_mps* m) {
     cudaFree(m->d_pre);
     cudaFree(m->d_planes);
     cudaFree(m->d_maps);
-    cudaFreeHost(m->h_out); cudaFreeHost(m->h_chi);
+    cudaFreeHost(m->h_out); cudaFreeHost(m->h_chi); cudaFreeHost(m->h_spec);
     for (auto& r : m->ring) {
         cudaFreeHost(r.desc); cudaFreeHost(r.s1); cudaFreeHost(r.gates);
         if (r.done) cudaEventDestroy(r.done);
@@ -635,6 +637,7 @@ tnsim_status tnsim_mps_create(int32_t n_qubits, tnsim_dtype dt, const tnsim_para
     ALLOC(m->d_ctl, 2 * sizeof(JacobiCtl));
     HALLOC(m->h_out, nG * sizeof(GateOut));
     HALLOC(m->h_chi, sizeof(int) * (n_qubits + 1));
+    HALLOC(m->h_spec, sizeof(double) * ((size_t)prm.chi_max + 1));
     for (auto& r : m->ring) {
         HALLOC(r.desc, nG * sizeof(GateDesc));
         HALLOC(r.s1, (size_t)n_qubits * sizeof(Site1Desc));
@@ -1173,12 +1176,17 @@ tnsim_status tnsim_bond_spectrum(tnsim_mps* m, int32_t bond, double* s_out, int3
     if (!m || !s_out || !k_out) return fail(TNSIM_EINVAL, "NULL argument");
     if (bond < 0 || bond > m->n) return fail(TNSIM_EINVAL, "bond out of range");
     DevGuard g(m->device);
+    // both copies in flight, one wait (two synchronous copies after a wait: 24 us a bond)
+    const size_t chi = (size_t)m->p.chi_max;
+    std::lock_guard<std::mutex> lock(m->spec_mu);
+    CUDA_TRY(cudaMemcpyAsync(m->h_spec, m->d_spec + (size_t)bond * chi, sizeof(double) * chi, cudaMemcpyDeviceToHost,
+                             m->stream));
+    CUDA_TRY(cudaMemcpyAsync(m->h_spec + chi, m->d_spec_k + bond, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
     CUDA_TRY(cudaStreamSynchronize(m->stream));
     int k = 0;
-    CUDA_TRY(cudaMemcpy(&k, m->d_spec_k + bond, sizeof(int), cudaMemcpyDeviceToHost));
+    std::memcpy(&k, m->h_spec + chi, sizeof(int));
     *k_out = k;
-    if (k > 0) CUDA_TRY(cudaMemcpy(s_out, m->d_spec + (size_t)bond * m->p.chi_max, sizeof(double) * k,
-                                   cudaMemcpyDeviceToHost));
+    if (k > 0) std::memcpy(s_out, m->h_spec, sizeof(double) * k);
     return TNSIM_OK;
 }
 
@@ -1216,20 +1224,54 @@ tnsim_status tnsim_import_sites(tnsim_mps* m, const int32_t* dims, const double*
     if (dims[0] != 1 || dims[m->n] != 1) return fail(TNSIM_EINVAL, "terminal bonds must be 1");
     for (int b = 1; b < m->n; ++b)
         if (dims[b] < 1 || dims[b] > m->cap[b]) return fail(TNSIM_EINVAL, "bond dimension exceeds capacity");
+    size_t total = 0;
+    for (int q = 0; q < m->n; ++q) {
+        const size_t cnt = (size_t)dims[q] * 2 * dims[q + 1];
+        if (!finite_all(data + 2 * total, 2 * cnt)) return fail(TNSIM_EINVAL, "non-finite site entry");
+        total += cnt;
+    }
+    auto convert = [&](char* dst, const double* src, size_t cnt) {
+        if (m->dt == TNSIM_C64) {
+            float* f = (float*)dst;
+            for (size_t i = 0; i < 2 * cnt; ++i) f[i] = (float)src[i];
+        } else {
+            std::memcpy(dst, src, cnt * 16);
+        }
+    };
     DevGuard g(m->device);
-    CUDA_TRY(cudaStreamSynchronize(m->stream));
     std::vector<char> buf;
+    const size_t ws_bytes = (size_t)m->G * 2 * m->ws_elems * m->esz;
+    if (total * m->esz <= std::min<size_t>(ws_bytes, 16 << 20)) {
+        // small states: one transfer into the gates' workspace (free between layers), and a
+        // kernel that puts the sites into their slots
+        buf.resize(total * m->esz);
+        convert(buf.data(), data, total);
+        CUDA_TRY(cudaMemcpyAsync(m->d_ws, buf.data(), buf.size(), cudaMemcpyHostToDevice, m->stream));
+        SiteCopies c;
+        c.src = m->d_ws;
+        c.count = 0;
+        size_t at = 0;
+        for (int q = 0; q < m->n; ++q) {
+            const size_t bytes = (size_t)dims[q] * 2 * dims[q + 1] * m->esz;
+            c.site[c.count++] = {site_ptr(m, q), (unsigned)(at / 16), (unsigned)(bytes / 16)};
+            at += bytes;
+            if (c.count == SiteCopies::kMax || q == m->n - 1) {
+                CUDA_TRY(launch_unpack_sites(c, m->stream));
+                c.count = 0;
+            }
+        }
+        CUDA_TRY(cudaMemcpyAsync(m->d_chi, dims, sizeof(int) * (m->n + 1), cudaMemcpyHostToDevice, m->stream));
+        CUDA_TRY(cudaMemsetAsync(m->d_spec_k, 0, sizeof(int) * (m->n + 1), m->stream));
+        CUDA_TRY(cudaStreamSynchronize(m->stream));   // buf and dims have been read
+        for (int b = 0; b <= m->n; ++b) m->ub[b] = dims[b];
+        return TNSIM_OK;
+    }
+    CUDA_TRY(cudaStreamSynchronize(m->stream));
     int64_t pos = 0;
     for (int q = 0; q < m->n; ++q) {
         const size_t cnt = (size_t)dims[q] * 2 * dims[q + 1];
-        if (!finite_all(data + pos, 2 * cnt)) return fail(TNSIM_EINVAL, "non-finite site entry");
         buf.resize(cnt * m->esz);
-        if (m->dt == TNSIM_C64) {
-            float* f = (float*)buf.data();
-            for (size_t i = 0; i < 2 * cnt; ++i) f[i] = (float)data[pos + i];
-        } else {
-            std::memcpy(buf.data(), data + pos, cnt * 16);
-        }
+        convert(buf.data(), data + pos, cnt);
         CUDA_TRY(cudaMemcpy(site_ptr(m, q), buf.data(), cnt * m->esz, cudaMemcpyHostToDevice));
         pos += (int64_t)cnt * 2;
     }

@@ -206,6 +206,14 @@ cudaError_t launch_sites_pre(const GateDesc* d, int n_gates, int m_max, int k_ma
 cudaError_t launch_left_pre_tc(const GateDesc* d, int n_gates, int m_max, int k_max, cudaStream_t s);
 template <typename T>
 cudaError_t launch_site1q(const Site1Desc* d, int n_sites, int cap_lr, cudaStream_t s);
+// Sites packed one after another, to their slots (sizes and places in 16-byte units).
+struct SiteCopies {
+    static constexpr int kMax = 128;
+    const void* src;
+    int count;
+    struct { void* dst; unsigned at, units; } site[kMax];
+};
+cudaError_t launch_unpack_sites(const SiteCopies& c, cudaStream_t s);
 
 // read-out
 template <typename T>
