@@ -1225,11 +1225,7 @@ tnsim_status tnsim_import_sites(tnsim_mps* m, const int32_t* dims, const double*
     for (int b = 1; b < m->n; ++b)
         if (dims[b] < 1 || dims[b] > m->cap[b]) return fail(TNSIM_EINVAL, "bond dimension exceeds capacity");
     size_t total = 0;
-    for (int q = 0; q < m->n; ++q) {
-        const size_t cnt = (size_t)dims[q] * 2 * dims[q + 1];
-        if (!finite_all(data + 2 * total, 2 * cnt)) return fail(TNSIM_EINVAL, "non-finite site entry");
-        total += cnt;
-    }
+    for (int q = 0; q < m->n; ++q) total += (size_t)dims[q] * 2 * dims[q + 1];
     auto convert = [&](char* dst, const double* src, size_t cnt) {
         if (m->dt == TNSIM_C64) {
             float* f = (float*)dst;
@@ -1244,6 +1240,7 @@ tnsim_status tnsim_import_sites(tnsim_mps* m, const int32_t* dims, const double*
     if (total * m->esz <= std::min<size_t>(ws_bytes, 16 << 20)) {
         // small states: one transfer into the gates' workspace (free between layers), and a
         // kernel that puts the sites into their slots
+        if (!finite_all(data, 2 * total)) return fail(TNSIM_EINVAL, "non-finite site entry");
         buf.resize(total * m->esz);
         convert(buf.data(), data, total);
         CUDA_TRY(cudaMemcpyAsync(m->d_ws, buf.data(), buf.size(), cudaMemcpyHostToDevice, m->stream));
@@ -1270,6 +1267,7 @@ tnsim_status tnsim_import_sites(tnsim_mps* m, const int32_t* dims, const double*
     int64_t pos = 0;
     for (int q = 0; q < m->n; ++q) {
         const size_t cnt = (size_t)dims[q] * 2 * dims[q + 1];
+        if (!finite_all(data + pos, 2 * cnt)) return fail(TNSIM_EINVAL, "non-finite site entry");
         buf.resize(cnt * m->esz);
         convert(buf.data(), data + pos, cnt);
         CUDA_TRY(cudaMemcpy(site_ptr(m, q), buf.data(), cnt * m->esz, cudaMemcpyHostToDevice));
