@@ -29,7 +29,7 @@
 // preconditioner that did not converge only costs sweeps.
 // FP64 enters where rounding would reach the result: in X, E and the second K.  The other
 // products are sums of FP32 pairs (48 bits) at a fifth of FP64's time: of small corrections
-// (K, F < 2^-9 of X), or where a few digits do.
+// (K, F < 2^-10 of X), or where a few digits do.
 // Measured: the SVD of 20 gates at m = n = 180, 139 ms without it, 29 without refinement
 // (12.2 and 4.7 FP64 sweeps per gate), 9.2 with the products in FP64, 6.2 so (1.5 sweeps,
 // 0.1 % of their pairs rotated; FP32 rotations 2.9, products 2.0, FP64 sweeps 1.1); 4 gates
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_sq(const GateDesc* __restr
 }
 
 // Step 0: I + F = (I + E/2 + 3/8 E^2) (I + K + K^2/2 - K^4/8), the second-order products in
-// FP32 (E ~ 1e-6, K < 2^-9); without K where K^2 is too large for K^6 to vanish.
+// FP32 (E ~ 1e-6, K < 2^-10); without K where K^2 is too large for K^6 to vanish.
 __global__ void __launch_bounds__(TILE_THREADS) k_mix_corr(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.z];
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];

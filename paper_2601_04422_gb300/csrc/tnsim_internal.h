@@ -131,10 +131,11 @@ __device__ __forceinline__ bool qr_active(const GateDesc& d, int m, int n) {
 constexpr int kMixMinCols = 10;
 constexpr int kMixMaxRows = 1024;
 constexpr double kMixTol = 2e-6;
-// Refinement steps (k_fp64.cu): the largest angle of a pair (the second step's, and its
-// fallback), and the largest row sums of |K^2| (first step) and of |K| (second) at which
+// Refinement steps (k_fp64.cu): the largest angle of a pair (a first step of up to 2^-9 was
+// given up by one gate of 180 columns in ~500 for its row sums, and one such gate took 20 ms
+// of FP64 sweeps; 30 layers of 2^-10: none), the second step's and its fallback, and the largest row sums of |K^2| (first step) and of |K| (second) at which
 // the neglected terms, K^6 / 16 and K^4 / 8, stay below 3e-17.
-constexpr float kRefCap0 = 0x1p-9f, kRefCap1 = 0x1p-14f, kRefCap2 = 0x1p-18f, kRefRow0 = 0x1p-17f, kRefRow1 = 0x1p-13f;
+constexpr float kRefCap0 = 0x1p-10f, kRefCap1 = 0x1p-14f, kRefCap2 = 0x1p-18f, kRefRow0 = 0x1p-17f, kRefRow1 = 0x1p-13f;
 #ifdef __CUDACC__
 // power of two that brings |theta|_F into [1, 2) in the FP32 copy of theta
 __device__ __forceinline__ double mix_scale(double frob2) {
