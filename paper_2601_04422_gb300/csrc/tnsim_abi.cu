@@ -1237,9 +1237,10 @@ tnsim_status tnsim_import_sites(tnsim_mps* m, const int32_t* dims, const double*
     DevGuard g(m->device);
     std::vector<char> buf;
     const size_t ws_bytes = (size_t)m->G * 2 * m->ws_elems * m->esz;
-    if (total * m->esz <= std::min<size_t>(ws_bytes, 16 << 20)) {
+    if (total * m->esz <= std::min<size_t>(ws_bytes, 1 << 20)) {
         // small states: one transfer into the gates' workspace (free between layers), and a
-        // kernel that puts the sites into their slots
+        // kernel that puts the sites into their slots (100 product-state sites: 743 -> 59 us;
+        // 13 MB of sites take 4 ms longer so, through a host buffer that no cache holds)
         if (!finite_all(data, 2 * total)) return fail(TNSIM_EINVAL, "non-finite site entry");
         buf.resize(total * m->esz);
         convert(buf.data(), data, total);
