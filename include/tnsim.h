@@ -262,9 +262,9 @@ tnsim_status tnsim_sample(tnsim_mps* m, int64_t n_shots, const double* uniforms,
                           int64_t* n_nodes_out);
 
 /* Launch configurations of the Jacobi SVD.  Bit 0: 0 -- 16-column blocks (8 for
- * complex128 at chi > 128), one persistent CTA per SM; 1 -- half-width blocks, two
- * CTAs per SM (barriers of the two CTAs are independent; a sweep has twice the
- * rounds).  Bit 1: QR preconditioning (Drmac and Veselic 2008) of every gate whose
+ * complex128), a cluster of CTAs per gate where all gates of the launch fit on the
+ * device, persistent CTAs otherwise; 1 -- half-width blocks on persistent CTAs (a sweep
+ * has twice the rounds).  Bit 1: QR preconditioning (Drmac and Veselic 2008) of every gate whose
  * gated block is square (2 chi_L == 2 chi_R <= 1536) in the paper's form: theta = Q R
  * by blocked Householder reflections, the Jacobi iteration runs on the columns of
  * R^H (fewer sweeps), the left site is theta V S^-1 and the right site S V^H is read

@@ -22,8 +22,9 @@
 // blocks back.  Each sweep therefore rotates every column pair exactly once.  A sweep
 // that rotates nothing ends the gate's iteration; reaching max_sweeps sets ENOCONV.
 //
-// Two kernels run this schedule with the same arithmetic: k_jacobi_cl, one cluster per gate,
-// where all gates are resident at once; else k_jacobi, a queue.
+// Three kernels run this schedule with the same arithmetic: k_jacobi_cl, one cluster per gate,
+// where all gates are resident at once; else k_jacobi, a queue, and beyond 256 rows in FP32
+// k_jacobi_pf, the queue with a prefetching warp.
 //
 // k_jacobi is persistent: as many CTAs as the SMs hold claim visits of
 // any gate from a device-side queue, so gates of different sizes and all rounds of
@@ -32,8 +33,9 @@
 // idle CTA polls with a sleep; if nothing progresses for spin_limit polls (default
 // 2^22, settable per state) it sets an error flag and leaves; every other CTA leaves
 // at its next claim, abandoning the claim, and the unfinished gates report status 5
-// (the host reports ETIMEOUT).  No other wait exists, and no CTA leaves with a copy
-// in flight.
+// (the host reports ETIMEOUT).  k_jacobi_pf also polls for its own copies and threads, with
+// a fixed limit and the same flag.  No other wait exists, and no CTA leaves with a copy in
+// flight.
 #include <float.h>
 
 #include <algorithm>
