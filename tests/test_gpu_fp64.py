@@ -1,7 +1,7 @@
-"""complex128 updates through the FP32-preconditioned SVD and the 16 x 16-tiled FP64 products.
+"""complex128 updates through the FP32-preconditioned, refined SVD and the 8 x 8-tiled FP64 products.
 
-Sizes around the edges of the tiles (16), of the column blocks (8, 4), of the smallest
-preconditioned block (16 columns) and of the largest (m + n = 1024 rows), rectangular
+Sizes around the edges of the tiles (8, 16), of the column blocks (8, 4), of the smallest
+preconditioned block (10 columns) and of the largest (m + n = 1024 rows), rectangular
 blocks, every contraction form, and spectra that FP32 cannot resolve.  The kept singular
 values must agree with LAPACK's within 64 eps s_max sqrt(rank) (both are backward stable:
 a few eps |theta|_2 each, and |theta|_F <= sqrt(rank) s_max), the new block with the best
@@ -64,7 +64,7 @@ def _update(T, cl, cm, cr, chi, cfg, decay=0.0, seed=1, dtype=None):
 
 
 @pytest.mark.parametrize("cfg", [0, 1, 2])
-@pytest.mark.parametrize("c", [(3, 4, 4), (7, 8, 7), (8, 8, 8), (8, 9, 9), (9, 16, 12), (16, 17, 17), (33, 33, 20),
+@pytest.mark.parametrize("c", [(3, 4, 4), (4, 5, 5), (7, 8, 7), (8, 8, 8), (8, 9, 9), (9, 16, 12), (16, 17, 17), (33, 33, 20),
                                (20, 33, 33), (64, 64, 65), (100, 60, 90)])
 def test_block_sizes(T, c, cfg):
     s, r, blk, blk_o, u = _update(T, *c, chi=1, cfg=cfg)
