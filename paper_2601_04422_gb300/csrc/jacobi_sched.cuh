@@ -115,12 +115,13 @@ __device__ __forceinline__ bool rot_params64(double a, double b, double gr, doub
 struct Tour {
     int m, n, nb, P, R, V;
 };
-template <int BC>
+// F64: a plain gate is one visit, whatever BC.
+template <int BC, bool F64 = false>
 __device__ __forceinline__ Tour tour_of(const GateDesc& d) {
     Tour t;
     t.m = 2 * d.chi[d.q];
     t.n = 2 * d.chi[d.q + 2];
-    t.nb = (t.n + BC - 1) / BC;
+    t.nb = F64 && plain64(t.m, t.n) ? 1 : (t.n + BC - 1) / BC;
     t.P = t.nb + (t.nb & 1);
     t.R = (t.nb == 1) ? 1 : t.P - 1;
     t.V = (t.nb == 1) ? 1 : t.P / 2;
@@ -133,7 +134,7 @@ constexpr int kScanTable = 2048;              // gates whose visit count is cach
 // Warp-parallel claim of one visit (warp 0): each lane checks one gate per pass (one
 // L2 round trip), the first claimable gate in descriptor order from gate scan0 on
 // (wrapping around) is tried with an atomic.  found = 0 when nothing is claimable now.
-template <int BC>
+template <int BC, bool F64 = false>
 __device__ __forceinline__ void claim_scan(const GateDesc* __restrict__ gd, int n_gates, const short* s_V, int scan0,
                                            int lane, int& found, int& fg, int& frnd, int& fv) {
     found = 0;
@@ -149,7 +150,7 @@ __device__ __forceinline__ void claim_scan(const GateDesc* __restrict__ gd, int 
         GateOut* o = nullptr;
         if (g < n_gates) {
             o = gd[g].out;
-            V = g < kScanTable ? (int)s_V[g] : tour_of<BC>(gd[g]).V;
+            V = g < kScanTable ? (int)s_V[g] : tour_of<BC, F64>(gd[g]).V;
             const int fin = *((volatile int*)&o->finished);
             const unsigned long long cur = *((volatile unsigned long long*)&o->claim);
             ok = !fin && (unsigned)(cur & 0xffffffffull) < (unsigned)V;

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_right64(const GateDesc* __rest
     const int lk = d.canon ? *d.lam_k : 0;
     double2 acc[1][1] = {};
     // tile rows: columns of R (they run along its rows in memory); tile columns: rows j
-    tile_product<double2, true, true, false, true, MulAdd>(
+    tile_product<double2, true, true, false, true, MulAddConj>(
         m,
         [&](int i, int row) {
             if (c0 + i >= n) return make_double2(0.0, 0.0);
@@ -148,12 +148,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_right64(const GateDesc* __rest
             }
             return w;
         },
-        [&](int row, int j) {
-            if (pj[j] < 0) return make_double2(0.0, 0.0);
-            const double2 v = Wm[(size_t)pj[j] * m + row];
-            return make_double2(v.x, -v.y);
-        },
-        acc);
+        [&](int row, int j) { return pj[j] < 0 ? make_double2(0.0, 0.0) : Wm[(size_t)pj[j] * m + row]; }, acc);
     double2* R = (double2*)d.siteB;
     const int jj = tid >> 3, col = c0 + (tid & 7);
     if (j0 + jj < k && col < n) R[(size_t)(j0 + jj) * n + col] = make_double2(acc[0][0].x * fj[jj], acc[0][0].y * fj[jj]);
@@ -163,7 +158,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_right64(const GateDesc* __rest
 // the preconditioner
 
 __device__ __forceinline__ bool mix_active(const GateDesc& d, int m, int n) {
-    return d.pre && n >= kMixMinCols && m + n <= kMixMaxRows;
+    return d.pre && n >= kMixMinCols && m + n <= kMixMaxRows && !plain64(m, n);
 }
 
 // FP32 pairs: h + l with |l| <= ulp(h), 48 bits; a complex number of two of them.
@@ -583,7 +578,7 @@ cudaError_t launch_right64(const GateDesc* d, int n_gates, int k_max, int n_max,
 
 cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, JacobiCtl* ctl, cudaStream_t s,
                        int n_lead, unsigned spin_limit) {
-    if (n_gates <= 0 || n_max < kMixMinCols) return cudaSuccess;
+    if (n_gates <= 0 || n_max < kMixMinCols || plain64(m_max, n_max)) return cudaSuccess;
     const int mt = m_max + n_max < kMixMaxRows ? m_max + n_max : kMixMaxRows;   // of an active gate
     const int mm = m_max < kMixMaxRows ? m_max : kMixMaxRows, nm = n_max < kMixMaxRows ? n_max : kMixMaxRows;
     int bx = (int)(((long long)mt * nm + 1023) / 1024);

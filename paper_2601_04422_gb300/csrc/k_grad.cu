@@ -193,6 +193,17 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
             k2 += __shfl_xor_sync(0xffffffffu, k2, o);
             nz = max(nz, __shfl_xor_sync(0xffffffffu, nz, o));
         }
+        if (sizeof(T) == 8 && plain64(m, n)) {
+            // in their order (see kPlain64): lane 0 all, lane 1 the kept ones
+            double t = 0.0;
+            const int top = tid == 0 ? n : tid == 1 ? k : 0;
+            for (int j = 0; j < n; ++j) {
+                const double v = d.s2[j];
+                if (j < top) t += v;
+            }
+            f2 = __shfl_sync(0xffffffffu, t, 0);
+            k2 = __shfl_sync(0xffffffffu, t, 1);
+        }
         if (tid == 0) {
             s_sc[0] = f2;
             s_sc[1] = k2;

@@ -39,7 +39,7 @@
 #include <float.h>
 
 #include <algorithm>
-#include <atomic>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -420,6 +420,196 @@ __device__ __forceinline__ void visit64(double2* __restrict__ XI, double2* __res
     }
 }
 
+// A plain gate (plain64: at most 30 rows and columns): all its sweeps in one visit, the
+// columns X (n x m) in shared memory.  Column blocks of 16 whatever the launch's: 15 steps
+// of the pairs inside the one or two blocks, whose norms are summed again for every pair,
+// then 16 of the cross pairs with tracked norms.  Every sum is the lanes' terms by halving
+// distances (a lane has row r, in the cross pairs 2 r and 2 r + 1), the parameters are IEEE
+// operations: see kPlain64.  A pair's sums are its warp's, four of them in six instead of
+// twenty additions.  The parameters of all 16 pairs are one warp's, two lanes each: of seven
+// divisions two of a pair share an issue slot three times, and the seventh, in the test, is
+// only made within rounding of the limit.
+// sw: the sweeps done; returns whether the last one still rotated.
+struct Plain64 {
+    double val[16][4];   // a, b, gr, gi of the step's pairs (cross pairs: gr, gi)
+    double nrm[32];      // cross pairs: tracked norms
+    Par64 par[16];
+};
+__device__ __forceinline__ void plain_pair(int s, int p, int n, int& ca, int& cb, bool& act) {
+    const int nI = min(16, n), nJ = n - nI;
+    if (s < 15) {
+        const int base = p < 8 ? 0 : 16, nblk = p < 8 ? nI : nJ;
+        int a, b;
+        rr_pair(16, s, p & 7, a, b);
+        act = a < nblk && b < nblk;
+        ca = base + a;
+        cb = base + b;
+    } else {
+        const int b = (p + s - 15) & 15;
+        act = p < nI && b < nJ;
+        ca = p;
+        cb = 16 + b;
+    }
+}
+// v[0..NV-1] summed over the warp's lanes: the sum of v[2 (lane >> 4 & 1) + (lane >> 3 & 1)]
+// (NV = 4) or v[lane >> 4 & 1] (NV = 2)
+template <int NV>
+__device__ __forceinline__ double plain_sums(const double (&v)[NV], int lane) {
+    const bool u4 = lane & 16, u3 = lane & 8;
+    double k;
+    if constexpr (NV == 4) {
+        double k0 = u4 ? v[2] : v[0], k1 = u4 ? v[3] : v[1];
+        k0 += __shfl_xor_sync(0xffffffffu, u4 ? v[0] : v[2], 16);
+        k1 += __shfl_xor_sync(0xffffffffu, u4 ? v[1] : v[3], 16);
+        k = u3 ? k1 : k0;
+        k += __shfl_xor_sync(0xffffffffu, u3 ? k0 : k1, 8);
+    } else {
+        k = u4 ? v[1] : v[0];
+        k += __shfl_xor_sync(0xffffffffu, u4 ? v[0] : v[1], 16);
+        k += __shfl_xor_sync(0xffffffffu, k, 8);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+    return k;
+}
+// g2 / b > lim a without the division unless the product is within rounding of g2
+__device__ __forceinline__ bool plain_above(double g2, double b, double la) {
+    const double p = la * b;
+    const long long ig = __double_as_longlong(g2), ip = __double_as_longlong(p);
+    constexpr long long lo = 0x0080000000000000ll, hi = 0x7f00000000000000ll;
+    if (ig > lo && ig < hi && ip > lo && ip < hi && (ig > ip + 64 || ig < ip - 64)) return ig > ip;
+    return g2 / b > la;
+}
+__device__ __noinline__ int plain64_sweeps(double2* X, int m, int n, int max_sweeps, double tol2, double zthr, Plain64& S,
+                                           int& sw, int& my_rot, int& my_vis) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int steps = n > 16 ? 31 : 15;
+    int rot_any = 0;
+    for (sw = 0; sw < max_sweeps;) {
+        int rots = 0;
+        for (int s = 0; s < steps; ++s) {
+            if (s == 15) {
+                // norms at the start of the cross pairs
+                for (int c = warp; c < n; c += nw) {
+                    const double2* x = X + (size_t)c * m;
+                    double a = 0.0;
+                    if (c < 16) {
+                        for (int k = 0; k < 2; ++k)
+                            if (2 * lane + k < m) {
+                                const double2 u = x[2 * lane + k];
+                                a = fma(u.x, u.x, fma(u.y, u.y, a));
+                            }
+                    } else if (lane < m) {
+                        const double2 u = x[lane];
+                        a = fma(u.x, u.x, fma(u.y, u.y, a));
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                    if (lane == 0) S.nrm[c] = a;
+                }
+            }
+            for (int p = warp; p < 16; p += nw) {
+                int ca, cb;
+                bool act;
+                plain_pair(s, p, n, ca, cb, act);
+                if (!act) continue;
+                const double2 *xa = X + (size_t)ca * m, *xb = X + (size_t)cb * m;
+                if (s < 15) {
+                    double v[4] = {0.0, 0.0, 0.0, 0.0};
+                    if (lane < m) {
+                        const double2 x = xa[lane], y = xb[lane];
+                        v[0] = fma(x.x, x.x, x.y * x.y);
+                        v[1] = fma(y.x, y.x, y.y * y.y);
+                        v[2] = fma(x.x, y.x, x.y * y.y);
+                        v[3] = fma(x.x, y.y, -x.y * y.x);
+                    }
+                    const double k = plain_sums<4>(v, lane);
+                    if ((lane & 7) == 0) S.val[p][lane >> 3] = k;
+                } else {
+                    double v[2] = {0.0, 0.0};
+#pragma unroll
+                    for (int k = 0; k < 2; ++k)
+                        if (2 * lane + k < m) {
+                            const double2 x = xa[2 * lane + k], y = xb[2 * lane + k];
+                            v[0] = fma(x.x, y.x, fma(x.y, y.y, v[0]));
+                            v[1] = fma(x.x, y.y, fma(-x.y, y.x, v[1]));
+                        }
+                    const double k = plain_sums<2>(v, lane);
+                    if ((lane & 15) == 0) S.val[p][2 + (lane >> 4)] = k;
+                }
+            }
+            __syncthreads();
+            if (warp == 0) {
+                const int p = lane >> 1;
+                const bool h = lane & 1;
+                int ca, cb;
+                bool act;
+                plain_pair(s, p, n, ca, cb, act);
+                const double gr = S.val[p][2], gi = S.val[p][3];
+                const double a = s < 15 ? S.val[p][0] : act ? S.nrm[ca] : 0.0;
+                const double b = s < 15 ? S.val[p][1] : act ? S.nrm[cb] : 0.0;
+                double g2 = 0.0;
+                bool rot = false;
+                if (act) {
+                    g2 = gr * gr + gi * gi;
+                    rot = a > zthr && b > zthr && plain_above(g2, b, tol2 * a);
+                }
+                const unsigned on = __ballot_sync(0xffffffffu, rot);
+                __syncwarp();
+                if (rot) {
+                    const double gabs = sqrt(g2);
+                    const double q1 = (h ? gr : b - a) / (h ? gabs : 2 * gabs);            // zeta; gr / |g|
+                    const double q2 = (h ? gi : copysign(1.0, q1)) /
+                                      (h ? gabs : fabs(q1) + sqrt(1.0 + q1 * q1));         // t; gi / |g|
+                    const double t = __shfl_sync(on, q2, lane & ~1);
+                    const double rr = sqrt(1.0 + t * t);
+                    const double q3 = (h ? t : -(t * t)) / (h ? rr : rr * (1.0 + rr));     // c - 1; s
+                    if (h) {
+                        S.par[p].sr = q3 * q1;
+                        S.par[p].si = q3 * q2;
+                    } else {
+                        S.par[p].cm1 = q3;
+                        if (s >= 15) {
+                            const double tg = __dmul_rn(t, gabs);   // rounded by itself
+                            S.nrm[ca] = __dsub_rn(a, tg);
+                            S.nrm[cb] = __dadd_rn(b, tg);
+                        }
+                    }
+                }
+                if (!h) S.par[p].rot = rot;
+                const int r = __popc(on) / 2, v = __popc(__ballot_sync(0xffffffffu, act && !h));
+                rots += r;
+                if (lane == 0) {
+                    my_rot += r;
+                    my_vis += v;
+                }
+            }
+            __syncthreads();
+            for (int p = warp; p < 16; p += nw) {
+                int ca, cb;
+                bool act;
+                plain_pair(s, p, n, ca, cb, act);
+                if (!act || !S.par[p].rot || lane >= m) continue;
+                const double cm1 = S.par[p].cm1, sr = S.par[p].sr, si = S.par[p].si;
+                double2 *xa = X + (size_t)ca * m + lane, *xb = X + (size_t)cb * m + lane;
+                const double2 u = *xa, v = *xb;
+                double2 nu, nv;
+                nu.x = u.x + fma(-si, v.y, fma(-sr, v.x, cm1 * u.x));
+                nu.y = u.y + fma(si, v.x, fma(-sr, v.y, cm1 * u.y));
+                nv.x = v.x + fma(-si, u.y, fma(sr, u.x, cm1 * v.x));
+                nv.y = v.y + fma(si, u.x, fma(sr, u.y, cm1 * v.y));
+                *xa = nu;
+                *xb = nv;
+            }
+            __syncthreads();
+        }
+        rot_any = __syncthreads_or(rots);
+        ++sw;
+        if (!rot_any) break;
+    }
+    return rot_any;
+}
+
 // Persistent kernel: every CTA repeatedly claims one visit (gate g, global round
 // number, block pair v) from the gates' claim words, processes it, and reports it.
 // The last visit of a round advances that gate to its next round (and, at the end
@@ -434,6 +624,7 @@ __global__ void __launch_bounds__(BC * LP, MINB)
 k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in, int max_sweeps,
          JacobiCtl* __restrict__ ctl, unsigned spin_limit) {
     using C = typename CT<T>::type;
+    constexpr bool F64 = sizeof(T) == 8;
     static_assert(BC * LP >= 64, "warp 0 claims while the others write back");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* X = reinterpret_cast<C*>(smem_raw);       // FP64: [2*BC][m], column-major
@@ -441,6 +632,7 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
     __shared__ T s_bn[2 * BC];                   // tracked squared norms (FP32: of block J's columns; FP64: of both)
     __shared__ double2 s_red[sizeof(T) == 8 ? BC * kRed64 : 1];
     __shared__ Par64 s_par[sizeof(T) == 8 ? BC : 1];
+    __shared__ typename std::conditional<F64, Plain64, int>::type s_plain;
     __shared__ short s_V[kScanTable];            // visits per round of each gate
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -451,7 +643,7 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
     // claimed, and from there on in descriptor order
     int scan0 = (int)(((long long)blockIdx.x * n_lead) / gridDim.x);
     for (int g = threadIdx.x; g < n_gates && g < kScanTable; g += blockDim.x)
-        s_V[g] = (short)tour_of<BC>(gd[g]).V;
+        s_V[g] = (short)tour_of<BC, F64>(gd[g]).V;
     __syncthreads();
 
     int have_next = 0, nxt_g = -1, nxt_rnd = 0, nxt_v = 0;   // warp 0: a claim made during the last visit
@@ -468,7 +660,7 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
                 have_next = 0;
             } else {
                 if (lane == 0) err = *((volatile int*)&ctl->error);
-                claim_scan<BC>(gd, n_gates, s_V, scan0, lane, found, fg, frnd, fv);
+                claim_scan<BC, F64>(gd, n_gates, s_V, scan0, lane, found, fg, frnd, fv);
             }
             if (found) scan0 = fg;
             if (lane == 0) {
@@ -506,7 +698,7 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
         const int g = s_g, rnd = s_rnd, v = s_v;
         const GateDesc& d = gd[g];
         GateOut* out = d.out;
-        const Tour tg = tour_of<BC>(d);
+        const Tour tg = tour_of<BC, F64>(d);
         const int md = tg.m, n = tg.n, nb = tg.nb, P = tg.P, R = tg.R;
         const int m = EXT ? md + n : md;   // rows of a stored column
         int sweep = rnd / R;
@@ -541,7 +733,18 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
         }
         const bool intra = (round == 0);
         int my_rot = 0, my_vis = 0;
-        if (J >= 0 || intra) {
+        bool plain = false;
+        if constexpr (F64) {
+            plain = plain64(md, n);
+            if (plain) {
+                copy_blocks_in(X, Wm, n * m, X, Wm, 0);
+                __syncthreads();
+                last_rot = plain64_sweeps(X, m, n, max_sweeps, tol2, zthr, s_plain, sweep, my_rot, my_vis);
+                --sweep;   // the last one's number
+                if (warp > 0) copy_block_out_from(Wm, X, n * m, 32);
+            }
+        }
+        if (!plain && (J >= 0 || intra)) {
             const int colI = I * BC, nI = min(BC, n - colI);
             const int colJ = J >= 0 ? J * BC : 0, nJ = J >= 0 ? min(BC, n - colJ) : 0;
             using V32 = Visit32<BC, LP, RPL, EXT>;
@@ -587,7 +790,7 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
         if (warp == 0) {
             int found, fg, frnd, fv;
             if (lane == 0) nxt_err = *((volatile int*)&ctl->error);
-            claim_scan<BC>(gd, n_gates, s_V, scan0, lane, found, fg, frnd, fv);
+            claim_scan<BC, F64>(gd, n_gates, s_V, scan0, lane, found, fg, frnd, fv);
             have_next = found;
             nxt_g = fg;
             nxt_rnd = frnd;
@@ -963,6 +1166,26 @@ k_jacobi_cl(const GateDesc* __restrict__ gd, double tol_in, int max_sweeps) {
     const bool seat = v <= last;
     const int tid = threadIdx.x, lane = tid & 31;
     if (tid == 0) s_rot = s_vis = 0;
+    if constexpr (sizeof(T) == 8) {
+        if (plain64(md, n)) {   // one CTA's work
+            if (v > 0) return;
+            __shared__ Plain64 s_plain;
+            C* const X = reinterpret_cast<C*>(smem_raw);
+            int sw, my_rot = 0, my_vis = 0;
+            copy_blocks_in(X, Wm, n * m, X, Wm, 0);
+            __syncthreads();
+            const int rs = plain64_sweeps(X, m, n, max_sweeps, tol2, zthr, s_plain, sw, my_rot, my_vis);
+            copy_block_out_from(Wm, X, n * m, 0);
+            if (tid == 0) {
+                atomicAdd(&out->rotations, (unsigned long long)my_rot);
+                atomicAdd(&out->visits, (unsigned long long)my_vis);
+                out->sweeps = sw;
+                if (rs != 0 && out->status < 4) out->status = 4;
+                out->finished = 1;
+            }
+            return;
+        }
+    }
 
     using V32 = Visit32<BC, LP, sizeof(T) == 4 ? RPL : 2, EXT>;
     // a block slot in 16-byte units (a multiple of two elements: m is even)
@@ -1154,7 +1377,9 @@ static cudaError_t launch_bc(const GateDesc* d, int n_gates, int n_lead, int m_m
                              int max_sweeps, JacobiCtl* ctl, cudaStream_t s, unsigned spin_limit) {
     using C = typename CT<T>::type;
     const auto kernel = k_jacobi<T, BC, LP, RPL, MINB, EXT>;
-    const size_t smem = sizeof(T) == 8 ? (size_t)2 * BC * m_max * sizeof(C) : (size_t)2 * BC * LP * RPL * sizeof(C);
+    // FP64: two blocks, or all columns of a plain gate
+    const size_t smem = sizeof(T) == 8 ? std::max((size_t)2 * BC * m_max, (size_t)std::min(n_max, kPlain64) * std::min(m_max, kPlain64)) * sizeof(C)
+                                       : (size_t)2 * BC * LP * RPL * sizeof(C);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;

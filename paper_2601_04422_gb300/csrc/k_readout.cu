@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_site_adj(const SiteAdjDesc* __
     const C* E = (const C*)d.E;
     const C* w = (const C*)d.w;
     C acc[R][R] = {};
-    tile_product<C, true, false, false, false, MulAdd>(
+    tile_product<C, true, false, false, false, MulAddIm>(
         cl, [&](int i, int k) { return i0 + i < cl ? E[(size_t)(i0 + i) * cl + k] : C{}; },
         [&](int k, int j) { return j0 + j < N ? w[(size_t)k * N + j0 + j] : C{}; }, acc);
     C* out = (C*)d.out;

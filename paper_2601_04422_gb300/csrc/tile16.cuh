@@ -11,6 +11,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "tnsim_internal.h"
+
 namespace tnsim {
 
 constexpr int TILE_THREADS = 64;
@@ -34,6 +36,13 @@ struct ConjMulAdd {
         acc.y = fma(-a.y, b.x, acc.y);
     }
 };
+// acc += a b, the products of the imaginary parts first
+struct MulAddIm {
+    template <typename C> static __device__ __forceinline__ void op(C& acc, const C& a, const C& b) {
+        acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
+        acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
+    }
+};
 struct MulAddConj {
     template <typename C> static __device__ __forceinline__ void op(C& acc, const C& a, const C& b) {
         ConjMulAdd::op(acc, b, a);
@@ -45,13 +54,14 @@ struct MulAddConj {
 // operands' elements for tile row i / tile column j (zero outside them); AK / BK: memory
 // runs along k (consecutive threads then load consecutive k).  k ascends; SPLIT sums every
 // K step by itself first (rounding grows with sqrt(16 + K / 16) instead of sqrt(K), for
-// 3 - 6 % more instructions).
+// 3 - 6 % more instructions); products of up to kPlain64 terms are one run of sums.
 template <typename C, bool AK, bool BK, bool PAIRED, bool SPLIT, typename OP, typename LA, typename LB>
 __device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[TileOf<C>::R][TileOf<C>::R]) {
     constexpr int E = TileOf<C>::E, R = TileOf<C>::R, TILE_K = TileOf<C>::K, PER = E * TILE_K / TILE_THREADS;
     __shared__ C As[TILE_K][E + 1], Bs[TILE_K][E + 1];
     const int tid = threadIdx.x, rx = tid & 7, cy = tid >> 3;
     C na[PER], nb[PER];
+    const bool split = SPLIT && K > kPlain64;
     // element e of a K step: (edge index, k) with k running fastest (KF) or slowest
     auto at = [](int e, bool kf, int& i, int& k) {
         if (kf) { k = e % TILE_K; i = e / TILE_K; }
@@ -82,6 +92,11 @@ __device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[TileO
         __syncthreads();
         if (k0 + TILE_K < K) fetch(k0 + TILE_K);
         C part[R][R] = {};
+        if (!split)
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+#pragma unroll
+                for (int j = 0; j < R; ++j) part[i][j] = acc[i][j];
         const int kn = min(TILE_K, K - k0);
 #pragma unroll 4
         for (int kk = 0; kk < kn; ++kk) {
@@ -94,14 +109,19 @@ __device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[TileO
 #pragma unroll
             for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int j = 0; j < R; ++j) OP::op(SPLIT ? part[i][j] : acc[i][j], a[i], b[j]);
+                for (int j = 0; j < R; ++j) OP::op(part[i][j], a[i], b[j]);
         }
-        if (SPLIT) {
 #pragma unroll
-            for (int i = 0; i < R; ++i)
+        for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int j = 0; j < R; ++j) { acc[i][j].x += part[i][j].x; acc[i][j].y += part[i][j].y; }
-        }
+            for (int j = 0; j < R; ++j) {
+                if (split) {
+                    acc[i][j].x += part[i][j].x;
+                    acc[i][j].y += part[i][j].y;
+                } else {
+                    acc[i][j] = part[i][j];
+                }
+            }
         __syncthreads();
     }
 }

@@ -175,7 +175,7 @@ tnsim_status check_params(const tnsim_params* p) {
 // that a state needs: under a process-wide cap, and beyond an eighth of the device's
 // memory over all states.
 void alloc_preconditioner(tnsim_mps* m) {
-    if (2 * m->capmax < kMixMinCols || 4 * m->capmax > kMixMaxRows || g_dev_cap.load() > 0) return;
+    if (2 * m->capmax <= kPlain64 || 4 * m->capmax > kMixMaxRows || g_dev_cap.load() > 0) return;
     const int64_t bytes = (int64_t)((size_t)m->G * 4 * m->ws_elems * m->esz);
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); return; }

@@ -130,6 +130,20 @@ __device__ __forceinline__ bool qr_active(const GateDesc& d, int m, int n) {
 // column blocks no longer fit in shared memory.
 constexpr int kMixMinCols = 10;
 constexpr int kMixMaxRows = 1024;
+// Complex128 gates of at most this many rows and columns keep one order of operations (plain64
+// in k_jacobi.cu, sums of one run in tile16.cuh): IEEE rotation parameters, norms summed
+// again for every pair inside a block.  What a circuit of small bonds returns can be decided
+// by every single rounding -- an amplitude that is exactly zero is the residue of the
+// roundings, a cutoff through two equal singular values keeps the one that rounding made
+// larger -- and so such results stay what they were.  It costs what the shorter parameters and
+// the preconditioner gained there: 100-qubit gate set 2.3 -> 3.1 ms (6.1 with the parameters
+// in every warp), ten-qubit circuit 4.4 -> 5.7, 30-qubit gradient 9.7 -> 15.9.  The line lies
+// below 32 x 32, the saturated gate of a random circuit at bond 16, whose flat spectrum has
+// no ties: with it the ten-qubit circuit takes 11.7 ms.
+constexpr int kPlain64 = 30;
+#ifdef __CUDACC__
+__host__ __device__ __forceinline__ bool plain64(int m, int n) { return m <= kPlain64 && n <= kPlain64; }
+#endif
 constexpr double kMixTol = 2e-6;
 // Refinement steps (k_fp64.cu): the largest angle of a pair (a first step of up to 2^-9 was
 // given up by one gate of 180 columns in ~500 for its row sums, and one such gate took 20 ms
