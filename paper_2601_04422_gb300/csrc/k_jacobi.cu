@@ -879,9 +879,9 @@ k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol
     __shared__ __align__(8) uint64_t s_full;
     const uint32_t bar = smem_u32(&s_full);
     const int lane = threadIdx.x & 31;
-    auto mid_arrive = [] { asm volatile("fence.proxy.async.shared::cta;\nbar.arrive 3, %0;" ::"n"(NT + 32) : "memory"); };
-    auto mid_wait = [] { asm volatile("bar.sync 3, %0;" ::"n"(NT + 32) : "memory"); };
-    auto ready = [] { asm volatile("fence.proxy.async.shared::cta;\nbar.sync 4, %0;" ::"n"(NT + 32) : "memory"); };
+    auto mid_arrive = [] { __syncwarp(); asm volatile("fence.proxy.async.shared::cta;\nbar.arrive 3, %0;" ::"n"(NT + 32) : "memory"); };
+    auto mid_wait = [] { __syncwarp(); asm volatile("bar.sync 3, %0;" ::"n"(NT + 32) : "memory"); };
+    auto ready = [] { __syncwarp(); asm volatile("fence.proxy.async.shared::cta;\nbar.sync 4, %0;" ::"n"(NT + 32) : "memory"); };
     for (int g = threadIdx.x; g < n_gates && g < kScanTable; g += blockDim.x)
         s_V[g] = (short)tour_of<BC>(gd[g]).V;
     if (threadIdx.x < 2) s_rot[threadIdx.x] = s_vis[threadIdx.x] = s_last[threadIdx.x] = 0;
@@ -958,6 +958,7 @@ k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol
             int found = 0, fg = -1, frnd = 0, fv = 0, leave = 0;
             for (;;) {
                 if (!reported && __all_sync(0xffffffffu, *((volatile int*)&s_done) == i * NW)) {
+                    __threadfence();   // their part, before block J is read and reported
                     store_J(p ^ 1);
                     report(p ^ 1);
                     reported = true;
@@ -1117,7 +1118,12 @@ k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol
         // a fence waits until the stores have landed: with the next visit in hand, later
         pending = true;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (*((volatile int*)&s_claimed) != i + 1) signal();
+        // one lane's reading for the warp: the prefetching warp writes it meanwhile, and lanes
+        // that read different values would part at signal's __syncwarp and the barrier
+        __syncwarp();
+        int ahead = lane == 0 ? *((volatile int*)&s_claimed) : 0;
+        ahead = __shfl_sync(0xffffffffu, ahead, 0);
+        if (ahead != i + 1) signal();
         ready();
     }
 }
