@@ -1330,7 +1330,8 @@ static cudaError_t launch_cl(const GateDesc* d, int n_gates, int m_max, int n_ma
     if (seats > 8) return cudaSuccess;
     const auto kernel = k_jacobi_cl<T, BC, LP, RPL, MINB, EXT>;
     const size_t smem = sizeof(T) == 4 ? (size_t)3 * BC * LP * RPL * sizeof(C) : (size_t)4 * BC * m_max * sizeof(C);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemLimit limit;
+    cudaError_t e = allow_dynamic_smem((const void*)kernel, limit);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
@@ -1350,7 +1351,6 @@ static cudaError_t launch_cl(const GateDesc* d, int n_gates, int m_max, int n_ma
         // one CTA per SM, where every SM's pipes and schedulers are its own: the cluster
         // scheduler otherwise packs two on an SM beside idle ones
         cfg.dynamicSmemBytes = kOneCta;
-        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOneCta)) != cudaSuccess) return e;
         if ((e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg)) != cudaSuccess) return e;
         if (n_gates > fit) cfg.dynamicSmemBytes = smem;
     }
@@ -1365,7 +1365,8 @@ static cudaError_t launch_pf(const GateDesc* d, int n_gates, int n_lead, int n_m
                              JacobiCtl* ctl, cudaStream_t s, unsigned spin_limit) {
     const auto kernel = k_jacobi_pf<BC, LP, RPL, EXT>;
     const size_t smem = (size_t)3 * BC * LP * RPL * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemLimit limit;
+    cudaError_t e = allow_dynamic_smem((const void*)kernel, limit);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1386,7 +1387,8 @@ static cudaError_t launch_bc(const GateDesc* d, int n_gates, int n_lead, int m_m
     // FP64: two blocks, or all columns of a plain gate
     const size_t smem = sizeof(T) == 8 ? std::max((size_t)2 * BC * m_max, (size_t)std::min(n_max, kPlain64) * std::min(m_max, kPlain64)) * sizeof(C)
                                        : (size_t)2 * BC * LP * RPL * sizeof(C);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemLimit limit;
+    cudaError_t e = allow_dynamic_smem((const void*)kernel, limit);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

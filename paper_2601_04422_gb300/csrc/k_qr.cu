@@ -430,7 +430,8 @@ cudaError_t launch_qr(const GateDesc* d, int n_gates, int m_max, cudaStream_t s)
     using C = typename CT<T>::type;
     // gates with m > kQrMaxRows are not preconditioned (qr_active) and need no panel
     const size_t smem = (size_t)NB * std::min(m_max, kQrMaxRows) * sizeof(C);
-    cudaError_t e = cudaFuncSetAttribute(k_qr<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemLimit limit;
+    cudaError_t e = allow_dynamic_smem((const void*)k_qr<T, NB>, limit);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(QT);

@@ -207,7 +207,8 @@ template <int S>
 static cudaError_t launch_amp_group(void* const* sites, const int* chi, int n, int ranks, int pitch,
                                     const uint8_t* bits, int64_t n_str, double* amps, cudaStream_t s) {
     const size_t smem = (size_t)2 * S * pitch * sizeof(float2) + (size_t)AG_ST * AG_K * 64 * sizeof(float4);
-    cudaError_t e = cudaFuncSetAttribute(k_amp_group<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemLimit limit;
+    cudaError_t e = allow_dynamic_smem((const void*)k_amp_group<S>, limit);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
@@ -244,8 +245,8 @@ cudaError_t launch_amplitudes(void* const* sites, const int* chi, int n_qubits, 
         }
     }
     const size_t smem = 2 * (size_t)chi_cap * sizeof(C);
-    cudaError_t e = cudaFuncSetAttribute(k_amplitudes<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    static SmemLimit limit;
+    cudaError_t e = allow_dynamic_smem((const void*)k_amplitudes<T>, limit);
     if (e != cudaSuccess) return e;
     k_amplitudes<T><<<(unsigned)n_str, 256, smem, s>>>(sites, chi, n_qubits, bits, amps, chi_cap);
     return cudaGetLastError();

@@ -5,7 +5,32 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace tnsim {
+
+// Lets `kernel` be launched with as much dynamic shared memory as a block can have beside its
+// static arrays.  The limit belongs to the function, not to a launch: set to what one launch
+// needs, it refuses another thread's that needs more.  So every call sets the same value.
+// limit: of this kernel, by device (zero at first).
+struct SmemLimit {
+    static constexpr int kDevices = 64;
+    std::atomic<int> bytes[kDevices];
+};
+inline cudaError_t allow_dynamic_smem(const void* kernel, SmemLimit& limit) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    int b = dev < SmemLimit::kDevices ? limit.bytes[dev].load() : 0;
+    if (b == 0) {
+        cudaFuncAttributes a;
+        if ((e = cudaDeviceGetAttribute(&b, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+        if ((e = cudaFuncGetAttributes(&a, kernel)) != cudaSuccess) return e;
+        b -= (int)a.sharedSizeBytes;
+        if (dev < SmemLimit::kDevices) limit.bytes[dev].store(b);
+    }
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+}
 
 // complex element type per arithmetic precision: interleaved (re, im)
 template <typename T> struct CT;
