@@ -377,15 +377,27 @@ __global__ void __launch_bounds__(TILE_THREADS) k_site_adj(const SiteAdjDesc* __
         }
 }
 
+// Steps of a list go to grid.y, which ends at 65535: f(first, count) for parts of a list.
+template <typename F>
+static cudaError_t in_parts(int count, F f) {
+    for (int first = 0; first < count; first += kMaxGridY) {
+        f(first, min(kMaxGridY, count - first));
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 template <typename T>
 cudaError_t launch_transfers(const TransferDesc* list, const TransferDesc& one, int count, int chi_cap,
                              cudaStream_t s) {
-    if (count <= 0) return cudaSuccess;
     constexpr int E = TileOf<typename CT<T>::type>::E;
     const int te = (chi_cap + E - 1) / E, th = (chi_cap + E / 2 - 1) / (E / 2);
-    k_transfer1<T><<<dim3(te * th, count), TILE_THREADS, 0, s>>>(list, one);
-    k_transfer2<T><<<dim3(te * te, count), TILE_THREADS, 0, s>>>(list, one);
-    return cudaGetLastError();
+    return in_parts(count, [&](int first, int part) {
+        const TransferDesc* l = list ? list + first : nullptr;
+        k_transfer1<T><<<dim3(te * th, part), TILE_THREADS, 0, s>>>(l, one);
+        k_transfer2<T><<<dim3(te * te, part), TILE_THREADS, 0, s>>>(l, one);
+    });
 }
 template <typename T>
 cudaError_t launch_transfer(const void* site, const int* chi, int q, const double* op,
@@ -396,12 +408,12 @@ cudaError_t launch_transfer(const void* site, const int* chi, int q, const doubl
 
 template <typename T>
 cudaError_t launch_site_adjs(const TransferDesc* t, const SiteAdjDesc* a, int count, int chi_cap, cudaStream_t s) {
-    if (count <= 0) return cudaSuccess;
     constexpr int E = TileOf<typename CT<T>::type>::E;
     const int te = (chi_cap + E - 1) / E, th = (chi_cap + E / 2 - 1) / (E / 2), t2 = (2 * chi_cap + E - 1) / E;
-    k_transfer1<T><<<dim3(te * th, count), TILE_THREADS, 0, s>>>(t, TransferDesc{});
-    k_site_adj<T><<<dim3(te * t2, count), TILE_THREADS, 0, s>>>(a);
-    return cudaGetLastError();
+    return in_parts(count, [&](int first, int part) {
+        k_transfer1<T><<<dim3(te * th, part), TILE_THREADS, 0, s>>>(t + first, TransferDesc{});
+        k_site_adj<T><<<dim3(te * t2, part), TILE_THREADS, 0, s>>>(a + first);
+    });
 }
 template cudaError_t launch_site_adjs<float>(const TransferDesc*, const SiteAdjDesc*, int, int, cudaStream_t);
 template cudaError_t launch_site_adjs<double>(const TransferDesc*, const SiteAdjDesc*, int, int, cudaStream_t);
@@ -470,7 +482,10 @@ __global__ void k_close_sum(const double* __restrict__ parts, int count, double*
 template <typename T>
 cudaError_t launch_close(const CloseDesc* list, int count, double* parts, double* out, cudaStream_t s) {
     if (count <= 0) return cudaSuccess;
-    k_close<T><<<dim3(CLOSE_PARTS, count), 256, 0, s>>>(list, parts);
+    const cudaError_t e = in_parts(count, [&](int first, int part) {
+        k_close<T><<<dim3(CLOSE_PARTS, part), 256, 0, s>>>(list + first, parts + (size_t)2 * CLOSE_PARTS * first);
+    });
+    if (e != cudaSuccess) return e;
     k_close_sum<<<(2 * count + 127) / 128, 128, 0, s>>>(parts, count, out);
     return cudaGetLastError();
 }

@@ -256,6 +256,7 @@ struct SiteCopies {
 };
 cudaError_t launch_unpack_sites(const SiteCopies& c, cudaStream_t s);
 
+constexpr int kMaxGridY = 65535;   // of grid.y and grid.z
 // read-out
 template <typename T>
 cudaError_t launch_amplitudes(void* const* sites, const int* chi, int n_qubits, int chi_cap,
