@@ -280,14 +280,15 @@ __device__ __forceinline__ int mix_exp(double frob2) {
     return frob2 > 0.0 && !isinf(frob2) ? (ilogb(frob2) >> 1) - 40 : -40;
 }
 
-// One launch, two products of V: X = W V (z < n_gates) and E = I - V^H V (Hermitian: tiles
-// on and above the diagonal, mirrored).  The first CTA of a gate's E also readies its
+// One launch, two products of V: X = W V (the first x_tiles of grid.x) and E = I - V^H V (the
+// rest; Hermitian: tiles on and above the diagonal, mirrored).  The first CTA of a gate's E also readies its
 // record for the FP64 launch: a sweep cap reached in FP32 is no error, a timeout is.
-__global__ void __launch_bounds__(TILE_THREADS) k_mix_first(const GateDesc* __restrict__ gd, int n_gates) {
-    const bool gram = blockIdx.z >= n_gates;
-    const GateDesc& d = gd[gram ? blockIdx.z - n_gates : blockIdx.z];
+__global__ void __launch_bounds__(TILE_THREADS) k_mix_first(const GateDesc* __restrict__ gd, int x_tiles) {
+    const bool gram = blockIdx.x >= x_tiles;
+    const int bx = gram ? blockIdx.x - x_tiles : blockIdx.x;
+    const GateDesc& d = gd[blockIdx.z];
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
-    if (gram && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    if (gram && bx == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
         GateOut* o = d.out;
         if (!o->finished) o->status = 5;
         else if (o->status == 4) o->status = 0;
@@ -297,7 +298,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_first(const GateDesc* __re
         o->claim = 0;
     }
     if (!mix_active(d, m, n)) return;
-    const int i0 = blockIdx.x * T64, j0 = blockIdx.y * T64;
+    const int i0 = bx * T64, j0 = blockIdx.y * T64;
     if (i0 >= (gram ? n : m) || j0 >= n || (gram && i0 > j0)) return;
     const int mt = m + n;
     const float2* V = (const float2*)d.pre + m;
@@ -588,7 +589,7 @@ cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, Jac
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_jacobi_mix(d, n_gates, mt, nm, ctl, s, n_lead, spin_limit);
     if (e != cudaSuccess) return e;
-    k_mix_first<<<dim3(max(tm, tn), tn, 2 * n_gates), TILE_THREADS, 0, s>>>(d, n_gates);
+    k_mix_first<<<dim3(tm + tn, tn, n_gates), TILE_THREADS, 0, s>>>(d, tm);
     k_mix_angle<0><<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_sq<0><<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_corr<<<dim3(tf, tf, n_gates), TILE_THREADS, 0, s>>>(d);
