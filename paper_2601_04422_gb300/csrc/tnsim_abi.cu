@@ -1347,28 +1347,54 @@ tnsim_status tnsim_expect_pauli(tnsim_mps* m, int32_t n_terms, const char* pauli
         l_need = std::max(l_need, a);
         r_need = std::min(r_need, b + 1);
     }
-    // One allocation: the environments L_0..L_n and R_0..R_n, two scratch buffers of the
-    // chains, per term of a batch two running environments and a scratch buffer, and the
-    // lists of the steps.  Terms of a batch advance together, one site per launch.
-    const int batch = (int)std::min<size_t>(n_terms, std::max<size_t>(1, ((size_t)256 << 20) / (4 * env)));
-    size_t off = 0;
-    auto take = [&](size_t bytes) { const size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
-    const size_t o_L = take(env * (n + 1)), o_R = take(env * (n + 1)), o_tmp = take(env * 4), o_ops = take(sizeof(ops));
-    const size_t o_term = take(env * 4 * batch), o_parts = take(sizeof(double) * 2 * CLOSE_PARTS * n_terms);
-    const size_t o_res = take(sizeof(double) * 2 * n_terms);
-    size_t n_steps = 2 * (size_t)n;
-    for (int t0 = 0; t0 < n_terms; t0 += batch) {
-        int len = 0;
-        for (int t = t0; t < std::min(n_terms, t0 + batch); ++t) len = std::max(len, sup[t].b - sup[t].a + 1);
-        n_steps += (size_t)len * batch;
-    }
-    const size_t o_list = take(sizeof(TransferDesc) * n_steps), o_close = take(sizeof(CloseDesc) * n_terms);
+    // Terms of a batch advance together, one site per launch: two running environments and a
+    // scratch buffer per term, and a list of the steps (every site of the longest support for
+    // every term), both bounded; where the device has less room, smaller batches.
+    constexpr size_t kTermBytes = (size_t)256 << 20, kStepBytes = (size_t)64 << 20;
+    struct Batch { int t0, nb, len; };
+    std::vector<Batch> batches;
+    size_t off = 0, o_L = 0, o_R = 0, o_tmp = 0, o_ops = 0, o_term = 0, o_parts = 0, o_res = 0, o_list = 0, o_close = 0;
+    size_t n_list = 0;
+    int nb_max = 1;
     char* base = nullptr;
-    CUDA_TRY(cudaMalloc((void**)&base, off));
+    int limit = (int)std::min<size_t>(n_terms, std::max<size_t>(1, kTermBytes / (4 * env)));
+    for (;;) {
+        batches.clear();
+        size_t n_steps = 0;
+        nb_max = 1;
+        for (int t0 = 0; t0 < n_terms;) {
+            Batch bt{t0, 0, 0};
+            while (bt.nb < limit && t0 + bt.nb < n_terms) {
+                const int len = std::max(bt.len, sup[t0 + bt.nb].b - sup[t0 + bt.nb].a + 1);
+                if (bt.nb > 0 && (size_t)len * (bt.nb + 1) * sizeof(TransferDesc) > kStepBytes) break;
+                bt.len = len;
+                ++bt.nb;
+            }
+            batches.push_back(bt);
+            n_steps = std::max(n_steps, (size_t)bt.len * bt.nb);
+            nb_max = std::max(nb_max, bt.nb);
+            t0 += bt.nb;
+        }
+        // One allocation: the environments L_0..L_n and R_0..R_n, two scratch buffers of the
+        // chains, a batch's terms, sums and lists
+        off = 0;
+        auto take = [&](size_t bytes) { const size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
+        n_list = 2 * (size_t)n + n_steps;
+        o_L = take(env * (n + 1)), o_R = take(env * (n + 1)), o_tmp = take(env * 4), o_ops = take(sizeof(ops));
+        o_term = take(env * 4 * nb_max), o_parts = take(sizeof(double) * 2 * CLOSE_PARTS * nb_max);
+        o_res = take(sizeof(double) * 2 * n_terms);
+        o_list = take(sizeof(TransferDesc) * n_list), o_close = take(sizeof(CloseDesc) * nb_max);
+        const cudaError_t em = cudaMalloc((void**)&base, off);
+        if (em == cudaSuccess) break;
+        if (em != cudaErrorMemoryAllocation || nb_max == 1) CUDA_TRY(em);
+        cudaGetLastError();
+        limit = std::max(1, nb_max / 8);
+    }
     char *d_L = base + o_L, *d_R = base + o_R;
     const double* d_ops = (const double*)(base + o_ops);
-    std::vector<TransferDesc> list(n_steps);
-    std::vector<CloseDesc> closes(n_terms);
+    // the chains' steps, then a batch's
+    std::vector<TransferDesc> list(n_list);
+    std::vector<CloseDesc> closes(nb_max);
     // both chains at once: step i takes L_i to L_{i+1} and R_{n-i} to R_{n-i-1}
     for (int i = 0; i < n; ++i) {
         const int q = n - 1 - i;
@@ -1376,34 +1402,6 @@ tnsim_status tnsim_expect_pauli(tnsim_mps* m, int32_t n_terms, const char* pauli
                        d_L + env * (i + 1), i, 1};
         list[2 * i + 1] = {q >= r_need ? site_ptr(m, q) : nullptr, m->d_chi, d_ops, d_R + env * (q + 1),
                            base + o_tmp + 2 * env, d_R + env * q, q, 0};
-    }
-    std::vector<std::pair<size_t, int>> launches;   // (first step of the list, how many)
-    size_t pos = 2 * (size_t)n;
-    for (int t0 = 0; t0 < n_terms; t0 += batch) {
-        const int nb = std::min(batch, n_terms - t0);
-        int len = 0;
-        for (int t = t0; t < t0 + nb; ++t) len = std::max(len, sup[t].b - sup[t].a + 1);
-        for (int step = 0; step < len; ++step) {
-            for (int t = t0; t < t0 + nb; ++t) {
-                char* buf = base + o_term + env * 4 * (t - t0);
-                const int q = sup[t].a + step;
-                TransferDesc& d = list[pos + (t - t0)];
-                d = {nullptr, m->d_chi, nullptr, nullptr, buf + 2 * env, buf + env * (step & 1), q, 1};
-                if (q > sup[t].b) continue;
-                d.site = site_ptr(m, q);
-                d.op = d_ops + 8 * opi(paulis[(size_t)t * n + q]);
-                d.e_in = step == 0 ? d_L + env * q : buf + env * ((step - 1) & 1);
-            }
-            launches.push_back({pos, nb});
-            pos += nb;
-        }
-        for (int t = t0; t < t0 + nb; ++t) {
-            const int steps = sup[t].b - sup[t].a + 1;
-            const char* buf = base + o_term + env * 4 * (t - t0);
-            closes[t] = {steps > 0 ? (const void*)(buf + env * ((steps - 1) & 1)) : (const void*)(d_L + env * n),
-                         d_R + env * (sup[t].b + 1), m->d_chi, sup[t].b + 1, 0};
-        }
-        launches.push_back({(size_t)t0, -nb});   // close this batch's terms
     }
     cudaStream_t st = m->stream;
     const bool c64 = m->dt == TNSIM_C64;
@@ -1414,30 +1412,52 @@ tnsim_status tnsim_expect_pauli(tnsim_mps* m, int32_t n_terms, const char* pauli
     cudaError_t e = cudaMemcpyAsync(base + o_ops, ops, sizeof(ops), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_L, one.data(), es, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_R + env * n, one.data(), es, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(base + o_list, list.data(), sizeof(TransferDesc) * n_steps, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(base + o_close, closes.data(), sizeof(CloseDesc) * n_terms, cudaMemcpyHostToDevice, st);
-    const TransferDesc* dl = (const TransferDesc*)(base + o_list);
-    const CloseDesc* dc = (const CloseDesc*)(base + o_close);
-    double* parts = (double*)(base + o_parts);
+    TransferDesc* dl = (TransferDesc*)(base + o_list);
+    CloseDesc* dc = (CloseDesc*)(base + o_close);
     double* res = (double*)(base + o_res);
     auto steps = [&](size_t first, int count) {
         return c64 ? launch_transfers<float>(dl + first, TransferDesc{}, count, chi_cap, st)
                    : launch_transfers<double>(dl + first, TransferDesc{}, count, chi_cap, st);
     };
-    for (int i = 0; i < n && e == cudaSuccess; ++i)
-        if (i < l_need || n - 1 - i >= r_need) e = steps(2 * (size_t)i, 2);
-    for (const auto& l : launches) {
+    for (const Batch& bt : batches) {
         if (e != cudaSuccess) break;
-        if (l.second > 0) {
-            e = steps(l.first, l.second);
-        } else {
-            const size_t t0 = l.first;
-            double* p = parts + 2 * CLOSE_PARTS * t0;
-            e = c64 ? launch_close<float>(dc + t0, -l.second, p, res + 2 * t0, st)
-                    : launch_close<double>(dc + t0, -l.second, p, res + 2 * t0, st);
+        const bool first = bt.t0 == 0;
+        // the copies of the batch before have read the host lists
+        if (!first && (e = cudaStreamSynchronize(st)) != cudaSuccess) break;
+        size_t pos = 2 * (size_t)n;
+        for (int step = 0; step < bt.len; ++step, pos += bt.nb) {
+            for (int i = 0; i < bt.nb; ++i) {
+                const int t = bt.t0 + i, q = sup[t].a + step;
+                char* buf = base + o_term + env * 4 * i;
+                TransferDesc& d = list[pos + i];
+                d = {nullptr, m->d_chi, nullptr, nullptr, buf + 2 * env, buf + env * (step & 1), q, 1};
+                if (q > sup[t].b) continue;
+                d.site = site_ptr(m, q);
+                d.op = d_ops + 8 * opi(paulis[(size_t)t * n + q]);
+                d.e_in = step == 0 ? d_L + env * q : buf + env * ((step - 1) & 1);
+            }
         }
+        for (int i = 0; i < bt.nb; ++i) {
+            const Sup& u = sup[bt.t0 + i];
+            const int len = u.b - u.a + 1;
+            const char* buf = base + o_term + env * 4 * i;
+            closes[i] = {len > 0 ? (const void*)(buf + env * ((len - 1) & 1)) : (const void*)(d_L + env * n),
+                         d_R + env * (u.b + 1), m->d_chi, u.b + 1, 0};
+        }
+        const size_t from = first ? 0 : 2 * (size_t)n;
+        if (pos > from)
+            e = cudaMemcpyAsync(dl + from, list.data() + from, sizeof(TransferDesc) * (pos - from), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(dc, closes.data(), sizeof(CloseDesc) * bt.nb, cudaMemcpyHostToDevice, st);
+        if (first)
+            for (int i = 0; i < n && e == cudaSuccess; ++i)
+                if (i < l_need || n - 1 - i >= r_need) e = steps(2 * (size_t)i, 2);
+        for (int step = 0; step < bt.len && e == cudaSuccess; ++step)
+            e = steps(2 * (size_t)n + (size_t)step * bt.nb, bt.nb);
+        double* parts = (double*)(base + o_parts);
+        if (e == cudaSuccess)
+            e = c64 ? launch_close<float>(dc, bt.nb, parts, res + 2 * (size_t)bt.t0, st)
+                    : launch_close<double>(dc, bt.nb, parts, res + 2 * (size_t)bt.t0, st);
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, res, sizeof(double) * 2 * n_terms, cudaMemcpyDeviceToHost, st);
     const cudaError_t es2 = cudaStreamSynchronize(st);   // the host lists are read by the copies

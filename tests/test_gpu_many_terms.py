@@ -54,3 +54,42 @@ def test_gradient_of_many_terms(T):  # noqa: F811
     tol = 40000 * np.finfo(float).eps * np.abs(c).sum()
     assert abs(e - e1) <= tol
     assert np.max(np.abs(np.concatenate([x.reshape(-1) for x in g]) - np.concatenate([x.reshape(-1) for x in g1]))) <= tol
+
+
+def test_memory_of_many_long_terms(T):  # noqa: F811
+    """60000 terms over 100 sites: the steps of all of them at once would be 336 MB.  A batch's
+    are 64 MB, its environments here less than 8 MB, and its sums less than 24; and each term
+    gets its value (a product state again)."""
+    torch = pytest.importorskip("torch")
+    import threading
+    import time
+
+    n, count = 100, 60000
+    rng = np.random.default_rng(6)
+    m = T.MPS(n, dtype=T.TNSIM_C64, chi_max=2)
+    plus = np.array([1, 1]).reshape(1, 2, 1) / np.sqrt(2)
+    zero = np.array([1, 0]).reshape(1, 2, 1)
+    m.import_sites([plus if q % 2 else zero for q in range(n)])
+    # X on |+>, Z on |0>: every value is 1 but those of a term with a Y or a Z on |+> (0)
+    kinds = ["".join("X" if q % 2 else "Z" for q in range(n)), "Z" + "I" * (n - 2) + "X", "Y" + "I" * (n - 2) + "X"]
+    paulis = [kinds[i] for i in rng.integers(0, 3, count)]
+    want = np.array([0.0 if p[0] == "Y" else 1.0 for p in paulis])
+    m.expect_pauli(paulis[:8])
+    free = [torch.cuda.mem_get_info()[0]]
+    stop = threading.Event()
+
+    def watch():
+        while not stop.is_set():
+            free.append(torch.cuda.mem_get_info()[0])
+            time.sleep(2e-4)
+
+    t = threading.Thread(target=watch)
+    t.start()
+    try:
+        got = m.expect_pauli(paulis)
+    finally:
+        stop.set()
+        t.join()
+    m.close()
+    assert np.max(np.abs(got - want)) <= 1e-5
+    assert free[0] - min(free) <= (64 + 8 + 24 + 32) << 20   # and 32 MB of slack for the allocator
