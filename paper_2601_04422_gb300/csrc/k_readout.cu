@@ -421,25 +421,10 @@ template cudaError_t launch_transfers<float>(const TransferDesc*, const Transfer
 template cudaError_t launch_transfers<double>(const TransferDesc*, const TransferDesc&, int, int, cudaStream_t);
 
 // Closure: out = sum_{x,y} E[x,y] Rt[y,x] over one bond, E and Rt both chi x chi.  CLOSE_PARTS
-// CTAs per pair, then one thread per pair adds their sums in order.  complex64 elements are
-// multiplied and summed in double-length FP32 (each product split exactly, about 2^-48
-// relative): FP64 issues once in 64 cycles per scheduler and took 10 of 16 us at chi 64.
-template <typename T> struct ProdAcc;
-template <> struct ProdAcc<float> {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float a, float b) {
-        const float p = a * b, e = fmaf(a, b, -p), t = s + p, z = t - s;
-        c += (s - (t - z)) + (p - z) + e;
-        s = t;
-    }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-template <> struct ProdAcc<double> {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
-    __device__ __forceinline__ double value() const { return s; }
-};
-
+// CTAs per pair, then one thread per pair adds their sums in order.  Products and sums are
+// FP64 for complex64 too: each environment of an unnormalised state may fill FP32's range by
+// itself.  (FP32 pairs are no faster -- 99 terms at chi 64 take 1.06 ms with both -- and give 0
+// or infinity below a squared norm of 1e-31 or above 1e38.)
 template <typename T>
 __global__ void __launch_bounds__(256) k_close(const CloseDesc* __restrict__ list, double* __restrict__ parts) {
     using C = typename CT<T>::type;
@@ -447,16 +432,16 @@ __global__ void __launch_bounds__(256) k_close(const CloseDesc* __restrict__ lis
     const int c = d.chi[d.bond];
     const C* E = (const C*)d.e;
     const C* Rt = (const C*)d.rt;
-    ProdAcc<T> re, im;
+    double a = 0.0, b = 0.0;
     for (int t = blockIdx.x * 256 + threadIdx.x; t < c * c; t += CLOSE_PARTS * 256) {
         const int x = t / c, y = t - x * c;
         const C e = E[t], r = Rt[(size_t)y * c + x];
-        re.add(e.x, r.x);
-        re.add(-e.y, r.y);
-        im.add(e.x, r.y);
-        im.add(e.y, r.x);
+        const double ex = e.x, ey = e.y, rx = r.x, ry = r.y;
+        a = fma(ex, rx, a);
+        a = fma(-ey, ry, a);
+        b = fma(ex, ry, b);
+        b = fma(ey, rx, b);
     }
-    double a = re.value(), b = im.value();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         a += __shfl_xor_sync(0xffffffffu, a, o);
