@@ -39,8 +39,9 @@ __device__ __forceinline__ bool rot_params_fast(float a, float b, float gr, floa
     if (!(a > zthr && b > zthr && g2 > (tol2 * a) * b)) return false;
     const float d = b - a, ad = fabsf(d);
     float h = fmaf(d, d, 4.f * g2);
-    // sqrt(h); beyond the range of h: |d| dominates
-    const float rt = h < 1e38f ? h * rsqrtf(h) : ad;
+    // sqrt(h); where h overflows, its larger part (norms that are equal leave 2 |g|)
+    float rt = h * rsqrtf(h);
+    if (h > 3e38f) rt = fmaxf(ad, 2.f * (g2 * rsqrtf(g2)));
     const float tau = copysignf(__fdividef(2.f, ad + rt), d);
     tg = tau * g2;                                        // the norms become a - t|g|, b + t|g|
     const float t2 = tg * tau;
