@@ -3,7 +3,7 @@
 //
 // GB300 issues FP64 at 1/64 of the FP32 rate, so an FP64 kernel's time is its FP64
 // instruction count over the SMs that it keeps busy, and everything else hides behind
-// it.  The products therefore use 8 x 8 tiles (tile16.cuh): with 64 x 64 tiles one SM per
+// it.  The products therefore use 8 x 8 tiles (tile8.cuh): with 64 x 64 tiles one SM per
 // gate did the work (theta and right site of 5 gates at m = n = 64: 88 + 136 -> 9 + 13 us;
 // of 20 gates at m = 180: 480 + 790 -> 330 + 350 us).
 //
@@ -39,7 +39,7 @@
 #include <float.h>
 
 #include "jacobi_sched.cuh"
-#include "tile16.cuh"
+#include "tile8.cuh"
 #include "tnsim_internal.h"
 
 namespace tnsim {
@@ -48,7 +48,7 @@ namespace {
 
 // ---------------------------------------------------------------------------
 // theta (see k_gemm.cu): 4 l x 4 r per CTA; tile rows (l, c), tile columns (d, r).
-constexpr int T64 = TileOf<double2>::E;   // 8
+constexpr int T64 = TILE_E;
 __global__ void __launch_bounds__(TILE_THREADS) k_theta64(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.z];
     const int q = d.q;
@@ -77,8 +77,8 @@ __global__ void __launch_bounds__(TILE_THREADS) k_theta64(const GateDesc* __rest
     const double2* A = (const double2*)d.siteA;
     const double2* B = (const double2*)d.siteB;
     const int m = 2 * chiL;
-    double2 acc[1][1] = {};
-    tile_product<double2, true, false, false, true, MulAdd>(
+    double2 acc = {};
+    tile_product<double2, true, false, true, MulAdd>(
         chiM,
         [&](int i, int k) {
             const int row = 2 * l0 + i;
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_theta64(const GateDesc* __rest
             return r < chiR ? B[((size_t)k * 2 + j / H) * chiR + r] : make_double2(0.0, 0.0);
         },
         acc);
-    tile_share<double2, false>(S, acc);
+    tile_share(S, acc);
     double2* Wm = (double2*)d.W;
     double2* T0 = (double2*)d.theta0;
     double fro = 0.0;
@@ -134,9 +134,9 @@ __global__ void __launch_bounds__(TILE_THREADS) k_right64(const GateDesc* __rest
     const double2* Wm = (const double2*)d.W;
     const double2* T0 = (const double2*)d.theta0;
     const int lk = d.canon ? *d.lam_k : 0;
-    double2 acc[1][1] = {};
+    double2 acc = {};
     // tile rows: columns of R (they run along its rows in memory); tile columns: rows j
-    tile_product<double2, true, true, false, true, MulAddConj>(
+    tile_product<double2, true, true, true, MulAddConj>(
         m,
         [&](int i, int row) {
             if (c0 + i >= n) return make_double2(0.0, 0.0);
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_right64(const GateDesc* __rest
         [&](int row, int j) { return pj[j] < 0 ? make_double2(0.0, 0.0) : Wm[(size_t)pj[j] * m + row]; }, acc);
     double2* R = (double2*)d.siteB;
     const int jj = tid >> 3, col = c0 + (tid & 7);
-    if (j0 + jj < k && col < n) R[(size_t)(j0 + jj) * n + col] = make_double2(acc[0][0].x * fj[jj], acc[0][0].y * fj[jj]);
+    if (j0 + jj < k && col < n) R[(size_t)(j0 + jj) * n + col] = make_double2(acc.x * fj[jj], acc.y * fj[jj]);
 }
 
 // ---------------------------------------------------------------------------
@@ -205,7 +205,6 @@ __device__ __forceinline__ Df to_df(const double2& v, int e, bool conj) {
     if (conj) { r.y = -r.y; r.yl = -r.yl; }
     return r;
 }
-constexpr int T32 = TileOf<float2>::E;    // 16
 
 // [W; I] in FP32; a gate outside the preconditioner counts as finished in its launch
 __global__ void __launch_bounds__(256) k_mix_build(const GateDesc* __restrict__ gd, JacobiCtl* __restrict__ ctl) {
@@ -309,16 +308,16 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_first(const GateDesc* __re
         const float2 v = V[(size_t)(j0 + c) * mt + k];
         return make_double2((double)v.x, (double)v.y);
     };
-    double2 acc[1][1] = {};
+    double2 acc = {};
     if (!gram) {
-        tile_product<double2, false, true, false, true, MulAdd>(
+        tile_product<double2, false, true, true, MulAdd>(
             n, [&](int r, int k) { return i0 + r < m ? Wm[(size_t)k * m + i0 + r] : make_double2(0.0, 0.0); }, lb, acc);
-        if (i < m && j < n) ((double2*)d.pre_x)[(size_t)j * m + i] = acc[0][0];
+        if (i < m && j < n) ((double2*)d.pre_x)[(size_t)j * m + i] = acc;
         return;
     }
     // the diagonal sums start from -1: they end near 0, and the last roundings are small
-    if (i0 == j0 && ti == tj) acc[0][0].x = -1.0;
-    tile_product<double2, true, true, false, true, MulAdd>(
+    if (i0 == j0 && ti == tj) acc.x = -1.0;
+    tile_product<double2, true, true, true, MulAdd>(
         n,
         [&](int c, int k) {
             if (i0 + c >= n) return make_double2(0.0, 0.0);
@@ -328,7 +327,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_first(const GateDesc* __re
         lb, acc);
     if (i >= n || j >= n) return;
     double2* E = (double2*)d.pre_b;
-    const double re = -acc[0][0].x, im = -acc[0][0].y;
+    const double re = -acc.x, im = -acc.y;
     E[(size_t)j * n + i] = make_double2(re, im);
     if (i0 != j0) E[(size_t)i * n + j] = make_double2(re, -im);
 }
@@ -351,15 +350,15 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_angle(const GateDesc* __re
     const int e = mix_exp(frob2);
     double2 g;
     if constexpr (STEP == 0) {
-        Df acc[1][1] = {};
-        tile_product<Df, true, true, false, false, DfMulAdd<true>>(
+        Df acc = {};
+        tile_product<Df, true, true, false, DfMulAdd<true>>(
             m,
             [&](int c, int k) { return i0 + c < n ? to_df(X[(size_t)(i0 + c) * m + k], e, true) : Df{}; },
             [&](int k, int c) { return j0 + c < n ? to_df(X[(size_t)(j0 + c) * m + k], e, false) : Df{}; }, acc);
-        g = from_df(acc[0][0]);
+        g = from_df(acc);
     } else {
-        double2 acc[1][1] = {};
-        tile_product<double2, true, true, false, true, MulAdd>(
+        double2 acc = {};
+        tile_product<double2, true, true, true, MulAdd>(
             m,
             [&](int c, int k) {
                 if (i0 + c >= n) return make_double2(0.0, 0.0);
@@ -367,7 +366,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_angle(const GateDesc* __re
                 return make_double2(v.x, -v.y);
             },
             [&](int k, int c) { return j0 + c < n ? X[(size_t)(j0 + c) * m + k] : make_double2(0.0, 0.0); }, acc);
-        g = acc[0][0];
+        g = acc;
     }
     // squared norms of the tile's 8 + 8 columns, four threads each
     __shared__ double nrm[2 * T64];
@@ -440,8 +439,8 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_sq(const GateDesc* __restr
         const float2 k = K[t];
         return STEP == 0 || fabsf(k.x) + fabsf(k.y) <= cap ? k : make_float2(0.f, 0.f);
     };
-    Df acc[1][1] = {};
-    tile_product<Df, true, true, false, false, DfMulAdd<false>>(
+    Df acc = {};
+    tile_product<Df, true, true, false, DfMulAdd<false>>(
         n,
         [&](int c, int k) {   // K[i, k] = -conj(K[k, i])
             if (i0 + c >= n) return Df{};
@@ -455,10 +454,10 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_sq(const GateDesc* __restr
         },
         acc);
     const int i = i0 + (threadIdx.x & 7), j = j0 + (threadIdx.x >> 3);
-    const double2 e2 = from_df(acc[0][0]);
+    const double2 e2 = from_df(acc);
     const bool in = i < n && j < n;
     if (STEP == 0) {
-        const float v = fabsf(acc[0][0].x) + fabsf(acc[0][0].y);
+        const float v = fabsf(acc.x) + fabsf(acc.y);
         mix_rows_add(mix_rows(d, n, 0), in ? v : 0.f, kRowUnit0, i, j, n, i0 != j0);
         if (!in) return;
         double2* D = (double2*)d.pre_d;
@@ -480,13 +479,12 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_corr(const GateDesc* __res
     const GateDesc& d = gd[blockIdx.z];
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
     if (!mix_active(d, m, n)) return;
-    const int i0 = blockIdx.x * T32, j0 = blockIdx.y * T32;
+    const int i0 = blockIdx.x * T64, j0 = blockIdx.y * T64;
     if (i0 >= n || j0 >= n) return;
     const double2 *E = (const double2*)d.pre_b, *Q = (const double2*)d.pre_d;
     const float2* K = (const float2*)d.pre;
     const bool skip = mix_rows_above(mix_rows(d, n, 0), n, kRowUnit0, kRefRow0);
-    constexpr int R = TileOf<float2>::R;
-    float2 acc[R][R] = {};
+    float2 acc = {};
     auto herm = [&](const double2* M, float f) {   // f M[i, k] = f conj(M[k, i])
         return [=](int c, int k) {
             if (i0 + c >= n) return make_float2(0.f, 0.f);
@@ -501,10 +499,10 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_corr(const GateDesc* __res
             return make_float2((float)e.x, (float)e.y);
         };
     };
-    tile_product<float2, true, true, false, true, MulAdd>(n, herm(E, 0.375f), cols(E), acc);
+    tile_product<float2, true, true, true, MulAdd>(n, herm(E, 0.375f), cols(E), acc);
     if (!skip) {
-        tile_product<float2, true, true, false, true, MulAdd>(n, herm(Q, -0.125f), cols(Q), acc);
-        tile_product<float2, true, true, false, true, MulAdd>(
+        tile_product<float2, true, true, true, MulAdd>(n, herm(Q, -0.125f), cols(Q), acc);
+        tile_product<float2, true, true, true, MulAdd>(
             n, herm(E, 0.5f),
             [&](int k, int c) {
                 if (j0 + c >= n) return make_float2(0.f, 0.f);
@@ -515,27 +513,21 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_corr(const GateDesc* __res
             acc);
     }
     Df* F = mix_bufs(d, 0).F;
-    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
-#pragma unroll
-    for (int jj = 0; jj < R; ++jj)
-#pragma unroll
-        for (int ii = 0; ii < R; ++ii) {
-            const int i = i0 + rx + 8 * ii, j = j0 + cy + 8 * jj;
-            if (i >= n || j >= n) continue;
-            const size_t t = (size_t)j * n + i;
-            double2 f = E[t];
-            if (!skip) {
-                f.x += Q[t].x;
-                f.y += Q[t].y;
-            }
-            f.x = fma(0.5, f.x, (double)acc[ii][jj].x);
-            f.y = fma(0.5, f.y, (double)acc[ii][jj].y);
-            if (!skip) {
-                f.x += (double)K[t].x;
-                f.y += (double)K[t].y;
-            }
-            F[t] = df_of(f.x, f.y);
-        }
+    const int i = i0 + (threadIdx.x & 7), j = j0 + (threadIdx.x >> 3);
+    if (i >= n || j >= n) return;
+    const size_t t = (size_t)j * n + i;
+    double2 f = E[t];
+    if (!skip) {
+        f.x += Q[t].x;
+        f.y += Q[t].y;
+    }
+    f.x = fma(0.5, f.x, (double)acc.x);
+    f.y = fma(0.5, f.y, (double)acc.y);
+    if (!skip) {
+        f.x += (double)K[t].x;
+        f.y += (double)K[t].y;
+    }
+    F[t] = df_of(f.x, f.y);
 }
 
 // dst = src + src F: F is at most 1e-3, so products and sums of FP32 pairs (2^-47) are as
@@ -549,14 +541,14 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_mul(const GateDesc* __rest
     if (i0 >= m || j0 >= n) return;
     const MixBufs b = mix_bufs(d, STEP);
     const int e = mix_exp(d.out->frob2);
-    Df acc[1][1] = {};
-    tile_product<Df, false, true, false, false, DfMulAdd<true>>(
+    Df acc = {};
+    tile_product<Df, false, true, false, DfMulAdd<true>>(
         n, [&](int c, int k) { return i0 + c < m ? to_df(b.src[(size_t)k * m + i0 + c], e, false) : Df{}; },
         [&](int k, int c) { return j0 + c < n ? b.F[(size_t)(j0 + c) * n + k] : Df{}; }, acc);
     const int i = i0 + (threadIdx.x & 7), j = j0 + (threadIdx.x >> 3);
     if (i >= m || j >= n) return;
     const size_t idx = (size_t)j * m + i;
-    const double2 x = b.src[idx], y = from_df(acc[0][0]);
+    const double2 x = b.src[idx], y = from_df(acc);
     const double sc = ldexp(1.0, e);
     b.dst[idx] = make_double2(fma(y.x, sc, x.x), fma(y.y, sc, x.y));
 }
@@ -584,7 +576,7 @@ cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, Jac
     const int mm = m_max < kMixMaxRows ? m_max : kMixMaxRows, nm = n_max < kMixMaxRows ? n_max : kMixMaxRows;
     int bx = (int)(((long long)mt * nm + 1023) / 1024);
     if (bx > 128) bx = 128;
-    const int tn = (nm + T64 - 1) / T64, tm = (mm + T64 - 1) / T64, tf = (nm + T32 - 1) / T32;
+    const int tn = (nm + T64 - 1) / T64, tm = (mm + T64 - 1) / T64;
     k_mix_build<<<dim3(bx, n_gates), 256, 0, s>>>(d, ctl);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_jacobi_mix(d, n_gates, mt, nm, ctl, s, n_lead, spin_limit);
@@ -592,7 +584,7 @@ cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, Jac
     k_mix_first<<<dim3(tm + tn, tn, n_gates), TILE_THREADS, 0, s>>>(d, tm);
     k_mix_angle<0><<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_sq<0><<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
-    k_mix_corr<<<dim3(tf, tf, n_gates), TILE_THREADS, 0, s>>>(d);
+    k_mix_corr<<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_mul<0><<<dim3(tm, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_angle<1><<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_sq<1><<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);

@@ -856,16 +856,16 @@ k_jacobi(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in
 struct VisitInfo {
     float2 *WI, *WJ;             // the two blocks' columns
     GateOut* out;
-    int nI, nJ, m, md;           // their columns (nI = 0: no work, nJ = 0: block I alone), stored rows, rows of the products
+    int nI, nJ, m;               // their columns (nI = 0: no work, nJ = 0: block I alone) and rows
     int intra, single;           // first round of a sweep; a gate of one block
     float tol2, zthr;
     int V, rnd, R, leave;        // visits of a round, round and rounds of a sweep (report); no more visits
 };
-template <int BC, int LP, int RPL, bool EXT>
+template <int BC, int LP, int RPL>
 __global__ void __launch_bounds__(BC * LP + 128, 1)
 k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol_in, int max_sweeps,
             JacobiCtl* __restrict__ ctl, unsigned spin_limit) {
-    using V32 = Visit32<BC, LP, RPL, EXT>;
+    using V32 = Visit32<BC, LP, RPL, false>;
     constexpr int NT = BC * LP, NW = NT / 32;
     constexpr unsigned kPolls = 1u << 24;   // of a wait for this CTA's own copies or threads
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -917,9 +917,9 @@ k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol
                 GateOut* out = q.out;
                 if (s_rot[p]) {
                     atomicAdd(&out->rot_sweep, s_rot[p]);
-                    if (!EXT) atomicAdd(&out->rotations, (unsigned long long)s_rot[p]);
+                    atomicAdd(&out->rotations, (unsigned long long)s_rot[p]);
                 }
-                if (s_vis[p] && !EXT) atomicAdd(&out->visits, (unsigned long long)s_vis[p]);
+                if (s_vis[p]) atomicAdd(&out->visits, (unsigned long long)s_vis[p]);
                 __threadfence();
                 if (atomicAdd(&out->done, 1) + 1 == q.V) {
                     out->done = 0;
@@ -991,7 +991,7 @@ k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol
                 __threadfence();   // order the claim before reading the blocks of the previous round
                 scan0 = fg;
                 const GateDesc& d = gd[fg];
-                const int md = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2], m = EXT ? md + n : md;
+                const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
                 const int nb = (n + BC - 1) / BC, P = nb + (nb & 1), R = nb == 1 ? 1 : P - 1, round = frnd % R;
                 int I = 0, J = -1;
                 if (nb > 1) {
@@ -1000,7 +1000,7 @@ k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol
                     else if (J >= nb) J = -1;
                 }
                 const int nI = J >= 0 || round == 0 ? min(BC, n - I * BC) : 0, nJ = J >= 0 ? min(BC, n - J * BC) : 0;
-                float2* W = EXT ? (float2*)d.pre : (float2*)d.W;
+                float2* W = (float2*)d.W;
                 float2 *WI = W + (size_t)I * BC * m, *WJ = W + (size_t)(J >= 0 ? J : 0) * BC * m;
                 if (nI > 0) {
                     asm volatile("fence.proxy.async;" ::: "memory");
@@ -1017,7 +1017,6 @@ k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol
                     q.nI = nI;
                     q.nJ = nJ;
                     q.m = m;
-                    q.md = md;
                     q.intra = round == 0;
                     q.single = nb == 1;
                     q.V = nb == 1 ? 1 : P / 2;
@@ -1027,12 +1026,7 @@ k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol
                     // tolerances: see k_jacobi
                     const double tol = tol_in > 0.0 ? tol_in : 2.0 * Eps<float>::v;
                     q.tol2 = (float)(tol * tol);
-                    double frob2 = d.out->frob2;
-                    if (EXT) {
-                        const double f = mix_scale(frob2);
-                        frob2 *= f * f;
-                    }
-                    q.zthr = (float)(Eps<float>::v * Eps<float>::v * (double)max(md, n) * frob2);
+                    q.zthr = (float)(Eps<float>::v * Eps<float>::v * (double)max(m, n) * d.out->frob2);
                 }
                 if (nI > 0) {
                     if (!__all_sync(0xffffffffu, mbar_wait(bar, phase, kPolls))) {
@@ -1079,7 +1073,7 @@ k_jacobi_pf(const GateDesc* __restrict__ gd, int n_gates, int n_lead, double tol
             if (pending) signal();
             return;
         }
-        const V32 vis(xs, xs + (size_t)(1 + p) * V32::BLOCK, q.md);
+        const V32 vis(xs, xs + (size_t)(1 + p) * V32::BLOCK, q.m);
         int my_rot = 0, my_vis = 0;
         if (q.nJ > 0) {
             const int nI = q.nI, nJ = q.nJ;
@@ -1360,10 +1354,10 @@ static cudaError_t launch_cl(const GateDesc* d, int n_gates, int m_max, int n_ma
     return cudaLaunchKernelEx(&cfg, kernel, d, tol, max_sweeps < 1 ? 1 : max_sweeps);
 }
 
-template <int BC, int LP, int RPL, bool EXT = false>
+template <int BC, int LP, int RPL>
 static cudaError_t launch_pf(const GateDesc* d, int n_gates, int n_lead, int n_max, double tol, int max_sweeps,
                              JacobiCtl* ctl, cudaStream_t s, unsigned spin_limit) {
-    const auto kernel = k_jacobi_pf<BC, LP, RPL, EXT>;
+    const auto kernel = k_jacobi_pf<BC, LP, RPL>;
     const size_t smem = (size_t)3 * BC * LP * RPL * sizeof(float2);
     static SmemLimit limit;
     cudaError_t e = allow_dynamic_smem((const void*)kernel, limit);

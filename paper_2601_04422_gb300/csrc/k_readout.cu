@@ -12,7 +12,7 @@
 //  k_close*     : sum_{x,y} E[x,y] Rt[y,x] of many (E, R) pairs.
 #include <cooperative_groups.h>
 
-#include "tile16.cuh"
+#include "tile8.cuh"
 #include "tnsim_internal.h"
 
 namespace cg = cooperative_groups;
@@ -267,7 +267,7 @@ cudaError_t launch_amplitudes(void* const* sites, const int* chi, int n_qubits, 
 template <typename T>
 __global__ void __launch_bounds__(TILE_THREADS) k_transfer1(const TransferDesc* __restrict__ list, TransferDesc one) {
     using C = typename CT<T>::type;
-    constexpr int E = TileOf<C>::E, R = TileOf<C>::R, H = E / 2;
+    constexpr int E = TILE_E, H = E / 2;
     const TransferDesc& d = list ? list[blockIdx.y] : one;
     if (!d.site) return;
     const int cl = d.chi[d.q], cr = d.chi[d.q + 1];
@@ -277,9 +277,9 @@ __global__ void __launch_bounds__(TILE_THREADS) k_transfer1(const TransferDesc* 
     if (x0 >= nx) return;
     const C* site = (const C*)d.site;
     const C* env = (const C*)d.e_in;
-    C acc[R][R] = {};
+    C acc = {};
     if (d.left)
-        tile_product<C, true, false, false, false, MulAdd>(
+        tile_product<C, true, false, false, MulAdd>(
             K, [&](int i, int k) { return x0 + i < cl ? env[(size_t)(x0 + i) * cl + k] : C{}; },
             [&](int k, int j) {
                 const int b = h0 + j % H;
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_transfer1(const TransferDesc* 
             },
             acc);
     else
-        tile_product<C, true, false, false, false, MulAdd>(
+        tile_product<C, true, false, false, MulAdd>(
             K,
             [&](int i, int k) {
                 const int y = h0 + i % H;
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_transfer1(const TransferDesc* 
             },
             [&](int k, int j) { return x0 + j < cr ? env[(size_t)k * cr + x0 + j] : C{}; }, acc);
     __shared__ C S[E][E + 1];
-    tile_share<C, false>(S, acc);
+    tile_share(S, acc);
     C o[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) { o[i].x = (T)d.op[2 * i]; o[i].y = (T)d.op[2 * i + 1]; }
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_transfer1(const TransferDesc* 
 template <typename T>
 __global__ void __launch_bounds__(TILE_THREADS) k_transfer2(const TransferDesc* __restrict__ list, TransferDesc one) {
     using C = typename CT<T>::type;
-    constexpr int TE = TileOf<C>::E, R = TileOf<C>::R;
+    constexpr int TE = TILE_E;
     const TransferDesc& d = list ? list[blockIdx.y] : one;
     if (!d.site) return;
     const int cl = d.chi[d.q], cr = d.chi[d.q + 1];
@@ -327,54 +327,42 @@ __global__ void __launch_bounds__(TILE_THREADS) k_transfer2(const TransferDesc* 
     if (i0 >= M) return;
     const C* A = (const C*)d.site;
     const C* w = (const C*)d.tmp;
-    C acc[R][R] = {};
+    C acc = {};
     if (d.left)
-        tile_product<C, false, false, false, false, ConjMulAdd>(
+        tile_product<C, false, false, false, ConjMulAdd>(
             K, [&](int i, int k) { return i0 + i < M ? A[(size_t)k * cr + i0 + i] : C{}; },
             [&](int k, int j) { return j0 + j < M ? w[(size_t)k * cr + j0 + j] : C{}; }, acc);
     else
-        tile_product<C, true, true, false, false, MulAddConj>(
+        tile_product<C, true, true, false, MulAddConj>(
             K, [&](int i, int k) { return i0 + i < M ? w[(size_t)(i0 + i) * K + k] : C{}; },
             [&](int k, int j) { return j0 + j < M ? A[(size_t)(2 * (j0 + j) + (k & 1)) * cr + (k >> 1)] : C{}; }, acc);
     C* out = (C*)d.e_out;
-    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
-#pragma unroll
-    for (int i = 0; i < R; ++i)
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-            const int r = i0 + rx + 8 * i, c = j0 + cy + 8 * j;
-            if (r < M && c < M) out[(size_t)r * M + c] = acc[i][j];
-        }
+    const int r = i0 + (threadIdx.x & 7), c = j0 + (threadIdx.x >> 3);
+    if (r < M && c < M) out[(size_t)r * M + c] = acc;
 }
 
 // out[l, p, r] += coef sum_{l'} E[l, l'] w[l', (r, p)]  (E: left environment, bra x ket)
 template <typename T>
 __global__ void __launch_bounds__(TILE_THREADS) k_site_adj(const SiteAdjDesc* __restrict__ list) {
     using C = typename CT<T>::type;
-    constexpr int TE = TileOf<C>::E, R = TileOf<C>::R;
+    constexpr int TE = TILE_E;
     const SiteAdjDesc& d = list[blockIdx.y];
     const int cl = d.chi[d.q], cr = d.chi[d.q + 1], N = 2 * cr;
     const int tn = (N + TE - 1) / TE, i0 = (int)(blockIdx.x / tn) * TE, j0 = (int)(blockIdx.x % tn) * TE;
     if (i0 >= cl) return;
     const C* E = (const C*)d.E;
     const C* w = (const C*)d.w;
-    C acc[R][R] = {};
-    tile_product<C, true, false, false, false, MulAddIm>(
+    C acc = {};
+    tile_product<C, true, false, false, MulAddIm>(
         cl, [&](int i, int k) { return i0 + i < cl ? E[(size_t)(i0 + i) * cl + k] : C{}; },
         [&](int k, int j) { return j0 + j < N ? w[(size_t)k * N + j0 + j] : C{}; }, acc);
     C* out = (C*)d.out;
     const T f = (T)d.coef;
-    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
-#pragma unroll
-    for (int i = 0; i < R; ++i)
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-            const int l = i0 + rx + 8 * i, c = j0 + cy + 8 * j;
-            if (l >= cl || c >= N) continue;
-            C* o = out + ((size_t)l * 2 + (c & 1)) * cr + (c >> 1);
-            o->x += f * acc[i][j].x;
-            o->y += f * acc[i][j].y;
-        }
+    const int l = i0 + (threadIdx.x & 7), c = j0 + (threadIdx.x >> 3);
+    if (l >= cl || c >= N) return;
+    C* o = out + ((size_t)l * 2 + (c & 1)) * cr + (c >> 1);
+    o->x += f * acc.x;
+    o->y += f * acc.y;
 }
 
 // Steps of a list go to grid.y, which ends at 65535: f(first, count) for parts of a list.
@@ -391,7 +379,7 @@ static cudaError_t in_parts(int count, F f) {
 template <typename T>
 cudaError_t launch_transfers(const TransferDesc* list, const TransferDesc& one, int count, int chi_cap,
                              cudaStream_t s) {
-    constexpr int E = TileOf<typename CT<T>::type>::E;
+    constexpr int E = TILE_E;
     const int te = (chi_cap + E - 1) / E, th = (chi_cap + E / 2 - 1) / (E / 2);
     return in_parts(count, [&](int first, int part) {
         const TransferDesc* l = list ? list + first : nullptr;
@@ -408,7 +396,7 @@ cudaError_t launch_transfer(const void* site, const int* chi, int q, const doubl
 
 template <typename T>
 cudaError_t launch_site_adjs(const TransferDesc* t, const SiteAdjDesc* a, int count, int chi_cap, cudaStream_t s) {
-    constexpr int E = TileOf<typename CT<T>::type>::E;
+    constexpr int E = TILE_E;
     const int te = (chi_cap + E - 1) / E, th = (chi_cap + E / 2 - 1) / (E / 2), t2 = (2 * chi_cap + E - 1) / E;
     return in_parts(count, [&](int first, int part) {
         k_transfer1<T><<<dim3(te * th, part), TILE_THREADS, 0, s>>>(t + first, TransferDesc{});

@@ -15,9 +15,8 @@
 
 namespace tnsim {
 
-constexpr int TILE_THREADS = 64;
-// edge, outputs per thread and side, K step
-template <typename C> struct TileOf { static constexpr int E = 8, R = 1, K = sizeof(C) == 8 ? 64 : 16; };
+constexpr int TILE_THREADS = 64, TILE_E = 8;   // threads, edge
+template <typename C> constexpr int TILE_K = sizeof(C) == 8 ? 64 : 16;   // K step
 
 // acc += a b; acc += conj(a) b; acc += a conj(b) -- one fixed order of the roundings
 struct MulAdd {
@@ -49,22 +48,22 @@ struct MulAddConj {
     }
 };
 
-// acc += sum over k < K of OP(la(i, k), lb(k, j)): thread (rx, cy) = (tid % 8, tid / 8)
-// holds rows rx + 8 i (PAIRED: 2 rx + i) and columns cy + 8 j, i, j < R.  la and lb give the
-// operands' elements for tile row i / tile column j (zero outside them); AK / BK: memory
-// runs along k (consecutive threads then load consecutive k).  k ascends; SPLIT sums every
-// K step by itself first (rounding grows with sqrt(16 + K / 16) instead of sqrt(K), for
-// 3 - 6 % more instructions); products of up to kPlain64 terms are one run of sums.
-template <typename C, bool AK, bool BK, bool PAIRED, bool SPLIT, typename OP, typename LA, typename LB>
-__device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[TileOf<C>::R][TileOf<C>::R]) {
-    constexpr int E = TileOf<C>::E, R = TileOf<C>::R, TILE_K = TileOf<C>::K, PER = E * TILE_K / TILE_THREADS;
-    __shared__ C As[TILE_K][E + 1], Bs[TILE_K][E + 1];
+// acc += sum over k < K of OP(la(i, k), lb(k, j)): thread tid holds row tid % 8 and column
+// tid / 8.  la and lb give the operands' elements for tile row i / tile column j (zero
+// outside them); AK / BK: memory runs along k (consecutive threads then load consecutive k).
+// k ascends; SPLIT sums every K step by itself first (rounding of 16-byte elements grows with
+// sqrt(16 + K / 16) instead of sqrt(K), for 3 - 6 % more instructions); products of up to
+// kPlain64 terms are one run of sums.
+template <typename C, bool AK, bool BK, bool SPLIT, typename OP, typename LA, typename LB>
+__device__ __forceinline__ void tile_product(int K, LA la, LB lb, C& acc) {
+    constexpr int E = TILE_E, KS = TILE_K<C>, PER = E * KS / TILE_THREADS;
+    __shared__ C As[KS][E + 1], Bs[KS][E + 1];
     const int tid = threadIdx.x, rx = tid & 7, cy = tid >> 3;
     C na[PER], nb[PER];
     const bool split = SPLIT && K > kPlain64;
     // element e of a K step: (edge index, k) with k running fastest (KF) or slowest
     auto at = [](int e, bool kf, int& i, int& k) {
-        if (kf) { k = e % TILE_K; i = e / TILE_K; }
+        if (kf) { k = e % KS; i = e / KS; }
         else { i = e % E; k = e / E; }
     };
     auto fetch = [&](int k0) {
@@ -80,7 +79,7 @@ __device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[TileO
         }
     };
     fetch(0);
-    for (int k0 = 0; k0 < K; k0 += TILE_K) {
+    for (int k0 = 0; k0 < K; k0 += KS) {
 #pragma unroll
         for (int t = 0; t < PER; ++t) {
             int i, k;
@@ -90,51 +89,26 @@ __device__ __forceinline__ void tile_product(int K, LA la, LB lb, C (&acc)[TileO
             Bs[k][i] = nb[t];
         }
         __syncthreads();
-        if (k0 + TILE_K < K) fetch(k0 + TILE_K);
-        C part[R][R] = {};
-        if (!split)
-#pragma unroll
-            for (int i = 0; i < R; ++i)
-#pragma unroll
-                for (int j = 0; j < R; ++j) part[i][j] = acc[i][j];
-        const int kn = min(TILE_K, K - k0);
+        if (k0 + KS < K) fetch(k0 + KS);
+        C part = {};
+        if (!split) part = acc;
+        const int kn = min(KS, K - k0);
 #pragma unroll 4
-        for (int kk = 0; kk < kn; ++kk) {
-            C a[R], b[R];
-#pragma unroll
-            for (int i = 0; i < R; ++i) {
-                a[i] = As[kk][PAIRED ? R * rx + i : rx + 8 * i];
-                b[i] = Bs[kk][cy + 8 * i];
-            }
-#pragma unroll
-            for (int i = 0; i < R; ++i)
-#pragma unroll
-                for (int j = 0; j < R; ++j) OP::op(part[i][j], a[i], b[j]);
+        for (int kk = 0; kk < kn; ++kk) OP::op(part, As[kk][rx], Bs[kk][cy]);
+        if (split) {
+            acc.x += part.x;
+            acc.y += part.y;
+        } else {
+            acc = part;
         }
-#pragma unroll
-        for (int i = 0; i < R; ++i)
-#pragma unroll
-            for (int j = 0; j < R; ++j) {
-                if (split) {
-                    acc[i][j].x += part[i][j].x;
-                    acc[i][j].y += part[i][j].y;
-                } else {
-                    acc[i][j] = part[i][j];
-                }
-            }
         __syncthreads();
     }
 }
 
 // The tile in shared memory, for outputs that mix entries of several threads.
-template <typename C, bool PAIRED>
-__device__ __forceinline__ void tile_share(C (*S)[TileOf<C>::E + 1], const C (&acc)[TileOf<C>::R][TileOf<C>::R]) {
-    constexpr int R = TileOf<C>::R;
-    const int rx = threadIdx.x & 7, cy = threadIdx.x >> 3;
-#pragma unroll
-    for (int i = 0; i < R; ++i)
-#pragma unroll
-        for (int j = 0; j < R; ++j) S[PAIRED ? R * rx + i : rx + 8 * i][cy + 8 * j] = acc[i][j];
+template <typename C>
+__device__ __forceinline__ void tile_share(C (*S)[TILE_E + 1], const C& acc) {
+    S[threadIdx.x & 7][threadIdx.x >> 3] = acc;
     __syncthreads();
 }
 
