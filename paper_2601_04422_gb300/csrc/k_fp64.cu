@@ -18,7 +18,8 @@
 //   k_mix_first  X = W V and E = I - V^H V in FP64 (V is unitary to ~1e-6 only);
 //   k_mix_angle  K, anti-Hermitian: the angles of the pairs of X's columns;
 //   k_mix_sq     K^2
-//   k_mix_corr   I + F = V's correction to a unitary matrix times K + (I + K^2)^{1/2},
+//   k_mix_r, k_mix_corr
+//                I + F = V's correction to a unitary matrix times K + (I + K^2)^{1/2},
 //                unitary to FP64 rounding;
 //   k_mix_mul    X + X F;
 //   k_mix_angle, k_mix_sq, k_mix_mul: a second refinement, whose angles are so small that
@@ -26,7 +27,8 @@
 // The FP64 Jacobi iteration then starts from W V' with V' unitary: the same SVD to the
 // same tolerance.  It usually only finds that the columns are orthogonal, and rotates the
 // pairs that the steps left out: those of singular values too close for a small angle.  A
-// preconditioner that did not converge only costs sweeps.
+// preconditioner that did not converge only costs sweeps; one whose V is not unitary enough
+// to be corrected (mix_off) is left out.
 // FP64 enters where rounding would reach the result: in X, E and the second K.  The other
 // products are sums of FP32 pairs (48 bits) at a fifth of FP64's time: of small corrections
 // (K, F < 2^-10 of X), or where a few digits do.
@@ -218,6 +220,8 @@ __global__ void __launch_bounds__(256) k_mix_build(const GateDesc* __restrict__ 
         return;
     }
     const int mt = m + n;
+    if (blockIdx.x == 0)
+        for (int t = threadIdx.x; t < kMixRows * n; t += blockDim.x) d.pre_rows[t] = 0;
     const double f = mix_scale(d.out->frob2);
     const double2* Wm = (const double2*)d.W;
     float2* Y = (float2*)d.pre;
@@ -249,12 +253,12 @@ __device__ __forceinline__ MixBufs mix_bufs(const GateDesc& d, int step) {
     if (step == 0) return {(const double2*)d.pre_x, (double2*)d.pre_b, (Df*)d.W};
     return {(const double2*)d.pre_b, (double2*)d.W, (Df*)d.pre_d};
 }
-// Row sums of a step's matrix, in fixed point (the order of the additions does not matter),
-// behind K: they bound its norm.
+// R of the correction (k_mix_r), behind K in the place of V
+__device__ __forceinline__ float2* mix_R(const GateDesc& d, int n) { return (float2*)d.pre + (size_t)n * n; }
+// Row sums of a matrix, in fixed point (the order of the additions does not matter): they
+// bound its norm.  0: K^2 of step 0; 1, 2: K of step 1, all angles and those up to kRefCap2; 3: E.
 constexpr float kRowUnit0 = 0x1p-38f, kRowUnit1 = 0x1p-36f;
-__device__ __forceinline__ unsigned* mix_rows(const GateDesc& d, int n, int step) {
-    return (unsigned*)((float2*)d.pre + (size_t)n * n) + step * n;
-}
+__device__ __forceinline__ unsigned* mix_rows(const GateDesc& d, int n, int which) { return d.pre_rows + which * n; }
 // the tile's elements of size v at (i, j), mirrored at (j, i) off the diagonal tiles
 __device__ __forceinline__ void mix_rows_add(unsigned* rows, float v, float unit, int i, int j, int n, bool mirror) {
     const float top = unit * 0x1p24f;
@@ -272,6 +276,10 @@ __device__ __forceinline__ bool mix_rows_above(const unsigned* rows, int n, floa
     bool over = false;
     for (int i = threadIdx.x; i < n; i += TILE_THREADS) over |= rows[i] > top;
     return __syncthreads_or(over);
+}
+// V too far from unitary for the series of its correction: the gate keeps W as it is
+__device__ __forceinline__ bool mix_off(const GateDesc& d, int n) {
+    return mix_rows_above(mix_rows(d, n, 3), n, kRowUnit1, kRefRowE);
 }
 // exponent that scales |W|_F into [2^40, 2^42): FP32 pairs then hold W's elements to 2^-48
 // of their size down to 2^-115 |W|_F
@@ -325,9 +333,11 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_first(const GateDesc* __re
             return make_double2((double)v.x, -(double)v.y);
         },
         lb, acc);
-    if (i >= n || j >= n) return;
-    double2* E = (double2*)d.pre_b;
     const double re = -acc.x, im = -acc.y;
+    const bool in = i < n && j < n;
+    mix_rows_add(mix_rows(d, n, 3), in ? fabsf((float)re) + fabsf((float)im) : 0.f, kRowUnit1, i, j, n, i0 != j0);
+    if (!in) return;
+    double2* E = (double2*)d.pre_b;
     E[(size_t)j * n + i] = make_double2(re, im);
     if (i0 != j0) E[(size_t)i * n + j] = make_double2(re, -im);
 }
@@ -342,9 +352,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_angle(const GateDesc* __re
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
     if (!mix_active(d, m, n)) return;
     const int i0 = blockIdx.x * T64, j0 = blockIdx.y * T64;
-    if (i0 >= n || j0 >= n || i0 > j0) return;
-    if (STEP == 0 && i0 == 0 && j0 == 0)
-        for (int t = threadIdx.x; t < 3 * n; t += TILE_THREADS) mix_rows(d, n, 0)[t] = 0;
+    if (i0 >= n || j0 >= n || i0 > j0 || mix_off(d, n)) return;
     const double2* X = mix_bufs(d, STEP).src;
     const double frob2 = d.out->frob2;
     const int e = mix_exp(frob2);
@@ -429,7 +437,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_sq(const GateDesc* __restr
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
     if (!mix_active(d, m, n)) return;
     const int i0 = blockIdx.x * T64, j0 = blockIdx.y * T64;
-    if (i0 >= n || j0 >= n || i0 > j0) return;
+    if (i0 >= n || j0 >= n || i0 > j0 || mix_off(d, n)) return;
     const float2* K = (const float2*)d.pre;
     // step 1: the angles in use, |Re K| + |Im K| at most this
     float cap = 1.f;
@@ -473,46 +481,71 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_sq(const GateDesc* __restr
     }
 }
 
-// Step 0: I + F = (I + E/2 + 3/8 E^2) (I + K + K^2/2 - K^4/8), the second-order products in
-// FP32 (E ~ 1e-6, K < 2^-10); without K where K^2 is too large for K^6 to vanish.
+// Step 0: I + F = (I + C) (I + B'), C = E/2 + 3/8 E^2 + 5/16 E^3 = (I - E)^{-1/2} - I and
+// B' = B - K^4/8 = K + (I + K^2)^{1/2} - I with B = K + K^2/2, without K where K^2 is too
+// large for K^6 to vanish.  F = E/2 + B' + E R with R = 3/8 E + B/2 + E (5/16 E + 3/8 B): two
+// products of E, in FP32 (E ~ 1e-6, K < 2^-10).  Left out: 35/128 E^4, 5/16 E^3 B, E K^4/16.
+// |E|_2 was 2e-6 .. 5e-6 at n = 64 .. 512 and |K|_2 is at most 2.8e-3, so these are below 2e-17;
+// at the largest row sums of E that are admitted (kRefRowE) below 2e-15.
+__device__ __forceinline__ float2 mix_B(const float2& k, const double2& q, bool skip) {
+    return skip ? make_float2(0.f, 0.f) : make_float2(fmaf(0.5f, (float)q.x, k.x), fmaf(0.5f, (float)q.y, k.y));
+}
+// f M[i, k] = f conj(M[k, i]) for rows i0 + c of a Hermitian matrix
+__device__ __forceinline__ float2 mix_herm(const double2* M, float f, int i, int k, int n) {
+    if (i >= n) return make_float2(0.f, 0.f);
+    const double2 e = M[(size_t)i * n + k];
+    return make_float2(f * (float)e.x, -f * (float)e.y);
+}
+__global__ void __launch_bounds__(TILE_THREADS) k_mix_r(const GateDesc* __restrict__ gd) {
+    const GateDesc& d = gd[blockIdx.z];
+    const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
+    if (!mix_active(d, m, n)) return;
+    const int i0 = blockIdx.x * T64, j0 = blockIdx.y * T64;
+    if (i0 >= n || j0 >= n || mix_off(d, n)) return;
+    const double2 *E = (const double2*)d.pre_b, *Q = (const double2*)d.pre_d;
+    const float2* K = (const float2*)d.pre;
+    const bool skip = mix_rows_above(mix_rows(d, n, 0), n, kRowUnit0, kRefRow0);
+    float2 acc = make_float2(0.f, 0.f);
+    tile_product<float2, true, true, true, MulAdd>(
+        n, [&](int c, int k) { return mix_herm(E, 1.f, i0 + c, k, n); },
+        [&](int k, int c) {
+            if (j0 + c >= n) return make_float2(0.f, 0.f);
+            const size_t t = (size_t)(j0 + c) * n + k;
+            const double2 e = E[t];
+            const float2 b = mix_B(K[t], Q[t], skip);
+            return make_float2(fmaf(0.375f, b.x, 0.3125f * (float)e.x), fmaf(0.375f, b.y, 0.3125f * (float)e.y));
+        },
+        acc);
+    const int i = i0 + (threadIdx.x & 7), j = j0 + (threadIdx.x >> 3);
+    if (i >= n || j >= n) return;
+    const size_t t = (size_t)j * n + i;
+    const double2 e = E[t];
+    const float2 b = mix_B(K[t], Q[t], skip);
+    mix_R(d, n)[t] = make_float2(fmaf(0.5f, b.x, fmaf(0.375f, (float)e.x, acc.x)),
+                                 fmaf(0.5f, b.y, fmaf(0.375f, (float)e.y, acc.y)));
+}
 __global__ void __launch_bounds__(TILE_THREADS) k_mix_corr(const GateDesc* __restrict__ gd) {
     const GateDesc& d = gd[blockIdx.z];
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
     if (!mix_active(d, m, n)) return;
     const int i0 = blockIdx.x * T64, j0 = blockIdx.y * T64;
-    if (i0 >= n || j0 >= n) return;
+    if (i0 >= n || j0 >= n || mix_off(d, n)) return;
     const double2 *E = (const double2*)d.pre_b, *Q = (const double2*)d.pre_d;
-    const float2* K = (const float2*)d.pre;
+    const float2 *K = (const float2*)d.pre, *Rm = mix_R(d, n);
     const bool skip = mix_rows_above(mix_rows(d, n, 0), n, kRowUnit0, kRefRow0);
-    float2 acc = {};
-    auto herm = [&](const double2* M, float f) {   // f M[i, k] = f conj(M[k, i])
-        return [=](int c, int k) {
-            if (i0 + c >= n) return make_float2(0.f, 0.f);
-            const double2 e = M[(size_t)(i0 + c) * n + k];
-            return make_float2(f * (float)e.x, -f * (float)e.y);
-        };
-    };
-    auto cols = [&](const double2* M) {
-        return [=](int k, int c) {
-            if (j0 + c >= n) return make_float2(0.f, 0.f);
-            const double2 e = M[(size_t)(j0 + c) * n + k];
-            return make_float2((float)e.x, (float)e.y);
-        };
-    };
-    tile_product<float2, true, true, true, MulAdd>(n, herm(E, 0.375f), cols(E), acc);
-    if (!skip) {
-        tile_product<float2, true, true, true, MulAdd>(n, herm(Q, -0.125f), cols(Q), acc);
+    float2 acc = make_float2(0.f, 0.f);
+    tile_product<float2, true, true, true, MulAdd>(
+        n, [&](int c, int k) { return mix_herm(E, 1.f, i0 + c, k, n); },
+        [&](int k, int c) { return j0 + c < n ? Rm[(size_t)(j0 + c) * n + k] : make_float2(0.f, 0.f); }, acc);
+    if (!skip)
         tile_product<float2, true, true, true, MulAdd>(
-            n, herm(E, 0.5f),
+            n, [&](int c, int k) { return mix_herm(Q, -0.125f, i0 + c, k, n); },
             [&](int k, int c) {
                 if (j0 + c >= n) return make_float2(0.f, 0.f);
-                const size_t t = (size_t)(j0 + c) * n + k;
-                const double2 e = Q[t];
-                return make_float2(fmaf(0.5f, (float)e.x, K[t].x), fmaf(0.5f, (float)e.y, K[t].y));
+                const double2 q = Q[(size_t)(j0 + c) * n + k];
+                return make_float2((float)q.x, (float)q.y);
             },
             acc);
-    }
-    Df* F = mix_bufs(d, 0).F;
     const int i = i0 + (threadIdx.x & 7), j = j0 + (threadIdx.x >> 3);
     if (i >= n || j >= n) return;
     const size_t t = (size_t)j * n + i;
@@ -527,7 +560,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_corr(const GateDesc* __res
         f.x += (double)K[t].x;
         f.y += (double)K[t].y;
     }
-    F[t] = df_of(f.x, f.y);
+    mix_bufs(d, 0).F[t] = df_of(f.x, f.y);
 }
 
 // dst = src + src F: F is at most 1e-3, so products and sums of FP32 pairs (2^-47) are as
@@ -538,7 +571,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_mix_mul(const GateDesc* __rest
     const int m = 2 * d.chi[d.q], n = 2 * d.chi[d.q + 2];
     if (!mix_active(d, m, n)) return;
     const int i0 = blockIdx.x * T64, j0 = blockIdx.y * T64;
-    if (i0 >= m || j0 >= n) return;
+    if (i0 >= m || j0 >= n || mix_off(d, n)) return;
     const MixBufs b = mix_bufs(d, STEP);
     const int e = mix_exp(d.out->frob2);
     Df acc = {};
@@ -584,6 +617,7 @@ cudaError_t launch_mix(const GateDesc* d, int n_gates, int m_max, int n_max, Jac
     k_mix_first<<<dim3(tm + tn, tn, n_gates), TILE_THREADS, 0, s>>>(d, tm);
     k_mix_angle<0><<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_sq<0><<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
+    k_mix_r<<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_corr<<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_mul<0><<<dim3(tm, tn, n_gates), TILE_THREADS, 0, s>>>(d);
     k_mix_angle<1><<<dim3(tn, tn, n_gates), TILE_THREADS, 0, s>>>(d);

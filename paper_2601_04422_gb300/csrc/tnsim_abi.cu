@@ -170,13 +170,18 @@ tnsim_status check_params(const tnsim_params* p) {
     return TNSIM_OK;
 }
 
+// The preconditioner's buffers of one gate: four matrices and row sums.
+size_t pre_slot_bytes(const tnsim_mps* m) {
+    return 4 * m->ws_elems * m->esz + (sizeof(unsigned) * kMixRows * 2 * m->capmax + 255) / 256 * 256;
+}
+
 // The FP32 preconditioner of a complex128 state is optional: a state without its buffers
 // takes more sweeps to the same result.  They are left out where they could take memory
 // that a state needs: under a process-wide cap, and beyond an eighth of the device's
 // memory over all states.
 void alloc_preconditioner(tnsim_mps* m) {
     if (2 * m->capmax <= kPlain64 || 4 * m->capmax > kMixMaxRows || g_dev_cap.load() > 0) return;
-    const int64_t bytes = (int64_t)((size_t)m->G * 4 * m->ws_elems * m->esz);
+    const int64_t bytes = (int64_t)((size_t)m->G * pre_slot_bytes(m));
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); return; }
     if (g_pre_held.fetch_add(bytes) + bytes > (int64_t)(total_b / 8) || bytes > (int64_t)(free_b / 2) ||
@@ -346,9 +351,11 @@ tnsim_status upload_desc(cudaStream_t st, const std::vector<GateJob>& jobs, Gate
         d.qr = qr_force >= 0 ? qr_force : (m->jac_cfg >> 1) & 1;
         d.wait_polls = m->tc_spin;
         if (m->d_pre) {
-            const size_t pb = m->ws_elems * es;   // [theta; I] in FP32: (m + n) n * 8 <= (2 capmax)^2 * 16 bytes
-            char* pre = m->d_pre + (size_t)j.slot * 4 * pb;
+            // [theta; I] in FP32: (m + n) n * 8 <= (2 capmax)^2 * 16 bytes; K and R: 2 n^2 * 8
+            const size_t pb = m->ws_elems * es;
+            char* pre = m->d_pre + (size_t)j.slot * pre_slot_bytes(m);
             d.pre = pre;
+            d.pre_rows = (unsigned*)(pre + 4 * pb);
             d.pre_x = pre + pb;
             d.pre_b = pre + 2 * pb;
             d.pre_d = pre + 3 * pb;

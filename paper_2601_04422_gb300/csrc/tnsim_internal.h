@@ -104,6 +104,7 @@ struct GateDesc {
     // complex128: the buffers of the mixed-precision preconditioner (k_fp64.cu), null = none:
     // [theta; I] in FP32 ((m + n) x n), then a step's angles; three FP64 matrices (m x n or n x n)
     void* pre;
+    unsigned* pre_rows;   // row sums of the preconditioner's matrices (kMixRows x n)
     void* pre_x;
     void* pre_b;
     void* pre_d;
@@ -169,12 +170,16 @@ constexpr int kPlain64 = 30;
 #ifdef __CUDACC__
 __host__ __device__ __forceinline__ bool plain64(int m, int n) { return m <= kPlain64 && n <= kPlain64; }
 #endif
+constexpr int kMixRows = 4;
 constexpr double kMixTol = 2e-6;
 // Refinement steps (k_fp64.cu): the largest angle of a pair (a first step of up to 2^-9 was
 // given up by one gate of 180 columns in ~500 for its row sums, and one such gate took 20 ms
 // of FP64 sweeps; 30 layers of 2^-10: none), the second step's and its fallback, and the largest row sums of |K^2| (first step) and of |K| (second) at which
 // the neglected terms, K^6 / 16 and K^4 / 8, stay below 3e-17.
 constexpr float kRefCap0 = 0x1p-10f, kRefCap1 = 0x1p-14f, kRefCap2 = 0x1p-18f, kRefRow0 = 0x1p-17f, kRefRow1 = 0x1p-13f;
+// and of |E| = |I - V^H V| at which V counts as unitary enough to be corrected; else the gate
+// keeps its columns as they were.  FP32 rotations leave 6e-5 at n = 512.
+constexpr float kRefRowE = 0x1p-13f;
 #ifdef __CUDACC__
 // power of two that brings |theta|_F into [1, 2) in the FP32 copy of theta
 __device__ __forceinline__ double mix_scale(double frob2) {
