@@ -301,10 +301,12 @@ tnsim_status tnsim_set_jacobi_config(tnsim_mps* m, int32_t cfg);
 tnsim_status tnsim_set_wait_limits(tnsim_mps* m, int64_t jacobi_idle_polls, int64_t mbarrier_polls);
 
 /* Process-wide cap on the device memory held by the states of this library (0 = no cap,
- * the default).  complex128 states made under a cap leave out the buffers of the SVD's FP32
- * preconditioner (the same results, more slowly).  tnsim_mps_create computes every device allocation of the new state
+ * the default).  tnsim_mps_create computes every device allocation of the new state
  * before making any, and returns ENOMEM, allocating nothing, when the bytes already held
- * plus the new state's would exceed the cap.  Errors: EINVAL (negative bytes). */
+ * plus the new state's would exceed the cap.  complex128 states made without a cap also
+ * hold buffers of the SVD's FP32 preconditioner (twice their workspace, together at most an
+ * eighth of the device's memory), which are not counted; states made under one leave them
+ * out (results equal to rounding, more slowly).  Errors: EINVAL (negative bytes). */
 tnsim_status tnsim_set_device_memory_cap(int64_t bytes);
 
 /* Device bytes held by the live states of this process (as counted for the cap). */

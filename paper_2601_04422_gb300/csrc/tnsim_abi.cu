@@ -49,7 +49,9 @@ constexpr int kRing = 4;           // pinned staging slots per state
 // Process-wide cap on the device memory that states hold (0 = none) and the bytes held.
 std::atomic<int64_t> g_dev_cap{0};
 std::atomic<int64_t> g_dev_held{0};
-std::atomic<int64_t> g_pre_held{0};   // of these, the preconditioner's buffers
+// bytes of the preconditioner's buffers by device (not among those above)
+constexpr int kPreDevices = 64;
+std::atomic<int64_t> g_pre_held[kPreDevices];
 constexpr int kMaxChi = 512;       // largest supported chi_max
 
 struct Staging {
@@ -95,7 +97,7 @@ struct tnsim_mps {
     int jac_cfg = 0;               // Jacobi launch configuration (tnsim_set_jacobi_config / tnsim_autotune)
     unsigned jac_spin = 0;         // idle polls of the Jacobi kernel before it gives up (0 = default)
     int tc_spin = 0;               // polls of a tensor-core mbarrier wait before it gives up (0 = default)
-    int64_t pre_bytes = 0;         // bytes of d_pre
+    int64_t pre_bytes = 0;         // bytes of d_pre (not in dev_bytes)
     int64_t dev_bytes = 0;         // device bytes held, counted against the process-wide cap
     // tensor-core contraction (complex64 with gemm TF32X3 / BF16X3)
     int tc_mode = -1;              // -1 none, 0 TF32 planes, 1 BF16 planes
@@ -177,23 +179,23 @@ size_t pre_slot_bytes(const tnsim_mps* m) {
 
 // The FP32 preconditioner of a complex128 state is optional: a state without its buffers
 // takes more sweeps to the same result.  They are left out where they could take memory
-// that a state needs: under a process-wide cap, and beyond an eighth of the device's
-// memory over all states.
+// that a state needs: under a process-wide cap (so that they do not count against one that
+// is set later), and beyond an eighth of the device's memory over all its states.
 void alloc_preconditioner(tnsim_mps* m) {
-    if (2 * m->capmax <= kPlain64 || 4 * m->capmax > kMixMaxRows || g_dev_cap.load() > 0) return;
+    if (2 * m->capmax <= kPlain64 || 4 * m->capmax > kMixMaxRows || g_dev_cap.load() > 0 || m->device >= kPreDevices)
+        return;
     const int64_t bytes = (int64_t)((size_t)m->G * pre_slot_bytes(m));
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); return; }
-    if (g_pre_held.fetch_add(bytes) + bytes > (int64_t)(total_b / 8) || bytes > (int64_t)(free_b / 2) ||
+    std::atomic<int64_t>& held = g_pre_held[m->device];
+    if (held.fetch_add(bytes) + bytes > (int64_t)(total_b / 8) || bytes > (int64_t)(free_b / 2) ||
         cudaMalloc((void**)&m->d_pre, (size_t)bytes) != cudaSuccess) {
         cudaGetLastError();
         m->d_pre = nullptr;
-        g_pre_held.fetch_sub(bytes);
+        held.fetch_sub(bytes);
         return;
     }
     m->pre_bytes = bytes;
-    m->dev_bytes += bytes;
-    g_dev_held.fetch_add(bytes);
 }
 
 void free_all(tnsim_mps* m) {
@@ -216,7 +218,7 @@ void free_all(tnsim_mps* m) {
     m->recs.clear();
     if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);
     g_dev_held.fetch_sub(m->dev_bytes);
-    g_pre_held.fetch_sub(m->pre_bytes);
+    if (m->pre_bytes) g_pre_held[m->device].fetch_sub(m->pre_bytes);
     m->dev_bytes = m->pre_bytes = 0;
 }
 
