@@ -1904,24 +1904,35 @@ tnsim_status tnsim_grad(const tnsim_circuit* c, const double* theta, const tnsim
     // per term 2 (len - 1) partials and 4 env, and one w = O A Rt (2 env) per site adjoint of
     // a launch (each launch takes at most one adjoint per site: their order is fixed).
     struct Adj { int q; const char* E; const double* op; const char* rt; double coef; char* out; };
-    const size_t max_scr = (size_t)512 << 20;
-    size_t scr_need = 0;
+    // Where the device has less room: fewer terms of a batch, fewer adjoints of a launch.
+    size_t max_scr = (size_t)512 << 20, scr_need = 0, adj_max = 2 * (size_t)n;
     std::vector<std::pair<size_t, size_t>> batches;
-    for (size_t t0 = 0; t0 < terms.size();) {
-        size_t t1 = t0, need = 0;
-        while (t1 < terms.size()) {
-            const size_t add = env * (2 * (size_t)(terms[t1].b - terms[t1].a) + 4);
-            if (t1 > t0 && need + add > max_scr) break;
-            need += add;
-            ++t1;
+    char* d_tscr = nullptr;
+    for (;;) {
+        batches.clear();
+        scr_need = 0;
+        size_t longest = 0;
+        for (size_t t0 = 0; t0 < terms.size();) {
+            size_t t1 = t0, need = 0;
+            while (t1 < terms.size()) {
+                const size_t add = env * (2 * (size_t)(terms[t1].b - terms[t1].a) + 4);
+                if (t1 > t0 && need + add > max_scr) break;
+                need += add;
+                ++t1;
+            }
+            scr_need = std::max(scr_need, need);
+            longest = std::max(longest, t1 - t0);
+            batches.push_back({t0, t1});
+            t0 = t1;
         }
-        scr_need = std::max(scr_need, need);
-        batches.push_back({t0, t1});
-        t0 = t1;
+        d_tscr = dalloc(scr_need + env * 2 * adj_max + 256);
+        if (d_tscr) break;
+        if (longest <= 1 && adj_max == 1) return fail(TNSIM_ENOMEM, "tnsim_grad: device allocation failed");
+        cudaGetLastError();
+        max_scr = std::min(max_scr, scr_need) / 8;
+        adj_max = std::max<size_t>(1, adj_max / 8);
     }
-    char* d_tscr = dalloc(scr_need + env * 2 * 2 * (size_t)n + 256);
-    if (!d_tscr) return fail(TNSIM_ENOMEM, "tnsim_grad: device allocation failed");
-    char* d_w = d_tscr + scr_need;             // 2 env for each of 2n site adjoints
+    char* d_w = d_tscr + scr_need;             // 2 env for each site adjoint of a launch
     auto add_adjoints = [&](const std::vector<Adj>& v) {
         // round r: the r-th adjoint of every (site, output)
         std::vector<int> seen(2 * (size_t)n, 0);
@@ -1934,10 +1945,10 @@ tnsim_status tnsim_grad(const tnsim_circuit* c, const double* theta, const tnsim
         for (const auto& r : rounds) {
             // transfer and adjoint lists advance together: the same index in both
             while (al.size() < tl.size()) al.push_back(SiteAdjDesc{});
-            plan.push_back({1, tl.size(), (int)r.size()});
             for (size_t k = 0; k < r.size(); ++k) {
+                if (k % adj_max == 0) plan.push_back({1, tl.size(), (int)std::min(adj_max, r.size() - k)});
                 const Adj& a = v[r[k]];
-                char* w = d_w + env * 2 * k;
+                char* w = d_w + env * 2 * (k % adj_max);
                 step(a.q, a.op, a.rt, w, nullptr, 0);
                 al.push_back({a.E, w, dchi, a.out + m->site_off[a.q], a.coef, a.q, 0});
             }
