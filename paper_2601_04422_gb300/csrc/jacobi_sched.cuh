@@ -70,7 +70,8 @@ __device__ __forceinline__ double f64_scaled(float x, int e) {
     return __hiloint2double((int)((b & 0x80000000u) | ((unsigned)min(ex, 2046) << 20) | ((b & 0x7fffffu) >> 3)),
                             (int)(b << 29));
 }
-// FP64: the test and a first tau in FP32 on values scaled by the larger norm's power of two;
+// FP64 (gates beyond kPlain64; the others: plain64_sweeps in k_jacobi.cu): the test and a first
+// tau in FP32 on values scaled by the larger norm's power of two;
 // one Newton step for tau (without it a gate took 0.6 sweeps more) and the quantities that
 // make the rotation unitary in FP64: 15 FP64 instructions while t < 2^-10 (where c - 1 is
 // its series), 20 beyond, against about 150 with FP64 square roots and divisions.

@@ -33,9 +33,10 @@
 // products are sums of FP32 pairs (48 bits) at a fifth of FP64's time: of small corrections
 // (K, F < 2^-10 of X), or where a few digits do.
 // Measured: the SVD of 20 gates at m = n = 180, 139 ms without it, 29 without refinement
-// (12.2 and 4.7 FP64 sweeps per gate), 9.2 with the products in FP64, 6.2 so (1.5 sweeps,
-// 0.1 % of their pairs rotated; FP32 rotations 2.9, products 2.0, FP64 sweeps 1.1); 4 gates
-// at m = n = 64, 3.2 ms without refinement, 0.8 with.  Singular values 6e-16 (relative)
+// (12.2 and 4.7 FP64 sweeps per gate), 9.2 with the products in FP64, 6.6 so (1.5 sweeps,
+// 0.1 % of their pairs rotated; FP32 rotations 2.9, products 2.1, FP64 sweeps 1.1; the layer's
+// small gates at its ends go with the last); 4 gates at m = n = 64, 3.2 ms without refinement,
+// 0.8 with.  Singular values 6e-16 (relative)
 // from LAPACK's throughout.  A second FP32 pass on the columns of X in place of the
 // refinement left 3.6 sweeps: 20 ms.
 #include <float.h>

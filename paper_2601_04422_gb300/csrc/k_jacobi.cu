@@ -24,7 +24,8 @@
 //
 // Three kernels run this schedule with the same arithmetic: k_jacobi_cl, one cluster per gate,
 // where all gates are resident at once; else k_jacobi, a queue, and beyond 256 rows in FP32
-// k_jacobi_pf, the queue with a prefetching warp.
+// k_jacobi_pf, the queue with a prefetching warp.  complex128 gates of up to kPlain64 rows and
+// columns run all their sweeps in one visit of either kernel (plain64_sweeps below).
 //
 // k_jacobi is persistent: as many CTAs as the SMs hold claim visits of
 // any gate from a device-side queue, so gates of different sizes and all rounds of
@@ -428,7 +429,8 @@ __device__ __forceinline__ void visit64(double2* __restrict__ XI, double2* __res
 // operations: see kPlain64.  A pair's sums are its warp's, four of them in six instead of
 // twenty additions.  The parameters of all 16 pairs are one warp's, two lanes each: of seven
 // divisions two of a pair share an issue slot three times, and the seventh, in the test, is
-// only made within rounding of the limit.
+// only made within rounding of the limit.  Bound by FP64 issue: 30 instructions per pair and
+// step over the schedulers and 75 of the one warp, 64 cycles each.
 // sw: the sweeps done; returns whether the last one still rotated.
 struct Plain64 {
     double val[16][4];   // a, b, gr, gi of the step's pairs (cross pairs: gr, gi)

@@ -150,10 +150,11 @@ __device__ __forceinline__ bool qr_active(const GateDesc& d, int m, int n) {
 }
 #endif
 
-// Mixed-precision preconditioner of the complex128 SVD: gates of fewer columns converge
-// in FP64 within the time of its launches (from 10 columns: ten-qubit circuit 4.4 ms, 30-qubit
-// gradient 10.4, 100-qubit gate set 2.3; from 16: 4.7, 11.9, 2.3; from 8: 4.1, 10.3, 2.6); of more rows (m + n, those of its columns) two
-// column blocks no longer fit in shared memory.
+// Mixed-precision preconditioner of the complex128 SVD: gates of fewer columns converge in
+// FP64 within the time of its launches (16 layers of gates of 10 to 32 columns: 10.4 ms from
+// 10 columns on, 11.9 from 16, 10.3 from 8, where layers of at most 8 columns took 2.6 ms
+// instead of 2.3; measured before the gates of kPlain64 were taken out); of more rows (m + n,
+// those of its columns) two column blocks no longer fit in shared memory.
 constexpr int kMixMinCols = 10;
 constexpr int kMixMaxRows = 1024;
 // Complex128 gates of at most this many rows and columns keep one order of operations (plain64
@@ -174,8 +175,9 @@ constexpr int kMixRows = 4;
 constexpr double kMixTol = 2e-6;
 // Refinement steps (k_fp64.cu): the largest angle of a pair (a first step of up to 2^-9 was
 // given up by one gate of 180 columns in ~500 for its row sums, and one such gate took 20 ms
-// of FP64 sweeps; 30 layers of 2^-10: none), the second step's and its fallback, and the largest row sums of |K^2| (first step) and of |K| (second) at which
-// the neglected terms, K^6 / 16 and K^4 / 8, stay below 3e-17.
+// of FP64 sweeps; 30 layers of 2^-10: none), the second step's and its fallback, and the
+// largest row sums of |K^2| (first step) and of |K| (second) at which the terms left out of
+// the root, K^6 / 16 and K^4 / 8, stay below 3e-17.
 constexpr float kRefCap0 = 0x1p-10f, kRefCap1 = 0x1p-14f, kRefCap2 = 0x1p-18f, kRefRow0 = 0x1p-17f, kRefRow1 = 0x1p-13f;
 // and of |E| = |I - V^H V| at which V counts as unitary enough to be corrected; else the gate
 // keeps its columns as they were.  FP32 rotations leave 6e-5 at n = 512.
