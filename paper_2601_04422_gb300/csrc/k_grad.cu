@@ -344,7 +344,11 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
     double gacc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) gacc[i] = 0.0;
-    for (int i = mid; i < chiL * chiR; i += gn) {
+    // a plain gate's at most 225 elements: 32 a rank in order, so that the sums below are those
+    // of its element's order (an adjoint at a degenerate cut cancels in them; see kPlain64)
+    const int lane = tid & 31, warp = tid >> 5;
+    const int at = sizeof(T) == 8 && plain64(m, n) ? (warp == 0 ? 32 * rank + lane : chiL * chiR) : mid;
+    for (int i = at; i < chiL * chiR; i += gn) {
         const int l = i / chiR, r = i % chiR;
         C tb[4], mm[4];
 #pragma unroll
@@ -370,7 +374,6 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
     }
     // sums of the 32 values over the warp: lane i ends up with value i (31 additions instead
     // of the 160 of 32 separate reductions), then over the warps and the ranks
-    const int lane = tid & 31, warp = tid >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
