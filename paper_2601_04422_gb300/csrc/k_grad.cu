@@ -344,8 +344,9 @@ __global__ void __launch_bounds__(256) k_gate_bwd(const GradGateDesc* __restrict
     double gacc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) gacc[i] = 0.0;
-    // a plain gate's at most 225 elements: 32 a rank in order, so that the sums below are those
-    // of its element's order (an adjoint at a degenerate cut cancels in them; see kPlain64)
+    // a plain gate's at most 225 elements: one per lane, 32 a rank in order, so the sums below are
+    // those of one block of 256 threads (at a degenerate cut they cancel, and their order
+    // shows; see kPlain64)
     const int lane = tid & 31, warp = tid >> 5;
     const int at = sizeof(T) == 8 && plain64(m, n) ? (warp == 0 ? 32 * rank + lane : chiL * chiR) : mid;
     for (int i = at; i < chiL * chiR; i += gn) {
